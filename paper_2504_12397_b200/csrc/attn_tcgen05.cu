@@ -39,6 +39,10 @@ constexpr int kAttnThreads = 384;   // 8 softmax warps, TMA producer for Q and K
 constexpr int kKeysPerTile = 128;   // keys per K/V stage in shared memory
 constexpr int kHalfKeys = 64;       // keys per score / probability tile in tensor memory
 constexpr int kKvStages = 3;
+// Of every 8 pairs of exponentials, the ones taken on the FMA pipe instead of the MUFU.  One in eight: each saves 16 cycles of
+// a scheduler's MUFU but costs 12 instructions, and the softmax warps are close to the issue limit (attention of 8 x (4096
+// + 256): none 149 us, one in eight 139, two 144, three 149).
+constexpr unsigned kPolyPairs = 0x80;
 
 struct AttnArgs {
     const AttnWork *items;
@@ -163,14 +167,6 @@ __device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, ui
         : "memory");
 }
 
-__device__ __forceinline__ void tmem_st_32x16(uint32_t taddr, const uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-          "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-        : "memory");
-}
 __device__ __forceinline__ void tmem_st_32x32(uint32_t taddr, const uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
@@ -219,17 +215,24 @@ __device__ __forceinline__ void add2(float &d0, float &d1, float a0, float a1) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(D), "l"(A));
     asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(d));
 }
-// 2^x for x <= 0 on the FMA pipe: x = n + f with n the nearest integer, a cubic for 2^f on [-0.5, 0.5] (relative
-// error 7.5e-5, below the bf16 rounding of the probabilities), n added to the exponent field
-__device__ __forceinline__ float exp2_poly(float x) {
-    x = fmaxf(x, -125.f);
-    const float magic = 12582912.f;
-    const float xr = x + magic;
-    const float f = x - (xr - magic);
-    float p = fmaf(f, 0.05517113f, 0.24261114f);
-    p = fmaf(p, f, 0.69326111f);
-    p = fmaf(p, f, 0.99992807f);
-    return __uint_as_float(__float_as_uint(p) + (__float_as_uint(xr) << 23));
+// 2^x of two x <= 0 on the FMA pipe: x = n + f with n the nearest integer, a cubic for 2^f on [-0.5, 0.5] (relative
+// error 7.5e-5, below the bf16 rounding of the probabilities), n added to the exponent field; two values per instruction
+__device__ __forceinline__ void exp2_poly2(float &p0, float &p1, float x0, float x1) {
+    x0 = fmaxf(x0, -125.f); x1 = fmaxf(x1, -125.f);
+    uint64_t x, xr, f, p, k;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(x0), "f"(x1));
+    auto pair = [](float c) { uint64_t r; asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(c)); return r; };
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(xr) : "l"(x), "l"(pair(12582912.f)));     // n in the low mantissa bits
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(k) : "l"(xr), "l"(pair(-12582912.f)));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(f) : "l"(k), "l"(pair(-1.f)), "l"(x));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(p) : "l"(f), "l"(pair(0.05517113f)), "l"(pair(0.24261114f)));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(p) : "l"(p), "l"(f), "l"(pair(0.69326111f)));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(p) : "l"(p), "l"(f), "l"(pair(0.99992807f)));
+    uint32_t r0, r1, n0, n1;
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(r0), "=r"(r1) : "l"(p));
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(n0), "=r"(n1) : "l"(xr));
+    p0 = __uint_as_float(r0 + (n0 << 23));
+    p1 = __uint_as_float(r1 + (n1 << 23));
 }
 // 4 x 4 transpose of 16-byte units across the 4 lanes of a quad (l = lane & 3): on entry u[0..3] are the units of
 // this lane's own row; on return u[j] is unit l of the row held by quad lane j.  Every lane of the warp takes part.
@@ -556,78 +559,69 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 tc::tc_fence_before();
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(s_free(g));
-                const bool masked = tbase + kKeysPerTile - 1 > pos;   // tile crosses this row's causal limit
-                bool bump = false;     // the exponent reference moved: O_g and the row sum are rescaled by alpha
-                float alpha = 1.f;
-                float l0 = 0.f, l1 = 0.f;
-                uint32_t pk[kHalfKeys / 2];   // probabilities (bf16 pairs); their row sum in fp32
-                auto row_max = [&]() {
+                const bool masked = __any_sync(0xffffffffu, tbase + kKeysPerTile - 1 > pos);   // crosses some row's causal limit
+                uint32_t pk[kHalfKeys / 2];   // probabilities (bf16 pairs)
+                // probabilities of the scores against the current reference; returns their sum in fp32
+                auto exponentials = [&](auto poly) {
+                    // (a piece that starts at an item's last tile can hold rows that see none of its keys so far)
+                    const float mb = m_ref == -INFINITY ? 0.f : m_ref * a.scale_log2;
+                    float l0 = 0.f, l1 = 0.f;
+#pragma unroll
+                    for (int e = 0; e < kHalfKeys; e += 2) {
+                        float x0, x1, p0, p1;
+                        fma2(x0, x1, __uint_as_float(sv[e]), __uint_as_float(sv[e + 1]), a.scale_log2, -mb);
+                        if (decltype(poly)::value && ((kPolyPairs >> ((e >> 1) & 7)) & 1)) exp2_poly2(p0, p1, x0, x1);
+                        else { p0 = fast_exp2(x0); p1 = fast_exp2(x1); }
+                        add2(l0, l1, p0, p1);
+                        pk[e >> 1] = pack_cvt(p0, p1);
+                    }
+                    return l0 + l1;
+                };
+                // P_g and O_g are still in use by the previous half tile's P V until it has completed
+                auto pv_wait = [&]() {
+                    if (i == 0) return true;
+                    const bool done = __all_sync(0xffffffffu, tc::mbar_wait(pv_done(g), (n_s - 1) & 1, abort_flag));
+                    tc::tc_fence_after();
+                    return done;
+                };
+                // No pass over the scores for their maximum: the exponentials are taken against the current
+                // reference, and only if their sum says that one of them may have left the safe range
+                // (> 2^14; also catches inf / NaN) is the true maximum taken and the half tile redone.  Half tiles
+                // that cross a causal limit and the first one of an item take their maximum first.  The two paths share
+                // no code: merging the registers of the probabilities would cost a move each.
+                bool fast = !masked && i != 0;
+                if (fast) {
+                    const float l = exponentials(std::true_type());
+                    if (__any_sync(0xffffffffu, !(l <= 16384.f))) {
+                        fast = false;
+                    } else {
+                        l_run += l;
+                        if (!pv_wait()) { ok = false; break; }
+                        tmem_st_32x32(p_addr, pk);
+                    }
+                }
+                if (!fast) {
+                    if (masked) {
+                        const int k0 = tbase + (perm ? hh * 8 : hh * kHalfKeys);
+#pragma unroll
+                        for (int e = 0; e < kHalfKeys; ++e)
+                            if (k0 + (perm ? (e >> 3) * 16 + (e & 7) : e) > pos) sv[e] = 0xff800000u;  // -inf
+                    }
                     float m0 = -INFINITY, m1 = -INFINITY;
 #pragma unroll
                     for (int e = 0; e < kHalfKeys; e += 4) {
                         m0 = max3(m0, __uint_as_float(sv[e]), __uint_as_float(sv[e + 1]));
                         m1 = max3(m1, __uint_as_float(sv[e + 2]), __uint_as_float(sv[e + 3]));
                     }
-                    return fmaxf(m0, m1);
-                };
-                auto move_reference = [&](float m_tile) {
-                    alpha = fast_exp2((m_ref - m_tile) * a.scale_log2);
-                    m_ref = m_tile;
-                    l_run *= alpha;
-                    bump = true;
-                };
-                if (masked) {
-                    float m_tile = -INFINITY;
-                    const int k0 = tbase + (perm ? hh * 8 : hh * kHalfKeys);
-#pragma unroll
-                    for (int e = 0; e < kHalfKeys; ++e) {
-                        const int key = k0 + (perm ? (e >> 3) * 16 + (e & 7) : e);
-                        if (key > pos) sv[e] = 0xff800000u;  // -inf
-                        m_tile = fmaxf(m_tile, __uint_as_float(sv[e]));
+                    const float m_tile = fmaxf(m0, m1);
+                    float alpha = 1.f;   // factor of O_g and the row sum when the reference moves
+                    if ((m_tile - m_ref) * a.scale_log2 > 8.f) {
+                        alpha = fast_exp2((m_ref - m_tile) * a.scale_log2);
+                        m_ref = m_tile;
                     }
-                    if ((m_tile - m_ref) * a.scale_log2 > 8.f) move_reference(m_tile);
-                    // (a piece that starts at an item's last tile can hold rows that see none of its keys so far)
-                    const float mb = m_ref == -INFINITY ? 0.f : m_ref * a.scale_log2;
-#pragma unroll
-                    for (int e = 0; e < kHalfKeys; e += 2) {
-                        const float p0 = fast_exp2(fmaf(__uint_as_float(sv[e]), a.scale_log2, -mb));
-                        const float p1 = fast_exp2(fmaf(__uint_as_float(sv[e + 1]), a.scale_log2, -mb));
-                        l0 += p0;
-                        l1 += p1;
-                        pk[e >> 1] = pack_cvt(p0, p1);
-                    }
-                } else {
-                    // No pass over the scores for their maximum: the exponentials are taken against the current
-                    // reference, and only if their sum says that one of them may have left the safe range
-                    // (> 2^14; also catches inf / NaN) is the true maximum taken and the half tile redone.  The
-                    // first half tile of an item has no reference yet and takes its maximum first.
-                    auto exponentials = [&]() {
-                        const float mb = m_ref * a.scale_log2;
-                        l0 = 0.f; l1 = 0.f;
-#pragma unroll
-                        for (int e = 0; e < kHalfKeys; e += 2) {
-                            float x0, x1, p0, p1;
-                            x0 = fmaf(__uint_as_float(sv[e]), a.scale_log2, -mb);
-                            x1 = fmaf(__uint_as_float(sv[e + 1]), a.scale_log2, -mb);
-                            if ((e & 7) == 6) { p0 = exp2_poly(x0); p1 = exp2_poly(x1); }   // a quarter of them on the FMA pipe
-                            else { p0 = fast_exp2(x0); p1 = fast_exp2(x1); }
-                            add2(l0, l1, p0, p1);
-                            pk[e >> 1] = pack_cvt(p0, p1);
-                        }
-                    };
-                    if (m_ref == -INFINITY) move_reference(row_max());
-                    exponentials();
-                    if (!(l0 + l1 <= 16384.f)) {
-                        move_reference(row_max());
-                        exponentials();
-                    }
-                }
-                l_run += l0 + l1;
-                // P_g and O_g are still in use by the previous half tile's P V until it has completed
-                if (i > 0) {
-                    if (!tc::mbar_wait(pv_done(g), (n_s - 1) & 1, abort_flag)) { ok = false; break; }
-                    tc::tc_fence_after();
-                    if (__any_sync(0xffffffffu, bump)) {
+                    l_run = fmaf(l_run, alpha, exponentials(std::false_type()));
+                    if (!pv_wait()) { ok = false; break; }
+                    if (i != 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
                         // O_g holds the earlier products relative to the old reference: scale the rows that moved
 #pragma unroll 1
                         for (int c = 0; c < HD; c += 32) {
@@ -639,9 +633,8 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                             tmem_st_32x32(o_addr + c, v);
                         }
                     }
+                    tmem_st_32x32(p_addr, pk);
                 }
-                tmem_st_32x16(p_addr, reinterpret_cast<uint32_t(&)[16]>(pk[0]));
-                tmem_st_32x16(p_addr + 16, reinterpret_cast<uint32_t(&)[16]>(pk[16]));
                 // V rows of keys at or beyond the item's causal limit are cleared before the tile's first P V uses them
                 // (thread `row` of each group clears key tbase + row)
                 if (tile_begin) kt += (i > 0);   // tile index of this half
