@@ -79,14 +79,17 @@ static alora_status run_layer(alora_ctx *ctx, int layer, const void *hidden, con
     if (!ctx->layers[layer].wqkv) return ALORA_ERR_NO_WEIGHTS;
     BatchArgs b = b_in;
     b.layer = layer;
-    b.few_row = project_is_few_row(ctx, layer, b.T) ? 1 : 0;
+    b.few_row = project_is_few_row(ctx, layer, b.T) ? 1 : 0;   // (n_layers > 1 only where all of them take that route)
     int n = 0, k;
     // The per-token arrays and the projection's lists first; the attention work lists are built beside the
     // projection (the few-row projection launches them between its two kernels, the other routes right after).
-    if ((k = launch_metadata(ctx, b, s, kMetaProjection)) < 0) return ALORA_ERR_UNSUPPORTED; n += k;
+    if (!(b.facts_ready & kMetaProjection)) {
+        if ((k = launch_metadata(ctx, b, s, kMetaProjection)) < 0) return ALORA_ERR_UNSUPPORTED;
+        n += k;
+    }
     bool kv_appended = false;
     const bool rope = ctx->d_rope_inv_freq != nullptr;   // the rotation comes between projection and append
-    ctx->pending_attn_meta = &b;
+    ctx->pending_attn_meta = (b.facts_ready & kMetaAttention) ? nullptr : &b;
     k = launch_project(ctx, layer, hidden, b.T, ctx->d_qkv, s, rope ? nullptr : pool, b.num_pages, &kv_appended);
     const bool attn_meta_pending = ctx->pending_attn_meta != nullptr;
     ctx->pending_attn_meta = nullptr;
@@ -219,7 +222,7 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
             ctx->max_split_items = kSplitItemsPerSm * ctx->sm_count + groups;
             ctx->max_split_rows = 16 * (kSplitItemsPerSm * ctx->sm_count + 4 * groups);
             alloc((void **)&ctx->d_split_items, (size_t)ctx->max_split_items * sizeof(AttnSplitWork));
-            alloc((void **)&ctx->d_req_scratch, (size_t)5 * c.max_requests * 4);
+            alloc((void **)&ctx->d_req_scratch, (size_t)kSplitScratch * c.max_requests * 4);
             alloc((void **)&ctx->d_prefix_groups, (size_t)2 * c.max_requests * 4);
             alloc((void **)&ctx->d_part_o, (size_t)ctx->max_split_rows * d.hd * 4);
             alloc((void **)&ctx->d_part_ml, (size_t)ctx->max_split_rows * 2 * 4);
@@ -237,7 +240,7 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
             const int ksplit = std::max(1, std::min(kb, ctx->sm_count / std::max(n_tiles, 1)));
             alloc((void **)&ctx->d_skinny_part, (size_t)ctx->skinny_max_items * 128 * 256 * 4);
             alloc((void **)&ctx->d_skinny_t, (size_t)ksplit * 128 * std::max(ctx->skinny_p_cap, 1) * 192 * 4);
-            alloc(&ctx->d_skinny_meta, sizeof(FewRowMeta));
+            alloc(&ctx->d_skinny_meta, (size_t)c.n_layers * sizeof(FewRowMeta));
         }
         alloc((void **)&ctx->d_row_delta, std::min<size_t>(Tm, kRowwiseMaxTokens) * d.N * 4);
         const size_t na = (size_t)std::max(1, c.max_adapters);
@@ -664,8 +667,15 @@ alora_status alora_forward_stack(alora_ctx *ctx, int mode, const void *d_hidden_
         }                                                                         \
         n += k;                                                                   \
     } while (0)
+    // The attention lists depend on the batch alone: the first layer builds them for all.  So do the few-row route's
+    // per-token arrays; its adapter facts of all layers are built in the first layer's launch.  (They were rebuilt by
+    // every layer: 63 of 240 us of a layer's decode step of 40 requests in prefix groups.)
+    bool all_few = true;
+    for (int l = 0; l < ctx->cfg.n_layers; ++l) all_few &= project_is_few_row(ctx, l, T);
+    b.n_layers = all_few ? ctx->cfg.n_layers : 1;
     for (int l = 0; l < ctx->cfg.n_layers; ++l) {
         const LayerWeights &lw = ctx->layers[l];
+        if (l > 0) b.facts_ready = kMetaAttention | (all_few ? kMetaProjection : 0);
         ALORA_STEP(launch_rmsnorm(ctx, h, lw.norm_attn, T, ctx->d_act[0], s));
         st = run_layer(ctx, l, ctx->d_act[0], b, h_paged_kv_layers[l], ctx->d_act[1], s);
         if (st != ALORA_OK) return st;

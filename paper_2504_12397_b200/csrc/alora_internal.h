@@ -84,6 +84,7 @@ struct AttnSplitWork {
                     // tokens only, up to each token's own position
 };
 constexpr int32_t kSplitOwnKeys = 0x40000000;
+constexpr int kSplitScratch = 7;       // per-request integers that the builder of the few-row list needs
 constexpr int kSplitItemsPerSm = 16;   // target number of (row tile, key range) pairs per SM
 
 // Few-row projection (batches of at most kFewRowMax rows): what its two kernels need to know about the batch's
@@ -163,7 +164,8 @@ struct alora_ctx {
                                   // [3] few-row attention items, [4] next unclaimed few-row item,
                                   // [5] 1 = the projection takes the row-wise route for this batch,
                                   // [6] key tiles of the attention items that are cut into runs, [7] tiles per run,
-                                  // [8] attention items taken whole (the first ones), [9] key tiles of those
+                                  // [8] attention items taken whole (the first ones), [9] key tiles of those,
+                                  // [10], [11] next unclaimed projection item and blocks done, [12] few-row attention blocks done
     int32_t *d_seg_scratch = nullptr;  // [14*max_requests+5] per-request values and merged row runs of the current batch
     int32_t *d_shrink_tiles = nullptr; // [max_tiles] indices of the row tiles with an adapter
     int32_t *d_t_ready = nullptr;      // [max_tiles] per row tile: epilogue warps that have published t
@@ -178,7 +180,7 @@ struct alora_ctx {
     float *d_attn_part_ml = nullptr;          // [2 * n_sm][2][256] their exponent references and row sums
     // few-row attention (requests with at most small_max_tokens new tokens): split-KV work list and partials
     alora::AttnSplitWork *d_split_items = nullptr;
-    int32_t *d_req_scratch = nullptr;   // [5][max_requests] items per request, item offset, partial-row offset, prefix groups
+    int32_t *d_req_scratch = nullptr;   // [kSplitScratch][max_requests] per-request values of the few-row list's builder
     int32_t *d_prefix_groups = nullptr; // [2][max_requests] per request of the last batch: first request of its prefix
                                         // group, keys the group shares (0: ungrouped)
     float *d_part_o = nullptr, *d_part_ml = nullptr;
@@ -189,7 +191,7 @@ struct alora_ctx {
     // few-row projection (batches of <= 128 rows): K-slice partial products and partial shrink results
     float *d_skinny_part = nullptr;   // [skinny_max_items][128][256] fp32
     float *d_skinny_t = nullptr;      // [slices of the q/k/v projection][128][skinny_p_cap][192] fp32
-    void *d_skinny_meta = nullptr;    // FewRowMeta of the current batch
+    void *d_skinny_meta = nullptr;    // [n_layers] FewRowMeta of the current batch
     const alora::BatchArgs *pending_attn_meta = nullptr;   // run_layer: attention lists still to be built for this batch
     int skinny_max_items = 0, skinny_p_cap = 0;
     void *d_qkv = nullptr;        // [max_tokens][N]
@@ -258,6 +260,8 @@ struct BatchArgs {
     int all_small;  // host-side knowledge that no request has more than small_max_tokens new tokens (decode)
     int layer = -1; // layer whose adapter table the gate is checked against (-1: no check)
     int few_row = 0; // the projection of this batch takes the few-row route: build FewRowMeta instead of row tiles
+    int n_layers = 1; // few-row route: layers from `layer` on whose FewRowMeta is built (a stack call builds all of them at once)
+    int facts_ready = 0; // bits (kMetaProjection, kMetaAttention): built by an earlier layer of the same stack call
 };
 
 // phases: bit 0 = per-token arrays and the projection's lists, bit 1 = the attention work lists.  A launch of

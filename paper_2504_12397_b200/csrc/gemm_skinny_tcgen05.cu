@@ -481,10 +481,10 @@ bool skinny_route(const alora_ctx *ctx, int T, int N, int K, bool lora, int Nq, 
 }
 
 // x[T][K] (T <= 128) times W[N][K]^T.  `lora`: the layer's adapter table, its B slab and its A-row tensor map (box of
-// 16 rows), or nullptr for a plain dense projection.  Returns kernels launched, or -1.
+// 16 rows) and `layer`, whose adapter facts are used, or nullptr for a plain dense projection.  Returns kernels launched, or -1.
 int launch_skinny_tc(alora_ctx *ctx, const void *x, const CUtensorMap &tmW, const CUtensorMap *tmA16,
                      const AdapterDev *adapters, const void *b_all, int T, int K, int N, int Nq, int Nkv, void *out,
-                     const void *residual, void *kv_pool, int num_pages, cudaStream_t s) {
+                     const void *residual, void *kv_pool, int num_pages, int layer, cudaStream_t s) {
     static bool attr_set[64] = {};
     const int dev = ctx->cfg.device;
     int extra_launches = 0;
@@ -509,7 +509,7 @@ int launch_skinny_tc(alora_ctx *ctx, const void *x, const CUtensorMap &tmW, cons
     if (a.n_stages < 2) return -1;
     a.part = ctx->d_skinny_part; a.t_part = ctx->d_skinny_t; a.p_cap = p_cap;
     a.row_adapter = lora ? ctx->d_row_adapter : nullptr;
-    a.meta = lora ? (const FewRowMeta *)ctx->d_skinny_meta : nullptr;
+    a.meta = lora ? (const FewRowMeta *)ctx->d_skinny_meta + layer : nullptr;
     a.max_adapters = ctx->cfg.max_adapters; a.status = ctx->d_status;
     const size_t smem = (size_t)a.n_stages * a.stage_bytes + 1024 + 256;
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {

@@ -512,7 +512,7 @@ int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T,
 bool skinny_route(const alora_ctx *ctx, int T, int N, int K, bool lora, int Nq, int Nkv);   // gemm_skinny_tcgen05.cu
 int launch_skinny_tc(alora_ctx *ctx, const void *x, const CUtensorMap &tmW, const CUtensorMap *tmA16,
                      const AdapterDev *adapters, const void *b_all, int T, int K, int N, int Nq, int Nkv, void *out,
-                     const void *residual, void *kv_pool, int num_pages, cudaStream_t s);
+                     const void *residual, void *kv_pool, int num_pages, int layer, cudaStream_t s);
 
 // Whether the q/k/v projection of a batch of T rows on this layer takes the few-row route (the batch-metadata step
 // then prepares that route's adapter facts instead of row tiles).
@@ -533,7 +533,7 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, void
         const AdapterDev *ads = ctx->d_adapters + (size_t)layer * ctx->cfg.max_adapters;
         return launch_skinny_tc(ctx, hidden, lm.wqkv[1], have_adapters ? &lm.a_all16 : nullptr,
                                 have_adapters ? ads : nullptr, ctx->tc_b_all[layer], T, d.H, d.N, d.Nq, d.Nkv, qkv, nullptr,
-                                kv_pool, num_pages, s);
+                                kv_pool, num_pages, layer, s);
     }
     if (ctx->tc_maps[layer].pair_ok) {   // many rows: two row tiles per block, 192-wide column tiles
         ProfScope prof(ctx, KK_PROJECT, s);
@@ -614,7 +614,7 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
     if (skinny_route(ctx, T, N, K, false, N, 0)) {
         CUtensorMap tmW256;
         if (!make_tensor_map_bf16(&tmW256, W, N, K, K, 256)) return -1;
-        return launch_skinny_tc(ctx, x, tmW256, nullptr, nullptr, nullptr, T, K, N, N, 0, y, residual, nullptr, 0, s);
+        return launch_skinny_tc(ctx, x, tmW256, nullptr, nullptr, nullptr, T, K, N, N, 0, y, residual, nullptr, 0, 0, s);
     }
     {
         const int r = launch_linear256_tc(ctx, x, W, T, K, N, y, residual, s);   // many rows: 256 x 256 tiles

@@ -27,7 +27,7 @@ __device__ __forceinline__ int find_request(const int32_t *qsl, int R, int t) {
 // page * page_size + position % page_size.  Findings (inconsistent positions, page id out of
 // range, adapter id out of range, an open gate on an adapter that was never registered on the layer) go
 // to the status word; the row then gets adapter -1 / slot -1 so that later kernels skip it.
-__device__ __forceinline__ void metadata_tokens(const int32_t *__restrict__ positions,
+__device__ __forceinline__ int metadata_token(int t, const int32_t *__restrict__ positions,
                                       const int32_t *__restrict__ a_req,
                                       const int32_t *__restrict__ adapter_ids,
                                       const int32_t *__restrict__ qsl, const int32_t *__restrict__ seq_lens,
@@ -36,8 +36,7 @@ __device__ __forceinline__ void metadata_tokens(const int32_t *__restrict__ posi
                                       int32_t *__restrict__ token_req, int32_t *__restrict__ row_adapter,
                                       int32_t *__restrict__ slot_map, const AdapterDev *__restrict__ adapters,
                                       int32_t *status) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
+    if (t >= T) return -1;
     int r = find_request(qsl, R, t);
     int p = positions[t];
     // positions of a request are consecutive and end at seq_len - 1
@@ -53,7 +52,8 @@ __device__ __forceinline__ void metadata_tokens(const int32_t *__restrict__ posi
         if (k >= 0 && adapters != nullptr && adapters[k].rank == 0) { report(status, ALORA_ERR_NO_WEIGHTS); k = -1; }
     }
     if (token_req) token_req[t] = r;
-    if (row_adapter) row_adapter[t] = ok ? k : -1;
+    k = ok ? k : -1;
+    if (row_adapter) row_adapter[t] = k;
     if (slot_map) {
         int slot = -1;
         if (ok && block_tables != nullptr) {
@@ -68,6 +68,7 @@ __device__ __forceinline__ void metadata_tokens(const int32_t *__restrict__ posi
         }
         slot_map[t] = slot;
     }
+    return k;
 }
 
 // Row tiles of the projection.  Each request contributes up to two runs of rows: its gated-off
@@ -325,18 +326,6 @@ __device__ __forceinline__ void metadata_attn_items(const int32_t *__restrict__ 
     }
 }
 
-// Work list of the few-row attention kernel: requests with 1 .. small_max new tokens.  Their score rows
-// (token, query head of the group) are cut into blocks of 16 * mt rows (mt = 1, 2 or 4 tiles, the
-// smallest that holds all rows, else 4), and the keys 0 .. causal limit of each block into ranges of
-// at most `chunk` 64-key units (see the choice of `chunk` below; at most kSplitItemsPerSm ranges per SM).
-// The ranges of one (block, KV head) are consecutive items.
-__device__ __forceinline__ void small_block_shape(int n_new, int G, int &mt, int &tok_per_blk, int &nblk) {
-    const int rows = n_new * G;
-    mt = rows <= 16 ? 1 : (rows <= 32 ? 2 : 4);
-    tok_per_blk = 16 * mt / G;
-    nblk = (n_new + tok_per_blk - 1) / tok_per_blk;
-}
-
 // Requests that read one shared prefix cache (several adapters invoked on the same conversation: their block tables
 // start with the same physical pages).  Neighbouring requests of the few-row route are put into one PREFIX GROUP when
 // they have leading pages in common, so that the attention reads those pages once for all of them:
@@ -354,8 +343,8 @@ __device__ __forceinline__ void metadata_prefix_groups(const int32_t *__restrict
                                                        int page_size, int G, int small_max,
                                                        int32_t *__restrict__ grp_first, int32_t *__restrict__ grp_shared) {
     // common(r) for all pairs.  First the pairs that can share at all (both on this route, same first page): most
-    // pairs of unrelated requests end here.  Then, pair after pair, all threads compare the table entries below the
-    // pair's limit at once and keep the smallest mismatching index; no thread waits for another pair's loads.
+    // pairs of unrelated requests end here.  Then a warp per pair compares the table entries below the pair's limit,
+    // 128 at a time with all loads in flight, up to the first mismatch.
     for (int r = threadIdx.x; r < R; r += blockDim.x) {
         int lim = 0;
         if (r > 0) {
@@ -369,12 +358,21 @@ __device__ __forceinline__ void metadata_prefix_groups(const int32_t *__restrict
         grp_shared[r] = max(lim, 0);   // for now: the first mismatching entry found so far (none yet)
     }
     __syncthreads();
-    for (int r = 1; r < R; ++r) {
-        const int lim = grp_first[r];
+    for (int r = 1 + (int)(threadIdx.x >> 5); r < R; r += (int)(blockDim.x >> 5)) {
+        const int lim = grp_first[r], lane = threadIdx.x & 31;
         if (lim <= 1) continue;
         const int32_t *ta = block_tables + (size_t)(r - 1) * max_blocks, *tb = block_tables + (size_t)r * max_blocks;
-        for (int b = 1 + (int)threadIdx.x; b < lim; b += blockDim.x)
-            if (ta[b] != tb[b]) atomicMin(&grp_shared[r], b);
+        int first = lim;   // first mismatching entry
+        for (int b0 = 1; b0 < lim && first == lim; b0 += 128) {
+            int mine = lim;
+#pragma unroll
+            for (int u = 3; u >= 0; --u) {
+                const int b = b0 + 32 * u + lane;
+                if (b < lim && ta[b] != tb[b]) mine = b;
+            }
+            first = __reduce_min_sync(0xffffffffu, mine);
+        }
+        if (lane == 0) grp_shared[r] = first;
     }
     __syncthreads();
     // keys in common with the left neighbour; most batches have no pair that shares enough: then nobody is grouped and
@@ -418,87 +416,88 @@ __device__ __forceinline__ void metadata_prefix_groups(const int32_t *__restrict
     __syncthreads();
 }
 
-// Work list of the few-row attention kernel.  A STREAM is one block of score rows with the keys it reads: for an
-// ungrouped request its blocks of up to 16 * mt rows over keys 0 .. causal limit; for a prefix group the stacked rows
-// of all members, over the shared prefix (read once, nothing masked) followed by every member's own keys beyond it
-// (masked so that only that member's rows see them).  A stream's keys are cut into ranges of at most `chunk` 64-key
-// units; the ranges of one (stream, KV head) are consecutive items and are merged by whichever block finishes last.
+// Work list of the few-row attention kernel: requests with 1 .. small_max new tokens (at most 16 score rows (token, query
+// head of the group) per KV head).  A STREAM is one block of score rows with the keys it reads: for an ungrouped
+// request its rows over keys 0 .. causal limit; for a prefix group the stacked rows of all members (16 * mt, mt = 1, 2
+// or 4), over the shared prefix (read once, nothing masked) followed by every member's own keys beyond it (masked so
+// that only that member's rows see them).  A stream's keys are cut into ranges of at most `chunk` 64-key units; the
+// ranges of one (stream, KV head) are consecutive items and are merged by whichever block finishes last.
 // A group is owned by its first request: that request accounts for all of the group's items.
-struct GroupShape {
-    int n_members, n_tok, shared, mt;
-};
-__device__ __forceinline__ GroupShape group_shape(const int32_t *qsl, const int32_t *grp_first, const int32_t *grp_shared,
-                                                  int R, int f, int G) {
-    GroupShape g;
-    g.shared = grp_shared[f];
-    int e = f + 1;
-    while (e < R && grp_first[e] == f) ++e;
-    g.n_members = e - f;
-    g.n_tok = qsl[e] - qsl[f];
-    const int rows = g.n_tok * G;
-    g.mt = rows <= 16 ? 1 : (rows <= 32 ? 2 : 4);
-    return g;
-}
-// ranges of request r's share of the list for a given range length; also the 64-key units (weighted by row tiles)
-__device__ __forceinline__ void request_ranges(const int32_t *qsl, const int32_t *seq_lens, const int32_t *grp_first,
-                                               const int32_t *grp_shared, int R, int r, int G, int small_max, int chunk,
-                                               int &n_ranges, int &weighted_units, int &mt_out) {
-    n_ranges = 0; weighted_units = 0; mt_out = 1;
-    const int n_new = qsl[r + 1] - qsl[r];
-    if (n_new <= 0 || n_new > small_max) return;
-    if (grp_first[r] != r) return;                       // a member of a group: accounted for by the group's owner
-    if (grp_shared[r] > 0) {
-        const GroupShape g = group_shape(qsl, grp_first, grp_shared, R, r, G);
-        const int pu = g.shared / 64;
-        int tu = 0;   // the members' own keys beyond the shared ones, member after member, in 64-key stages
-        for (int m = r; m < r + g.n_members; ++m) tu += (seq_lens[m] - g.shared + 63) / 64;
-        n_ranges = (pu + chunk - 1) / chunk + (tu + chunk - 1) / chunk;
-        weighted_units = (pu + tu) * g.mt;
-        mt_out = g.mt;
-        return;
+//
+// What bounds it: latency, in front of the attention of the first layer.  Everything that is needed more than once per
+// request (units, members, row tiles) is computed once in parallel; sums and offsets are block-wide scans.
+__device__ __forceinline__ int units_to_ranges(int units, int chunk) { return (units + chunk - 1) / chunk; }
+
+// Exclusive sums of v[0 .. R) and w[0 .. R) in place; returns the totals.  All threads of a block of whole warps.
+__device__ __forceinline__ int2 block_scan2(int32_t *v, int32_t *w, int R) {
+    __shared__ int2 warp_tot[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, n_warps = (int)blockDim.x >> 5;
+    int2 carry = make_int2(0, 0);
+    for (int base = 0; base < R; base += (int)blockDim.x) {
+        const int r = base + (int)threadIdx.x;
+        const int2 x = r < R ? make_int2(v[r], w[r]) : make_int2(0, 0);
+        int2 inc = x;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int a = __shfl_up_sync(0xffffffffu, inc.x, o), b = __shfl_up_sync(0xffffffffu, inc.y, o);
+            if (lane >= o) { inc.x += a; inc.y += b; }
+        }
+        if (lane == 31) warp_tot[wid] = inc;
+        __syncthreads();
+        int2 before = carry;
+        for (int i = 0; i < n_warps; ++i) {
+            const int2 t = warp_tot[i];
+            if (i < wid) { before.x += t.x; before.y += t.y; }
+            carry.x += t.x; carry.y += t.y;
+        }
+        if (r < R) { v[r] = before.x + inc.x - x.x; w[r] = before.y + inc.y - x.y; }
+        __syncthreads();
     }
-    int mt, tpb, nblk;
-    small_block_shape(n_new, G, mt, tpb, nblk);
-    for (int blk = 0; blk < nblk; ++blk) {
-        const int kv_end = seq_lens[r] - n_new + min(n_new, (blk + 1) * tpb);
-        const int u = (kv_end + 63) / 64;
-        weighted_units += u * mt;
-        n_ranges += (u + chunk - 1) / chunk;
-    }
-    mt_out = mt;
+    return carry;
 }
 
 __device__ __forceinline__ void metadata_split_items(const int32_t *__restrict__ qsl, const int32_t *__restrict__ seq_lens,
                                                      const int32_t *__restrict__ block_tables, int max_blocks, int page_size,
                                                      int R, int Hkv, int G, int n_sm, int small_max, int max_items, int max_rows,
                                                      AttnSplitWork *__restrict__ items, int32_t *__restrict__ counts,
-                                                     int32_t *req_scratch /* [5][R] */,
+                                                     int32_t *req_scratch /* [kSplitScratch][R] */,
                                                      int32_t *__restrict__ group_done, int32_t *__restrict__ groups_out,
                                                      int part, int n_parts, int32_t *status) {
     // (several blocks may build the list together: each repeats the cheap per-request passes and fills the items
     // part, part + n_parts, ..; block `part` 0 alone writes the counts and reports findings)
-    __shared__ unsigned long long tot_units;
-    __shared__ int chunk_units, total_items, few_ranges;
+    __shared__ int chunk_units, total_items, few_ranges, max_units, best1, best2;
     small_max = few_row_limit(qsl, R, Hkv, n_sm, small_max);
-    int32_t *req_cnt = req_scratch, *req_off = req_scratch + R, *req_row = req_scratch + 2 * R;
-    int32_t *grp_first = req_scratch + 3 * R, *grp_shared = req_scratch + 4 * R;
+    int32_t *req_off = req_scratch, *req_row = req_scratch + R, *grp_first = req_scratch + 2 * R, *grp_shared = req_scratch + 3 * R;
+    int32_t *u_shared = req_scratch + 4 * R;   // 64-key units of the stream (of the shared prefix, for a group's owner)
+    int32_t *u_own = req_scratch + 5 * R;      // a group's units beyond the shared prefix, member after member
+    int32_t *shape = req_scratch + 6 * R;      // members * 8 + row tiles; 0: the request owns no items
     metadata_prefix_groups(qsl, seq_lens, block_tables, max_blocks, R, page_size, G, small_max, grp_first, grp_shared);
     if (groups_out != nullptr && part == 0)
         for (int r = threadIdx.x; r < R; r += blockDim.x) { groups_out[r] = grp_first[r]; groups_out[R + r] = grp_shared[r]; }
-    // 64-key units of all streams, weighted by their row tiles (an item of mt tiles needs mt * 16 partial rows):
-    // per request in parallel, summed by one thread (a shared 64-bit atomic under contention is far slower)
+    if (threadIdx.x == 0) { max_units = 4; best1 = 0x7fffffff; best2 = 0x7fffffff; }
+    __syncthreads();
     for (int r = threadIdx.x; r < R; r += blockDim.x) {
-        int n, wu, mt;
-        request_ranges(qsl, seq_lens, grp_first, grp_shared, R, r, G, small_max, 1 << 20, n, wu, mt);
-        req_cnt[r] = wu * Hkv;
+        const int n_new = qsl[r + 1] - qsl[r];
+        int us = 0, uo = 0, sh = 0;
+        if (n_new > 0 && n_new <= small_max && grp_first[r] == r) {
+            const int shared = grp_shared[r];
+            int e = r + 1;
+            if (shared > 0) {
+                us = shared / 64;
+                uo = (seq_lens[r] - shared + 63) / 64;
+                for (; e < R && grp_first[e] == r; ++e) uo += (seq_lens[e] - shared + 63) / 64;
+            } else {
+                us = (seq_lens[r] + 63) / 64;
+            }
+            const int rows = (qsl[e] - qsl[r]) * G;
+            sh = (e - r) * 8 + (rows <= 16 ? 1 : (rows <= 32 ? 2 : 4));
+        }
+        u_shared[r] = us; u_own[r] = uo; shape[r] = sh;
+        // units weighted by the row tiles (an item of mt tiles needs mt * 16 partial rows), for the sum below
+        req_off[r] = (us + uo) * (sh & 7) * Hkv; req_row[r] = 0;
+        if (max(us, uo) > 4) atomicMax(&max_units, max(us, uo));
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long sum = 0ull;
-        for (int r = 0; r < R; ++r) sum += (unsigned long long)req_cnt[r];
-        tot_units = sum;
-    }
-    __syncthreads();
+    const int tot_units = block_scan2(req_off, req_row, R).x;
     if (threadIdx.x == 0) {
         // Range length: a range costs a fixed time beyond its streaming time (item claim, first table window and
         // first copies, query fetch, combining the warps, publishing the partial result, a share of the merge), and
@@ -508,8 +507,8 @@ __device__ __forceinline__ void metadata_split_items(const int32_t *__restrict__
         // to 64 requests with 4096 to 32768 cached tokens run fastest with (3 us: 5 .. 16 % slower on the small ones).
         const float t_us = (float)tot_units * 0.74f / (float)max(n_sm, 1);
         const float per_sm = fminf(fmaxf(sqrtf(t_us / 12.f), 1.f), (float)kSplitItemsPerSm);
-        const unsigned long long target = (unsigned long long)ceilf(per_sm * (float)max(n_sm, 1));
-        chunk_units = (int)max(4ull, (tot_units + target - 1) / target);
+        const int target = (int)ceilf(per_sm * (float)max(n_sm, 1));
+        chunk_units = max(4, (int)(((long long)tot_units + target - 1) / target));
         few_ranges = (tot_units > 0 && per_sm < 2.5f) ? 1 : 0;
     }
     __syncthreads();
@@ -520,21 +519,12 @@ __device__ __forceinline__ void metadata_split_items(const int32_t *__restrict__
     if (few_ranges) {
         // every thread tries one candidate length (a grid over 4 .. the longest stream) and counts the ranges of the
         // whole batch for it; the shortest candidates that fit one round and two rounds are kept
-        __shared__ int max_units, best1, best2;
-        if (threadIdx.x == 0) { max_units = 4; best1 = 0x7fffffff; best2 = 0x7fffffff; }
-        __syncthreads();
-        int mu = 0;
-        for (int r = threadIdx.x; r < R; r += blockDim.x) mu = max(mu, (seq_lens[r] + 63) / 64);
-        if (mu > 4) atomicMax(&max_units, mu);
-        __syncthreads();
-        const int step = (max_units - 4 + (int)blockDim.x - 1) / (int)blockDim.x + 0, cand = 4 + (int)threadIdx.x * max(step, 1);
-        if (cand <= max_units + max(step, 1)) {
+        const int step = max((max_units - 4 + (int)blockDim.x - 1) / (int)blockDim.x, 1), cand = 4 + (int)threadIdx.x * step;
+        if (cand <= max_units + step) {
             int cnt = 0;
-            for (int r = 0; r < R; ++r) {
-                int n, wu, mt;
-                request_ranges(qsl, seq_lens, grp_first, grp_shared, R, r, G, small_max, cand, n, wu, mt);
-                cnt += n * Hkv;
-            }
+#pragma unroll 4
+            for (int r = 0; r < R; ++r) cnt += units_to_ranges(u_shared[r], cand) + units_to_ranges(u_own[r], cand);
+            cnt *= Hkv;
             if (cnt <= n_sm) atomicMin(&best1, cand);
             if (cnt <= 2 * n_sm) atomicMin(&best2, cand);
         }
@@ -548,26 +538,21 @@ __device__ __forceinline__ void metadata_split_items(const int32_t *__restrict__
     }
     const int chunk = chunk_units;
     for (int r = threadIdx.x; r < R; r += blockDim.x) {
-        int n, wu, mt;
-        request_ranges(qsl, seq_lens, grp_first, grp_shared, R, r, G, small_max, chunk, n, wu, mt);
-        req_cnt[r] = n * Hkv;
-        req_row[r] = n * Hkv * 16 * mt;
+        const int n = (units_to_ranges(u_shared[r], chunk) + units_to_ranges(u_own[r], chunk)) * Hkv;
+        req_off[r] = n;
+        req_row[r] = n * 16 * (shape[r] & 7);
     }
     __syncthreads();
+    const int2 total = block_scan2(req_off, req_row, R);
     if (threadIdx.x == 0) {
-        int acc = 0, rows = 0;
-        for (int r = 0; r < R; ++r) {
-            const int c = req_cnt[r], n = req_row[r];
-            req_off[r] = acc; req_row[r] = rows;
-            acc += c; rows += n;
-        }
-        if (acc > max_items || rows > max_rows) {
+        int n = total.x;
+        if (n > max_items || total.y > max_rows) {
             if (part == 0) report(status, ALORA_ERR_CAPACITY);
-            acc = 0;
+            n = 0;
         }
-        total_items = acc;
+        total_items = n;
         if (part == 0) {
-            counts[3] = acc;
+            counts[3] = n;
             counts[4] = 0;   // work counter of the few-row kernel
         }
     }
@@ -575,85 +560,51 @@ __device__ __forceinline__ void metadata_split_items(const int32_t *__restrict__
     if (total_items == 0) return;
     // one item per thread and step: owner request by binary search over the item offsets, then stream / KV head / range
     for (int i = part * (int)blockDim.x + (int)threadIdx.x; i < total_items; i += n_parts * (int)blockDim.x) {
-        int lo = 0, hi = R;   // largest r with req_off[r] <= i among requests that own items
+        int lo = 0, hi = R;   // the largest r with req_off[r] <= i owns item i (requests without items share their successor's offset)
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
             if (req_off[mid] <= i) lo = mid; else hi = mid;
         }
-        const int r = lo;
-        int local = i - req_off[r], row0 = req_row[r];
+        const int r = lo, n_mem = shape[r] >> 3, mt = shape[r] & 7;
+        const int local = i - req_off[r], us = u_shared[r], uo = u_own[r];
+        const int np = units_to_ranges(us, chunk), n_splits = np + units_to_ranges(uo, chunk);
+        const int kvh = local / n_splits, sp = local % n_splits;
+        const int shared = grp_shared[r], n_tok = qsl[r + n_mem] - qsl[r];
         AttnSplitWork w;
-        if (grp_shared[r] > 0) {
-            // ---- a prefix group: per KV head [ranges of the shared prefix | ranges of the members' own keys]; the own
-            // keys of all members form one sequence of 64-key stages (member after member) that is cut like any other
-            const GroupShape g = group_shape(qsl, grp_first, grp_shared, R, r, G);
-            const int pu = g.shared / 64, np = (pu + chunk - 1) / chunk;
-            int tu = 0;
-            for (int m = r; m < r + g.n_members; ++m) tu += (seq_lens[m] - g.shared + 63) / 64;
-            const int nt = (tu + chunk - 1) / chunk;
-            const int n_splits = np + nt;
-            const int kvh = local / n_splits, sp = local % n_splits;
-            w.q_start = qsl[r]; w.q_count = g.n_tok; w.kv_head = kvh; w.mt = g.mt; w.split = sp; w.n_splits = n_splits;
-            w.part_row0 = row0 + local * 16 * g.mt;
-            if (sp < np) {
-                const int per = (pu + np - 1) / np;
-                w.req = r; w.kv_start = sp * per * 64; w.kv_end = min(g.shared, (sp + 1) * per * 64);
-                w.pos0 = g.shared;    // every row sees every key of the shared prefix
-                w.pad_ = 0;
-            } else {
-                // stages [kv_start / 64, kv_end / 64) of the members' own keys (not key positions: the kernel walks the
-                // members to find each stage's request, key positions and rows)
-                const int sp2 = sp - np, per = (tu + nt - 1) / nt;
-                w.req = r; w.kv_start = sp2 * per * 64; w.kv_end = min(tu, (sp2 + 1) * per) * 64;
-                w.pos0 = g.shared;
-                w.pad_ = kSplitOwnKeys | g.n_members;
-            }
-            group_done[i] = 0;
-            items[i] = w;
-            continue;
-        }
-        const int n_new = qsl[r + 1] - qsl[r];
-        int mt, tpb, nblk;
-        small_block_shape(n_new, G, mt, tpb, nblk);
-        for (int blk = 0; blk < nblk; ++blk) {
-            const int q_count = min(tpb, n_new - blk * tpb);
-            const int pos0 = seq_lens[r] - n_new + blk * tpb;
-            const int kv_end = pos0 + q_count;   // last token's position + 1
-            const int units = (kv_end + 63) / 64;
-            const int n_splits = (units + chunk - 1) / chunk;
-            if (local >= n_splits * Hkv && blk + 1 < nblk) {
-                local -= n_splits * Hkv;
-                row0 += n_splits * Hkv * 16 * mt;
-                continue;
-            }
-            const int per = (units + n_splits - 1) / n_splits;   // equal ranges rather than full ones and a stub
-            const int kvh = local / n_splits, sp = local % n_splits;
-            w.req = r; w.q_start = qsl[r] + blk * tpb; w.q_count = q_count; w.kv_head = kvh;
+        w.req = r; w.q_start = qsl[r]; w.q_count = n_tok; w.kv_head = kvh; w.mt = mt; w.split = sp; w.n_splits = n_splits;
+        w.part_row0 = req_row[r] + local * 16 * mt;
+        if (sp < np) {   // (equal ranges rather than full ones and a stub)
+            const int per = (us + np - 1) / np;
+            const int kv_end = shared > 0 ? shared : seq_lens[r];   // last visible position + 1
             w.kv_start = sp * per * 64; w.kv_end = min(kv_end, (sp + 1) * per * 64);
-            w.pos0 = pos0; w.mt = mt; w.split = sp; w.n_splits = n_splits; w.part_row0 = row0 + local * 16 * mt; w.pad_ = 0;
-            group_done[i] = 0;
-            items[i] = w;
-            break;
+            w.pos0 = shared > 0 ? shared : seq_lens[r] - n_tok;     // every row sees every key of a shared prefix
+            w.pad_ = 0;
+        } else {
+            // a prefix group: per KV head [ranges of the shared prefix | ranges of the members' own keys].  Stages
+            // [kv_start / 64, kv_end / 64) of the own keys (not key positions: the kernel walks the members to find each
+            // stage's request, key positions and rows)
+            const int sp2 = sp - np, nt = n_splits - np, per = (uo + nt - 1) / nt;
+            w.kv_start = sp2 * per * 64; w.kv_end = min(uo, (sp2 + 1) * per) * 64;
+            w.pos0 = shared;
+            w.pad_ = kSplitOwnKeys | n_mem;
         }
+        group_done[i] = 0;
+        items[i] = w;
     }
 }
 
-// FewRowMeta of a batch of at most kFewRowMax rows (all of them in block 0): the adapters that occur in
-// row_adapter[0 .. T), ascending, each one's padded rank and scale, and every row's slot.  Called by all
-// threads of block 0 after they have written row_adapter.
-__device__ __forceinline__ void metadata_few_row(const int32_t *row_adapter, const AdapterDev *__restrict__ adapters,
-                                                 int T, int max_adapters, FewRowMeta *__restrict__ meta) {
+// FewRowMeta of a batch of at most kFewRowMax rows, thread t's applied adapter being k_mine (-1: none, or no such
+// row): the adapters that occur, ascending, each one's padded rank and scale, and every row's slot.  Called by all
+// kFewRowMax threads of a block.
+__device__ __forceinline__ void metadata_few_row(int k_mine, const AdapterDev *__restrict__ adapters, int max_adapters,
+                                                 FewRowMeta *__restrict__ meta) {
     __shared__ uint32_t bits[32];
     __shared__ int16_t ids[kFewRowMax];
     __shared__ int n_present;
     if (threadIdx.x < 32) bits[threadIdx.x] = 0u;
-    __syncthreads();   // (also orders this block's row_adapter writes before the reads below)
-    int k_mine = -1;
-    if ((int)threadIdx.x < T && (int)threadIdx.x < kFewRowMax) {
-        k_mine = row_adapter[threadIdx.x];
-        if (k_mine >= 0 && k_mine < max_adapters && k_mine < 1024) atomicOr(&bits[k_mine >> 5], 1u << (k_mine & 31));
-        else k_mine = -1;
-    }
+    __syncthreads();
+    if (k_mine >= 0 && k_mine < max_adapters && k_mine < 1024) atomicOr(&bits[k_mine >> 5], 1u << (k_mine & 31));
+    else k_mine = -1;
     __syncthreads();
     if (threadIdx.x == 0) {
         int n = 0;
@@ -700,7 +651,7 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
                 AttnSplitWork *__restrict__ split_items,
                 int32_t *req_scratch, int32_t *__restrict__ group_done, int rowwise_cap,
                 int32_t *__restrict__ attn_cta_start, const AdapterDev *__restrict__ adapters, int phases,
-                FewRowMeta *__restrict__ few_row_meta, int32_t *__restrict__ prefix_groups, int32_t *status) {
+                int32_t *__restrict__ prefix_groups, int32_t *status) {
     // The per-request inputs are read many times (binary searches, list builders): one parallel pass stages them
     // in shared memory, so that the later steps do not each pay a round trip to global memory.
     __shared__ int32_t s_req[4 * kMetaStageR + 1];
@@ -719,8 +670,8 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
         if (a_req) a_req = s_areq;
     }
     if (phases & kMetaProjection)
-        metadata_tokens(positions, a_req, adapter_ids, qsl, seq_lens, block_tables, max_blocks, num_pages, page_size,
-                        max_adapters, T, R, mode, token_req, row_adapter, slot_map, adapters, status);
+        metadata_token((int)(blockIdx.x * blockDim.x + threadIdx.x), positions, a_req, adapter_ids, qsl, seq_lens, block_tables,
+                       max_blocks, num_pages, page_size, max_adapters, T, R, mode, token_req, row_adapter, slot_map, adapters, status);
     // The three list builders are independent of one another: blocks 0, 1 and 2 take one each (a launch of both
     // phases has at least three blocks, one of the attention phase alone two).
     const int nb = (int)gridDim.x;
@@ -741,11 +692,8 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
     if (14 * R + 5 <= kMetaSmemInts) seg_scratch = blk_off = req_scratch = smem_scratch;
     __syncthreads();
     if ((int)blockIdx.x == b_tiles) {
-        if (few_row_meta != nullptr && adapters != nullptr && row_adapter != nullptr)
-            metadata_few_row(row_adapter, adapters, T, max_adapters, few_row_meta);   // the few-row route has no row tiles
-        else
-            metadata_tiles(a_req, adapter_ids, qsl, seq_lens, R, mode, max_adapters, max_tiles, tiles, counts, seg_scratch,
-                           T, rowwise_cap, shrink_tiles, t_ready, status);
+        metadata_tiles(a_req, adapter_ids, qsl, seq_lens, R, mode, max_adapters, max_tiles, tiles, counts, seg_scratch,
+                       T, rowwise_cap, shrink_tiles, t_ready, status);
         __syncthreads();  // a builder that follows in this block reuses the scratch
     }
     if ((int)blockIdx.x == b_attn && items != nullptr && block_tables != nullptr) {
@@ -760,9 +708,12 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
     if (!proj) tc::grid_dep_wait();
 }
 
-// The projection phase for a batch on the few-row route (at most kFewRowMax tokens, one block): per-token arrays
-// and the adapter facts, nothing else.  A kernel of its own because every step of a decode loop waits for it: it
-// runs once per call on one SM, so what it costs is mostly the fetch of its instructions, and this one is short.
+// The projection phase for a batch on the few-row route (at most kFewRowMax tokens): per-token arrays and the adapter
+// facts, nothing else.  A kernel of its own because every step of a decode loop waits for it: what it costs is mostly
+// the fetch of its instructions, and this one is short.  Block l writes the facts of layer l of the call (a stack call
+// builds those of all layers in one launch: with a launch per layer each layer waited 10 us for it), block 0 also the
+// per-token arrays.  row_adapter holds the adapter of every row whose gate is open; whether it is registered on a layer
+// (else: base output and a finding) goes into that layer's facts.
 __global__ void __launch_bounds__(kFewRowMax)
 metadata_few_row_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, const int32_t *adapter_ids,
                         const int32_t *qsl, const int32_t *seq_lens, const int32_t *__restrict__ block_tables,
@@ -785,9 +736,15 @@ metadata_few_row_kernel(const int32_t *__restrict__ positions, const int32_t *a_
         if (adapter_ids) adapter_ids = s_ids;
         if (a_req) a_req = s_areq;
     }
-    metadata_tokens(positions, a_req, adapter_ids, qsl, seq_lens, block_tables, max_blocks, num_pages, page_size,
-                    max_adapters, T, R, mode, token_req, row_adapter, slot_map, adapters, status);
-    if (few_row_meta != nullptr) metadata_few_row(row_adapter, adapters, T, max_adapters, few_row_meta);
+    const bool first = blockIdx.x == 0;
+    int k = metadata_token((int)threadIdx.x, positions, a_req, adapter_ids, qsl, seq_lens, first ? block_tables : nullptr,
+                           max_blocks, num_pages, page_size, max_adapters, T, R, mode, first ? token_req : nullptr,
+                           first ? row_adapter : nullptr, first ? slot_map : nullptr, nullptr, status);
+    if (few_row_meta != nullptr) {
+        const AdapterDev *ads = adapters + (size_t)blockIdx.x * max_adapters;
+        if (k >= 0 && ads[k].rank == 0) { report(status, ALORA_ERR_NO_WEIGHTS); k = -1; }
+        metadata_few_row(k, ads, max_adapters, few_row_meta + blockIdx.x);
+    }
 }
 
 int launch_metadata(alora_ctx *ctx, const BatchArgs &b, cudaStream_t s, int phases, bool timed) {
@@ -806,9 +763,9 @@ int launch_metadata(alora_ctx *ctx, const BatchArgs &b, cudaStream_t s, int phas
     constexpr int kSplitBuilders = 8;
     const int grid = attn_only ? (14 * b.R + 5 <= kMetaSmemInts ? 1 + kSplitBuilders : 2) : std::max((phases & kMetaAttention) ? 3 : 1, (b.T + threads - 1) / threads);
     const AdapterDev *ads = b.layer >= 0 ? ctx->d_adapters + (size_t)b.layer * ctx->cfg.max_adapters : nullptr;
-    FewRowMeta *few = (b.few_row && ads != nullptr) ? (FewRowMeta *)ctx->d_skinny_meta : nullptr;
     if (phases == kMetaProjection && b.few_row && b.T <= kFewRowMax) {
-        metadata_few_row_kernel<<<1, kFewRowMax, 0, s>>>(
+        FewRowMeta *few = ads != nullptr ? (FewRowMeta *)ctx->d_skinny_meta + b.layer : nullptr;
+        metadata_few_row_kernel<<<b.n_layers, kFewRowMax, 0, s>>>(
             b.positions, b.activation_offsets, b.adapter_ids, b.query_start_loc, b.seq_lens, b.block_tables, b.max_blocks,
             b.num_pages, ctx->d.page, ctx->cfg.max_adapters, b.T, b.R, b.mode, ctx->d_token_req, ctx->d_row_adapter,
             ctx->d_slot, ads, few, ctx->d_status);
@@ -822,7 +779,7 @@ int launch_metadata(alora_ctx *ctx, const BatchArgs &b, cudaStream_t s, int phas
         ctx->d.Hkv, ctx->attn_q_block, ctx->max_attn_items, ctx->d_attn_items, ctx->d_attn_off, ctx->d.G,
         ctx->sm_count, ctx->small_max_tokens, ctx->max_split_items, ctx->max_split_rows, ctx->d_split_items,
         ctx->d_req_scratch, ctx->d_group_done, ctx->d_row_delta ? kRowwiseMaxTokens : 0,
-        ctx->d_attn_cta_start, ads, phases, few, ctx->d_prefix_groups, ctx->d_status);
+        ctx->d_attn_cta_start, ads, phases, ctx->d_prefix_groups, ctx->d_status);
     return e == cudaSuccess ? 1 : -1;
 }
 
