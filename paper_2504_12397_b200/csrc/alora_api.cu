@@ -226,7 +226,7 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
             alloc((void **)&ctx->d_prefix_groups, (size_t)2 * c.max_requests * 4);
             alloc((void **)&ctx->d_part_o, (size_t)ctx->max_split_rows * d.hd * 4);
             alloc((void **)&ctx->d_part_ml, (size_t)ctx->max_split_rows * 2 * 4);
-            alloc((void **)&ctx->d_group_done, (size_t)ctx->max_split_items * 4);
+            alloc((void **)&ctx->d_group_done, (size_t)(ctx->max_split_rows / 16) * 4);
         }
     }
     if (c.dtype == ALORA_DTYPE_BF16) {

@@ -71,8 +71,8 @@ constexpr int kAttnSpreadMinGain = 24; // fewer items than blocks: spread them o
 
 // One unit of few-row (decode / short suffix) attention work: score rows of `q_count` tokens starting at
 // flat token q_start (rows are (token, query head of the group) pairs, `mt` tiles of 16 rows), one KV
-// head, keys [kv_start, kv_end) of the request.  The `n_splits` key ranges of the same rows are
-// consecutive items; their partial results are merged afterwards.
+// head, keys [kv_start, kv_end) of the request.  The `n_splits` key ranges of the same rows have consecutive
+// blocks of 16 * mt partial rows (range `split` the split-th one); their partial results are merged afterwards.
 struct AttnSplitWork {
     int32_t req, q_start, q_count, kv_head;
     int32_t kv_start, kv_end, pos0, mt;      // pos0 = position of the first token of the block
@@ -84,7 +84,7 @@ struct AttnSplitWork {
                     // tokens only, up to each token's own position
 };
 constexpr int32_t kSplitOwnKeys = 0x40000000;
-constexpr int kSplitScratch = 7;       // per-request integers that the builder of the few-row list needs
+constexpr int kSplitScratch = 8;       // per-request integers that the builder of the few-row list needs
 constexpr int kSplitItemsPerSm = 16;   // target number of (row tile, key range) pairs per SM
 
 // Few-row projection (batches of at most kFewRowMax rows): what its two kernels need to know about the batch's
@@ -184,7 +184,7 @@ struct alora_ctx {
     int32_t *d_prefix_groups = nullptr; // [2][max_requests] per request of the last batch: first request of its prefix
                                         // group, keys the group shares (0: ungrouped)
     float *d_part_o = nullptr, *d_part_ml = nullptr;
-    int32_t *d_group_done = nullptr;    // [max_split_items] finished key ranges per group (first item's index)
+    int32_t *d_group_done = nullptr;    // [max_split_rows / 16] finished key ranges per (stream, KV head), at its first partial row / 16
     int32_t max_split_items = 0, max_split_rows = 0, small_max_tokens = 0;
     void *d_t = nullptr;          // [max_tokens][3][RP] rank-r intermediate
     float *d_row_delta = nullptr; // [min(max_tokens, kRowwiseMaxTokens)][N] fp32 delta rows (bf16 row-wise route)

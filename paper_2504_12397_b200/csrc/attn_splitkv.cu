@@ -49,7 +49,7 @@ struct SplitArgs {
     float *part_ml;             // [partial row][2]: maximum (scaled, log2 units), sum
     int32_t *work_counter;      // next unclaimed item (zero between launches)
     int32_t *blocks_done;       // blocks that have finished (zero between launches)
-    int32_t *group_done;        // [item] per group (indexed by its first item): key ranges finished so far (zero between launches)
+    int32_t *group_done;        // per (stream, KV head), at its first partial row / 16: key ranges finished so far (zero between launches)
     int32_t *status;
 };
 
@@ -121,30 +121,33 @@ __device__ __forceinline__ void own_key_stage(const int32_t *seq_lens, int f, in
 }
 
 // Merge of the key ranges of one block of rows: out = sum_s O_s 2^(m_s - M) / sum_s l_s 2^(m_s - M).
-// `w` is the group's first range; called by 128 threads (threadIdx.x 0..127).
+// `row0` is the first partial row of the block's first range; called by the 256 consumer threads (32 rows at a time).
+// It sits at the end of a launch: the loads of four ranges are in flight together.
 template <int HD>
-__device__ __forceinline__ void merge_group(const AttnSplitWork w, const float *part_o, const float *part_ml, int G,
+__device__ __forceinline__ void merge_group(const AttnSplitWork &w, int row0, const float *part_o, const float *part_ml, int G,
                                             int Nq, __nv_bfloat16 *out) {
     constexpr int kCols = HD / 8;
-    const int t = threadIdx.x, r = t >> 3, c0 = (t & 7) * kCols;
+    const int c0 = (threadIdx.x & 7) * kCols;
     const int rows = 16 * w.mt;  // partial rows per key range of this group
-    for (int mt = 0; mt < w.mt; ++mt) {
-        const int rg = mt * 16 + r;
+    for (int rg = threadIdx.x >> 3; rg < rows; rg += 32) {
         const int tok = rg / G;
-        if (tok >= w.q_count) continue;
+        if (tok >= w.q_count) break;
+        const float2 *ml = reinterpret_cast<const float2 *>(part_ml) + row0 + rg;
+        const float *src = part_o + ((size_t)row0 + rg) * HD + c0;
         float M = -INFINITY;
-        for (int s = 0; s < w.n_splits; ++s) M = fmaxf(M, __ldcg(part_ml + ((size_t)w.part_row0 + (size_t)s * rows + rg) * 2));
+#pragma unroll 4
+        for (int s = 0; s < w.n_splits; ++s) M = fmaxf(M, __ldcg(ml + (size_t)s * rows).x);
         float L = 0.f, acc[kCols];
 #pragma unroll
         for (int c = 0; c < kCols; ++c) acc[c] = 0.f;
+#pragma unroll 4
         for (int s = 0; s < w.n_splits; ++s) {
-            const float *ml = part_ml + ((size_t)w.part_row0 + (size_t)s * rows + rg) * 2;
-            const float wgt = ex2(__ldcg(ml) - M);
-            L += __ldcg(ml + 1) * wgt;
-            const float *src = part_o + ((size_t)w.part_row0 + (size_t)s * rows + rg) * HD + c0;
+            const float2 v2 = __ldcg(ml + (size_t)s * rows);
+            const float wgt = ex2(v2.x - M);
+            L += v2.y * wgt;
 #pragma unroll
             for (int c = 0; c < kCols; c += 4) {
-                const float4 v = __ldcg(reinterpret_cast<const float4 *>(src + c));
+                const float4 v = __ldcg(reinterpret_cast<const float4 *>(src + (size_t)s * rows * HD + c));
                 acc[c] += v.x * wgt; acc[c + 1] += v.y * wgt; acc[c + 2] += v.z * wgt; acc[c + 3] += v.w * wgt;
             }
         }
@@ -501,12 +504,12 @@ attn_splitkv_kernel(const __grid_constant__ CUtensorMap tmKV, const SplitArgs a)
                 }
             }
             if (consumer_barrier_or(!ok)) break;  // a wait expired somewhere: all consumers leave together
-            if (warp < 4) {
+            {
                 const int n_src = 4 / mt_cnt;             // warps 0..3 that hold the same row tile
                 constexpr int kCols = HD / 8;             // columns per thread: 8 threads cover a row
-                const int t = threadIdx.x;                // 0..127
+                const int t = threadIdx.x & 127;
                 const int r = t >> 3, c0 = (t & 7) * kCols;
-                for (int mt = 0; mt < mt_cnt; ++mt) {
+                for (int mt = threadIdx.x >> 7; mt < mt_cnt; mt += 2) {   // a row tile per four warps
                     float M = -INFINITY;
                     for (int g = 0; g < n_src; ++g) M = fmaxf(M, ml_s[((mt + mt_cnt * g) * 16 + r) * 2]);
                     const float Mu = M == -INFINITY ? 0.f : M;
@@ -553,16 +556,18 @@ attn_splitkv_kernel(const __grid_constant__ CUtensorMap tmKV, const SplitArgs a)
             if (w.n_splits > 1) {
                 // the block that completes the last key range of a group merges the group (ranges in index order,
                 // whichever block does it: the result does not depend on timing)
+                const int row0 = w.part_row0 - w.split * 16 * w.mt;
                 __threadfence();
                 consumer_barrier();
                 if (threadIdx.x == 0) {
-                    *merge_flag = atomicAdd(a.group_done + (it - w.split), 1) == w.n_splits - 1;
-                    if (*merge_flag) a.group_done[it - w.split] = 0;   // for the next layer that uses the list
+                    int32_t *done = a.group_done + row0 / 16;
+                    *merge_flag = atomicAdd(done, 1) == w.n_splits - 1;
+                    if (*merge_flag) *done = 0;   // for the next layer that uses the list
                 }
                 consumer_barrier();
-                if (*merge_flag && warp < 4) {
+                if (*merge_flag) {
                     __threadfence();
-                    merge_group<HD>(a.items[it - w.split], a.part_o, a.part_ml, a.G, a.Nq, a.out);
+                    merge_group<HD>(w, row0, a.part_o, a.part_ml, a.G, a.Nq, a.out);
                 }
             } else {
                 consumer_barrier();  // the exchange buffers are rewritten by the next item

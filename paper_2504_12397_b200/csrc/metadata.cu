@@ -420,8 +420,9 @@ __device__ __forceinline__ void metadata_prefix_groups(const int32_t *__restrict
 // head of the group) per KV head).  A STREAM is one block of score rows with the keys it reads: for an ungrouped
 // request its rows over keys 0 .. causal limit; for a prefix group the stacked rows of all members (16 * mt, mt = 1, 2
 // or 4), over the shared prefix (read once, nothing masked) followed by every member's own keys beyond it (masked so
-// that only that member's rows see them).  A stream's keys are cut into ranges of at most `chunk` 64-key units; the
-// ranges of one (stream, KV head) are consecutive items and are merged by whichever block finishes last.
+// that only that member's rows see them).  A stream's keys are cut into ranges of at most `chunk` 64-key units, which are
+// merged by whichever block finishes last.  The list holds the ranges of whole streams and shared prefixes first and
+// the groups' own keys after them: those are short and fill the blocks that have no long range left.
 // A group is owned by its first request: that request accounts for all of the group's items.
 //
 // What bounds it: latency, in front of the attention of the first layer.  Everything that is needed more than once per
@@ -464,16 +465,17 @@ __device__ __forceinline__ void metadata_split_items(const int32_t *__restrict__
                                                      int part, int n_parts, int32_t *status) {
     // (several blocks may build the list together: each repeats the cheap per-request passes and fills the items
     // part, part + n_parts, ..; block `part` 0 alone writes the counts and reports findings)
-    __shared__ int chunk_units, total_items, few_ranges, max_units, best1, best2;
+    __shared__ int chunk_units, total_items, few_ranges, max_units;
+    __shared__ unsigned long long best;
     small_max = few_row_limit(qsl, R, Hkv, n_sm, small_max);
-    int32_t *req_off = req_scratch, *req_row = req_scratch + R, *grp_first = req_scratch + 2 * R, *grp_shared = req_scratch + 3 * R;
+    int32_t *req_off = req_scratch, *own_off = req_scratch + 7 * R, *req_row = req_scratch + R, *grp_first = req_scratch + 2 * R, *grp_shared = req_scratch + 3 * R;
     int32_t *u_shared = req_scratch + 4 * R;   // 64-key units of the stream (of the shared prefix, for a group's owner)
     int32_t *u_own = req_scratch + 5 * R;      // a group's units beyond the shared prefix, member after member
     int32_t *shape = req_scratch + 6 * R;      // members * 8 + row tiles; 0: the request owns no items
     metadata_prefix_groups(qsl, seq_lens, block_tables, max_blocks, R, page_size, G, small_max, grp_first, grp_shared);
     if (groups_out != nullptr && part == 0)
         for (int r = threadIdx.x; r < R; r += blockDim.x) { groups_out[r] = grp_first[r]; groups_out[R + r] = grp_shared[r]; }
-    if (threadIdx.x == 0) { max_units = 4; best1 = 0x7fffffff; best2 = 0x7fffffff; }
+    if (threadIdx.x == 0) { max_units = 4; best = ~0ull; }
     __syncthreads();
     for (int r = threadIdx.x; r < R; r += blockDim.x) {
         const int n_new = qsl[r + 1] - qsl[r];
@@ -513,40 +515,44 @@ __device__ __forceinline__ void metadata_split_items(const int32_t *__restrict__
     }
     __syncthreads();
     // With only one or two ranges per SM the rule above ignores how the ranges fall into rounds over the SMs: 192
-    // equal ranges on 148 SMs take as long as 296.  Such batches (a few requests) instead take the shortest range
-    // length whose ranges fit into exactly one round, or into two, whichever the same cost model says is faster:
-    // rounds x (12 us + range length x 0.74 us).  The range count for a given length is a sum over the requests.
+    // equal ranges on 148 SMs take as long as 296.  Such batches (a few requests) instead take the range length that the
+    // same cost model finds fastest: whole rounds of the long ranges, 12 us + length x 0.74 us each, and the groups' own
+    // keys in the gaps of the last round, or after it where they do not fit.
     if (few_ranges) {
-        // every thread tries one candidate length (a grid over 4 .. the longest stream) and counts the ranges of the
-        // whole batch for it; the shortest candidates that fit one round and two rounds are kept
+        // every thread tries one candidate length (a grid over 4 .. the longest stream)
         const int step = max((max_units - 4 + (int)blockDim.x - 1) / (int)blockDim.x, 1), cand = 4 + (int)threadIdx.x * step;
         if (cand <= max_units + step) {
-            int cnt = 0;
+            int n_long = 0, n_own = 0, own_units = 0;
 #pragma unroll 4
-            for (int r = 0; r < R; ++r) cnt += units_to_ranges(u_shared[r], cand) + units_to_ranges(u_own[r], cand);
-            cnt *= Hkv;
-            if (cnt <= n_sm) atomicMin(&best1, cand);
-            if (cnt <= 2 * n_sm) atomicMin(&best2, cand);
+            for (int r = 0; r < R; ++r) {
+                n_long += units_to_ranges(u_shared[r], cand);
+                n_own += units_to_ranges(u_own[r], cand);
+                own_units += u_own[r];
+            }
+            n_long *= Hkv; n_own *= Hkv; own_units *= Hkv;
+            const float t_long = 12.f + 0.74f * (float)cand;
+            const float t_own = n_own > 0 ? 12.f + 0.74f * (float)own_units / (float)n_own : 0.f;
+            const float rounds = (float)((n_long + n_sm - 1) / n_sm) * t_long;
+            const float all = ((float)n_long * t_long + (float)n_own * t_own) / (float)n_sm + 0.5f * t_own;
+            atomicMin(&best, ((unsigned long long)(unsigned)(fmaxf(rounds, all) * 16.f) << 32) | (unsigned)cand);
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            const float c1 = 12.f + 0.74f * (float)best1, c2 = 2.f * (12.f + 0.74f * (float)best2);
-            if (best1 != 0x7fffffff && c1 <= c2) chunk_units = best1;
-            else if (best2 != 0x7fffffff) chunk_units = best2;
-        }
+        if (threadIdx.x == 0) chunk_units = (int)(best & 0xffffffffu);
         __syncthreads();
     }
     const int chunk = chunk_units;
     for (int r = threadIdx.x; r < R; r += blockDim.x) {
-        const int n = (units_to_ranges(u_shared[r], chunk) + units_to_ranges(u_own[r], chunk)) * Hkv;
-        req_off[r] = n;
-        req_row[r] = n * 16 * (shape[r] & 7);
+        const int n = units_to_ranges(u_shared[r], chunk) * Hkv, n_own = units_to_ranges(u_own[r], chunk) * Hkv;
+        req_off[r] = n; own_off[r] = n_own;
+        req_row[r] = (n + n_own) * 16 * (shape[r] & 7);
+        grp_first[r] = 0;   // (not needed any more: second array of the row scan)
     }
     __syncthreads();
-    const int2 total = block_scan2(req_off, req_row, R);
+    const int2 total = block_scan2(req_off, own_off, R);
+    const int total_rows = block_scan2(req_row, grp_first, R).x;
     if (threadIdx.x == 0) {
-        int n = total.x;
-        if (n > max_items || total.y > max_rows) {
+        int n = total.x + total.y;
+        if (n > max_items || total_rows > max_rows) {
             if (part == 0) report(status, ALORA_ERR_CAPACITY);
             n = 0;
         }
@@ -557,38 +563,40 @@ __device__ __forceinline__ void metadata_split_items(const int32_t *__restrict__
         }
     }
     __syncthreads();
-    if (total_items == 0) return;
     // one item per thread and step: owner request by binary search over the item offsets, then stream / KV head / range
     for (int i = part * (int)blockDim.x + (int)threadIdx.x; i < total_items; i += n_parts * (int)blockDim.x) {
-        int lo = 0, hi = R;   // the largest r with req_off[r] <= i owns item i (requests without items share their successor's offset)
+        const bool own = i >= total.x;
+        const int32_t *off = own ? own_off : req_off;
+        const int idx = own ? i - total.x : i;
+        int lo = 0, hi = R;   // the largest r with off[r] <= idx owns the item (requests without items share their successor's offset)
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
-            if (req_off[mid] <= i) lo = mid; else hi = mid;
+            if (off[mid] <= idx) lo = mid; else hi = mid;
         }
         const int r = lo, n_mem = shape[r] >> 3, mt = shape[r] & 7;
-        const int local = i - req_off[r], us = u_shared[r], uo = u_own[r];
-        const int np = units_to_ranges(us, chunk), n_splits = np + units_to_ranges(uo, chunk);
-        const int kvh = local / n_splits, sp = local % n_splits;
+        const int us = u_shared[r], uo = u_own[r];
+        const int np = units_to_ranges(us, chunk), nt = units_to_ranges(uo, chunk), per_head = own ? nt : np;
+        const int local = idx - off[r], kvh = local / per_head, sp = local % per_head;
         const int shared = grp_shared[r], n_tok = qsl[r + n_mem] - qsl[r];
         AttnSplitWork w;
-        w.req = r; w.q_start = qsl[r]; w.q_count = n_tok; w.kv_head = kvh; w.mt = mt; w.split = sp; w.n_splits = n_splits;
-        w.part_row0 = req_row[r] + local * 16 * mt;
-        if (sp < np) {   // (equal ranges rather than full ones and a stub)
+        w.req = r; w.q_start = qsl[r]; w.q_count = n_tok; w.kv_head = kvh; w.mt = mt; w.n_splits = np + nt;
+        w.split = own ? np + sp : sp;
+        w.part_row0 = req_row[r] + (kvh * (np + nt) + w.split) * 16 * mt;
+        if (!own) {   // (equal ranges rather than full ones and a stub)
             const int per = (us + np - 1) / np;
             const int kv_end = shared > 0 ? shared : seq_lens[r];   // last visible position + 1
             w.kv_start = sp * per * 64; w.kv_end = min(kv_end, (sp + 1) * per * 64);
             w.pos0 = shared > 0 ? shared : seq_lens[r] - n_tok;     // every row sees every key of a shared prefix
             w.pad_ = 0;
         } else {
-            // a prefix group: per KV head [ranges of the shared prefix | ranges of the members' own keys].  Stages
-            // [kv_start / 64, kv_end / 64) of the own keys (not key positions: the kernel walks the members to find each
-            // stage's request, key positions and rows)
-            const int sp2 = sp - np, nt = n_splits - np, per = (uo + nt - 1) / nt;
-            w.kv_start = sp2 * per * 64; w.kv_end = min(uo, (sp2 + 1) * per) * 64;
+            // a prefix group's members' own keys: stages [kv_start / 64, kv_end / 64) (not key positions: the kernel walks
+            // the members to find each stage's request, key positions and rows)
+            const int per = (uo + nt - 1) / nt;
+            w.kv_start = sp * per * 64; w.kv_end = min(uo, (sp + 1) * per) * 64;
             w.pos0 = shared;
             w.pad_ = kSplitOwnKeys | n_mem;
         }
-        group_done[i] = 0;
+        if (w.split == 0) group_done[w.part_row0 / 16] = 0;
         items[i] = w;
     }
 }
