@@ -18,7 +18,7 @@ int launch_project_simt(alora_ctx *, int, const void *, int, void *, cudaStream_
 int launch_linear_simt(alora_ctx *, const void *, const void *, int, int, int, void *, const void *, cudaStream_t);
 int launch_attend_simt(alora_ctx *, const void *, const BatchArgs &, const void *, void *, cudaStream_t);
 
-int launch_project_tc(alora_ctx *, int, const void *, int, void *, cudaStream_t, void *, int);
+int launch_project_tc(alora_ctx *, int, const void *, int, int, void *, cudaStream_t, void *, int);
 int launch_linear_tc(alora_ctx *, const void *, const void *, int, int, int, void *, const void *, cudaStream_t);
 int launch_repack_mlp(const void *, const void *, const void *, const void *, int, int, int, int, int, void *, void *,
                       cudaStream_t);   // mlp_adapter.cu
@@ -33,11 +33,11 @@ int launch_attend_tc(alora_ctx *, const void *, const BatchArgs &, const void *,
 // bf16 runs on the tensor cores; the fp32 data type (tiny exact-precision configurations) on CUDA cores.
 // With a page pool given, the bf16 projection also writes the k / v columns of every row to the row's cache slot
 // (the KV append fused into its epilogue) and sets *kv_appended.
-int launch_project(alora_ctx *ctx, int layer, const void *hidden, int T, void *qkv, cudaStream_t s, void *kv_pool,
+int launch_project(alora_ctx *ctx, int layer, const void *hidden, int T, int R, void *qkv, cudaStream_t s, void *kv_pool,
                    int num_pages, bool *kv_appended) {
     if (kv_appended) *kv_appended = false;
     if (ctx->cfg.dtype == ALORA_DTYPE_BF16) {
-        const int n = launch_project_tc(ctx, layer, hidden, T, qkv, s, kv_pool, num_pages);
+        const int n = launch_project_tc(ctx, layer, hidden, T, R, qkv, s, kv_pool, num_pages);
         if (kv_appended && n >= 0 && kv_pool != nullptr) *kv_appended = true;
         return n;
     }
@@ -90,7 +90,7 @@ static alora_status run_layer(alora_ctx *ctx, int layer, const void *hidden, con
     bool kv_appended = false;
     const bool rope = ctx->d_rope_inv_freq != nullptr;   // the rotation comes between projection and append
     ctx->pending_attn_meta = (b.facts_ready & kMetaAttention) ? nullptr : &b;
-    k = launch_project(ctx, layer, hidden, b.T, ctx->d_qkv, s, rope ? nullptr : pool, b.num_pages, &kv_appended);
+    k = launch_project(ctx, layer, hidden, b.T, b.R, ctx->d_qkv, s, rope ? nullptr : pool, b.num_pages, &kv_appended);
     const bool attn_meta_pending = ctx->pending_attn_meta != nullptr;
     ctx->pending_attn_meta = nullptr;
     if (k < 0) return ALORA_ERR_UNSUPPORTED;
@@ -183,17 +183,19 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, c.device) == cudaSuccess) ctx->sm_count = prop.multiProcessorCount;
     const size_t Tm = (size_t)c.max_tokens;
-    ctx->max_tiles = (int)(Tm / 128 + 2 * (size_t)c.max_requests + 2);
+    ctx->max_pairs = pair_bound(ctx, c.max_tokens, c.max_requests);
+    if (c.dtype == ALORA_DTYPE_BF16)
+        ctx->t_slots = std::max(ctx->max_pairs, 2 * pair_bound(ctx, std::min(c.max_tokens, kSplitTTokens), c.max_requests));
     alloc((void **)&ctx->d_adapters, n_ad * sizeof(AdapterDev));
     alloc((void **)&ctx->d_token_req, Tm * 4);
     alloc((void **)&ctx->d_row_adapter, Tm * 4);
     alloc((void **)&ctx->d_slot, Tm * 4);
-    alloc((void **)&ctx->d_tiles, (size_t)ctx->max_tiles * sizeof(ProjTile));
+    alloc((void **)&ctx->d_pairs, (size_t)ctx->max_pairs * sizeof(TilePair));
+    alloc((void **)&ctx->d_pair_off, (Tm / kTileRows + 2) * 4);
     alloc((void **)&ctx->d_counts, 16 * 4);
     alloc((void **)&ctx->d_seg_scratch, ((size_t)14 * c.max_requests + 5) * 4);
-    alloc((void **)&ctx->d_shrink_tiles, (size_t)ctx->max_tiles * 4);
-    alloc((void **)&ctx->d_t_ready, (size_t)ctx->max_tiles * 4);
-    alloc(&ctx->d_t, Tm * 3 * d.RP * 4);
+    alloc((void **)&ctx->d_t_ready, (size_t)ctx->max_pairs * 4);
+    alloc(&ctx->d_t, c.dtype == ALORA_DTYPE_BF16 ? (size_t)ctx->t_slots * kTileRows * 3 * d.RP * 2 : Tm * 3 * d.RP * 4);
     alloc(&ctx->d_qkv, Tm * d.N * es);
     alloc((void **)&ctx->d_status, 4);
     if (c.rope_theta != 0.f) alloc((void **)&ctx->d_rope_inv_freq, (size_t)(c.head_dim / 2) * sizeof(double));
@@ -242,7 +244,6 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
             alloc((void **)&ctx->d_skinny_t, (size_t)ksplit * 128 * std::max(ctx->skinny_p_cap, 1) * 192 * 4);
             alloc(&ctx->d_skinny_meta, (size_t)c.n_layers * sizeof(FewRowMeta));
         }
-        alloc((void **)&ctx->d_row_delta, std::min<size_t>(Tm, kRowwiseMaxTokens) * d.N * 4);
         const size_t na = (size_t)std::max(1, c.max_adapters);
         ctx->tc_a_all.assign(c.n_layers, nullptr);
         ctx->tc_b_all.assign(c.n_layers, nullptr);
@@ -274,6 +275,7 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
         e = cudaMemset(ctx->d_status, 0, 4);
         if (e == cudaSuccess) e = cudaMemset(ctx->d_adapters, 0, n_ad * sizeof(AdapterDev));
         if (e == cudaSuccess) e = cudaMemset(ctx->d_counts, 0, 64);
+        if (e == cudaSuccess) e = cudaMemset(ctx->d_t_ready, 0, (size_t)ctx->max_pairs * 4);
         if (e == cudaSuccess && ctx->d_rope_inv_freq) {
             std::vector<double> f((size_t)c.head_dim / 2);
             for (size_t i = 0; i < f.size(); ++i) f[i] = pow((double)c.rope_theta, -2.0 * (double)i / (double)c.head_dim);
@@ -303,10 +305,10 @@ alora_status alora_destroy(alora_ctx *ctx) {
     if (ctx->d_mlp_t) cudaFree(ctx->d_mlp_t);
     if (ctx->d_mlp_part) cudaFree(ctx->d_mlp_part);
     if (ctx->d_mlp_done) cudaFree(ctx->d_mlp_done);
-    void *ptrs[] = {ctx->d_adapters, ctx->d_token_req, ctx->d_row_adapter, ctx->d_slot, ctx->d_tiles, ctx->d_counts,
-                    ctx->d_seg_scratch, ctx->d_shrink_tiles, ctx->d_t_ready, ctx->d_t, ctx->d_qkv, ctx->d_status, ctx->d_act[0], ctx->d_act[1],
+    void *ptrs[] = {ctx->d_adapters, ctx->d_token_req, ctx->d_row_adapter, ctx->d_slot, ctx->d_pairs, ctx->d_pair_off, ctx->d_counts,
+                    ctx->d_seg_scratch, ctx->d_t_ready, ctx->d_t, ctx->d_qkv, ctx->d_status, ctx->d_act[0], ctx->d_act[1],
                     ctx->d_act[2], ctx->d_act[3], ctx->d_iota, ctx->d_attn_items, ctx->d_attn_off, ctx->d_split_items,
-                    ctx->d_req_scratch, ctx->d_part_o, ctx->d_part_ml, ctx->d_group_done, ctx->d_row_delta,
+                    ctx->d_req_scratch, ctx->d_part_o, ctx->d_part_ml, ctx->d_group_done,
                     ctx->d_skinny_part, ctx->d_skinny_t, ctx->d_skinny_meta, ctx->d_rope_inv_freq, ctx->d_prefix_groups,
                     ctx->d_attn_cta_start, ctx->d_attn_part_o, ctx->d_attn_part_ml};
     for (void *p : ptrs) if (p) cudaFree(p);
@@ -526,7 +528,7 @@ alora_status alora_project_qkv(alora_ctx *ctx, int layer, int mode, const void *
     b.few_row = project_is_few_row(ctx, layer, T) ? 1 : 0;
     int n = launch_metadata(ctx, b, s, kMetaProjection), k;
     if (n < 0) return ALORA_ERR_UNSUPPORTED;
-    if ((k = launch_project(ctx, layer, d_hidden, T, d_qkv, s, nullptr, 0, nullptr)) < 0) return ALORA_ERR_UNSUPPORTED;
+    if ((k = launch_project(ctx, layer, d_hidden, T, R, d_qkv, s, nullptr, 0, nullptr)) < 0) return ALORA_ERR_UNSUPPORTED;
     if (ctx->d_rope_inv_freq != nullptr) {   // the rows handed out are the rotated ones, as they would be cached
         int k2 = launch_rope(ctx, d_qkv, d_positions, T, nullptr, 0, s);
         if (k2 < 0) return ALORA_ERR_UNSUPPORTED;
@@ -667,15 +669,16 @@ alora_status alora_forward_stack(alora_ctx *ctx, int mode, const void *d_hidden_
         }                                                                         \
         n += k;                                                                   \
     } while (0)
-    // The attention lists depend on the batch alone: the first layer builds them for all.  So do the few-row route's
-    // per-token arrays; its adapter facts of all layers are built in the first layer's launch.  (They were rebuilt by
-    // every layer: 63 of 240 us of a layer's decode step of 40 requests in prefix groups.)
-    bool all_few = true;
-    for (int l = 0; l < ctx->cfg.n_layers; ++l) all_few &= project_is_few_row(ctx, l, T);
-    b.n_layers = all_few ? ctx->cfg.n_layers : 1;
+    // The batch's lists depend on the batch alone: the first layer builds them for all, with the few-row route's adapter
+    // facts of all layers.  (They were rebuilt by every layer: 63 of 240 us of a layer's decode step of 40 requests in
+    // prefix groups.)  Only where the layers' projections take different routes does each build its own.
+    int n_few = 0;
+    for (int l = 0; l < ctx->cfg.n_layers; ++l) n_few += project_is_few_row(ctx, l, T) ? 1 : 0;
+    const bool one_route = n_few == 0 || n_few == ctx->cfg.n_layers;
+    b.n_layers = one_route ? ctx->cfg.n_layers : 1;
     for (int l = 0; l < ctx->cfg.n_layers; ++l) {
         const LayerWeights &lw = ctx->layers[l];
-        if (l > 0) b.facts_ready = kMetaAttention | (all_few ? kMetaProjection : 0);
+        if (l > 0) b.facts_ready = kMetaAttention | (one_route ? kMetaProjection : 0);
         ALORA_STEP(launch_rmsnorm(ctx, h, lw.norm_attn, T, ctx->d_act[0], s));
         st = run_layer(ctx, l, ctx->d_act[0], b, h_paged_kv_layers[l], ctx->d_act[1], s);
         if (st != ALORA_OK) return st;

@@ -14,7 +14,6 @@
 namespace alora {
 
 constexpr int kRankPadMax = 64;  // adapters are stored padded to a multiple of 16 rows, <= 64
-constexpr int kRowwiseMaxTokens = 1024;  // largest batch that may take the row-wise delta route of the projection
 constexpr int kMlpChunk = 8192;   // tokens per MLP pass of the stack entry (bounds the gate/up buffer)
 
 // Per (layer, adapter) record as the kernels see it.  A is [3][rpad_max][H] (q, k, v blocks, rows
@@ -40,15 +39,17 @@ struct LayerWeights {
     const void *norm_attn = nullptr, *norm_mlp = nullptr;
 };
 
-// One row-tile of the projection: rows [row_start, row_start + row_count) of the batch, all with
-// the same applied adapter (or -1).  A tile never spans two different applied adapters, so rows
-// whose gate is closed run through tiles that execute the base-only instruction sequence.
-struct ProjTile {
-    int32_t row_start;
-    int32_t row_count;
-    int32_t adapter;  // applied adapter id, -1 = none
-    int32_t pad_;
+// The projection works on dense tiles of kTileRows rows.  A row tile meets the adapters applied to its rows (gate open)
+// one after another: one TilePair per (row tile, adapter that occurs in it).  The pair's t = s A x is kept for the whole
+// tile with the rows of other adapters and the rows with a closed gate set to zero, so the expand step t B^T adds
+// nothing to them.
+constexpr int kTileRows = 128;
+struct TilePair {
+    int32_t tile, adapter;
 };
+// Batches of at most this many rows carry t as the sum of two bf16 values (16 significant bits, for the few rows of a
+// handful of requests), larger ones as one.
+constexpr int kSplitTTokens = 1024;
 
 // One unit of attention work: query tokens [q_start, q_start + q_count) of request `req` (flat
 // token indices), one KV head, keys [kv_start, kv_end) of the request's sequence.
@@ -63,7 +64,6 @@ struct AttnWork {
     int32_t n_splits;
 };
 constexpr int kAttnKeysPerTile = 128;   // keys per K/V tile of the tensor-core attention kernel
-constexpr int kRowwiseAlwaysRows = 24;  // batches of at most this many rows always take the projection's row-wise route
 constexpr int kAttnMinRunTiles = 8;     // shortest run of key tiles given to one block
 constexpr int kAttnCutMinTiles = 128;   // items are cut into runs only when a block has at least this many tiles to do
 constexpr int kAttnCutMinWaves = 3;     // ... and the items make at least this many full rounds over the blocks
@@ -159,18 +159,18 @@ struct alora_ctx {
 
     // per-call workspaces
     int32_t *d_token_req = nullptr, *d_row_adapter = nullptr, *d_slot = nullptr;
-    alora::ProjTile *d_tiles = nullptr;
-    int32_t *d_counts = nullptr;  // [0] projection row tiles, [1] attention work items, [2] row tiles with an adapter,
+    alora::TilePair *d_pairs = nullptr;       // [max_pairs] (row tile, adapter) pairs of the batch, tile after tile
+    int32_t *d_pair_off = nullptr;            // [row tiles + 1] first pair of each row tile
+    int32_t *d_counts = nullptr;  // [1] attention work items, [2] (row tile, adapter) pairs,
                                   // [3] few-row attention items, [4] next unclaimed few-row item,
-                                  // [5] 1 = the projection takes the row-wise route for this batch,
                                   // [6] key tiles of the attention items that are cut into runs, [7] tiles per run,
                                   // [8] attention items taken whole (the first ones), [9] key tiles of those,
                                   // [10], [11] next unclaimed projection item and blocks done, [12] few-row attention blocks done
     int32_t *d_seg_scratch = nullptr;  // [14*max_requests+5] per-request values and merged row runs of the current batch
-    int32_t *d_shrink_tiles = nullptr; // [max_tiles] indices of the row tiles with an adapter
-    int32_t *d_t_ready = nullptr;      // [max_tiles] per row tile: epilogue warps that have published t
+    int32_t *d_t_ready = nullptr;      // [max_pairs] per pair: epilogue warps that have published t (zero between launches)
     int32_t *d_iota = nullptr;         // 0..max_requests: query_start_loc of a decode batch
-    int32_t max_tiles = 0;
+    int32_t max_pairs = 0;
+    int t_slots = 0;                   // 128-row slots of d_t (bf16)
     alora::AttnWork *d_attn_items = nullptr;  // tensor-core attention work list (bf16)
     int32_t *d_attn_off = nullptr;            // [max_requests+1] block offsets per request
     int32_t max_attn_items = 0, attn_q_block = 0;
@@ -186,8 +186,7 @@ struct alora_ctx {
     float *d_part_o = nullptr, *d_part_ml = nullptr;
     int32_t *d_group_done = nullptr;    // [max_split_rows / 16] finished key ranges per (stream, KV head), at its first partial row / 16
     int32_t max_split_items = 0, max_split_rows = 0, small_max_tokens = 0;
-    void *d_t = nullptr;          // [max_tokens][3][RP] rank-r intermediate
-    float *d_row_delta = nullptr; // [min(max_tokens, kRowwiseMaxTokens)][N] fp32 delta rows (bf16 row-wise route)
+    void *d_t = nullptr;          // rank-r intermediate: fp32 [max_tokens][3][RP]; bf16 [pair][1 or 2 summands][128][3][RP]
     // few-row projection (batches of <= 128 rows): K-slice partial products and partial shrink results
     float *d_skinny_part = nullptr;   // [skinny_max_items][128][256] fp32
     float *d_skinny_t = nullptr;      // [slices of the q/k/v projection][128][skinny_p_cap][192] fp32
@@ -260,7 +259,7 @@ struct BatchArgs {
     int all_small;  // host-side knowledge that no request has more than small_max_tokens new tokens (decode)
     int layer = -1; // layer whose adapter table the gate is checked against (-1: no check)
     int few_row = 0; // the projection of this batch takes the few-row route: build FewRowMeta instead of row tiles
-    int n_layers = 1; // few-row route: layers from `layer` on whose FewRowMeta is built (a stack call builds all of them at once)
+    int n_layers = 1; // layers from `layer` on that the projection's facts are built for (a stack call: all of them at once)
     int facts_ready = 0; // bits (kMetaProjection, kMetaAttention): built by an earlier layer of the same stack call
 };
 
@@ -273,8 +272,16 @@ int launch_metadata(alora_ctx *ctx, const BatchArgs &b, cudaStream_t s, int phas
 int launch_repack_adapter(alora_ctx *ctx, int rank, const void *Aq, const void *Bq, const void *Ak,
                           const void *Bk, const void *Av, const void *Bv, void *A_dst, void *B_dst,
                           cudaStream_t s);
-int launch_project(alora_ctx *ctx, int layer, const void *hidden, int T, void *qkv, cudaStream_t s, void *kv_pool,
+int launch_project(alora_ctx *ctx, int layer, const void *hidden, int T, int R, void *qkv, cudaStream_t s, void *kv_pool,
                    int num_pages, bool *kv_appended);
+// Most (row tile, adapter) pairs that a batch of T rows and R requests can have.
+inline int pair_bound(const alora_ctx *ctx, int T, int R) {
+    const long long n_m = (T + kTileRows - 1) / kTileRows, na = ctx->cfg.max_adapters > 0 ? ctx->cfg.max_adapters : 1;
+    long long n = n_m + R;
+    if (n > T) n = T;
+    if (n > n_m * na) n = n_m * na;
+    return (int)n;
+}
 int launch_kv_append(alora_ctx *ctx, const void *qkv, int T, int num_pages, void *pool, cudaStream_t s);
 int launch_cow_tail_pages(alora_ctx *ctx, const int32_t *qsl, const int32_t *seq_lens, int32_t *block_tables, int max_blocks,
                           int num_pages, int R, const int32_t *fresh_pages, void *pool, cudaStream_t s);

@@ -1,8 +1,8 @@
 // Gated multi-adapter q/k/v projection (Eq. 2 / Eq. 5) for batches of many rows: 256 x 192 output tiles.
 //
-// Same computation and the same work list as gemm_tcgen05.cu's tile route (row tiles of up to 128 rows segmented by
-// (adapter, gate); t = s A_k x from leading "shrink items" of the same launch; an adapter tile appends t B_k^T to its
-// K loop; optional KV append in the epilogue), with another tile shape: a block owns TWO row tiles that share the
+// Same computation and the same work list as gemm_tcgen05.cu's tile route (dense row tiles of 128 rows and the
+// (row tile, adapter) pairs that occur; t = s A_k x from leading "shrink items" of the same launch; a tile appends
+// t B_k^T of each of its adapters to its K loop; optional KV append in the epilogue), with another tile shape: a block owns TWO row tiles that share the
 // W tile, 56 KB of operands per 64-wide K block for 8 x 96 tensor-pipe cycles instead of 48 KB for 4 x 128, i.e.
 // 1.3 x the flops per operand byte (one SM cannot fill its shared memory fast enough for the 128 x 256 tile), and
 // 192-wide column tiles so that 2048 rows x 6144 columns make 256 tiles: two rounds over 148 blocks at 86 %.
@@ -10,7 +10,7 @@
 // under the epilogue and its MMAs start on a half as soon as that half has been drained).
 //
 // A 192-wide column tile can straddle the q | k | v boundaries of the fused row.  The expand step therefore takes
-// one K block per (row tile, q/k/v block that the column tile touches): A = that block's 64 (padded-rank) columns
+// one K block per (pair, q/k/v block that the column tile touches): A = that block's 64 (padded-rank) columns
 // of t, B = the adapter's B rows of that block through a 3-D tensor map (rank column, row inside the block,
 // adapter) whose out-of-range rows read as zero, so the columns of the other block get no contribution.
 //
@@ -38,16 +38,16 @@ constexpr int kSmemTotalP = kItemRingOffP + 128 + 1024;
 constexpr int kShrinkColsP = 3 * kTensorRP;        // 192 columns of t = one column tile
 
 struct PairArgs {
-    const ProjTile *tiles;
-    const int32_t *n_row_tiles;
-    int N, K, Nq, Nkv;
+    const TilePair *pairs;          // (row tile, adapter) pairs, nullptr: no adapters in this launch
+    const int32_t *pair_off;        // [row tiles + 1] first pair of each row tile
+    int M, N, K, Nq, Nkv;
     __nv_bfloat16 *out;
     int ldo;
     const AdapterDev *adapters;
-    const int32_t *shrink_tiles;    // row-tile indices that have an adapter ...
-    const int32_t *n_shrink_tiles;  // ... and their count
-    int32_t *t_ready;               // [row tile] epilogue warps that have published their part of t
-    __nv_bfloat16 *t_out;           // [tokens][192]
+    const int32_t *n_pairs;         // shrink items of this launch: one per pair (nullptr: t is there already)
+    const int32_t *row_adapter;     // [M] applied adapter per row (shrink items: which rows of t are kept)
+    int32_t *t_ready;               // [pair] epilogue warps that have published their part of t
+    __nv_bfloat16 *t_out;           // [pair][128][192]
     // KV append fused into the epilogue (nullptr: off), as in gemm_tcgen05.cu
     __nv_bfloat16 *kv_pool;
     const int32_t *slot_map;
@@ -71,28 +71,31 @@ __device__ __forceinline__ void tma_load_3d_p(uint32_t smem_dst, const CUtensorM
 
 // One work item: a shrink item (row tile m[0] only) or two row tiles (m[1] = -1: none) x one column tile.
 struct PairItem {
-    ProjTile t[2];
     int m[2];
-    int n0;
+    int p0[2], p1[2];    // pairs of each row tile
+    int n0, adapter;
     bool shrink;
 };
 __device__ __forceinline__ PairItem decode_pair(const PairArgs &a, int item, int n_shrink, int n_m, int n_n) {
     PairItem g;
-    g.t[1].row_start = 0; g.t[1].row_count = 0; g.t[1].adapter = -1; g.t[1].pad_ = 0;
-    if (item < n_shrink) {
-        g.m[0] = a.shrink_tiles[item];
-        g.m[1] = -1;
-        g.n0 = 0;
-        g.shrink = true;
+    g.n0 = 0; g.adapter = -1; g.m[1] = -1;
+    g.p0[0] = g.p1[0] = g.p0[1] = g.p1[1] = 0;
+    g.shrink = item < n_shrink;
+    if (g.shrink) {
+        const TilePair p = a.pairs[item];
+        g.m[0] = p.tile;
+        g.adapter = p.adapter;
     } else {
         const int j = item - n_shrink;
         g.m[0] = 2 * (j / n_n);
         g.m[1] = g.m[0] + 1 < n_m ? g.m[0] + 1 : -1;
         g.n0 = (j % n_n) * kBNp;
-        g.shrink = false;
+        if (a.pairs) {
+            g.p0[0] = a.pair_off[g.m[0]];
+            g.p1[0] = g.p0[1] = a.pair_off[g.m[0] + 1];
+            g.p1[1] = g.m[1] >= 0 ? a.pair_off[g.m[0] + 2] : g.p0[1];
+        }
     }
-    g.t[0] = a.tiles[g.m[0]];
-    if (g.m[1] >= 0) g.t[1] = a.tiles[g.m[1]];
     return g;
 }
 // first row of q/k/v block `blk` in the fused row, and one past its last
@@ -142,9 +145,9 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
     tc::grid_dep_launch();
     tc::grid_dep_wait();   // the metadata step's lists, the activations: all written by earlier kernels of the stream
 
-    const int n_m = *a.n_row_tiles;
+    const int n_m = (a.M + 127) / 128;
     const int n_n = (a.N + kBNp - 1) / kBNp;
-    const int n_shrink = *a.n_shrink_tiles;
+    const int n_shrink = a.n_pairs ? *a.n_pairs : 0;
     const int total = n_shrink + ((n_m + 1) / 2) * n_n;
     const int kb_main = (a.K + kBKp - 1) / kBKp;
 
@@ -188,33 +191,39 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                     if (!tc::mbar_wait(empty_bar(s), ((kc / kStagesP) & 1) ^ 1, abort_flag)) { ok = false; break; }
                     const uint32_t sa = smem_base + s * kStageBytesP, sb = sa + 2 * kHalfAp;
                     tc::mbar_arrive_expect_tx(full_bar(s), (two ? 2 : 1) * kHalfAp + kBBytesP);
-                    tc::tma_load_2d(sa, &tmX, full_bar(s), kb * kBKp, g.t[0].row_start);
-                    if (two) tc::tma_load_2d(sa + kHalfAp, &tmX, full_bar(s), kb * kBKp, g.t[1].row_start);
-                    if (g.shrink) tc::tma_load_2d(sb, &tmS, full_bar(s), kb * kBKp, g.t[0].adapter * kShrinkColsP);
+                    tc::tma_load_2d(sa, &tmX, full_bar(s), kb * kBKp, g.m[0] * 128);
+                    if (two) tc::tma_load_2d(sa + kHalfAp, &tmX, full_bar(s), kb * kBKp, g.m[1] * 128);
+                    if (g.shrink) tc::tma_load_2d(sb, &tmS, full_bar(s), kb * kBKp, g.adapter * kShrinkColsP);
                     else tc::tma_load_2d(sb, &tmW, full_bar(s), kb * kBKp, g.n0);
                 }
                 if (g.shrink) continue;
-                // expand: per row tile with an adapter, one K block per q/k/v block the column tile touches
+                // expand: per pair of the row tiles, one K block per q/k/v block the column tile touches
                 for (int h = 0; h < 2 && ok; ++h) {
-                    if (g.m[h] < 0 || g.t[h].adapter < 0) continue;
-                    // t of this row tile is written by a shrink item (earlier in the list, so claimed by a running
-                    // block): wait until its four epilogue warps have published, then order the TMA read after it
-                    const long long t0 = clock64();
-                    while (ld_acquire_p(a.t_ready + g.m[h]) < 4) {
-                        if (*abort_flag || clock64() - t0 > tc::kWaitCycleLimit) { *abort_flag = 1; ok = false; break; }
-                    }
-                    if (!ok) break;
-                    asm volatile("fence.proxy.async.global;" ::: "memory");
-                    for (int blk = 0; blk < 3 && ok; ++blk) {
-                        if (!touches(a, g.n0, blk)) continue;
-                        const int s = kc % kStagesP;
-                        if (!tc::mbar_wait(empty_bar(s), ((kc / kStagesP) & 1) ^ 1, abort_flag)) { ok = false; break; }
-                        const uint32_t sa = smem_base + s * kStageBytesP, sb = sa + 2 * kHalfAp;
-                        tc::mbar_arrive_expect_tx(full_bar(s), kHalfAp + kBBytesP);
-                        tc::tma_load_2d(sa + h * kHalfAp, &tmT, full_bar(s), blk * kTensorRP, g.t[h].row_start);
-                        tma_load_3d_p(sb, blk == 0 ? &tmB0 : (blk == 1 ? &tmB1 : &tmB2), full_bar(s), 0,
-                                      g.n0 - blk_start(a, blk), g.t[h].adapter);
-                        ++kc;
+                    int next_ad = g.p0[h] < g.p1[h] ? a.pairs[g.p0[h]].adapter : -1;
+                    for (int p = g.p0[h]; p < g.p1[h] && ok; ++p) {
+                        const int adapter = next_ad;
+                        if (p + 1 < g.p1[h]) next_ad = a.pairs[p + 1].adapter;   // (in flight while this pair is waited for)
+                        if (n_shrink > 0) {
+                            // t of this pair is written by a shrink item (earlier in the list, so claimed by a running
+                            // block): wait until its four epilogue warps have published, then order the TMA read after it
+                            const long long t0 = clock64();
+                            while (ld_acquire_p(a.t_ready + p) < 4) {
+                                if (*abort_flag || clock64() - t0 > tc::kWaitCycleLimit) { *abort_flag = 1; ok = false; break; }
+                            }
+                            if (!ok) break;
+                            asm volatile("fence.proxy.async.global;" ::: "memory");
+                        }
+                        for (int blk = 0; blk < 3 && ok; ++blk) {
+                            if (!touches(a, g.n0, blk)) continue;
+                            const int s = kc % kStagesP;
+                            if (!tc::mbar_wait(empty_bar(s), ((kc / kStagesP) & 1) ^ 1, abort_flag)) { ok = false; break; }
+                            const uint32_t sa = smem_base + s * kStageBytesP, sb = sa + 2 * kHalfAp;
+                            tc::mbar_arrive_expect_tx(full_bar(s), kHalfAp + kBBytesP);
+                            tc::tma_load_2d(sa + h * kHalfAp, &tmT, full_bar(s), blk * kTensorRP, p * 128);
+                            tma_load_3d_p(sb, blk == 0 ? &tmB0 : (blk == 1 ? &tmB1 : &tmB2), full_bar(s), 0,
+                                          g.n0 - blk_start(a, blk), adapter);
+                            ++kc;
+                        }
                     }
                 }
             }
@@ -242,6 +251,8 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
             if (item < 0) { ok = item == -1; break; }
             const PairItem g = decode_pair(a, item, n_shrink, n_m, n_n);
             const bool two = g.m[1] >= 0;
+            // MMA steps of the row tiles' adapters, one per lane, loaded while the main loop runs
+            const int my_steps = g.p0[0] + lane < g.p1[1] ? a.adapters[a.pairs[g.p0[0] + lane].adapter].rpad / 16 : 0;
             for (int kb = 0; kb < kb_main && ok; ++kb, ++kc) {
                 const int s = kc % kStagesP;
                 if (!wait_all(full_bar(s), (kc / kStagesP) & 1)) { ok = false; break; }
@@ -267,10 +278,10 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                 }
             }
             if (!ok) break;
-            if (!g.shrink) {
-                for (int h = 0; h < 2 && ok; ++h) {
-                    if (g.m[h] < 0 || g.t[h].adapter < 0) continue;
-                    const int steps = a.adapters[g.t[h].adapter].rpad / 16;
+            for (int h = 0; h < 2 && ok; ++h) {
+                for (int p = g.p0[h]; p < g.p1[h] && ok; ++p) {
+                    const int at = p - g.p0[0];   // (the pairs of the two row tiles follow one another)
+                    const int steps = at < 32 ? __shfl_sync(0xffffffffu, my_steps, at) : a.adapters[a.pairs[p].adapter].rpad / 16;
                     for (int blk = 0; blk < 3 && ok; ++blk) {
                         if (!touches(a, g.n0, blk)) continue;
                         const int s = kc % kStagesP;
@@ -286,8 +297,8 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                         ++kc;
                     }
                 }
-                if (!ok) break;
             }
+            if (!ok) break;
             if (leader) tc::mma_commit(accf_bar);      // accumulators complete
         }
         if (!ok && leader) {
@@ -315,27 +326,17 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                 continue;
             }
             if (g.shrink) {
-                // t = s A x of this row tile: 192 columns, scaled, rounded to bf16
-                const ProjTile t = g.t[0];
-                const bool row_ok = r < t.row_count;
-                const float scale = a.adapters[t.adapter].scale;
-                __nv_bfloat16 *trow = a.t_out + (size_t)(t.row_start + r) * kShrinkColsP;
+                // t = s A x of this pair: 192 columns, zero in the rows that do not use the adapter
+                const int row = g.m[0] * 128 + r;
+                const bool use = row < a.M && a.row_adapter[row] == g.adapter;
+                const float scale = a.adapters[g.adapter].scale;
+                __nv_bfloat16 *trow = a.t_out + ((size_t)item * 128 + r) * kShrinkColsP;
 #pragma unroll 1
                 for (int c = 0; c < kShrinkColsP; c += 32) {
                     uint32_t v[32];
                     tc::tmem_ld_32x32(tmem_base + c + ((uint32_t)(q * 32) << 16), v);
                     tc::tmem_ld_wait();
-                    if (row_ok) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            uint4 o;
-                            o.x = tc::pack_bf16(__uint_as_float(v[8 * j]) * scale, __uint_as_float(v[8 * j + 1]) * scale);
-                            o.y = tc::pack_bf16(__uint_as_float(v[8 * j + 2]) * scale, __uint_as_float(v[8 * j + 3]) * scale);
-                            o.z = tc::pack_bf16(__uint_as_float(v[8 * j + 4]) * scale, __uint_as_float(v[8 * j + 5]) * scale);
-                            o.w = tc::pack_bf16(__uint_as_float(v[8 * j + 6]) * scale, __uint_as_float(v[8 * j + 7]) * scale);
-                            *reinterpret_cast<uint4 *>(trow + c + 8 * j) = o;
-                        }
-                    }
+                    tc::store_t<32>(reinterpret_cast<float(&)[32]>(v), scale, use, trow + c, nullptr);
                 }
                 tc::tc_fence_before();
                 // publish: the rows are read by other blocks through TMA (async proxy)
@@ -343,7 +344,7 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                 __threadfence();
                 __syncwarp();
                 if (lane == 0) {
-                    atomicAdd(a.t_ready + g.m[0], 1);
+                    atomicAdd(a.t_ready + item, 1);
                     tc::mbar_arrive(acce_bar(0));
                 }
                 continue;
@@ -351,13 +352,13 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
             {
                 const int h = my_h;
                 if (g.m[h] >= 0) {
-                    const ProjTile t = g.t[h];
-                    const bool row_ok = r < t.row_count;
-                    __nv_bfloat16 *orow = a.out + (size_t)(t.row_start + r) * a.ldo + g.n0;
+                    const int row = g.m[h] * 128 + r;
+                    const bool row_ok = row < a.M;
+                    __nv_bfloat16 *orow = a.out + (size_t)row * a.ldo + g.n0;
                     // fused KV append: where this row's k / v columns go in the page pool
                     int kv_page = -1, kv_row = 0;
                     if (a.kv_pool != nullptr && row_ok && g.n0 + kBNp > a.Nq) {
-                        const int slot = a.slot_map[t.row_start + r];
+                        const int slot = a.slot_map[row];
                         if (slot >= 0) {
                             kv_page = slot / a.kv_page_size;
                             kv_row = slot % a.kv_page_size;
@@ -401,7 +402,7 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
     tc::tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && *abort_flag) report(a.status, ALORA_ERR_TIMEOUT);
-    if (threadIdx.x == 0) tc::item_counter_release(a.item_counters);
+    if (threadIdx.x == 0) tc::item_counter_release(a.item_counters, a.t_ready, n_shrink);
     if (warp == 1) {
         tc::tc_fence_after();
         tc::tmem_dealloc(tmem_base, 512);
@@ -441,13 +442,17 @@ bool build_pair_maps(alora_ctx *ctx, int layer) {
     return ok;
 }
 
-// Returns the kernels launched (1), 0 when the batch is better served by the 128-row kernel (nothing launched) or
-// -1 on error.  Only for batches too large for the row-wise route (the decision must not depend on the mode, so
-// that rows with a closed gate come out bit-identical to the base-only projection of the same batch).
-int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T, void *qkv, cudaStream_t s,
+bool launch_shrink_tc(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap &tmA, const AdapterDev *adapters,
+                      int T, int K, int max_pairs, int t_parts, cudaStream_t s);  // shrink_tcgen05.cu
+bool shrink_apart(const alora_ctx *ctx, int T, int R, int items);                  // gemm_tcgen05.cu
+
+// Returns the kernels launched, 0 when the batch is better served by the 128-row kernel (nothing launched) or
+// -1 on error.  Only for batches of more than kSplitTTokens rows (one summand of t; the decision must not depend on the
+// mode, so that rows with a closed gate come out bit-identical to the base-only projection of the same batch).
+int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int R, void *qkv, cudaStream_t s,
                            void *kv_pool, int num_pages) {
     const Dims &d = ctx->d;
-    if (T <= kRowwiseMaxTokens || d.H % 8 != 0 || d.N % 8 != 0 || d.Nq % 8 != 0 || d.Nkv % 8 != 0) return 0;
+    if (T <= kSplitTTokens || d.H % 8 != 0 || d.N % 8 != 0 || d.Nq % 8 != 0 || d.Nkv % 8 != 0) return 0;
     const int G = ctx->sm_count;
     const int n_n = (d.N + kBNp - 1) / kBNp, n_n256 = (d.N + 255) / 256;
     const int items = ((T + 255) / 256) * n_n, items128 = ((T + 127) / 128) * n_n256;
@@ -457,7 +462,7 @@ int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T,
     const TcLayerMaps &lm = ctx->tc_maps[layer];
     CUtensorMap tmX, tmT;
     if (!make_tensor_map_bf16(&tmX, hidden, T, d.H, d.H, 128)) return -1;
-    if (!make_tensor_map_bf16(&tmT, ctx->d_t, ctx->cfg.max_tokens, 3 * kTensorRP, 3 * kTensorRP, 128)) return -1;
+    if (!make_tensor_map_bf16(&tmT, ctx->d_t, (uint64_t)ctx->t_slots * 128, 3 * kTensorRP, 3 * kTensorRP, 128)) return -1;
     static bool attr_set[64] = {};
     const int dev = ctx->cfg.device;
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
@@ -467,11 +472,17 @@ int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T,
         attr_set[dev] = true;
     }
     PairArgs g{};
-    g.tiles = ctx->d_tiles; g.n_row_tiles = ctx->d_counts; g.N = d.N; g.K = d.H; g.Nq = d.Nq; g.Nkv = d.Nkv;
+    g.M = T; g.N = d.N; g.K = d.H; g.Nq = d.Nq; g.Nkv = d.Nkv;
     g.out = (__nv_bfloat16 *)qkv; g.ldo = d.N;
     g.adapters = ctx->d_adapters + (size_t)layer * ctx->cfg.max_adapters;
-    g.shrink_tiles = ctx->d_shrink_tiles; g.n_shrink_tiles = ctx->d_counts + 2;
-    g.t_ready = ctx->d_t_ready; g.t_out = (__nv_bfloat16 *)ctx->d_t;
+    const bool have_adapters = ctx->layer_has_adapter[layer] != 0;
+    const bool apart = have_adapters && shrink_apart(ctx, T, R, items);
+    const int max_pairs = have_adapters ? pair_bound(ctx, T, R) : 0;
+    if (have_adapters) { g.pairs = ctx->d_pairs; g.pair_off = ctx->d_pair_off; }
+    if (have_adapters && !apart) {
+        g.n_pairs = ctx->d_counts + 2; g.row_adapter = ctx->d_row_adapter;
+        g.t_ready = ctx->d_t_ready; g.t_out = (__nv_bfloat16 *)ctx->d_t;
+    }
     g.item_counters = ctx->d_counts + 10;
     if (kv_pool != nullptr) {
         int shift = 0;
@@ -480,13 +491,12 @@ int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T,
         g.kv_page_size = d.page; g.kv_num_pages = num_pages;
     }
     g.status = ctx->d_status;
-    const int max_row_tiles = std::min(std::min(ctx->max_tiles, T / 128 + 2 * ctx->cfg.max_requests + 2), T);
-    const int max_items = max_row_tiles + ((max_row_tiles + 1) / 2) * n_n;
-    const int grid = std::max(1, std::min(G, max_items));
+    const int grid = std::max(1, std::min(G, items + (apart ? 0 : max_pairs)));
+    if (apart && !launch_shrink_tc(ctx, tmX, lm.a_all, g.adapters, T, d.H, max_pairs, 1, s)) return -1;
     if (launch_kernel(gemm_pair_tcgen05_kernel, dim3(grid), dim3(kThreadsP), kSmemTotalP, s, true, tmX, lm.wqkv192, tmT,
                       lm.a_all, lm.b_blk[0], lm.b_blk[1], lm.b_blk[2], g) != cudaSuccess)
         return -1;
-    return 1;
+    return apart ? 2 : 1;
 }
 
 }  // namespace alora

@@ -11,20 +11,20 @@
 //                      add / scale, round to bf16, 16-byte row-predicated stores.  The second
 //                      accumulator lets the next tile's main loop overlap this epilogue.
 //
-// Row tiles come from the batch-metadata step: all rows of a tile have the same applied adapter.
-// For a tile with an adapter the main K loop (the base term W x of Eq. 5) is followed by one more
-// K block whose operands are t = s A x (rows of the tile) and the adapter's B rows of this column
-// tile, i.e. the delta s B (A x) is accumulated by the same tensor-core instruction stream.  Tiles
-// without an adapter execute exactly the base-only sequence: that is what makes gated-off rows
-// bit-identical to a base-only call (Prop. 1).
+// Row tiles are dense.  For every adapter that some row of the tile uses (the (row tile, adapter) pairs of the
+// batch-metadata step) the main K loop (the base term W x of Eq. 5) is followed by further K blocks whose operands are
+// t = s A x and the adapter's B rows of this column tile, i.e. the delta s B (A x) is accumulated by the same
+// tensor-core instruction stream.  The rows of t that do not use the adapter (another adapter, or a closed gate) are
+// zero, so those rows of the accumulator are added zeros: a row whose gate is closed keeps the bits of a base-only
+// call (Prop. 1).  (Cutting the row tiles at every change of adapter instead left most tiles of a batch of short
+// requests nearly empty, and a per-row delta beside dense tiles took 190 us for 742 rows.)
 //
-// Where t = s A x comes from.  With 256-wide column tiles the shrink is part of this kernel: the first
-// work items of the launch are one "shrink item" per adapter row tile, whose B operand is the adapter's
-// 192 A rows (q, k, v blocks, rank padded to 64) and whose epilogue writes t and then raises a per-tile
-// ready counter in global memory.  A projection item of an adapter tile waits (bounded) for that
-// counter before it loads t for its extra K block; since every block walks the item list in increasing
-// order and shrink items come first, the block that owns a shrink item never waits before finishing it.
-// With 128-wide column tiles the shrink runs as a separate cluster split-K kernel (shrink_tcgen05.cu).
+// Where t = s A x comes from.  With 256-wide column tiles the shrink can be part of this kernel: the first
+// work items of the launch are one "shrink item" per pair, whose B operand is the adapter's
+// 192 A rows (q, k, v blocks, rank padded to 64) and whose epilogue writes t and then raises a per-pair
+// ready counter in global memory.  A projection item waits (bounded) for the counters of its row tile's pairs
+// before it loads their t; shrink items are claimed first (claim_order.h).  With 128-wide column tiles, and where the
+// shrink items would add a round over the blocks, the shrink is a cluster split-K kernel before (shrink_tcgen05.cu).
 // No split-K, no atomics in the arithmetic: results are run-to-run deterministic.
 //
 // Every wait is bounded (tc::mbar_wait); on expiry the block records ALORA_ERR_TIMEOUT, drains its
@@ -45,8 +45,8 @@ struct GemmArgs {
     // 64-row box: the other half of the tile in shared memory is never filled, the accumulator rows it feeds are
     // never read, and the shared-memory fill of a stage, which bounds this shape, drops by a third.
     int a_tile_bytes;
-    const ProjTile *tiles;        // nullptr: dense row tiles 0..ceil(M/128)-1, no adapters
-    const int32_t *n_row_tiles;   // device count of `tiles` entries (when tiles != nullptr)
+    const TilePair *pairs;          // (row tile, adapter) pairs of the batch, nullptr: no adapters in this launch
+    const int32_t *pair_off;        // [row tiles + 1] first pair of each row tile
     int M, N, K;
     __nv_bfloat16 *out;
     int ldo;
@@ -54,16 +54,11 @@ struct GemmArgs {
     const AdapterDev *adapters;     // this layer's adapter table (expand), or nullptr
     int Nq, Nkv;                    // block boundaries of the fused output row (expand)
     int total_adapter_rows;         // rows per adapter in the B_all map (= N of the layer)
-    const int32_t *shrink_tiles;    // fused shrink: row-tile indices that have an adapter ...
-    const int32_t *n_shrink_tiles;  // ... and their count (nullptr: no shrink items in this launch)
-    int32_t *t_ready;               // [row tile] epilogue warps that have published their part of t
-    __nv_bfloat16 *t_out;           // [tokens][192]
-    // Row-wise route (batches of few rows per tile): when *rowwise_flag is set by the metadata step the launch
-    // ignores the tile list, walks dense row tiles without any adapter, and its epilogue adds row_delta[row][n]
-    // (fp32, made by lora_delta_rows_kernel) to the rows whose row_adapter is >= 0.
-    const int32_t *rowwise_flag;
-    const float *row_delta;
-    const int32_t *row_adapter;
+    const int32_t *n_pairs;         // shrink items in this launch: one per pair (nullptr: t is there already)
+    const int32_t *row_adapter;     // [M] applied adapter per row (shrink items: which rows of t are kept)
+    int32_t *t_ready;               // [pair] epilogue warps that have published their part of t
+    __nv_bfloat16 *t_out;           // [pair][t_parts][128][192]
+    int t_parts;                    // t is the sum of this many bf16 values (1 or 2)
     // KV append fused into the epilogue (nullptr: off): columns Nq .. N of row t also go to the paged cache,
     // pool[page][plane][head][row in page][:] with page * page_size + row = slot_map[t] (-1: token rejected, skipped)
     __nv_bfloat16 *kv_pool;
@@ -86,39 +81,31 @@ struct GemmSmem {
     static constexpr int kTotal = kItemRingOffset + 128 + 1024;  // barriers, item ring, slack for 1024-byte alignment
 };
 
-__device__ __forceinline__ ProjTile load_tile(const GemmArgs &a, int m, bool dense) {
-    if (a.tiles && !dense) return a.tiles[m];
-    ProjTile t;
-    t.row_start = m * kBM;
-    t.row_count = min(kBM, a.M - m * kBM);
-    t.adapter = -1;
-    t.pad_ = 0;
-    return t;
-}
-
 constexpr int kShrinkCols = 3 * kTensorRP;  // 192 columns of t: q, k, v blocks of 64 padded rank columns
 
-// Work item `item` of a launch: shrink items first (one per adapter row tile), then the projection's
+// Work item `item` of a launch: shrink items first (one per pair), then the projection's
 // (row tile, column tile) pairs.
 struct GemmItem {
-    ProjTile t;
-    int m;        // row-tile index
-    int n0;       // first output column (projection items)
+    int m;            // row-tile index
+    int n0;           // first output column (projection items)
+    int p0, p1;       // projection items: the row tile's pairs
+    int adapter;      // shrink items
     bool shrink;
 };
-__device__ __forceinline__ GemmItem decode_item(const GemmArgs &a, int item, int n_shrink, int n_n, int BN, bool dense) {
+__device__ __forceinline__ GemmItem decode_item(const GemmArgs &a, int item, int n_shrink, int n_n, int BN) {
     GemmItem g;
-    if (item < n_shrink) {
-        g.m = a.shrink_tiles[item];
-        g.n0 = 0;
-        g.shrink = true;
+    g.n0 = 0; g.p0 = 0; g.p1 = 0; g.adapter = -1;
+    g.shrink = item < n_shrink;
+    if (g.shrink) {
+        const TilePair p = a.pairs[item];
+        g.m = p.tile;
+        g.adapter = p.adapter;
     } else {
         const int j = item - n_shrink;
         g.m = j / n_n;
         g.n0 = (j % n_n) * BN;
-        g.shrink = false;
+        if (a.pairs) { g.p0 = a.pair_off[g.m]; g.p1 = a.pair_off[g.m + 1]; }
     }
-    g.t = load_tile(a, g.m, dense);
     return g;
 }
 
@@ -172,10 +159,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     tc::grid_dep_launch();
     tc::grid_dep_wait();   // the metadata step's lists, the activations: all written by earlier kernels of the stream
 
-    const bool dense = a.rowwise_flag != nullptr && *a.rowwise_flag != 0;
-    const int n_m = (a.tiles && !dense) ? *a.n_row_tiles : (a.M + kBM - 1) / kBM;
+    const int n_m = (a.M + kBM - 1) / kBM;
     const int n_n = (a.N + BN - 1) / BN;
-    const int n_shrink = (BN >= kShrinkCols && a.n_shrink_tiles && !dense) ? *a.n_shrink_tiles : 0;
+    const int n_shrink = (BN >= kShrinkCols && a.n_pairs) ? *a.n_pairs : 0;
     const int total = n_shrink + n_m * n_n;
     const int kb_main = (a.K + kBK - 1) / kBK;
 
@@ -213,38 +199,41 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 }
                 if (!ring.put(item, abort_flag)) { ok = false; break; }
                 if (item < 0) break;
-                const GemmItem g = decode_item(a, item, n_shrink, n_n, BN, dense);
-                const ProjTile t = g.t;
-                const int n0 = g.n0;
-                const int extra = (!g.shrink && t.adapter >= 0) ? 1 : 0;
-                for (int kb = 0; kb < kb_main + extra; ++kb, ++kc) {
+                const GemmItem g = decode_item(a, item, n_shrink, n_n, BN);
+                const int row0 = g.m * kBM, n0 = g.n0;
+                for (int kb = 0; kb < kb_main; ++kb, ++kc) {
                     const int s = kc % kStages;
                     if (!tc::mbar_wait(empty_bar(s), ((kc / kStages) & 1) ^ 1, abort_flag)) { ok = false; break; }
                     const uint32_t sa = smem_base + s * S::kStageBytes, sb = sa + S::kABytes;
-                    if (g.shrink) {
-                        tc::mbar_arrive_expect_tx(full_bar(s), a_bytes + kShrinkCols * kBK * 2);
-                        tc::tma_load_2d(sa, &tmA, full_bar(s), kb * kBK, t.row_start);
-                        tc::tma_load_2d(sb, &tmS, full_bar(s), kb * kBK, t.adapter * kShrinkCols);
-                    } else if (kb < kb_main) {
-                        tc::mbar_arrive_expect_tx(full_bar(s), a_bytes + S::kBBytes);
-                        tc::tma_load_2d(sa, &tmA, full_bar(s), kb * kBK, t.row_start);
-                        tc::tma_load_2d(sb, &tmB, full_bar(s), kb * kBK, n0);
-                    } else {
-                        if (n_shrink > 0) {
-                            // t of this row tile is written by a shrink item, which comes earlier in the list and has
-                            // therefore been claimed by a running block: wait until its four epilogue warps have
-                            // published, then order the TMA read after their writes
-                            const long long t0 = clock64();
-                            while (ld_acquire(a.t_ready + g.m) < 4) {
-                                if (*abort_flag || clock64() - t0 > tc::kWaitCycleLimit) { *abort_flag = 1; ok = false; break; }
-                            }
-                            if (!ok) break;
-                            fence_proxy_async_global();
+                    tc::mbar_arrive_expect_tx(full_bar(s), a_bytes + (g.shrink ? kShrinkCols * kBK * 2 : S::kBBytes));
+                    tc::tma_load_2d(sa, &tmA, full_bar(s), kb * kBK, row0);
+                    if (g.shrink) tc::tma_load_2d(sb, &tmS, full_bar(s), kb * kBK, g.adapter * kShrinkCols);
+                    else tc::tma_load_2d(sb, &tmB, full_bar(s), kb * kBK, n0);
+                }
+                // expand: per adapter of the row tile one K block for each summand of t
+                int next_ad = g.p0 < g.p1 ? a.pairs[g.p0].adapter : -1;
+                for (int p = g.p0; p < g.p1 && ok; ++p) {
+                    const int adapter = next_ad;
+                    if (p + 1 < g.p1) next_ad = a.pairs[p + 1].adapter;   // (in flight while this pair is waited for)
+                    if (n_shrink > 0) {
+                        // t of this pair is written by a shrink item, which comes earlier in the list and has
+                        // therefore been claimed by a running block: wait until its four epilogue warps have
+                        // published, then order the TMA read after their writes
+                        const long long t0 = clock64();
+                        while (ld_acquire(a.t_ready + p) < 4) {
+                            if (*abort_flag || clock64() - t0 > tc::kWaitCycleLimit) { *abort_flag = 1; ok = false; break; }
                         }
+                        if (!ok) break;
+                        fence_proxy_async_global();
+                    }
+                    const int blk = n0 < a.Nq ? 0 : (n0 < a.Nq + a.Nkv ? 1 : 2);
+                    for (int part = 0; part < a.t_parts; ++part, ++kc) {
+                        const int s = kc % kStages;
+                        if (!tc::mbar_wait(empty_bar(s), ((kc / kStages) & 1) ^ 1, abort_flag)) { ok = false; break; }
+                        const uint32_t sa = smem_base + s * S::kStageBytes, sb = sa + S::kABytes;
                         tc::mbar_arrive_expect_tx(full_bar(s), S::kStageBytes);
-                        const int blk = n0 < a.Nq ? 0 : (n0 < a.Nq + a.Nkv ? 1 : 2);
-                        tc::tma_load_2d(sa, &tmT, full_bar(s), blk * kTensorRP, t.row_start);
-                        tc::tma_load_2d(sb, &tmL, full_bar(s), 0, t.adapter * a.total_adapter_rows + n0);
+                        tc::tma_load_2d(sa, &tmT, full_bar(s), blk * kTensorRP, (p * a.t_parts + part) * kBM);
+                        tc::tma_load_2d(sb, &tmL, full_bar(s), 0, adapter * a.total_adapter_rows + n0);
                     }
                 }
             }
@@ -275,30 +264,40 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             while (ok) {
                 const int item = ring.take(abort_flag);
                 if (item < 0) { ok = item == -1; break; }
-                const GemmItem g = decode_item(a, item, n_shrink, n_n, BN, dense);
-                const ProjTile t = g.t;
-                const int extra = (!g.shrink && t.adapter >= 0) ? 1 : 0;
-                const int extra_steps = extra ? a.adapters[t.adapter].rpad / 16 : 0;
+                const GemmItem g = decode_item(a, item, n_shrink, n_n, BN);
+                // MMA steps of the row tile's adapters, one per lane, loaded while the main loop runs
+                const int my_steps = g.p0 + lane < g.p1 ? a.adapters[a.pairs[g.p0 + lane].adapter].rpad / 16 : 0;
                 const uint32_t idesc = g.shrink ? idesc_shrink : idesc_main;
                 const uint32_t acc = it & 1;
                 if (!wait_all(acce_bar(acc), ((it >> 1) & 1) ^ 1)) { ok = false; break; }
                 tc::tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * BN;
-                for (int kb = 0; kb < kb_main + extra; ++kb, ++kc) {
+                for (int kb = 0; kb < kb_main; ++kb, ++kc) {
                     const int s = kc % kStages;
                     if (!wait_all(full_bar(s), (kc / kStages) & 1)) { ok = false; break; }
                     tc::tc_fence_after();
                     const uint32_t sa = smem_base + s * S::kStageBytes, sb = sa + S::kABytes;
                     const uint64_t da = tc::smem_desc_k_sw128(sa), db = tc::smem_desc_k_sw128(sb);
                     if (leader) {
-                        if (kb < kb_main) {
 #pragma unroll
-                            for (int k = 0; k < kBK / 16; ++k)
-                                tc::mma_bf16(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
-                        } else {
-                            for (int k = 0; k < extra_steps; ++k) tc::mma_bf16(d_tmem, da + 2 * k, db + 2 * k, idesc, 1u);
-                        }
+                        for (int k = 0; k < kBK / 16; ++k)
+                            tc::mma_bf16(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
                         tc::mma_commit(empty_bar(s));  // slot reusable once these MMAs have read it
+                    }
+                }
+                for (int p = g.p0; p < g.p1 && ok; ++p) {
+                    const int at = p - g.p0;
+                    const int steps = at < 32 ? __shfl_sync(0xffffffffu, my_steps, at) : a.adapters[a.pairs[p].adapter].rpad / 16;
+                    for (int part = 0; part < a.t_parts; ++part, ++kc) {
+                        const int s = kc % kStages;
+                        if (!wait_all(full_bar(s), (kc / kStages) & 1)) { ok = false; break; }
+                        tc::tc_fence_after();
+                        const uint32_t sa = smem_base + s * S::kStageBytes, sb = sa + S::kABytes;
+                        const uint64_t da = tc::smem_desc_k_sw128(sa), db = tc::smem_desc_k_sw128(sb);
+                        if (leader) {
+                            for (int k = 0; k < steps; ++k) tc::mma_bf16(d_tmem, da + 2 * k, db + 2 * k, idesc, 1u);
+                            tc::mma_commit(empty_bar(s));
+                        }
                     }
                 }
                 if (!ok) break;
@@ -319,34 +318,24 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         while (ok) {
             const int item = ring.take(abort_flag);
             if (item < 0) break;
-            const GemmItem g = decode_item(a, item, n_shrink, n_n, BN, dense);
-            const ProjTile t = g.t;
-            const int n0 = g.n0;
+            const GemmItem g = decode_item(a, item, n_shrink, n_n, BN);
+            const int n0 = g.n0, row = g.m * kBM + q * 32 + lane;   // this thread's row
             const uint32_t acc = it & 1;
             if (!tc::mbar_wait(accf_bar(acc), (it >> 1) & 1, abort_flag)) { ok = false; break; }
             tc::tc_fence_after();
-            const int r = q * 32 + lane;
-            const bool row_ok = r < t.row_count;
+            const bool row_ok = row < a.M;
             if (g.shrink) {
-                // t = s A x of this row tile: 192 columns, scaled, rounded to bf16
-                const float scale = a.adapters[t.adapter].scale;
-                __nv_bfloat16 *trow = a.t_out + (size_t)(t.row_start + r) * kShrinkCols;
+                // t = s A x of this pair: 192 columns, zero in the rows that do not use the adapter
+                const float scale = a.adapters[g.adapter].scale;
+                const bool use = row_ok && a.row_adapter[row] == g.adapter;
+                __nv_bfloat16 *trow = a.t_out + ((size_t)item * a.t_parts * kBM + q * 32 + lane) * kShrinkCols;
+                __nv_bfloat16 *tlow = a.t_parts > 1 ? trow + (size_t)kBM * kShrinkCols : nullptr;
 #pragma unroll 1
                 for (int c = 0; c < kShrinkCols && c < BN; c += 32) {
                     uint32_t v[32];
                     tc::tmem_ld_32x32(tmem_base + acc * BN + c + ((uint32_t)(q * 32) << 16), v);
                     tc::tmem_ld_wait();
-                    if (row_ok) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            uint4 o;
-                            o.x = tc::pack_bf16(__uint_as_float(v[8 * j]) * scale, __uint_as_float(v[8 * j + 1]) * scale);
-                            o.y = tc::pack_bf16(__uint_as_float(v[8 * j + 2]) * scale, __uint_as_float(v[8 * j + 3]) * scale);
-                            o.z = tc::pack_bf16(__uint_as_float(v[8 * j + 4]) * scale, __uint_as_float(v[8 * j + 5]) * scale);
-                            o.w = tc::pack_bf16(__uint_as_float(v[8 * j + 6]) * scale, __uint_as_float(v[8 * j + 7]) * scale);
-                            *reinterpret_cast<uint4 *>(trow + c + 8 * j) = o;
-                        }
-                    }
+                    tc::store_t<32>(reinterpret_cast<float(&)[32]>(v), scale, use, trow + c, tlow ? tlow + c : nullptr);
                 }
                 tc::tc_fence_before();
                 // publish: the rows are read by other blocks through TMA (async proxy)
@@ -354,21 +343,18 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 __threadfence();
                 __syncwarp();
                 if (lane == 0) {
-                    atomicAdd(a.t_ready + g.m, 1);
+                    atomicAdd(a.t_ready + item, 1);
                     tc::mbar_arrive(acce_bar(acc));
                 }
                 ++it;
                 continue;
             }
-            __nv_bfloat16 *orow = a.out + (size_t)(t.row_start + r) * a.ldo + n0;
-            const __nv_bfloat16 *rrow = a.residual ? a.residual + (size_t)(t.row_start + r) * a.ldo + n0 : nullptr;
-            // row-wise delta: only rows with an applied adapter add anything (a gated-off row never sees "+ 0")
-            const float *drow = (dense && row_ok && a.row_adapter[t.row_start + r] >= 0)
-                                    ? a.row_delta + (size_t)(t.row_start + r) * a.N + n0 : nullptr;
+            __nv_bfloat16 *orow = a.out + (size_t)row * a.ldo + n0;
+            const __nv_bfloat16 *rrow = a.residual ? a.residual + (size_t)row * a.ldo + n0 : nullptr;
             // fused KV append: where this row's k / v columns go in the page pool
             int kv_page = -1, kv_row = 0;
             if (a.kv_pool != nullptr && row_ok && n0 + BN > a.Nq) {
-                const int slot = a.slot_map[t.row_start + r];
+                const int slot = a.slot_map[row];
                 if (slot >= 0) {
                     kv_page = slot / a.kv_page_size;
                     kv_row = slot % a.kv_page_size;
@@ -387,12 +373,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         float f[8];
 #pragma unroll
                         for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[8 * j + e]);
-                        if (drow) {
-                            const float4 d0 = *reinterpret_cast<const float4 *>(drow + c + 8 * j);
-                            const float4 d1 = *reinterpret_cast<const float4 *>(drow + c + 8 * j + 4);
-                            f[0] += d0.x; f[1] += d0.y; f[2] += d0.z; f[3] += d0.w;
-                            f[4] += d1.x; f[5] += d1.y; f[6] += d1.z; f[7] += d1.w;
-                        }
                         if (rrow) {
                             const uint4 rv = *reinterpret_cast<const uint4 *>(rrow + c + 8 * j);
                             const uint32_t rw[4] = {rv.x, rv.y, rv.z, rv.w};
@@ -428,7 +408,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     tc::tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && *abort_flag) report(a.status, ALORA_ERR_TIMEOUT);
-    if (threadIdx.x == 0) tc::item_counter_release(a.item_counters);
+    if (threadIdx.x == 0) tc::item_counter_release(a.item_counters, a.t_ready, n_shrink);
     if (warp == 1) {
         tc::tc_fence_after();
         tc::tmem_dealloc(tmem_base, kTmemCols);
@@ -488,9 +468,8 @@ static bool launch_gemm_bn(alora_ctx *ctx, const CUtensorMap &tmA, const CUtenso
     return true;
 }
 
-int launch_lora_delta_rows(alora_ctx *ctx, int layer, const void *hidden, int T, cudaStream_t s);  // simt_kernels.cu
 bool launch_shrink_tc(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap &tmA, const AdapterDev *adapters,
-                      int K, int max_row_tiles, cudaStream_t s);  // shrink_tcgen05.cu
+                      int T, int K, int max_pairs, int t_parts, cudaStream_t s);  // shrink_tcgen05.cu
 
 // Picks the column-tile width: 256 when the q/k/v block boundaries allow it, else 128; 64 for batches of at most
 // 128 rows, where the kernel streams the weights once and more, narrower tiles put more SMs to work.
@@ -504,10 +483,20 @@ static int pick_bn(int N, int Nq, int Nkv, bool lora, int T) {
     return (N % 256 == 0 || N > 1024) ? 256 : 128;
 }
 
-// q/k/v projection of one layer on the tensor cores: shrink (t = s A x on adapter tiles), then the
+// q/k/v projection of one layer on the tensor cores: shrink (t = s A x of the (row tile, adapter) pairs), then the
 // base GEMM with the expand step fused.  Returns kernels launched, or -1 when the shape is unsupported.
-int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T, void *qkv, cudaStream_t s,
+int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int R, void *qkv, cudaStream_t s,
                            void *kv_pool, int num_pages);  // gemm_pair_tcgen05.cu
+
+// Whether the shrink of a launch of `items` projection items is a kernel of its own.  As leading items of the projection
+// it is free unless it makes another round over the blocks of a launch of one or two rounds (a round is 27 us at
+// hidden 4096, a kernel for a few pairs 8 us); a kernel for many pairs takes rounds of its own.  The number of pairs is
+// an upper bound from the row and request counts, so that the choice does not depend on the mode.
+bool shrink_apart(const alora_ctx *ctx, int T, int R, int items) {
+    const int G = ctx->sm_count, n = pair_bound(ctx, T, R);
+    const int rounds = (items + G - 1) / G;
+    return rounds <= 2 && (items + n + G - 1) / G > rounds && n * 8 <= 4 * G;
+}
 
 bool skinny_route(const alora_ctx *ctx, int T, int N, int K, bool lora, int Nq, int Nkv);   // gemm_skinny_tcgen05.cu
 int launch_skinny_tc(alora_ctx *ctx, const void *x, const CUtensorMap &tmW, const CUtensorMap *tmA16,
@@ -522,7 +511,7 @@ bool project_is_few_row(const alora_ctx *ctx, int layer, int T) {
     return skinny_route(ctx, T, d.N, d.H, ctx->layer_has_adapter[layer] != 0, d.Nq, d.Nkv);
 }
 
-int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, void *qkv, cudaStream_t s, void *kv_pool,
+int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int R, void *qkv, cudaStream_t s, void *kv_pool,
                       int num_pages) {
     if (T == 0) return 0;
     const Dims &d = ctx->d;
@@ -537,7 +526,7 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, void
     }
     if (ctx->tc_maps[layer].pair_ok) {   // many rows: two row tiles per block, 192-wide column tiles
         ProfScope prof(ctx, KK_PROJECT, s);
-        const int r = launch_project_pair_tc(ctx, layer, hidden, T, qkv, s, kv_pool, num_pages);
+        const int r = launch_project_pair_tc(ctx, layer, hidden, T, R, qkv, s, kv_pool, num_pages);
         if (r != 0) return r;
     }
     const int BN = pick_bn(d.N, d.Nq, d.Nkv, true, T);
@@ -546,25 +535,16 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, void
     if (!make_tensor_map_bf16(&tmX, hidden, T, d.H, d.H, kBM)) return -1;
     const bool half_box = T <= kBM / 2;   // see GemmArgs::a_tile_bytes
     if (half_box && !make_tensor_map_bf16(&tmX64, hidden, T, d.H, d.H, kBM / 2)) return -1;
-    if (!make_tensor_map_bf16(&tmTt, ctx->d_t, ctx->cfg.max_tokens, 3 * kTensorRP, 3 * kTensorRP, kBM)) return -1;
+    if (!make_tensor_map_bf16(&tmTt, ctx->d_t, (uint64_t)ctx->t_slots * kBM, 3 * kTensorRP, 3 * kTensorRP, kBM)) return -1;
     const TcLayerMaps &lm = ctx->tc_maps[layer];
     const AdapterDev *ads = ctx->d_adapters + (size_t)layer * ctx->cfg.max_adapters;
-    // every row tile holds at least one row; a request contributes at most two partial tiles
-    const int max_row_tiles = std::min(std::min(ctx->max_tiles, T / kBM + 2 * ctx->cfg.max_requests + 2), T);
+    const int t_parts = T <= kSplitTTokens ? 2 : 1, max_pairs = have_adapters ? pair_bound(ctx, T, R) : 0;
+    const int proj_items = ((T + kBM - 1) / kBM) * ((d.N + BN - 1) / BN);
+    const bool fuse_shrink = have_adapters && BN == 256 && !shrink_apart(ctx, T, R, proj_items);
     int n = 0;
-    // Batches whose row tiles would hold only a few rows each may be switched to the row-wise route by the
-    // metadata step (a device-side decision): the delta rows are prepared here, and both kernels read the flag.
-    const bool may_rowwise = have_adapters && T <= kRowwiseMaxTokens && ctx->d_row_delta != nullptr;
-    if (may_rowwise) {
+    if (have_adapters && !fuse_shrink) {
         ProfScope prof(ctx, KK_SHRINK, s);
-        n += launch_lora_delta_rows(ctx, layer, hidden, T, s);
-    }
-    const bool fuse_shrink = have_adapters && BN == 256;
-    // (a batch of at most kRowwiseAlwaysRows rows always takes the row-wise route when it has adapter rows: no shrink
-    // launch; otherwise the shrink kernel looks at the flag itself)
-    if (have_adapters && !fuse_shrink && !(may_rowwise && T <= kRowwiseAlwaysRows)) {
-        ProfScope prof(ctx, KK_SHRINK, s);
-        if (!launch_shrink_tc(ctx, tmX, lm.a_all, ads, d.H, max_row_tiles, s)) return -1;
+        if (!launch_shrink_tc(ctx, tmX, lm.a_all, ads, T, d.H, max_pairs, t_parts, s)) return -1;
         ++n;
     }
     {
@@ -572,13 +552,11 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, void
         GemmArgs g{};
         g.a_tile_bytes = half_box ? (kBM / 2) * kBK * 2 : 0;
         const CUtensorMap &tmXg = half_box ? tmX64 : tmX;
-        g.tiles = ctx->d_tiles; g.n_row_tiles = ctx->d_counts; g.M = T; g.N = d.N; g.K = d.H;
+        g.M = T; g.N = d.N; g.K = d.H;
         g.out = (__nv_bfloat16 *)qkv; g.ldo = d.N; g.residual = nullptr; g.adapters = ads;
         g.Nq = d.Nq; g.Nkv = d.Nkv; g.total_adapter_rows = d.N; g.status = ctx->d_status;
         g.item_counters = ctx->d_counts + 10;
-        if (may_rowwise) {
-            g.rowwise_flag = ctx->d_counts + 5; g.row_delta = ctx->d_row_delta; g.row_adapter = ctx->d_row_adapter;
-        }
+        if (have_adapters) { g.pairs = ctx->d_pairs; g.pair_off = ctx->d_pair_off; g.t_parts = t_parts; }
         if (kv_pool != nullptr) {
             int shift = 0;
             while ((1 << shift) < d.hd) ++shift;
@@ -586,10 +564,10 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, void
             g.kv_page_size = d.page; g.kv_num_pages = num_pages;
         }
         if (fuse_shrink) {
-            g.shrink_tiles = ctx->d_shrink_tiles; g.n_shrink_tiles = ctx->d_counts + 2;
+            g.n_pairs = ctx->d_counts + 2; g.row_adapter = ctx->d_row_adapter;
             g.t_ready = ctx->d_t_ready; g.t_out = (__nv_bfloat16 *)ctx->d_t;
         }
-        const int items = max_row_tiles * ((d.N + BN - 1) / BN + (fuse_shrink ? 1 : 0));
+        const int items = proj_items + (fuse_shrink ? max_pairs : 0);
         const bool ok = BN == 256
                             ? launch_gemm_bn<256>(ctx, tmXg, lm.wqkv[1], tmTt, lm.b_all_bn[1], lm.a_all, g, items, s)
                             : BN == 128
@@ -627,7 +605,7 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
     if (!make_tensor_map_bf16(&tmW, W, N, K, K, BN)) return -1;
     GemmArgs g{};
     g.a_tile_bytes = half_box ? (kBM / 2) * kBK * 2 : 0;
-    g.tiles = nullptr; g.n_row_tiles = nullptr; g.M = T; g.N = N; g.K = K; g.out = (__nv_bfloat16 *)y; g.ldo = N;
+    g.M = T; g.N = N; g.K = K; g.out = (__nv_bfloat16 *)y; g.ldo = N;
     g.residual = (const __nv_bfloat16 *)residual; g.adapters = nullptr; g.Nq = N; g.Nkv = 0;
     g.total_adapter_rows = 0; g.status = ctx->d_status; g.item_counters = ctx->d_counts + 10;
     const int items = ((T + kBM - 1) / kBM) * ((N + BN - 1) / BN);

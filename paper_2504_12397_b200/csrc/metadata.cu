@@ -1,5 +1,5 @@
 // Batch metadata: per-token request / applied-adapter / KV-slot arrays and the projection's
-// row-tile list.  Integer work only; every output is compared exactly against the CPU oracle.
+// (row tile, adapter) pairs.  Integer work only; every output is compared exactly against the CPU oracle.
 #include <algorithm>
 #include <climits>
 #include "alora_internal.h"
@@ -7,7 +7,6 @@
 
 namespace alora {
 
-constexpr int kProjTileRows = 128;
 constexpr int kMetaSmemInts = 7168;   // 28 KB of builder scratch: batches of up to 511 requests
 constexpr int kMetaStageR = 1024;     // per-request inputs of up to this many requests are staged in shared memory
 
@@ -25,8 +24,8 @@ __device__ __forceinline__ int find_request(const int32_t *qsl, int R, int t) {
 // Per token: request index, adapter applied to the row (the gate of Eq. 5: position >= activation
 // offset; always open in full-LoRA mode, always closed in base mode), and the token slot
 // page * page_size + position % page_size.  Findings (inconsistent positions, page id out of
-// range, adapter id out of range, an open gate on an adapter that was never registered on the layer) go
-// to the status word; the row then gets adapter -1 / slot -1 so that later kernels skip it.
+// range, adapter id out of range) go to the status word; the row then gets adapter -1 / slot -1 so that later kernels
+// skip it.  (Whether the adapter is registered on a layer is not looked at here: one that is not has rank 0 there.)
 __device__ __forceinline__ int metadata_token(int t, const int32_t *__restrict__ positions,
                                       const int32_t *__restrict__ a_req,
                                       const int32_t *__restrict__ adapter_ids,
@@ -34,8 +33,7 @@ __device__ __forceinline__ int metadata_token(int t, const int32_t *__restrict__
                                       const int32_t *__restrict__ block_tables, int max_blocks,
                                       int num_pages, int page_size, int max_adapters, int T, int R, int mode,
                                       int32_t *__restrict__ token_req, int32_t *__restrict__ row_adapter,
-                                      int32_t *__restrict__ slot_map, const AdapterDev *__restrict__ adapters,
-                                      int32_t *status) {
+                                      int32_t *__restrict__ slot_map, int32_t *status) {
     if (t >= T) return -1;
     int r = find_request(qsl, R, t);
     int p = positions[t];
@@ -48,8 +46,6 @@ __device__ __forceinline__ int metadata_token(int t, const int32_t *__restrict__
         k = adapter_ids[r];
         if (k >= max_adapters || k < -1) { report(status, ALORA_ERR_BAD_BATCH); k = -1; }
         if (k >= 0 && mode == ALORA_MODE_ALORA && p < a_req[r]) k = -1;
-        // a row whose gate is open needs its adapter's weights on this layer
-        if (k >= 0 && adapters != nullptr && adapters[k].rank == 0) { report(status, ALORA_ERR_NO_WEIGHTS); k = -1; }
     }
     if (token_req) token_req[t] = r;
     k = ok ? k : -1;
@@ -71,99 +67,100 @@ __device__ __forceinline__ int metadata_token(int t, const int32_t *__restrict__
     return k;
 }
 
-// Row tiles of the projection.  Each request contributes up to two runs of rows: its gated-off
-// rows (applied adapter -1) and its gated-on rows; neighbouring runs with the same applied adapter
-// are merged across requests, and every merged run is cut into tiles of at most kProjTileRows rows.
-// One block; R is small (a scheduler batch).
-__device__ __forceinline__ void metadata_tiles(const int32_t *__restrict__ a_req, const int32_t *__restrict__ adapter_ids,
-                                      const int32_t *__restrict__ qsl, const int32_t *__restrict__ seq_lens,
-                                      int R, int mode, int max_adapters, int max_tiles,
-                                      ProjTile *__restrict__ tiles, int32_t *__restrict__ counts,
-                                      int32_t *seg_scratch /* [14R + 5] */, int T, int rowwise_cap, int32_t *__restrict__ shrink_tiles,
-                                      int32_t *__restrict__ t_ready, int32_t *status) {
-    int32_t *seg_start = seg_scratch, *seg_len = seg_scratch + (2 * R + 1);
-    int32_t *seg_adapter = seg_scratch + 2 * (2 * R + 1), *seg_tile0 = seg_scratch + 3 * (2 * R + 1);
-    int32_t *seg_shrink0 = seg_scratch + 4 * (2 * R + 1);  // adapter tiles before the segment
-    int32_t *rq_start = seg_scratch + 5 * (2 * R + 1), *rq_new = rq_start + R, *rq_off = rq_new + R, *rq_k = rq_off + R;
-    __shared__ int n_seg, n_tiles;
-    // per request, in parallel: first row, new rows, gated-off rows, adapter
+// The (row tile, adapter) pairs of the projection: for every tile of kTileRows rows the adapters whose gate is open on
+// some row of it, in the order of their first request, each once.  One block; a warp per tile, a lane per request.  Also
+// reports a request whose open rows name an adapter that some layer of the call has not registered.
+__device__ __forceinline__ void metadata_pairs(const int32_t *__restrict__ a_req, const int32_t *__restrict__ adapter_ids,
+                                               const int32_t *__restrict__ qsl, const int32_t *__restrict__ seq_lens,
+                                               int R, int mode, int max_adapters, int T, int max_pairs,
+                                               TilePair *__restrict__ pairs, int32_t *__restrict__ pair_off,
+                                               int32_t *__restrict__ counts, int32_t *scratch /* [3R] */,
+                                               const AdapterDev *__restrict__ adapters, int n_layers, int32_t *status) {
+    constexpr int kBatch = 128;   // tiles per round
+    __shared__ int r_lo[kBatch], r_hi[kBatch], cnt[kBatch], off_s[kBatch];
+    __shared__ int total_s;
+    int32_t *on0 = scratch, *on1 = scratch + R, *on_k = scratch + 2 * R;   // per request: rows with an open gate, adapter (-1: none)
+    bool any = false;
     for (int r = threadIdx.x; r < R; r += blockDim.x) {
         const int n_new = qsl[r + 1] - qsl[r];
         int k = (mode == ALORA_MODE_BASE || adapter_ids == nullptr) ? -1 : adapter_ids[r];
         if (k >= max_adapters || k < -1) k = -1;
         int n_off = 0;
-        if (k < 0) n_off = max(n_new, 0);
-        else if (mode == ALORA_MODE_ALORA) {
-            const int p_first = seq_lens[r] - n_new;
-            const long long d = (long long)a_req[r] - p_first;
+        if (k >= 0 && mode == ALORA_MODE_ALORA) {
+            const long long d = (long long)a_req[r] - (seq_lens[r] - n_new);
             n_off = d <= 0 ? 0 : (d >= n_new ? n_new : (int)d);
         }
-        rq_start[r] = qsl[r]; rq_new[r] = n_new; rq_off[r] = n_off; rq_k[r] = k;
+        if (n_off >= n_new) k = -1;
+        on0[r] = qsl[r] + n_off; on1[r] = qsl[r + 1]; on_k[r] = k;
+        any |= k >= 0;
+        if (k >= 0 && adapters != nullptr)
+            for (int l = 0; l < n_layers; ++l)
+                if (adapters[(size_t)l * max_adapters + k].rank == 0) report(status, ALORA_ERR_NO_WEIGHTS);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ns = 0, nt = 0;
-        int cur_start = 0, cur_len = 0, cur_ad = -1;   // the run being grown, kept in registers
-        bool have = false;
-#pragma unroll 4
-        for (int r = 0; r < R; ++r) {
-            const int n_new = rq_new[r];
-            if (n_new <= 0) continue;
-            const int n_off = rq_off[r];
-            const int start[2] = {rq_start[r], rq_start[r] + n_off};
-            const int len[2] = {n_off, n_new - n_off};
-            const int ad[2] = {-1, rq_k[r]};
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                if (len[i] <= 0) continue;
-                if (have && cur_ad == ad[i] && cur_start + cur_len == start[i]) {
-                    cur_len += len[i];
-                } else {
-                    if (have) { seg_start[ns] = cur_start; seg_len[ns] = cur_len; seg_adapter[ns] = cur_ad; ++ns; }
-                    cur_start = start[i]; cur_len = len[i]; cur_ad = ad[i];
-                    have = true;
+    any = __syncthreads_or(any);
+    const int n_tiles = (T + kTileRows - 1) / kTileRows;
+    if (!any) {   // base model only
+        for (int i = threadIdx.x; i <= n_tiles; i += blockDim.x) pair_off[i] = 0;
+        if (threadIdx.x == 0) counts[2] = 0;
+        return;
+    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = (int)blockDim.x >> 5;
+    // adapters of tile `t` (requests lo .. hi): counted, or written from pairs[at] on; called by whole warps
+    auto walk = [&](int t, int lo, int hi, bool write, int at) {
+        const int row0 = t * kTileRows, row1 = min(row0 + kTileRows, T);
+        int n = 0;
+        for (int base = lo; base <= hi; base += 32) {
+            const int r = base + lane;
+            int k = -1;
+            if (r <= hi && on0[r] < row1 && on1[r] > row0) k = on_k[r];
+            const unsigned same = __match_any_sync(0xffffffffu, k);   // (every lane takes part)
+            bool fresh = k >= 0 && __ffs(same) - 1 == lane;
+            for (int q = lo; fresh && q < base; ++q)   // (only a tile with more than 32 requests)
+                fresh = !(on_k[q] == k && on0[q] < row1 && on1[q] > row0);
+            __syncwarp();
+            const unsigned m = __ballot_sync(0xffffffffu, fresh);
+            const int slot = at + n + __popc(m & ((1u << lane) - 1u));
+            if (write && fresh && slot < max_pairs) { pairs[slot].tile = t; pairs[slot].adapter = k; }
+            n += __popc(m);
+        }
+        return n;
+    };
+    int carry = 0;
+    for (int t0 = 0; t0 < n_tiles; t0 += kBatch) {
+        const int nb = min(kBatch, n_tiles - t0);
+        for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+            r_lo[i] = find_request(qsl, R, (t0 + i) * kTileRows);
+            r_hi[i] = find_request(qsl, R, min((t0 + i + 1) * kTileRows, T) - 1);
+        }
+        __syncthreads();
+        for (int i = warp; i < nb; i += n_warps) {
+            const int n = walk(t0 + i, r_lo[i], r_hi[i], false, 0);
+            if (lane == 0) cnt[i] = n;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            int acc = carry;
+            for (int i = 0; i < nb; i += 32) {
+                const int x = i + lane < nb ? cnt[i + lane] : 0;
+                int inc = x;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (lane >= o) inc += v;
                 }
+                if (i + lane < nb) { off_s[i + lane] = acc + inc - x; pair_off[t0 + i + lane] = min(acc + inc - x, max_pairs); }
+                acc += __shfl_sync(0xffffffffu, inc, 31);
             }
+            if (lane == 0) total_s = acc;
         }
-        if (have) { seg_start[ns] = cur_start; seg_len[ns] = cur_len; seg_adapter[ns] = cur_ad; ++ns; }
-        int n_ad = 0;
-        for (int s = 0; s < ns; ++s) {
-            seg_tile0[s] = nt;
-            seg_shrink0[s] = n_ad;
-            const int n = (seg_len[s] + kProjTileRows - 1) / kProjTileRows;
-            nt += n;
-            if (seg_adapter[s] >= 0) n_ad += n;
-        }
-        seg_tile0[ns] = nt;
-        if (nt > max_tiles) { report(status, ALORA_ERR_CAPACITY); nt = 0; ns = 0; n_ad = 0; }
-        n_seg = ns; n_tiles = nt;
-        counts[0] = nt;
-        counts[2] = n_ad;
-        // Row tiles that hold only a few rows each (decode steps, short suffixes of many requests with different
-        // adapters) waste the tensor cores: when the tiles cover more than twice the batch's rows, and always when
-        // the batch has at most kRowwiseAlwaysRows rows, the projection takes the row-wise route (dense row tiles + a
-        // per-row delta) instead.  (The per-row delta costs about 0.4 us per row, the tensor-core shrink of a few
-        // tiles about 8 us whatever their rows.)
-        const bool wasteful = (long long)nt * kProjTileRows > 2ll * T + 2 * kProjTileRows;
-        counts[5] = (n_ad > 0 && T <= rowwise_cap && (T <= kRowwiseAlwaysRows || wasteful)) ? 1 : 0;
+        __syncthreads();
+        carry = total_s;
+        for (int i = warp; i < nb; i += n_warps) walk(t0 + i, r_lo[i], r_hi[i], true, off_s[i]);
+        __syncthreads();
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < n_tiles; i += blockDim.x) {
-        int lo = 0, hi = n_seg;  // seg_tile0[lo] <= i < seg_tile0[hi]
-        while (hi - lo > 1) {
-            int mid = (lo + hi) >> 1;
-            if (seg_tile0[mid] <= i) lo = mid; else hi = mid;
-        }
-        int off = (i - seg_tile0[lo]) * kProjTileRows;
-        ProjTile pt;
-        pt.row_start = seg_start[lo] + off;
-        pt.row_count = min(kProjTileRows, seg_len[lo] - off);
-        pt.adapter = seg_adapter[lo];
-        pt.pad_ = 0;
-        tiles[i] = pt;
-        // list of the tiles that need t = s A x, and their "t is ready" counters, cleared for this batch
-        if (pt.adapter >= 0) shrink_tiles[seg_shrink0[lo] + (i - seg_tile0[lo])] = i;
-        t_ready[i] = 0;
+    if (threadIdx.x == 0) {
+        if (carry > max_pairs) report(status, ALORA_ERR_CAPACITY);
+        pair_off[n_tiles] = min(carry, max_pairs);
+        counts[2] = min(carry, max_pairs);
     }
 }
 
@@ -642,7 +639,7 @@ __device__ __forceinline__ void metadata_few_row(int k_mine, const AdapterDev *_
 }
 
 // The metadata step.  Phase bit 0: every block handles 256 tokens (request, applied adapter, slot); block 0 then
-// builds the projection's row-tile list, or the few-row route's adapter facts.  Phase bit 1: the two attention
+// builds the projection's (row tile, adapter) pairs.  Phase bit 1: the two attention
 // work lists, one block each (their serial parts are O(R)).  Both phases in one launch: blocks 0, 1, 2 take one
 // builder each.  The attention phase alone is launched as a programmatic dependent of the projection kernel, beside
 // which it runs (it reads nothing that kernel writes); its blocks wait for that kernel before they exit, so that
@@ -652,13 +649,13 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
                 const int32_t *qsl, const int32_t *seq_lens, const int32_t *__restrict__ block_tables, int max_blocks,
                 int num_pages, int page_size, int max_adapters, int T, int R, int mode,
                 int32_t *__restrict__ token_req, int32_t *__restrict__ row_adapter, int32_t *__restrict__ slot_map,
-                int max_tiles, ProjTile *__restrict__ tiles, int32_t *__restrict__ counts, int32_t *seg_scratch,
-                int32_t *__restrict__ shrink_tiles, int32_t *__restrict__ t_ready,
+                int max_pairs, TilePair *__restrict__ pairs, int32_t *__restrict__ pair_off, int32_t *__restrict__ counts,
+                int32_t *seg_scratch,
                 int Hkv, int q_block, int max_items, AttnWork *__restrict__ items, int32_t *blk_off,
                 int G, int n_sm, int small_max, int max_split_items, int max_split_rows,
                 AttnSplitWork *__restrict__ split_items,
-                int32_t *req_scratch, int32_t *__restrict__ group_done, int rowwise_cap,
-                int32_t *__restrict__ attn_cta_start, const AdapterDev *__restrict__ adapters, int phases,
+                int32_t *req_scratch, int32_t *__restrict__ group_done,
+                int32_t *__restrict__ attn_cta_start, const AdapterDev *__restrict__ adapters, int n_layers, int phases,
                 int32_t *__restrict__ prefix_groups, int32_t *status) {
     // The per-request inputs are read many times (binary searches, list builders): one parallel pass stages them
     // in shared memory, so that the later steps do not each pay a round trip to global memory.
@@ -679,18 +676,18 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
     }
     if (phases & kMetaProjection)
         metadata_token((int)(blockIdx.x * blockDim.x + threadIdx.x), positions, a_req, adapter_ids, qsl, seq_lens, block_tables,
-                       max_blocks, num_pages, page_size, max_adapters, T, R, mode, token_req, row_adapter, slot_map, adapters, status);
+                       max_blocks, num_pages, page_size, max_adapters, T, R, mode, token_req, row_adapter, slot_map, status);
     // The three list builders are independent of one another: blocks 0, 1 and 2 take one each (a launch of both
     // phases has at least three blocks, one of the attention phase alone two).
     const int nb = (int)gridDim.x;
     const bool proj = (phases & kMetaProjection) != 0, attn = (phases & kMetaAttention) != 0;
-    const int b_tiles = proj ? 0 : -1;
+    const int b_pairs = proj && pairs != nullptr ? 0 : -1;
     const int b_attn = !attn ? -1 : (proj ? (nb > 1 ? 1 : 0) : 0);
     const int b_split = !attn ? -1 : (proj ? (nb > 2 ? 2 : 0) : (nb > 1 ? 1 : 0));
     // the attention phase alone: block 0 builds the tensor-core kernel's list, all the others share the few-row list
     const int split_parts = (!proj && attn && nb > 1) ? nb - 1 : 1;
     const bool split_helper = !proj && attn && (int)blockIdx.x > b_split;
-    if ((int)blockIdx.x != b_tiles && (int)blockIdx.x != b_attn && (int)blockIdx.x != b_split && !split_helper) {
+    if ((int)blockIdx.x != b_pairs && (int)blockIdx.x != b_attn && (int)blockIdx.x != b_split && !split_helper) {
         if (!proj) tc::grid_dep_wait();
         return;
     }
@@ -699,9 +696,9 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
     __shared__ int32_t smem_scratch[kMetaSmemInts];
     if (14 * R + 5 <= kMetaSmemInts) seg_scratch = blk_off = req_scratch = smem_scratch;
     __syncthreads();
-    if ((int)blockIdx.x == b_tiles) {
-        metadata_tiles(a_req, adapter_ids, qsl, seq_lens, R, mode, max_adapters, max_tiles, tiles, counts, seg_scratch,
-                       T, rowwise_cap, shrink_tiles, t_ready, status);
+    if ((int)blockIdx.x == b_pairs) {
+        metadata_pairs(a_req, adapter_ids, qsl, seq_lens, R, mode, max_adapters, T, max_pairs, pairs, pair_off, counts,
+                       seg_scratch, adapters, n_layers, status);
         __syncthreads();  // a builder that follows in this block reuses the scratch
     }
     if ((int)blockIdx.x == b_attn && items != nullptr && block_tables != nullptr) {
@@ -747,7 +744,7 @@ metadata_few_row_kernel(const int32_t *__restrict__ positions, const int32_t *a_
     const bool first = blockIdx.x == 0;
     int k = metadata_token((int)threadIdx.x, positions, a_req, adapter_ids, qsl, seq_lens, first ? block_tables : nullptr,
                            max_blocks, num_pages, page_size, max_adapters, T, R, mode, first ? token_req : nullptr,
-                           first ? row_adapter : nullptr, first ? slot_map : nullptr, nullptr, status);
+                           first ? row_adapter : nullptr, first ? slot_map : nullptr, status);
     if (few_row_meta != nullptr) {
         const AdapterDev *ads = adapters + (size_t)blockIdx.x * max_adapters;
         if (k >= 0 && ads[k].rank == 0) { report(status, ALORA_ERR_NO_WEIGHTS); k = -1; }
@@ -782,12 +779,11 @@ int launch_metadata(alora_ctx *ctx, const BatchArgs &b, cudaStream_t s, int phas
     const cudaError_t e = launch_kernel(metadata_kernel, dim3(grid), dim3(threads), 0, s, attn_only,
         b.positions, b.activation_offsets, b.adapter_ids, b.query_start_loc, b.seq_lens, b.block_tables,
         b.max_blocks, b.num_pages, ctx->d.page, ctx->cfg.max_adapters, b.T, b.R, b.mode, ctx->d_token_req,
-        ctx->d_row_adapter, ctx->d_slot, ctx->max_tiles, ctx->d_tiles, ctx->d_counts, ctx->d_seg_scratch,
-        ctx->d_shrink_tiles, ctx->d_t_ready,
+        ctx->d_row_adapter, ctx->d_slot, ctx->max_pairs, ctx->d_pairs, ctx->d_pair_off, ctx->d_counts, ctx->d_seg_scratch,
         ctx->d.Hkv, ctx->attn_q_block, ctx->max_attn_items, ctx->d_attn_items, ctx->d_attn_off, ctx->d.G,
         ctx->sm_count, ctx->small_max_tokens, ctx->max_split_items, ctx->max_split_rows, ctx->d_split_items,
-        ctx->d_req_scratch, ctx->d_group_done, ctx->d_row_delta ? kRowwiseMaxTokens : 0,
-        ctx->d_attn_cta_start, ads, phases, ctx->d_prefix_groups, ctx->d_status);
+        ctx->d_req_scratch, ctx->d_group_done,
+        ctx->d_attn_cta_start, ads, b.n_layers, phases, ctx->d_prefix_groups, ctx->d_status);
     return e == cudaSuccess ? 1 : -1;
 }
 

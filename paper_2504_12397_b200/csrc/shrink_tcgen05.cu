@@ -1,14 +1,13 @@
 // Rank-r shrink t = s A_k x on the tensor cores (the inner product of the low-rank delta of Eq. 5),
 // split along the hidden dimension over a thread-block cluster.
 //
-// The shrink has few output tiles (one 128 x 192 tile per row tile: 3 blocks q/k/v of 64 padded rank
-// columns) but a long contraction (the hidden dimension), so each row tile is given to a cluster of
+// The shrink has few output tiles (one 128 x 192 tile per (row tile, adapter) pair: 3 blocks q/k/v of 64 padded rank
+// columns) but a long contraction (the hidden dimension), so each pair is given to a cluster of
 // kShrinkSplits blocks.  Block c of the cluster contracts hidden columns of its own K range with
 // tcgen05.mma into tensor memory, copies its fp32 partial tile into its shared memory, and after a
 // cluster barrier reduces a 24-column slice of the tile over all blocks' shared memory (distributed
 // shared memory loads) in the fixed order 0, 1, ..., 7.  The order does not depend on timing, so the
-// result is run-to-run deterministic.  Row tiles without an applied adapter are skipped by their
-// whole cluster.
+// result is run-to-run deterministic.
 #include <algorithm>
 
 #include "alora_internal.h"
@@ -25,10 +24,12 @@ constexpr int kShrinkThreads = 192;     // warp 0 TMA, warp 1 MMA, warps 2-5 epi
 constexpr int kShrinkSlice = kShrinkBN / kShrinkSplits;  // 24 columns reduced by each block
 
 struct ShrinkArgs {
-    const ProjTile *tiles;
-    const int32_t *n_row_tiles;
+    const TilePair *pairs;
+    const int32_t *n_pairs;
+    const int32_t *row_adapter;   // [T] applied adapter per row
     const AdapterDev *adapters;
-    __nv_bfloat16 *t;   // [tokens][192]
+    __nv_bfloat16 *t;   // [pair][t_parts][128][192]
+    int t_parts, T;
     int K;              // hidden
     int32_t *status;
 };
@@ -64,10 +65,11 @@ __global__ void __cluster_dims__(kShrinkSplits, 1, 1) __launch_bounds__(kShrinkT
 shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmA,
                       const ShrinkArgs a) {
     using S = ShrinkSmem;
-    // the whole cluster takes the same decision: blockIdx.y selects the row tile
-    if ((int)blockIdx.y >= *a.n_row_tiles || a.n_row_tiles[5] != 0) return;  // [5]: batch takes the row-wise route
-    const ProjTile tile = a.tiles[blockIdx.y];
-    if (tile.adapter < 0) return;
+    tc::grid_dep_launch();
+    tc::grid_dep_wait();   // the pairs and the row -> adapter map come from the metadata kernel, x from the kernel before
+    // the whole cluster takes the same decision: blockIdx.y selects the pair
+    if ((int)blockIdx.y >= *a.n_pairs) return;
+    const TilePair pair = a.pairs[blockIdx.y];
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (tc::smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -113,8 +115,8 @@ shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                 if (!tc::mbar_wait(empty_bar(s), ((kc / kShrinkStages) & 1) ^ 1, abort_flag)) { ok = false; break; }
                 const uint32_t sa = smem_base + s * S::kStageBytes, sb = sa + S::kABytes;
                 tc::mbar_arrive_expect_tx(full_bar(s), S::kStageBytes);
-                tc::tma_load_2d(sa, &tmX, full_bar(s), (kb0 + kc) * kShrinkBK, tile.row_start);
-                tc::tma_load_2d(sb, &tmA, full_bar(s), (kb0 + kc) * kShrinkBK, tile.adapter * kShrinkBN);
+                tc::tma_load_2d(sa, &tmX, full_bar(s), (kb0 + kc) * kShrinkBK, pair.tile * kShrinkBM);
+                tc::tma_load_2d(sb, &tmA, full_bar(s), (kb0 + kc) * kShrinkBK, pair.adapter * kShrinkBN);
             }
             if (!ok) {
                 // copies already in flight must land before the shared memory is reused or released
@@ -170,7 +172,7 @@ shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     if (warp >= 2) {
         const int q = warp & 3;
         const int r = q * 32 + lane;
-        const float scale = a.adapters[tile.adapter].scale;
+        const float scale = a.adapters[pair.adapter].scale;
         const int c0 = (int)crank * kShrinkSlice;
         float acc[kShrinkSlice];
 #pragma unroll
@@ -181,18 +183,10 @@ shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
             for (int j = 0; j < kShrinkSlice; ++j)
                 acc[j] += ld_dsmem_f32(tc::smem_u32(partial + (c0 + j) * kShrinkBM + r), src);
         }
-        if (r < tile.row_count) {
-            __nv_bfloat16 *orow = a.t + (size_t)(tile.row_start + r) * kShrinkBN + c0;
-#pragma unroll
-            for (int j = 0; j < kShrinkSlice; j += 8) {
-                uint4 o;
-                o.x = tc::pack_bf16(acc[j] * scale, acc[j + 1] * scale);
-                o.y = tc::pack_bf16(acc[j + 2] * scale, acc[j + 3] * scale);
-                o.z = tc::pack_bf16(acc[j + 4] * scale, acc[j + 5] * scale);
-                o.w = tc::pack_bf16(acc[j + 6] * scale, acc[j + 7] * scale);
-                *reinterpret_cast<uint4 *>(orow + j) = o;
-            }
-        }
+        const int row = pair.tile * kShrinkBM + r;
+        __nv_bfloat16 *orow = a.t + ((size_t)blockIdx.y * a.t_parts * kShrinkBM + r) * kShrinkBN + c0;
+        tc::store_t<kShrinkSlice>(acc, scale, row < a.T && a.row_adapter[row] == pair.adapter, orow,
+                                  a.t_parts > 1 ? orow + (size_t)kShrinkBM * kShrinkBN : nullptr);
     }
 
     cluster_sync_all();  // no block may release its shared memory while another still reads it
@@ -203,9 +197,10 @@ shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     }
 }
 
-// t = s A x for the adapter row tiles of the current batch.  Returns false if the launch could not be set up.
+// t = s A x of the (row tile, adapter) pairs of the current batch, of which there are at most max_pairs.  Returns false
+// if the launch could not be set up.
 bool launch_shrink_tc(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap &tmA, const AdapterDev *adapters,
-                      int K, int max_row_tiles, cudaStream_t s) {
+                      int T, int K, int max_pairs, int t_parts, cudaStream_t s) {
     static bool attr_set[64] = {};
     const int dev = ctx->cfg.device;
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
@@ -214,10 +209,9 @@ bool launch_shrink_tc(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap 
             return false;
         attr_set[dev] = true;
     }
-    ShrinkArgs a{ctx->d_tiles, ctx->d_counts, adapters, (__nv_bfloat16 *)ctx->d_t, K, ctx->d_status};
-    dim3 grid(kShrinkSplits, std::max(1, max_row_tiles));
-    shrink_tcgen05_kernel<<<grid, kShrinkThreads, ShrinkSmem::kTotal, s>>>(tmX, tmA, a);
-    return true;
+    ShrinkArgs a{ctx->d_pairs, ctx->d_counts + 2, ctx->d_row_adapter, adapters, (__nv_bfloat16 *)ctx->d_t, t_parts, T, K, ctx->d_status};
+    return launch_kernel(shrink_tcgen05_kernel, dim3(kShrinkSplits, std::max(1, max_pairs)), dim3(kShrinkThreads),
+                         ShrinkSmem::kTotal, s, true, tmX, tmA, a) == cudaSuccess;
 }
 
 }  // namespace alora

@@ -86,105 +86,6 @@ __global__ void shrink_simt_kernel(const T *__restrict__ x, const int32_t *__res
 }
 
 // ---------------------------------------------------------------------------------------------
-// Row-wise low-rank delta for batches of few rows per adapter (bf16):
-//     delta[row][n] = s * sum_i B[n][i] (A x_row)[blk(n)][i]          (Eq. 5, the term behind the gate)
-// for every row with an applied adapter, in fp32.  One block per (row, q/k/v block): the row of x is staged in
-// shared memory, each of 32 warps forms one or two of the block's `rank` inner products with A (16-byte loads,
-// several in flight per lane), then each thread forms outputs of the block's columns from its B rows.  Adapter storage is the rank-padded tensor-core layout A[3][64][H], B[N][64].  The kernel does
-// nothing unless the metadata step chose the row-wise route for this batch (*rowwise_flag).
-// ---------------------------------------------------------------------------------------------
-constexpr int kDeltaThreads = 1024;  // 32 warps: one or two inner products per warp, many loads in flight per SM
-
-__global__ void __launch_bounds__(kDeltaThreads)
-lora_delta_rows_kernel(const __nv_bfloat16 *__restrict__ x, const int32_t *__restrict__ row_adapter,
-                       const AdapterDev *__restrict__ adapters, const int32_t *__restrict__ rowwise_flag, int H,
-                       int Nq, int Nkv, int N, float *__restrict__ delta) {
-    extern __shared__ uint4 x_s4[];  // H bf16
-    __shared__ float t_s[kRankPadMax];
-    tc::grid_dep_launch();
-    tc::grid_dep_wait();   // the flag and the row -> adapter map come from the metadata kernel
-    if (*rowwise_flag == 0) return;
-    const int row = blockIdx.x, blk = blockIdx.y;
-    const int k = row_adapter[row];
-    if (k < 0) return;
-    const AdapterDev ad = adapters[k];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int hv = H / 8;  // 16-byte vectors per row
-    const uint4 *xg = reinterpret_cast<const uint4 *>(x + (size_t)row * H);
-    for (int i = threadIdx.x; i < hv; i += blockDim.x) x_s4[i] = xg[i];
-    __syncthreads();
-    {
-        // inner products warp and warp + 32 (rank <= 64)
-        const uint4 *A4 = reinterpret_cast<const uint4 *>(ad.A) + (size_t)blk * kRankPadMax * hv;
-        const bool on0 = warp < ad.rank, on1 = warp + 32 < ad.rank;
-        const uint4 *a0 = A4 + (size_t)warp * hv, *a1 = A4 + (size_t)(warp + 32) * hv;
-        float acc0 = 0.f, acc1 = 0.f;
-        if (on0) {
-#pragma unroll 2
-            for (int v = lane; v < hv; v += 32) {
-                const uint4 xv = x_s4[v];
-                const uint4 av0 = a0[v];
-                const uint4 av1 = on1 ? a1[v] : make_uint4(0, 0, 0, 0);
-                const __nv_bfloat162 *x2 = reinterpret_cast<const __nv_bfloat162 *>(&xv);
-                const __nv_bfloat162 *p0 = reinterpret_cast<const __nv_bfloat162 *>(&av0);
-                const __nv_bfloat162 *p1 = reinterpret_cast<const __nv_bfloat162 *>(&av1);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 xf = __bfloat1622float2(x2[e]);
-                    const float2 f0 = __bfloat1622float2(p0[e]), f1 = __bfloat1622float2(p1[e]);
-                    acc0 = fmaf(f0.x, xf.x, acc0); acc0 = fmaf(f0.y, xf.y, acc0);
-                    acc1 = fmaf(f1.x, xf.x, acc1); acc1 = fmaf(f1.y, xf.y, acc1);
-                }
-            }
-        }
-        for (int off = 16; off; off >>= 1) {
-            acc0 += __shfl_xor_sync(0xffffffffu, acc0, off);
-            acc1 += __shfl_xor_sync(0xffffffffu, acc1, off);
-        }
-        if (lane == 0) {
-            t_s[warp] = on0 ? acc0 * ad.scale : 0.f;          // zero beyond the rank
-            t_s[warp + 32] = on1 ? acc1 * ad.scale : 0.f;
-        }
-    }
-    __syncthreads();
-    const int n_begin = blk == 0 ? 0 : (blk == 1 ? Nq : Nq + Nkv);
-    const int n_end = blk == 0 ? Nq : (blk == 1 ? Nq + Nkv : N);
-    const uint4 *B4 = reinterpret_cast<const uint4 *>(ad.B);
-    const int rv = (ad.rank + 7) / 8;  // 16-byte vectors of a B row that hold non-zero columns (padding is zero)
-    for (int n = n_begin + threadIdx.x; n < n_end; n += blockDim.x) {
-        const uint4 *brow = B4 + (size_t)n * (kRankPadMax / 8);
-        float acc = 0.f;
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {   // four 16-byte vectors (32 rank columns) at a time, loads first
-            if (half * 4 >= rv) break;
-            uint4 b[4];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) b[v] = half * 4 + v < rv ? brow[half * 4 + v] : make_uint4(0, 0, 0, 0);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const __nv_bfloat162 *p = reinterpret_cast<const __nv_bfloat162 *>(&b[v]);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 f = __bfloat1622float2(p[e]);
-                    acc = fmaf(f.x, t_s[(half * 4 + v) * 8 + 2 * e], acc);
-                    acc = fmaf(f.y, t_s[(half * 4 + v) * 8 + 2 * e + 1], acc);
-                }
-            }
-        }
-        delta[(size_t)row * N + n] = acc;
-    }
-}
-
-int launch_lora_delta_rows(alora_ctx *ctx, int layer, const void *hidden, int T, cudaStream_t s) {
-    const Dims &d = ctx->d;
-    const AdapterDev *ads = ctx->d_adapters + (size_t)layer * ctx->cfg.max_adapters;
-    launch_kernel(lora_delta_rows_kernel, dim3(T, 3), dim3(kDeltaThreads), (size_t)d.H * 2, s, true, (const __nv_bfloat16 *)hidden, (const int32_t *)ctx->d_row_adapter, ads,
-                                                                   ctx->d_counts + 5, d.H, d.Nq, d.Nkv, d.N,
-                                                                   ctx->d_row_delta);
-    return 1;
-}
-
-// ---------------------------------------------------------------------------------------------
 // CUDA-core projection y[row][n] = sum_h W[n][h] x[row][h]  (+ sum_i B[n][i] t[row][blk(n)][i] when the
 // row has an applied adapter).  64x64 output tile per block, 16x16 threads, 4x4 outputs each,
 // K staged through shared memory 16 columns at a time.  The base sum of a row is formed by the

@@ -200,13 +200,36 @@ struct ItemRing {
     }
 };
 // At the end of a kernel that hands items out through a global counter: the last block to get here clears
-// the counter for the next launch.  counters[0] = next item, counters[1] = blocks that have finished.
-__device__ __forceinline__ void item_counter_release(int32_t *counters) {
+// the counter, and the n ready counters of the items' results, for the next launch.  counters[0] = next item,
+// counters[1] = blocks that have finished.
+__device__ __forceinline__ void item_counter_release(int32_t *counters, int32_t *ready, int n) {
     __threadfence();
     if (atomicAdd(counters + 1, 1) == (int)gridDim.x - 1) {
+        for (int i = 0; i < n; ++i) ready[i] = 0;
         counters[0] = 0;
         counters[1] = 0;
         __threadfence();
+    }
+}
+
+// t of a (row tile, adapter) pair as the operand of the expand step: `n` (a multiple of 8) fp32 columns of one row, times
+// the adapter's scale, rounded to bf16; with `lo` also what the rounding left, rounded again (their sum has 16
+// significant bits).  A row that does not use the adapter gets zeros.
+template <int n>
+__device__ __forceinline__ void store_t(const float (&v)[n], float scale, bool use, __nv_bfloat16 *hi, __nv_bfloat16 *lo) {
+#pragma unroll
+    for (int j = 0; j < n; j += 8) {
+        uint32_t h[4], l[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float a = use ? v[j + 2 * e] * scale : 0.f, b = use ? v[j + 2 * e + 1] * scale : 0.f;
+            const __nv_bfloat162 r = __floats2bfloat162_rn(a, b);
+            const __nv_bfloat162 q = __floats2bfloat162_rn(a - __low2float(r), b - __high2float(r));
+            h[e] = *reinterpret_cast<const uint32_t *>(&r);
+            l[e] = *reinterpret_cast<const uint32_t *>(&q);
+        }
+        *reinterpret_cast<uint4 *>(hi + j) = make_uint4(h[0], h[1], h[2], h[3]);
+        if (lo) *reinterpret_cast<uint4 *>(lo + j) = make_uint4(l[0], l[1], l[2], l[3]);
     }
 }
 
