@@ -63,7 +63,14 @@ struct AttnArgs {
     float *part_ml;             // [2 * blocks][2][256] exponent reference and row sum of a part
 };
 
-// A block's work: whole items blockIdx, blockIdx + blocks, ... below n_whole, then the pieces of its run (tiles
+// The item a block takes whole in its `round`: dealt back and forth, so that with the list longest first no block gets
+// the longer item of every round.
+__device__ __forceinline__ int whole_item(int round) {
+    const int n = (int)gridDim.x, b = (int)blockIdx.x;
+    return round * n + ((round & 1) ? n - 1 - b : b);
+}
+
+// A block's work: whole items (one of each round of `blocks` items) below n_whole, then the pieces of its run (tiles
 // [blockIdx * len, +len) of the concatenated key tiles of the items from n_whole on).  One piece = tiles [t0, t1)
 // of one item.  An item cut by run boundaries is worked on by n_parts consecutive blocks (this block holds part
 // `part`, the first of them is block c_first); each writes its partial result to a slot and a merge kernel adds
@@ -73,21 +80,21 @@ struct RunPiece {
     int item, t0, t1, n_parts, part, c_first;
 };
 struct RunIter {
-    int gt, gt_end, it, len, off, n_whole, whole;
+    int gt, gt_end, it, len, off, n_whole, round = 0;
     __device__ explicit RunIter(const AttnArgs &a) {
         const int total = a.run_counts[0];
         len = a.run_counts[1];
         n_whole = a.run_counts[2];
         off = a.run_counts[3];
-        whole = (int)blockIdx.x;
         gt = min(total, (int)blockIdx.x * len);
         gt_end = min(total, gt + len);
         it = gt < gt_end ? a.cta_start[blockIdx.x] : 0;
     }
     __device__ bool next(const AttnArgs &a, RunPiece &p) {
+        const int whole = whole_item(round);
         if (whole < n_whole) {
+            ++round;
             p.item = whole;
-            whole += (int)gridDim.x;
             p.w = a.items[p.item];
             p.t0 = 0;
             p.t1 = (p.w.kv_end + kKeysPerTile - 1) / kKeysPerTile;
@@ -110,14 +117,15 @@ struct RunIter {
     }
 };
 // The same interface for batches whose items are all taken whole (what the host can tell in advance for short
-// batches): items blockIdx, blockIdx + blocks, ...
+// batches).
 struct WholeIter {
-    int whole, n_items;
-    __device__ explicit WholeIter(const AttnArgs &a) : whole((int)blockIdx.x), n_items(*a.n_items) {}
+    int round = 0, n_items;
+    __device__ explicit WholeIter(const AttnArgs &a) : n_items(*a.n_items) {}
     __device__ bool next(const AttnArgs &a, RunPiece &p) {
+        const int whole = whole_item(round);
         if (whole >= n_items) return false;
+        ++round;
         p.item = whole;
-        whole += (int)gridDim.x;
         p.w = a.items[p.item];
         p.t0 = 0;
         p.t1 = (p.w.kv_end + kKeysPerTile - 1) / kKeysPerTile;

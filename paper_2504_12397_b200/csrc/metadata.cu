@@ -165,10 +165,11 @@ __device__ __forceinline__ void metadata_pairs(const int32_t *__restrict__ a_req
 }
 
 // Which requests the few-row kernel takes (1 .. returned limit new tokens; the others go to the tensor-core
-// kernel).  Normally the limit is small_max.  When the requests with 2 .. small_max new tokens alone make at least
-// two KV streams per SM, they fill the tensor-core kernel's blocks, which then reads the cache faster than the
-// few-row kernel (64 requests x 4 tokens on 4096 cached ones: 0.82 against 0.67 of the HBM bandwidth), and the limit
-// is 1.  Called by all threads of a block; both list builders take the same decision.
+// kernel).  Normally the limit is small_max.  When the requests with 2 and more new tokens make at least two KV streams
+// per SM, they fill the tensor-core kernel's blocks, and the limit is 1: that kernel then reads the cache faster than the
+// few-row kernel (64 requests x 4 tokens on 4096 cached ones: 0.82 against 0.67 of the HBM bandwidth), and a few
+// requests of 2 .. small_max tokens among longer ones would make a launch of their own behind it (48 requests of 3 .. 29
+// tokens: 30 us).  Called by all threads of a block; both list builders take the same decision.
 __device__ __forceinline__ int few_row_limit(const int32_t *__restrict__ qsl, int R, int Hkv, int n_sm, int small_max) {
     __shared__ int n_multi;
     if (threadIdx.x == 0) n_multi = 0;
@@ -176,7 +177,7 @@ __device__ __forceinline__ int few_row_limit(const int32_t *__restrict__ qsl, in
     int mine = 0;
     for (int r = threadIdx.x; r < R; r += blockDim.x) {
         const int n_new = qsl[r + 1] - qsl[r];
-        mine += n_new >= 2 && n_new <= small_max;
+        mine += n_new >= 2;
     }
     if (mine) atomicAdd(&n_multi, mine);
     __syncthreads();
@@ -189,17 +190,32 @@ __device__ __forceinline__ int few_row_limit(const int32_t *__restrict__ qsl, in
 // `q_block` tokens; one item per (request, KV head, block), blocks of the same KV stream adjacent so
 // that blocks running at the same time share their K/V pages in L2.  Keys 0 .. position of the
 // block's last token are visible to the block (causal limit); per-row limits are applied in the kernel.
+// Requests are taken longest first (`order`, where the scratch has room for it), a request's last block first: dealt to
+// the blocks back and forth (attn_tcgen05.cu), items of very different length then end at about the same time.
 __device__ __forceinline__ void metadata_attn_items(const int32_t *__restrict__ qsl, const int32_t *__restrict__ seq_lens,
                                            int R, int Hkv, int q_block, int small_max, int max_items,
                                            AttnWork *__restrict__ items, int32_t *__restrict__ counts,
-                                           int32_t *blk_off /* [R+1] */, int n_blocks, int32_t *__restrict__ cta_start,
-                                           int32_t *status) {
+                                           int32_t *blk_off /* [R+1] */, int32_t *order /* [2R] or nullptr */, int n_blocks,
+                                           int32_t *__restrict__ cta_start, int32_t *status) {
     __shared__ int total;
     small_max = few_row_limit(qsl, R, Hkv, n_blocks, small_max);
-    for (int r = threadIdx.x; r < R; r += blockDim.x) {
+    auto blocks_of = [&](int r) {   // (short requests: few-row list)
         const int n_new = qsl[r + 1] - qsl[r];
-        blk_off[r] = n_new > small_max ? (n_new + q_block - 1) / q_block : 0;  // short requests: few-row list
+        return n_new > small_max ? (n_new + q_block - 1) / q_block : 0;
+    };
+    if (order != nullptr) {
+        int32_t *key = order + R;
+        for (int r = threadIdx.x; r < R; r += blockDim.x) key[r] = blocks_of(r) > 0 ? seq_lens[r] : 0;
+        __syncthreads();
+        for (int r = threadIdx.x; r < R; r += blockDim.x) {
+            const int mine = key[r];
+            int at = 0;
+            for (int q = 0; q < R; ++q) at += key[q] > mine || (key[q] == mine && q < r);
+            order[at] = r;
+        }
+        __syncthreads();
     }
+    for (int i = threadIdx.x; i < R; i += blockDim.x) blk_off[i] = blocks_of(order != nullptr ? order[i] : i);
     __syncthreads();
     if (threadIdx.x == 0) {
         int acc = 0;
@@ -222,10 +238,10 @@ __device__ __forceinline__ void metadata_attn_items(const int32_t *__restrict__ 
             const int mid = (lo + hi) >> 1;
             if (blk_off[mid] * Hkv <= i) lo = mid; else hi = mid;
         }
-        const int r = lo;
-        const int nblk = blk_off[r + 1] - blk_off[r];
-        const int rem = i - blk_off[r] * Hkv;
-        const int kvh = rem / nblk, blk = rem % nblk;
+        const int r = order != nullptr ? order[lo] : lo;
+        const int nblk = blk_off[lo + 1] - blk_off[lo];
+        const int rem = i - blk_off[lo] * Hkv;
+        const int kvh = rem / nblk, blk = nblk - 1 - rem % nblk;
         const int n_new = qsl[r + 1] - qsl[r];
         AttnWork w;
         w.req = r;
@@ -703,7 +719,7 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
     }
     if ((int)blockIdx.x == b_attn && items != nullptr && block_tables != nullptr) {
         metadata_attn_items(qsl, seq_lens, R, Hkv, q_block, small_max, max_items, items, counts, blk_off,
-                            n_sm, attn_cta_start, status);
+                            blk_off == smem_scratch ? smem_scratch + R + 1 : nullptr, n_sm, attn_cta_start, status);
         __syncthreads();
     }
     if (((int)blockIdx.x == b_split || split_helper) && split_items != nullptr && block_tables != nullptr)

@@ -264,6 +264,19 @@ def test_projection_row_wise_route_many_short_requests(oracle64):
     _check_projection(oracle64, MID, w, ads, b)
 
 
+@pytest.mark.parametrize("n_req,each", [(129, 1), (140, 1), (33, 5), (257, 4)])
+def test_projection_row_tiles_with_many_adapters(oracle64, n_req, each):
+    """More requests and more adapters in a row tile than a warp has lanes, a last tile of one row, requests across the
+    tile boundary, with t in two summands (up to 1024 rows) and in one (257 x 4 rows)."""
+    rng = np.random.default_rng(49)
+    w = wl.make_wqkv(MID, rng)
+    ads = _boosted_adapters(MID, rng, tuple((8, 0.5 + 0.1 * (i % 7)) for i in range(36)))
+    P = [(i * 37) % 200 for i in range(n_req)]
+    ids = [(i * 5) % 37 - 1 for i in range(n_req)]
+    b = wl.make_batch(MID, P, [each] * n_req, ids, rng, activation_offsets=[p + (i % 6 == 0) for i, p in enumerate(P)])
+    _check_projection(oracle64, MID, w, ads, b)
+
+
 @pytest.mark.parametrize("T", [1, 24, 33, 64, 65, 128])
 def test_projection_few_row_route_mixed_adapters(oracle64, T):
     """Batches of at most 128 rows (decode steps): the weight-streaming route, K split over the SMs, the shrink of
