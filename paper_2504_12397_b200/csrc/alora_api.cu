@@ -19,7 +19,8 @@ int launch_linear_simt(alora_ctx *, const void *, const void *, int, int, int, v
 int launch_attend_simt(alora_ctx *, const void *, const BatchArgs &, const void *, void *, cudaStream_t);
 
 int launch_project_tc(alora_ctx *, int, const void *, int, int, void *, cudaStream_t, void *, int);
-int launch_linear_tc(alora_ctx *, const void *, const void *, int, int, int, void *, const void *, cudaStream_t);
+int launch_linear_tc(alora_ctx *, const void *, const void *, int, int, int, void *, const void *, const LinearDelta *,
+                     cudaStream_t);
 int launch_repack_mlp(const void *, const void *, const void *, const void *, int, int, int, int, int, void *, void *,
                       cudaStream_t);   // mlp_adapter.cu
 int launch_mlp_expand(alora_ctx *, void *, int, int, const void *, int, const void *, int, int, int, const int32_t *,
@@ -44,8 +45,8 @@ int launch_project(alora_ctx *ctx, int layer, const void *hidden, int T, int R, 
     return launch_project_simt(ctx, layer, hidden, T, qkv, s);
 }
 int launch_linear(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
-                  const void *residual, cudaStream_t s) {
-    if (ctx->cfg.dtype == ALORA_DTYPE_BF16) return launch_linear_tc(ctx, x, W, T, K, N, y, residual, s);
+                  const void *residual, cudaStream_t s, const LinearDelta *delta) {
+    if (ctx->cfg.dtype == ALORA_DTYPE_BF16) return launch_linear_tc(ctx, x, W, T, K, N, y, residual, delta, s);
     return launch_linear_simt(ctx, x, W, T, K, N, y, residual, s);
 }
 int launch_attend(alora_ctx *ctx, const void *qkv, const BatchArgs &b, const void *pool, void *out,
@@ -402,9 +403,10 @@ alora_status alora_register_mlp_adapter(alora_ctx *ctx, int adapter_id, int laye
         ALORA_CUDA(ctx, cudaMemsetAsync(ctx->d_mlp_adapters, 0, bytes, s));
     }
     if (!ctx->d_mlp_t) {
-        const size_t rows = (size_t)std::min(std::max(ctx->cfg.max_tokens, 1), kMlpChunk);
+        // (shrink kernel and its partials: only for the projections of at most kFewRowMax rows)
+        const size_t rows = (size_t)std::min(std::max(ctx->cfg.max_tokens, 1), kFewRowMax);
         const size_t rows_pad = (rows + 63) / 64 * 64;
-        ALORA_CUDA(ctx, cudaMalloc(&ctx->d_mlp_t, rows * na * 2 * d.RP * es));
+        ALORA_CUDA(ctx, cudaMalloc(&ctx->d_mlp_t, std::max(rows * na, (size_t)ctx->max_pairs * kTileRows) * 2 * d.RP * es));
         // K-slice partials of the shrink kernel: room for four slices of the widest result, at most 64 MB (the
         // kernel takes fewer slices when a batch's partials would not fit)
         ctx->mlp_part_floats = std::min<size_t>(4 * rows_pad * na * 2 * d.RP, (size_t)16 << 20);
@@ -688,13 +690,18 @@ alora_status alora_forward_stack(alora_ctx *ctx, int mode, const void *d_hidden_
             const int tc = std::min(kMlpChunk, T - t0);
             const char *xm = (const char *)ctx->d_act[0] + (size_t)t0 * d.H * ctx->esize;
             char *hc = h + (size_t)t0 * d.H * ctx->esize;
-            // adapters on the MLP block: shrink against all of the layer's A rows (one launch), then the expand
-            // step adds each open-gate row's delta in place (the row's applied adapter comes from this layer's
-            // batch metadata; base-model batches and closed gates have none)
+            // adapters on the MLP block: part of the projections' launches; on the few-row route a shrink against all of
+            // the layer's A rows (one launch) and an expand step that adds each open-gate row's delta in place
             const int n_mlp = (mode != ALORA_MODE_BASE && !ctx->mlp_n_adapters.empty()) ? ctx->mlp_n_adapters[l] : 0;
             const MlpAdapterDev *mlp_tab = n_mlp ? ctx->d_mlp_adapters + (size_t)l * std::max(1, ctx->cfg.max_adapters) : nullptr;
-            ALORA_STEP(launch_linear(ctx, xm, lw.wgate_up, tc, d.H, 2 * d.I, ctx->d_act[2], nullptr, s));
-            if (n_mlp) {
+            const bool fused = n_mlp && linear_takes_delta(ctx, tc, d.H, 2 * d.I) && linear_takes_delta(ctx, tc, d.I, d.H);
+            LinearDelta gu{}, dn{};
+            if (fused) {
+                gu = LinearDelta{ctx->mlp_a_gu[l], ctx->mlp_b_gu[l], 2, mlp_tab, t0 / kTileRows, ctx->d_row_adapter + t0, ctx->d_mlp_t};
+                dn = LinearDelta{ctx->mlp_a_dn[l], ctx->mlp_b_dn[l], 1, mlp_tab, t0 / kTileRows, ctx->d_row_adapter + t0, ctx->d_mlp_t};
+            }
+            ALORA_STEP(launch_linear(ctx, xm, lw.wgate_up, tc, d.H, 2 * d.I, ctx->d_act[2], nullptr, s, fused ? &gu : nullptr));
+            if (n_mlp && !fused) {
                 const int tw = n_mlp * 2 * d.RP;
                 ALORA_STEP(launch_mlp_shrink(ctx, xm, ctx->mlp_a_gu[l], tc, d.H, tw, ctx->d_mlp_t, ctx->d_mlp_part,
                                              ctx->mlp_part_floats, ctx->d_mlp_done, ctx->mlp_done_ints, s));
@@ -702,8 +709,8 @@ alora_status alora_forward_stack(alora_ctx *ctx, int mode, const void *d_hidden_
                                              d.I, 2, ctx->d_row_adapter + t0, mlp_tab, n_mlp, s));
             }
             ALORA_STEP(launch_swiglu(ctx, ctx->d_act[2], tc, ctx->d_act[3], s));
-            ALORA_STEP(launch_linear(ctx, ctx->d_act[3], lw.wdown, tc, d.I, d.H, hc, hc, s));  // h += down(...)
-            if (n_mlp) {
+            ALORA_STEP(launch_linear(ctx, ctx->d_act[3], lw.wdown, tc, d.I, d.H, hc, hc, s, fused ? &dn : nullptr));  // h += down(...)
+            if (n_mlp && !fused) {
                 const int tw = n_mlp * d.RP;
                 ALORA_STEP(launch_mlp_shrink(ctx, ctx->d_act[3], ctx->mlp_a_dn[l], tc, d.I, tw, ctx->d_mlp_t, ctx->d_mlp_part,
                                              ctx->mlp_part_floats, ctx->d_mlp_done, ctx->mlp_done_ints, s));

@@ -151,7 +151,8 @@ struct alora_ctx {
     std::vector<int> mlp_n_adapters;                 // [layer] highest registered MLP adapter id + 1
     std::vector<alora::MlpAdapterDev> h_mlp_adapters;   // [layer * max_adapters + id], mirrors d_mlp_adapters
     alora::MlpAdapterDev *d_mlp_adapters = nullptr;
-    void *d_mlp_t = nullptr;                         // [min(max_tokens, kMlpChunk)][max_adapters * 2 * RP] shrink results
+    void *d_mlp_t = nullptr;                         // t of the MLP adapters: [max_pairs][128][2 * RP], or (few-row route)
+                                                     // [kFewRowMax][max_adapters * 2 * RP]
     float *d_mlp_part = nullptr;                     // K-slice partials of the shrink kernel
     size_t mlp_part_floats = 0;
     int32_t *d_mlp_done = nullptr;                   // per 64 x 64 tile of the shrink result: slices stored (zero between launches)
@@ -288,8 +289,20 @@ int launch_cow_tail_pages(alora_ctx *ctx, const int32_t *qsl, const int32_t *seq
 int launch_rope(alora_ctx *ctx, void *qkv, const int32_t *positions, int T, void *pool, int num_pages, cudaStream_t s);
 int launch_attend(alora_ctx *ctx, const void *qkv, const BatchArgs &b, const void *pool, void *out,
                   cudaStream_t s);
+// A gated low-rank delta on a dense projection (adapters on the MLP block): the A and B slabs of all adapters of the layer
+// (64 padded rank columns per adapted matrix, n_blk matrices side by side in the output row), the layer's table, the
+// batch's row tile of the projection's first row, the applied adapter of its rows, room for t ([max_pairs][128][64 n_blk]).
+struct LinearDelta {
+    const void *A, *B;
+    int n_blk;
+    const MlpAdapterDev *table;
+    int tile0;
+    const int32_t *row_adapter;
+    void *t;
+};
 int launch_linear(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
-                  const void *residual, cudaStream_t s);
+                  const void *residual, cudaStream_t s, const LinearDelta *delta = nullptr);
+bool linear_takes_delta(const alora_ctx *ctx, int T, int K, int N);   // gemm_tcgen05.cu
 int launch_rmsnorm(alora_ctx *ctx, const void *x, const void *w, int T, void *y, cudaStream_t s);
 int launch_swiglu(alora_ctx *ctx, const void *gate_up, int T, void *y, cudaStream_t s);
 

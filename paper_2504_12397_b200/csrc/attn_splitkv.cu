@@ -47,8 +47,8 @@ struct SplitArgs {
     __nv_bfloat16 *out;         // [T][Nq]
     float *part_o;              // [partial row][HD], unnormalised, relative to the row's maximum in the item
     float *part_ml;             // [partial row][2]: maximum (scaled, log2 units), sum
-    int32_t *work_counter;      // next unclaimed item (zero between launches)
-    int32_t *blocks_done;       // blocks that have finished (zero between launches)
+    int32_t *work_counter;      // next unclaimed item (cleared by the metadata step)
+    int32_t *blocks_done;       // blocks that have finished (zero between launches); nullptr: a launch that does not share its list
     int32_t *group_done;        // per (stream, KV head), at its first partial row / 16: key ranges finished so far (zero between launches)
     int32_t *status;
 };
@@ -576,8 +576,8 @@ attn_splitkv_kernel(const __grid_constant__ CUtensorMap tmKV, const SplitArgs a)
     }
     __syncthreads();
     if (threadIdx.x == 0 && *abort_flag) report(a.status, ALORA_ERR_TIMEOUT);
-    // the last block to finish clears the claim counter: the layers of a stack call share one work list
-    if (threadIdx.x == 0) {
+    // the layers of a stack call share one work list: there the last block to finish clears the claim counter
+    if (threadIdx.x == 0 && a.blocks_done != nullptr) {
         __threadfence();
         if (atomicAdd(a.blocks_done, 1) == (int)gridDim.x - 1) { *a.work_counter = 0; *a.blocks_done = 0; __threadfence(); }
     }
@@ -615,7 +615,7 @@ int launch_attend_splitkv(alora_ctx *ctx, const void *qkv, const BatchArgs &b, c
     a.max_blocks = b.max_blocks; a.num_pages = b.num_pages; a.Hkv = d.Hkv; a.G = d.G; a.page_size = d.page;
     a.box_rows = box_rows; a.N = d.N; a.Nq = d.Nq; a.scale_log2 = d.softmax_scale * 1.4426950408889634f;
     a.qkv = (const __nv_bfloat16 *)qkv; a.out = (__nv_bfloat16 *)out; a.part_o = ctx->d_part_o;
-    a.part_ml = ctx->d_part_ml; a.work_counter = ctx->d_counts + 4; a.blocks_done = ctx->d_counts + 12; a.group_done = ctx->d_group_done;
+    a.part_ml = ctx->d_part_ml; a.work_counter = ctx->d_counts + 4; a.blocks_done = b.n_layers > 1 || b.facts_ready ? ctx->d_counts + 12 : nullptr; a.group_done = ctx->d_group_done;
     a.status = ctx->d_status;
     static bool attr_set[2][64] = {};
     const int dev = ctx->cfg.device, hi = d.hd == 128;

@@ -1,20 +1,26 @@
-// Gated multi-adapter q/k/v projection (Eq. 2 / Eq. 5) for batches of many rows: 256 x 192 output tiles.
+// Dense contractions of many rows with the aLoRA delta fused in: the gated q/k/v projection (Eq. 2 / Eq. 5) with 256 x 192
+// output tiles, and the o_proj / MLP matrices of the layer stack with 256 x 256 tiles (residual in the epilogue; with
+// adapters on the MLP block the same gated delta).
 //
 // Same computation and the same work list as gemm_tcgen05.cu's tile route (dense row tiles of 128 rows and the
 // (row tile, adapter) pairs that occur; t = s A_k x from leading "shrink items" of the same launch; a tile appends
-// t B_k^T of each of its adapters to its K loop; optional KV append in the epilogue), with another tile shape: a block owns TWO row tiles that share the
-// W tile, 56 KB of operands per 64-wide K block for 8 x 96 tensor-pipe cycles instead of 48 KB for 4 x 128, i.e.
-// 1.3 x the flops per operand byte (one SM cannot fill its shared memory fast enough for the 128 x 256 tile), and
-// 192-wide column tiles so that 2048 rows x 6144 columns make 256 tiles: two rounds over 148 blocks at 86 %.
+// t B_k^T of each of its adapters to its K loop; optional KV append in the epilogue), with another tile shape: a block
+// owns TWO row tiles that share the W tile.  256 x 192: 56 KB of operands per 64-wide K block for 8 x 96 tensor-pipe
+// cycles instead of 48 KB for 4 x 128, i.e. 1.3 x the flops per operand byte (one SM cannot fill its shared memory fast
+// enough for the 128 x 256 tile), and 192-wide column tiles so that 2048 rows x 6144 columns make 256 tiles: two rounds
+// over 148 blocks at 86 %.  256 x 256: 64 KB for 8 x 128 cycles, 1.5 x the flops per byte.
 // The two row tiles accumulate in the two halves of tensor memory (not double-buffered; the next item's loads run
 // under the epilogue and its MMAs start on a half as soon as that half has been drained).
+//
+// The MLP deltas as further K blocks cost next to nothing: 2048 rows of 8 x (8192 + 256) through two adapted layers took
+// 174 us a layer for them when the shrink and the update of the finished gate / up / down rows were kernels of their own.
 //
 // A 192-wide column tile can straddle the q | k | v boundaries of the fused row.  The expand step therefore takes
 // one K block per (pair, q/k/v block that the column tile touches): A = that block's 64 (padded-rank) columns
 // of t, B = the adapter's B rows of that block through a 3-D tensor map (rank column, row inside the block,
 // adapter) whose out-of-range rows read as zero, so the columns of the other block get no contribution.
 //
-//   warp 0   TMA producer (4 slots of 56 KB)      warp 1   MMA issuer (whole warp walks, elected lane issues)
+//   warp 0   TMA producer (4 slots of 56 KB or 3 of 64 KB)      warp 1   MMA issuer (whole warp walks, elected lane issues)
 //   warps 2-5 / 6-9  epilogue of the first / second row tile: tcgen05.ld one row per thread, bf16, 16-byte stores,
 //              KV append, or t for shrink items
 // All waits are bounded; on expiry ALORA_ERR_TIMEOUT is recorded and the block leaves normally.
@@ -27,27 +33,36 @@
 namespace alora {
 
 namespace {
-constexpr int kBNp = 192, kBKp = 64, kStagesP = 4, kThreadsP = 320;   // producer, issuer, 2 x 4 epilogue warps
+constexpr int kBKp = 64, kThreadsP = 320;          // producer, issuer, 2 x 4 epilogue warps
+constexpr int kBNqkv = 192;                        // column tile of the q/k/v projection
 constexpr int kTensorRP = 64;                      // the tensor path stores adapters padded to 64 rank columns
 constexpr int kHalfAp = 128 * kBKp * 2;            // one row tile's x (or t) block: 16 KB
-constexpr int kBBytesP = kBNp * kBKp * 2;          // 24 KB
-constexpr int kStageBytesP = 2 * kHalfAp + kBBytesP;
-constexpr int kBarOffP = kStagesP * kStageBytesP;
-constexpr int kItemRingOffP = kBarOffP + 256;
-constexpr int kSmemTotalP = kItemRingOffP + 128 + 1024;
-constexpr int kShrinkColsP = 3 * kTensorRP;        // 192 columns of t = one column tile
+template <int BN>
+struct PairSmem {
+    static constexpr int kStages = BN <= 192 ? 4 : 3;
+    static constexpr int kBBytes = BN * kBKp * 2;
+    static constexpr int kStageBytes = 2 * kHalfAp + kBBytes;
+    static constexpr int kBarOff = kStages * kStageBytes;
+    static constexpr int kItemRingOff = kBarOff + 256;
+    static constexpr int kTotal = kItemRingOff + 128 + 1024;
+};
 
 struct PairArgs {
     const TilePair *pairs;          // (row tile, adapter) pairs, nullptr: no adapters in this launch
     const int32_t *pair_off;        // [row tiles + 1] first pair of each row tile
-    int M, N, K, Nq, Nkv;
+    int tile0;                      // row tile of the batch that holds this launch's first row
+    int shrink;                     // the launch has shrink items, one per pair of its row tiles (0: t is there already)
+    int t_cols;                     // columns of t: 64 padded rank columns per adapted matrix
+    const int32_t *adapters;        // per adapter `ad_stride` words, the first two: padded rank, scale (float)
+    int ad_stride;
+    int M, N, K, Nq, Nkv;           // Nq, Nkv: the q/k/v blocks of the fused row
+    int blk_cols;                   // other launches: columns per adapted matrix
     __nv_bfloat16 *out;
     int ldo;
-    const AdapterDev *adapters;
-    const int32_t *n_pairs;         // shrink items of this launch: one per pair (nullptr: t is there already)
+    const __nv_bfloat16 *residual;  // optional, same layout as out, may alias it
     const int32_t *row_adapter;     // [M] applied adapter per row (shrink items: which rows of t are kept)
     int32_t *t_ready;               // [pair] epilogue warps that have published their part of t
-    __nv_bfloat16 *t_out;           // [pair][128][192]
+    __nv_bfloat16 *t_out;           // [pair][128][t_cols]
     // KV append fused into the epilogue (nullptr: off), as in gemm_tcgen05.cu
     __nv_bfloat16 *kv_pool;
     const int32_t *slot_map;
@@ -69,31 +84,38 @@ __device__ __forceinline__ void tma_load_3d_p(uint32_t smem_dst, const CUtensorM
         : "memory");
 }
 
-// One work item: a shrink item (row tile m[0] only) or two row tiles (m[1] = -1: none) x one column tile.
+__device__ __forceinline__ int rank_steps(const PairArgs &a, int adapter) { return a.adapters[adapter * a.ad_stride] / 16; }
+
+// One work item: a shrink item (pair p0[0], row tile m[0]) or two row tiles (m[1] = -1: none) x one column tile.
 struct PairItem {
     int m[2];
     int p0[2], p1[2];    // pairs of each row tile
     int n0, adapter;
     bool shrink;
 };
-__device__ __forceinline__ PairItem decode_pair(const PairArgs &a, int item, int n_shrink, int n_m, int n_n) {
+// kQkv: the column tiles of a row-tile pair are neighbours in the list; else the row tiles of a column tile (the blocks
+// that run together share a W tile).
+template <int BN, bool kQkv>
+__device__ __forceinline__ PairItem decode_pair(const PairArgs &a, int item, int n_shrink, int p_base, int n_m, int n_n) {
     PairItem g;
     g.n0 = 0; g.adapter = -1; g.m[1] = -1;
     g.p0[0] = g.p1[0] = g.p0[1] = g.p1[1] = 0;
     g.shrink = item < n_shrink;
     if (g.shrink) {
-        const TilePair p = a.pairs[item];
-        g.m[0] = p.tile;
+        const TilePair p = a.pairs[p_base + item];
+        g.m[0] = p.tile - a.tile0;
         g.adapter = p.adapter;
+        g.p0[0] = g.p1[0] = g.p0[1] = g.p1[1] = p_base + item;
     } else {
-        const int j = item - n_shrink;
-        g.m[0] = 2 * (j / n_n);
+        const int j = item - n_shrink, n_mp = (n_m + 1) / 2;
+        g.m[0] = 2 * (kQkv ? j / n_n : j % n_mp);
         g.m[1] = g.m[0] + 1 < n_m ? g.m[0] + 1 : -1;
-        g.n0 = (j % n_n) * kBNp;
+        g.n0 = (kQkv ? j % n_n : j / n_mp) * BN;
         if (a.pairs) {
-            g.p0[0] = a.pair_off[g.m[0]];
-            g.p1[0] = g.p0[1] = a.pair_off[g.m[0] + 1];
-            g.p1[1] = g.m[1] >= 0 ? a.pair_off[g.m[0] + 2] : g.p0[1];
+            const int32_t *off = a.pair_off + a.tile0 + g.m[0];
+            g.p0[0] = off[0];
+            g.p1[0] = g.p0[1] = off[1];
+            g.p1[1] = g.m[1] >= 0 ? off[2] : g.p0[1];
         }
     }
     return g;
@@ -103,19 +125,23 @@ __device__ __forceinline__ int blk_start(const PairArgs &a, int blk) { return bl
 __device__ __forceinline__ int blk_end(const PairArgs &a, int blk) { return blk == 0 ? a.Nq : (blk == 1 ? a.Nq + a.Nkv : a.N); }
 // does the column tile at n0 touch block blk?
 __device__ __forceinline__ bool touches(const PairArgs &a, int n0, int blk) {
-    return n0 < blk_end(a, blk) && n0 + kBNp > blk_start(a, blk);
+    return n0 < blk_end(a, blk) && n0 + kBNqkv > blk_start(a, blk);
 }
 
+template <int BN, bool kQkv>
 __global__ void __launch_bounds__(kThreadsP, 1)
 gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                          const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmS,
                          const __grid_constant__ CUtensorMap tmB0, const __grid_constant__ CUtensorMap tmB1,
                          const __grid_constant__ CUtensorMap tmB2, const PairArgs a) {
+    using S = PairSmem<BN>;
+    constexpr int kStagesP = S::kStages, kBBytesP = S::kBBytes, kStageBytesP = S::kStageBytes;
+    constexpr int kBarOffP = S::kBarOff, kItemRingOffP = S::kItemRingOff;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (tc::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_al = smem_raw + (smem_base - tc::smem_u32(smem_raw));
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem_al + kBarOffP);
-    // barrier words: full[4], empty[4], acc_full, acc_empty[2] (one per half), drain
+    // barrier words: full[stages], empty[stages], acc_full, acc_empty[2] (one per half), drain
     const uint32_t bar0 = smem_base + kBarOffP;
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
     auto empty_bar = [&](int s) { return bar0 + 8u * (kStagesP + s); };
@@ -146,8 +172,9 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
     tc::grid_dep_wait();   // the metadata step's lists, the activations: all written by earlier kernels of the stream
 
     const int n_m = (a.M + 127) / 128;
-    const int n_n = (a.N + kBNp - 1) / kBNp;
-    const int n_shrink = a.n_pairs ? *a.n_pairs : 0;
+    const int n_n = (a.N + BN - 1) / BN;
+    const int p_base = a.shrink ? a.pair_off[a.tile0] : 0;
+    const int n_shrink = a.shrink ? a.pair_off[a.tile0 + n_m] - p_base : 0;
     const int total = n_shrink + ((n_m + 1) / 2) * n_n;
     const int kb_main = (a.K + kBKp - 1) / kBKp;
 
@@ -184,21 +211,21 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                 }
                 if (!ring.put(item, abort_flag)) { ok = false; break; }
                 if (item < 0) break;
-                const PairItem g = decode_pair(a, item, n_shrink, n_m, n_n);
+                const PairItem g = decode_pair<BN, kQkv>(a, item, n_shrink, p_base, n_m, n_n);
                 const bool two = g.m[1] >= 0;
                 for (int kb = 0; kb < kb_main && ok; ++kb, ++kc) {
                     const int s = kc % kStagesP;
                     if (!tc::mbar_wait(empty_bar(s), ((kc / kStagesP) & 1) ^ 1, abort_flag)) { ok = false; break; }
                     const uint32_t sa = smem_base + s * kStageBytesP, sb = sa + 2 * kHalfAp;
-                    tc::mbar_arrive_expect_tx(full_bar(s), (two ? 2 : 1) * kHalfAp + kBBytesP);
+                    tc::mbar_arrive_expect_tx(full_bar(s), (two ? 2 : 1) * kHalfAp + (g.shrink ? a.t_cols * kBKp * 2 : kBBytesP));
                     tc::tma_load_2d(sa, &tmX, full_bar(s), kb * kBKp, g.m[0] * 128);
                     if (two) tc::tma_load_2d(sa + kHalfAp, &tmX, full_bar(s), kb * kBKp, g.m[1] * 128);
-                    if (g.shrink) tc::tma_load_2d(sb, &tmS, full_bar(s), kb * kBKp, g.adapter * kShrinkColsP);
+                    if (g.shrink) tc::tma_load_2d(sb, &tmS, full_bar(s), kb * kBKp, g.adapter * a.t_cols);
                     else tc::tma_load_2d(sb, &tmW, full_bar(s), kb * kBKp, g.n0);
                 }
                 if (g.shrink) continue;
-                // expand: per pair of the row tiles, one K block per q/k/v block the column tile touches
-                for (int h = 0; h < 2 && ok; ++h) {
+                // expand: per pair of the row tiles, one K block per adapted matrix (q / k / v block) the column tile touches
+                for (int h = 0; h < 2 && ok && !g.shrink; ++h) {
                     int next_ad = g.p0[h] < g.p1[h] ? a.pairs[g.p0[h]].adapter : -1;
                     for (int p = g.p0[h]; p < g.p1[h] && ok; ++p) {
                         const int adapter = next_ad;
@@ -213,15 +240,17 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                             if (!ok) break;
                             asm volatile("fence.proxy.async.global;" ::: "memory");
                         }
-                        for (int blk = 0; blk < 3 && ok; ++blk) {
-                            if (!touches(a, g.n0, blk)) continue;
+                        for (int blk = 0; blk < (kQkv ? 3 : 1) && ok; ++blk) {
+                            if (kQkv && !touches(a, g.n0, blk)) continue;
                             const int s = kc % kStagesP;
                             if (!tc::mbar_wait(empty_bar(s), ((kc / kStagesP) & 1) ^ 1, abort_flag)) { ok = false; break; }
                             const uint32_t sa = smem_base + s * kStageBytesP, sb = sa + 2 * kHalfAp;
                             tc::mbar_arrive_expect_tx(full_bar(s), kHalfAp + kBBytesP);
-                            tc::tma_load_2d(sa + h * kHalfAp, &tmT, full_bar(s), blk * kTensorRP, p * 128);
-                            tma_load_3d_p(sb, blk == 0 ? &tmB0 : (blk == 1 ? &tmB1 : &tmB2), full_bar(s), 0,
-                                          g.n0 - blk_start(a, blk), adapter);
+                            const int t_blk = kQkv ? blk : g.n0 / a.blk_cols;
+                            tc::tma_load_2d(sa + h * kHalfAp, &tmT, full_bar(s), t_blk * kTensorRP, p * 128);
+                            if (kQkv) tma_load_3d_p(sb, blk == 0 ? &tmB0 : (blk == 1 ? &tmB1 : &tmB2), full_bar(s), 0,
+                                                    g.n0 - blk_start(a, blk), adapter);
+                            else tc::tma_load_2d(sb, &tmB0, full_bar(s), 0, adapter * a.N + g.n0);
                             ++kc;
                         }
                     }
@@ -243,16 +272,18 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
         auto wait_all = [&](uint32_t bar, uint32_t parity) {
             return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort_flag));
         };
-        constexpr uint32_t idesc = tc::idesc_bf16_f32(128, kBNp);
+        constexpr uint32_t idesc_main = tc::idesc_bf16_f32(128, BN);
+        const uint32_t idesc_shrink = tc::idesc_bf16_f32(128, a.t_cols);
         uint32_t kc = 0, it = 0;
         bool ok = true;
         for (;; ++it) {
             const int item = ring.take(abort_flag);
             if (item < 0) { ok = item == -1; break; }
-            const PairItem g = decode_pair(a, item, n_shrink, n_m, n_n);
+            const PairItem g = decode_pair<BN, kQkv>(a, item, n_shrink, p_base, n_m, n_n);
             const bool two = g.m[1] >= 0;
             // MMA steps of the row tiles' adapters, one per lane, loaded while the main loop runs
-            const int my_steps = g.p0[0] + lane < g.p1[1] ? a.adapters[a.pairs[g.p0[0] + lane].adapter].rpad / 16 : 0;
+            const int my_steps = g.p0[0] + lane < g.p1[1] ? rank_steps(a, a.pairs[g.p0[0] + lane].adapter) : 0;
+            const uint32_t idesc = g.shrink ? idesc_shrink : idesc_main;
             for (int kb = 0; kb < kb_main && ok; ++kb, ++kc) {
                 const int s = kc % kStagesP;
                 if (!wait_all(full_bar(s), (kc / kStagesP) & 1)) { ok = false; break; }
@@ -281,9 +312,9 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
             for (int h = 0; h < 2 && ok; ++h) {
                 for (int p = g.p0[h]; p < g.p1[h] && ok; ++p) {
                     const int at = p - g.p0[0];   // (the pairs of the two row tiles follow one another)
-                    const int steps = at < 32 ? __shfl_sync(0xffffffffu, my_steps, at) : a.adapters[a.pairs[p].adapter].rpad / 16;
-                    for (int blk = 0; blk < 3 && ok; ++blk) {
-                        if (!touches(a, g.n0, blk)) continue;
+                    const int steps = at < 32 ? __shfl_sync(0xffffffffu, my_steps, at) : rank_steps(a, a.pairs[p].adapter);
+                    for (int blk = 0; blk < (kQkv ? 3 : 1) && ok; ++blk) {
+                        if (kQkv && !touches(a, g.n0, blk)) continue;
                         const int s = kc % kStagesP;
                         if (!wait_all(full_bar(s), (kc / kStagesP) & 1)) { ok = false; break; }
                         tc::tc_fence_after();
@@ -315,7 +346,7 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
         for (;; ++it) {
             const int item = ring.take(abort_flag);
             if (item < 0) break;
-            const PairItem g = decode_pair(a, item, n_shrink, n_m, n_n);
+            const PairItem g = decode_pair<BN, kQkv>(a, item, n_shrink, p_base, n_m, n_n);
             if (!tc::mbar_wait(accf_bar, it & 1, abort_flag)) { ok = false; break; }
             tc::tc_fence_after();
             const int r = q * 32 + lane;
@@ -326,13 +357,13 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                 continue;
             }
             if (g.shrink) {
-                // t = s A x of this pair: 192 columns, zero in the rows that do not use the adapter
+                // t = s A x of this pair, zero in the rows that do not use the adapter
                 const int row = g.m[0] * 128 + r;
                 const bool use = row < a.M && a.row_adapter[row] == g.adapter;
-                const float scale = a.adapters[g.adapter].scale;
-                __nv_bfloat16 *trow = a.t_out + ((size_t)item * 128 + r) * kShrinkColsP;
+                const float scale = __int_as_float(a.adapters[g.adapter * a.ad_stride + 1]);
+                __nv_bfloat16 *trow = a.t_out + ((size_t)g.p0[0] * 128 + r) * a.t_cols;
 #pragma unroll 1
-                for (int c = 0; c < kShrinkColsP; c += 32) {
+                for (int c = 0; c < a.t_cols; c += 32) {
                     uint32_t v[32];
                     tc::tmem_ld_32x32(tmem_base + c + ((uint32_t)(q * 32) << 16), v);
                     tc::tmem_ld_wait();
@@ -344,7 +375,7 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                 __threadfence();
                 __syncwarp();
                 if (lane == 0) {
-                    atomicAdd(a.t_ready + item, 1);
+                    atomicAdd(a.t_ready + g.p0[0], 1);
                     tc::mbar_arrive(acce_bar(0));
                 }
                 continue;
@@ -355,9 +386,10 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                     const int row = g.m[h] * 128 + r;
                     const bool row_ok = row < a.M;
                     __nv_bfloat16 *orow = a.out + (size_t)row * a.ldo + g.n0;
+                    const __nv_bfloat16 *rrow = a.residual ? a.residual + (size_t)row * a.ldo + g.n0 : nullptr;
                     // fused KV append: where this row's k / v columns go in the page pool
                     int kv_page = -1, kv_row = 0;
-                    if (a.kv_pool != nullptr && row_ok && g.n0 + kBNp > a.Nq) {
+                    if (kQkv && a.kv_pool != nullptr && row_ok && g.n0 + BN > a.Nq) {
                         const int slot = a.slot_map[row];
                         if (slot >= 0) {
                             kv_page = slot / a.kv_page_size;
@@ -366,7 +398,7 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                         }
                     }
 #pragma unroll 1
-                    for (int c = 0; c < kBNp; c += 32) {
+                    for (int c = 0; c < BN; c += 32) {
                         uint32_t v[32];
                         tc::tmem_ld_32x32(tmem_base + h * 256 + c + ((uint32_t)(q * 32) << 16), v);
                         tc::tmem_ld_wait();
@@ -374,12 +406,24 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
 #pragma unroll
                             for (int j = 0; j < 4; ++j) {
                                 if (g.n0 + c + 8 * j >= a.N) break;
+                                float f[8];
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[8 * j + e]);
+                                if (!kQkv && rrow) {
+                                    const uint4 rv = *reinterpret_cast<const uint4 *>(rrow + c + 8 * j);
+                                    const uint32_t rw[4] = {rv.x, rv.y, rv.z, rv.w};
+#pragma unroll
+                                    for (int e = 0; e < 4; ++e) {
+                                        const __nv_bfloat162 b2 = *reinterpret_cast<const __nv_bfloat162 *>(&rw[e]);
+                                        f[2 * e] += __low2float(b2);
+                                        f[2 * e + 1] += __high2float(b2);
+                                    }
+                                }
                                 uint4 o;
-                                o.x = tc::pack_bf16(__uint_as_float(v[8 * j]), __uint_as_float(v[8 * j + 1]));
-                                o.y = tc::pack_bf16(__uint_as_float(v[8 * j + 2]), __uint_as_float(v[8 * j + 3]));
-                                o.z = tc::pack_bf16(__uint_as_float(v[8 * j + 4]), __uint_as_float(v[8 * j + 5]));
-                                o.w = tc::pack_bf16(__uint_as_float(v[8 * j + 6]), __uint_as_float(v[8 * j + 7]));
+                                o.x = tc::pack_bf16(f[0], f[1]); o.y = tc::pack_bf16(f[2], f[3]);
+                                o.z = tc::pack_bf16(f[4], f[5]); o.w = tc::pack_bf16(f[6], f[7]);
                                 *reinterpret_cast<uint4 *>(orow + c + 8 * j) = o;
+                                if (!kQkv) continue;
                                 const int kcol = g.n0 + c + 8 * j - a.Nq;   // column inside [k | v]
                                 if (kv_page >= 0 && kcol >= 0) {
                                     const int plane = kcol >= a.Nkv ? 1 : 0, c2 = kcol - plane * a.Nkv;
@@ -402,7 +446,7 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
     tc::tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && *abort_flag) report(a.status, ALORA_ERR_TIMEOUT);
-    if (threadIdx.x == 0) tc::item_counter_release(a.item_counters, a.t_ready, n_shrink);
+    if (threadIdx.x == 0) tc::item_counter_release(a.item_counters, a.t_ready + p_base, n_shrink);
     if (warp == 1) {
         tc::tc_fence_after();
         tc::tmem_dealloc(tmem_base, 512);
@@ -424,7 +468,7 @@ bool build_pair_maps(alora_ctx *ctx, int layer) {
     TcLayerMaps &lm = ctx->tc_maps[layer];
     const LayerWeights &lw = ctx->layers[layer];
     bool ok = true;
-    if (lw.wqkv) ok &= make_tensor_map_bf16(&lm.wqkv192, lw.wqkv, d.N, d.H, d.H, kBNp);
+    if (lw.wqkv) ok &= make_tensor_map_bf16(&lm.wqkv192, lw.wqkv, d.N, d.H, d.H, kBNqkv);
     EncodeTiledFn enc = tensor_map_encoder();
     if (!enc) return false;
     const size_t na = (size_t)std::max(1, ctx->cfg.max_adapters);
@@ -432,7 +476,7 @@ bool build_pair_maps(alora_ctx *ctx, int layer) {
     for (int blk = 0; blk < 3; ++blk) {
         cuuint64_t dims[3] = {(cuuint64_t)kTensorRP, (cuuint64_t)rows[blk], (cuuint64_t)na};
         cuuint64_t strides[2] = {(cuuint64_t)kTensorRP * 2, (cuuint64_t)d.N * kTensorRP * 2};
-        cuuint32_t box[3] = {(cuuint32_t)kTensorRP, (cuuint32_t)kBNp, 1};
+        cuuint32_t box[3] = {(cuuint32_t)kTensorRP, (cuuint32_t)kBNqkv, 1};
         cuuint32_t es[3] = {1, 1, 1};
         void *base = (char *)ctx->tc_b_all[layer] + (size_t)starts[blk] * kTensorRP * 2;
         ok &= enc(&lm.b_blk[blk], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, es,
@@ -440,6 +484,16 @@ bool build_pair_maps(alora_ctx *ctx, int layer) {
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     }
     return ok;
+}
+
+template <int BN, bool kQkv>
+static bool pair_kernel_ready(alora_ctx *ctx) {
+    static bool attr_set[64] = {};   // one per instantiation
+    const int dev = ctx->cfg.device;
+    if (dev < 0 || dev >= 64 || attr_set[dev]) return true;
+    attr_set[dev] = cudaFuncSetAttribute(gemm_pair_tcgen05_kernel<BN, kQkv>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         PairSmem<BN>::kTotal) == cudaSuccess;
+    return attr_set[dev];
 }
 
 bool launch_shrink_tc(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap &tmA, const AdapterDev *adapters,
@@ -454,7 +508,7 @@ int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T,
     const Dims &d = ctx->d;
     if (T <= kSplitTTokens || d.H % 8 != 0 || d.N % 8 != 0 || d.Nq % 8 != 0 || d.Nkv % 8 != 0) return 0;
     const int G = ctx->sm_count;
-    const int n_n = (d.N + kBNp - 1) / kBNp, n_n256 = (d.N + 255) / 256;
+    const int n_n = (d.N + kBNqkv - 1) / kBNqkv, n_n256 = (d.N + 255) / 256;
     const int items = ((T + 255) / 256) * n_n, items128 = ((T + 127) / 128) * n_n256;
     const double eff = (double)items / ((double)((items + G - 1) / G) * G);
     const double eff128 = (double)items128 / ((double)((items128 + G - 1) / G) * G);
@@ -463,24 +517,19 @@ int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T,
     CUtensorMap tmX, tmT;
     if (!make_tensor_map_bf16(&tmX, hidden, T, d.H, d.H, 128)) return -1;
     if (!make_tensor_map_bf16(&tmT, ctx->d_t, (uint64_t)ctx->t_slots * 128, 3 * kTensorRP, 3 * kTensorRP, 128)) return -1;
-    static bool attr_set[64] = {};
-    const int dev = ctx->cfg.device;
-    if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        if (cudaFuncSetAttribute(gemm_pair_tcgen05_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTotalP) !=
-            cudaSuccess)
-            return -1;
-        attr_set[dev] = true;
-    }
+    if (!pair_kernel_ready<kBNqkv, true>(ctx)) return -1;
     PairArgs g{};
     g.M = T; g.N = d.N; g.K = d.H; g.Nq = d.Nq; g.Nkv = d.Nkv;
     g.out = (__nv_bfloat16 *)qkv; g.ldo = d.N;
-    g.adapters = ctx->d_adapters + (size_t)layer * ctx->cfg.max_adapters;
+    const AdapterDev *ads = ctx->d_adapters + (size_t)layer * ctx->cfg.max_adapters;
+    g.adapters = &ads->rpad;   // (address arithmetic only: padded rank and scale of an AdapterDev are neighbours)
+    g.ad_stride = sizeof(AdapterDev) / 4; g.t_cols = 3 * kTensorRP;
     const bool have_adapters = ctx->layer_has_adapter[layer] != 0;
     const bool apart = have_adapters && shrink_apart(ctx, T, R, items);
     const int max_pairs = have_adapters ? pair_bound(ctx, T, R) : 0;
     if (have_adapters) { g.pairs = ctx->d_pairs; g.pair_off = ctx->d_pair_off; }
     if (have_adapters && !apart) {
-        g.n_pairs = ctx->d_counts + 2; g.row_adapter = ctx->d_row_adapter;
+        g.shrink = 1; g.row_adapter = ctx->d_row_adapter;
         g.t_ready = ctx->d_t_ready; g.t_out = (__nv_bfloat16 *)ctx->d_t;
     }
     g.item_counters = ctx->d_counts + 10;
@@ -492,11 +541,48 @@ int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T,
     }
     g.status = ctx->d_status;
     const int grid = std::max(1, std::min(G, items + (apart ? 0 : max_pairs)));
-    if (apart && !launch_shrink_tc(ctx, tmX, lm.a_all, g.adapters, T, d.H, max_pairs, 1, s)) return -1;
-    if (launch_kernel(gemm_pair_tcgen05_kernel, dim3(grid), dim3(kThreadsP), kSmemTotalP, s, true, tmX, lm.wqkv192, tmT,
-                      lm.a_all, lm.b_blk[0], lm.b_blk[1], lm.b_blk[2], g) != cudaSuccess)
+    if (apart && !launch_shrink_tc(ctx, tmX, lm.a_all, ads, T, d.H, max_pairs, 1, s)) return -1;
+    if (launch_kernel(gemm_pair_tcgen05_kernel<kBNqkv, true>, dim3(grid), dim3(kThreadsP), PairSmem<kBNqkv>::kTotal, s, true, tmX,
+                      lm.wqkv192, tmT, lm.a_all, lm.b_blk[0], lm.b_blk[1], lm.b_blk[2], g) != cudaSuccess)
         return -1;
     return apart ? 2 : 1;
+}
+
+// Plain dense projection y = x W^T (+ residual) with many rows, optionally with a gated low-rank delta: 256 x 256 tiles.
+// Returns 1 (launched), 0 (shape better served by the 128-row kernel: not launched) or -1 (error).
+int launch_linear256_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
+                        const void *residual, const LinearDelta *delta, cudaStream_t s) {
+    constexpr int BN = 256;
+    const int n_n = (N + BN - 1) / BN, G = ctx->sm_count;
+    const int items = ((T + 255) / 256) * n_n, items128 = ((T + 127) / 128) * n_n;
+    // Rounds over the blocks x cycles of a tile's K block: 1230 here (0.83 of the tensor pipe), 790 for the 128 x 256 tile
+    // (shared-memory fill rate).
+    const long long here = (long long)((items + G - 1) / G) * 1230, other = (long long)((items128 + G - 1) / G) * 790;
+    if (T <= 256 || K % 8 != 0 || N % 8 != 0 || here > other) return 0;
+    CUtensorMap tmX, tmW, tmT, tmA, tmB;
+    if (!make_tensor_map_bf16(&tmX, x, T, K, K, 128)) return -1;
+    if (!make_tensor_map_bf16(&tmW, W, N, K, K, BN)) return -1;
+    tmT = tmX; tmA = tmW; tmB = tmW;
+    PairArgs g{};
+    g.M = T; g.N = N; g.K = K; g.Nq = N; g.Nkv = 0; g.blk_cols = N; g.t_cols = kTensorRP;
+    g.out = (__nv_bfloat16 *)y; g.residual = (const __nv_bfloat16 *)residual; g.ldo = N;
+    g.item_counters = ctx->d_counts + 10; g.status = ctx->d_status;
+    if (delta != nullptr) {
+        const uint64_t na = (uint64_t)std::max(1, ctx->cfg.max_adapters);
+        g.t_cols = delta->n_blk * kTensorRP; g.blk_cols = N / delta->n_blk;
+        if (!make_tensor_map_bf16(&tmT, delta->t, (uint64_t)ctx->max_pairs * 128, g.t_cols, g.t_cols, 128)) return -1;
+        if (!make_tensor_map_bf16(&tmA, delta->A, na * g.t_cols, K, K, g.t_cols)) return -1;
+        if (!make_tensor_map_bf16(&tmB, delta->B, na * N, kTensorRP, kTensorRP, BN)) return -1;
+        g.pairs = ctx->d_pairs; g.pair_off = ctx->d_pair_off; g.tile0 = delta->tile0; g.shrink = 1;
+        g.adapters = &delta->table->rpad; g.ad_stride = sizeof(MlpAdapterDev) / 4;
+        g.row_adapter = delta->row_adapter; g.t_ready = ctx->d_t_ready; g.t_out = (__nv_bfloat16 *)delta->t;
+    }
+    if (!pair_kernel_ready<BN, false>(ctx)) return -1;
+    const int grid = std::max(1, std::min(G, items + (delta != nullptr ? ctx->max_pairs : 0)));
+    if (launch_kernel(gemm_pair_tcgen05_kernel<BN, false>, dim3(grid), dim3(kThreadsP), PairSmem<BN>::kTotal, s, true, tmX, tmW,
+                      tmT, tmA, tmB, tmB, tmB, g) != cudaSuccess)
+        return -1;
+    return 1;
 }
 
 }  // namespace alora

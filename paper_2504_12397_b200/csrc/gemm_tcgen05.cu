@@ -47,17 +47,20 @@ struct GemmArgs {
     int a_tile_bytes;
     const TilePair *pairs;          // (row tile, adapter) pairs of the batch, nullptr: no adapters in this launch
     const int32_t *pair_off;        // [row tiles + 1] first pair of each row tile
+    int tile0;                      // row tile of the batch that holds this launch's first row
+    int shrink;                     // the launch has shrink items, one per pair of its row tiles (0: t is there already)
+    int t_cols;                     // columns of t: 64 padded rank columns per adapted matrix
+    const int32_t *adapters;        // per adapter `ad_stride` words, the first two: padded rank, scale (float)
+    int ad_stride;
     int M, N, K;
     __nv_bfloat16 *out;
     int ldo;
     const __nv_bfloat16 *residual;  // optional, same layout as out, may alias it
-    const AdapterDev *adapters;     // this layer's adapter table (expand), or nullptr
-    int Nq, Nkv;                    // block boundaries of the fused output row (expand)
+    int Nq, Nkv;                    // block boundaries of the fused output row (expand; gate | up: Nq = Nkv = half)
     int total_adapter_rows;         // rows per adapter in the B_all map (= N of the layer)
-    const int32_t *n_pairs;         // shrink items in this launch: one per pair (nullptr: t is there already)
     const int32_t *row_adapter;     // [M] applied adapter per row (shrink items: which rows of t are kept)
     int32_t *t_ready;               // [pair] epilogue warps that have published their part of t
-    __nv_bfloat16 *t_out;           // [pair][t_parts][128][192]
+    __nv_bfloat16 *t_out;           // [pair][t_parts][128][t_cols]
     int t_parts;                    // t is the sum of this many bf16 values (1 or 2)
     // KV append fused into the epilogue (nullptr: off): columns Nq .. N of row t also go to the paged cache,
     // pool[page][plane][head][row in page][:] with page * page_size + row = slot_map[t] (-1: token rejected, skipped)
@@ -81,30 +84,31 @@ struct GemmSmem {
     static constexpr int kTotal = kItemRingOffset + 128 + 1024;  // barriers, item ring, slack for 1024-byte alignment
 };
 
-constexpr int kShrinkCols = 3 * kTensorRP;  // 192 columns of t: q, k, v blocks of 64 padded rank columns
+__device__ __forceinline__ int rank_steps(const GemmArgs &a, int adapter) { return a.adapters[adapter * a.ad_stride] / 16; }
 
 // Work item `item` of a launch: shrink items first (one per pair), then the projection's
 // (row tile, column tile) pairs.
 struct GemmItem {
     int m;            // row-tile index
     int n0;           // first output column (projection items)
-    int p0, p1;       // projection items: the row tile's pairs
+    int p0, p1;       // projection items: the row tile's pairs; shrink items: p0 = p1 = its pair
     int adapter;      // shrink items
     bool shrink;
 };
-__device__ __forceinline__ GemmItem decode_item(const GemmArgs &a, int item, int n_shrink, int n_n, int BN) {
+__device__ __forceinline__ GemmItem decode_item(const GemmArgs &a, int item, int n_shrink, int p_base, int n_n, int BN) {
     GemmItem g;
     g.n0 = 0; g.p0 = 0; g.p1 = 0; g.adapter = -1;
     g.shrink = item < n_shrink;
     if (g.shrink) {
-        const TilePair p = a.pairs[item];
-        g.m = p.tile;
+        const TilePair p = a.pairs[p_base + item];
+        g.m = p.tile - a.tile0;
         g.adapter = p.adapter;
+        g.p0 = g.p1 = p_base + item;
     } else {
         const int j = item - n_shrink;
         g.m = j / n_n;
         g.n0 = (j % n_n) * BN;
-        if (a.pairs) { g.p0 = a.pair_off[g.m]; g.p1 = a.pair_off[g.m + 1]; }
+        if (a.pairs) { g.p0 = a.pair_off[a.tile0 + g.m]; g.p1 = a.pair_off[a.tile0 + g.m + 1]; }
     }
     return g;
 }
@@ -161,7 +165,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 
     const int n_m = (a.M + kBM - 1) / kBM;
     const int n_n = (a.N + BN - 1) / BN;
-    const int n_shrink = (BN >= kShrinkCols && a.n_pairs) ? *a.n_pairs : 0;
+    const int p_base = (BN == 256 && a.shrink) ? a.pair_off[a.tile0] : 0;
+    const int n_shrink = (BN == 256 && a.shrink) ? a.pair_off[a.tile0 + n_m] - p_base : 0;
     const int total = n_shrink + n_m * n_n;
     const int kb_main = (a.K + kBK - 1) / kBK;
 
@@ -199,15 +204,15 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 }
                 if (!ring.put(item, abort_flag)) { ok = false; break; }
                 if (item < 0) break;
-                const GemmItem g = decode_item(a, item, n_shrink, n_n, BN);
+                const GemmItem g = decode_item(a, item, n_shrink, p_base, n_n, BN);
                 const int row0 = g.m * kBM, n0 = g.n0;
                 for (int kb = 0; kb < kb_main; ++kb, ++kc) {
                     const int s = kc % kStages;
                     if (!tc::mbar_wait(empty_bar(s), ((kc / kStages) & 1) ^ 1, abort_flag)) { ok = false; break; }
                     const uint32_t sa = smem_base + s * S::kStageBytes, sb = sa + S::kABytes;
-                    tc::mbar_arrive_expect_tx(full_bar(s), a_bytes + (g.shrink ? kShrinkCols * kBK * 2 : S::kBBytes));
+                    tc::mbar_arrive_expect_tx(full_bar(s), a_bytes + (g.shrink ? a.t_cols * kBK * 2 : S::kBBytes));
                     tc::tma_load_2d(sa, &tmA, full_bar(s), kb * kBK, row0);
-                    if (g.shrink) tc::tma_load_2d(sb, &tmS, full_bar(s), kb * kBK, g.adapter * kShrinkCols);
+                    if (g.shrink) tc::tma_load_2d(sb, &tmS, full_bar(s), kb * kBK, g.adapter * a.t_cols);
                     else tc::tma_load_2d(sb, &tmB, full_bar(s), kb * kBK, n0);
                 }
                 // expand: per adapter of the row tile one K block for each summand of t
@@ -258,15 +263,15 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort_flag));
             };
             constexpr uint32_t idesc_main = tc::idesc_bf16_f32(kBM, BN);
-            constexpr uint32_t idesc_shrink = tc::idesc_bf16_f32(kBM, BN >= kShrinkCols ? kShrinkCols : BN);
+            const uint32_t idesc_shrink = tc::idesc_bf16_f32(kBM, a.t_cols);
             uint32_t kc = 0, it = 0;
             bool ok = true;
             while (ok) {
                 const int item = ring.take(abort_flag);
                 if (item < 0) { ok = item == -1; break; }
-                const GemmItem g = decode_item(a, item, n_shrink, n_n, BN);
+                const GemmItem g = decode_item(a, item, n_shrink, p_base, n_n, BN);
                 // MMA steps of the row tile's adapters, one per lane, loaded while the main loop runs
-                const int my_steps = g.p0 + lane < g.p1 ? a.adapters[a.pairs[g.p0 + lane].adapter].rpad / 16 : 0;
+                const int my_steps = g.p0 + lane < g.p1 ? rank_steps(a, a.pairs[g.p0 + lane].adapter) : 0;
                 const uint32_t idesc = g.shrink ? idesc_shrink : idesc_main;
                 const uint32_t acc = it & 1;
                 if (!wait_all(acce_bar(acc), ((it >> 1) & 1) ^ 1)) { ok = false; break; }
@@ -287,7 +292,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 }
                 for (int p = g.p0; p < g.p1 && ok; ++p) {
                     const int at = p - g.p0;
-                    const int steps = at < 32 ? __shfl_sync(0xffffffffu, my_steps, at) : a.adapters[a.pairs[p].adapter].rpad / 16;
+                    const int steps = at < 32 ? __shfl_sync(0xffffffffu, my_steps, at) : rank_steps(a, a.pairs[p].adapter);
                     for (int part = 0; part < a.t_parts; ++part, ++kc) {
                         const int s = kc % kStages;
                         if (!wait_all(full_bar(s), (kc / kStages) & 1)) { ok = false; break; }
@@ -318,20 +323,20 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         while (ok) {
             const int item = ring.take(abort_flag);
             if (item < 0) break;
-            const GemmItem g = decode_item(a, item, n_shrink, n_n, BN);
+            const GemmItem g = decode_item(a, item, n_shrink, p_base, n_n, BN);
             const int n0 = g.n0, row = g.m * kBM + q * 32 + lane;   // this thread's row
             const uint32_t acc = it & 1;
             if (!tc::mbar_wait(accf_bar(acc), (it >> 1) & 1, abort_flag)) { ok = false; break; }
             tc::tc_fence_after();
             const bool row_ok = row < a.M;
             if (g.shrink) {
-                // t = s A x of this pair: 192 columns, zero in the rows that do not use the adapter
-                const float scale = a.adapters[g.adapter].scale;
+                // t = s A x of this pair, zero in the rows that do not use the adapter
+                const float scale = __int_as_float(a.adapters[g.adapter * a.ad_stride + 1]);
                 const bool use = row_ok && a.row_adapter[row] == g.adapter;
-                __nv_bfloat16 *trow = a.t_out + ((size_t)item * a.t_parts * kBM + q * 32 + lane) * kShrinkCols;
-                __nv_bfloat16 *tlow = a.t_parts > 1 ? trow + (size_t)kBM * kShrinkCols : nullptr;
+                __nv_bfloat16 *trow = a.t_out + ((size_t)g.p0 * a.t_parts * kBM + q * 32 + lane) * a.t_cols;
+                __nv_bfloat16 *tlow = a.t_parts > 1 ? trow + (size_t)kBM * a.t_cols : nullptr;
 #pragma unroll 1
-                for (int c = 0; c < kShrinkCols && c < BN; c += 32) {
+                for (int c = 0; c < a.t_cols && c < BN; c += 32) {
                     uint32_t v[32];
                     tc::tmem_ld_32x32(tmem_base + acc * BN + c + ((uint32_t)(q * 32) << 16), v);
                     tc::tmem_ld_wait();
@@ -343,7 +348,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 __threadfence();
                 __syncwarp();
                 if (lane == 0) {
-                    atomicAdd(a.t_ready + item, 1);
+                    atomicAdd(a.t_ready + g.p0, 1);
                     tc::mbar_arrive(acce_bar(acc));
                 }
                 ++it;
@@ -408,7 +413,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     tc::tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && *abort_flag) report(a.status, ALORA_ERR_TIMEOUT);
-    if (threadIdx.x == 0) tc::item_counter_release(a.item_counters, a.t_ready, n_shrink);
+    if (threadIdx.x == 0) tc::item_counter_release(a.item_counters, a.t_ready + p_base, n_shrink);
     if (warp == 1) {
         tc::tc_fence_after();
         tc::tmem_dealloc(tmem_base, kTmemCols);
@@ -553,7 +558,9 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
         g.a_tile_bytes = half_box ? (kBM / 2) * kBK * 2 : 0;
         const CUtensorMap &tmXg = half_box ? tmX64 : tmX;
         g.M = T; g.N = d.N; g.K = d.H;
-        g.out = (__nv_bfloat16 *)qkv; g.ldo = d.N; g.residual = nullptr; g.adapters = ads;
+        g.out = (__nv_bfloat16 *)qkv; g.ldo = d.N; g.residual = nullptr;
+        g.adapters = &ads->rpad;   // (address arithmetic only: padded rank and scale of an AdapterDev are neighbours)
+        g.ad_stride = sizeof(AdapterDev) / 4; g.t_cols = 3 * kTensorRP;
         g.Nq = d.Nq; g.Nkv = d.Nkv; g.total_adapter_rows = d.N; g.status = ctx->d_status;
         g.item_counters = ctx->d_counts + 10;
         if (have_adapters) { g.pairs = ctx->d_pairs; g.pair_off = ctx->d_pair_off; g.t_parts = t_parts; }
@@ -564,7 +571,7 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
             g.kv_page_size = d.page; g.kv_num_pages = num_pages;
         }
         if (fuse_shrink) {
-            g.n_pairs = ctx->d_counts + 2; g.row_adapter = ctx->d_row_adapter;
+            g.shrink = 1; g.row_adapter = ctx->d_row_adapter;
             g.t_ready = ctx->d_t_ready; g.t_out = (__nv_bfloat16 *)ctx->d_t;
         }
         const int items = proj_items + (fuse_shrink ? max_pairs : 0);
@@ -580,14 +587,19 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
 }
 
 int launch_linear256_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
-                        const void *residual, cudaStream_t s);  // gemm256_tcgen05.cu
+                        const void *residual, const LinearDelta *delta, cudaStream_t s);  // gemm_pair_tcgen05.cu
 bool build_pair_maps(alora_ctx *ctx, int layer);                 // gemm_pair_tcgen05.cu
 
-// Plain dense projection y = x W^T (+ residual) for o_proj and the MLP matrices.
+// Whether launch_linear_tc can add a gated delta to a projection of this shape (not on the few-row route).
+bool linear_takes_delta(const alora_ctx *ctx, int T, int K, int N) { return !skinny_route(ctx, T, N, K, false, N, 0); }
+
+// Dense projection y = x W^T (+ residual) for o_proj and the MLP matrices, with the gated delta of the MLP adapters where
+// `delta` is given.
 int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
-                     const void *residual, cudaStream_t s) {
+                     const void *residual, const LinearDelta *delta, cudaStream_t s) {
     if (T == 0) return 0;
     if (K % 8 != 0 || N % 8 != 0) return -1;
+    if (delta != nullptr && (!linear_takes_delta(ctx, T, K, N) || (N / delta->n_blk) % 256 != 0)) return -1;
     ProfScope prof(ctx, KK_LINEAR, s);
     if (skinny_route(ctx, T, N, K, false, N, 0)) {
         CUtensorMap tmW256;
@@ -595,10 +607,10 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
         return launch_skinny_tc(ctx, x, tmW256, nullptr, nullptr, nullptr, T, K, N, N, 0, y, residual, nullptr, 0, 0, s);
     }
     {
-        const int r = launch_linear256_tc(ctx, x, W, T, K, N, y, residual, s);   // many rows: 256 x 256 tiles
+        const int r = launch_linear256_tc(ctx, x, W, T, K, N, y, residual, delta, s);   // many rows: 256 x 256 tiles
         if (r != 0) return r;
     }
-    const int BN = pick_bn(N, N, 0, false, T);
+    const int BN = delta != nullptr ? 256 : pick_bn(N, N, 0, false, T);
     CUtensorMap tmX, tmW;
     const bool half_box = T <= kBM / 2;   // see GemmArgs::a_tile_bytes
     if (!make_tensor_map_bf16(&tmX, x, T, K, K, half_box ? kBM / 2 : kBM)) return -1;
@@ -606,10 +618,22 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
     GemmArgs g{};
     g.a_tile_bytes = half_box ? (kBM / 2) * kBK * 2 : 0;
     g.M = T; g.N = N; g.K = K; g.out = (__nv_bfloat16 *)y; g.ldo = N;
-    g.residual = (const __nv_bfloat16 *)residual; g.adapters = nullptr; g.Nq = N; g.Nkv = 0;
-    g.total_adapter_rows = 0; g.status = ctx->d_status; g.item_counters = ctx->d_counts + 10;
-    const int items = ((T + kBM - 1) / kBM) * ((N + BN - 1) / BN);
-    const bool ok = BN == 256 ? launch_gemm_bn<256>(ctx, tmX, tmW, tmX, tmW, tmW, g, items, s)
+    g.residual = (const __nv_bfloat16 *)residual; g.Nq = N; g.Nkv = 0; g.t_cols = kTensorRP;
+    g.total_adapter_rows = N; g.status = ctx->d_status; g.item_counters = ctx->d_counts + 10;
+    CUtensorMap tmT = tmX, tmA = tmW, tmB = tmW;
+    if (delta != nullptr) {
+        const uint64_t na = (uint64_t)std::max(1, ctx->cfg.max_adapters);
+        g.t_cols = delta->n_blk * kTensorRP; g.t_parts = 1;
+        if (delta->n_blk == 2) g.Nq = g.Nkv = N / 2;
+        if (!make_tensor_map_bf16(&tmT, delta->t, (uint64_t)ctx->max_pairs * kBM, g.t_cols, g.t_cols, kBM)) return -1;
+        if (!make_tensor_map_bf16(&tmA, delta->A, na * g.t_cols, K, K, g.t_cols)) return -1;
+        if (!make_tensor_map_bf16(&tmB, delta->B, na * N, kTensorRP, kTensorRP, BN)) return -1;
+        g.pairs = ctx->d_pairs; g.pair_off = ctx->d_pair_off; g.tile0 = delta->tile0; g.shrink = 1;
+        g.adapters = &delta->table->rpad; g.ad_stride = sizeof(MlpAdapterDev) / 4;
+        g.row_adapter = delta->row_adapter; g.t_ready = ctx->d_t_ready; g.t_out = (__nv_bfloat16 *)delta->t;
+    }
+    const int items = ((T + kBM - 1) / kBM) * ((N + BN - 1) / BN) + (delta != nullptr ? ctx->max_pairs : 0);
+    const bool ok = BN == 256 ? launch_gemm_bn<256>(ctx, tmX, tmW, tmT, tmB, tmA, g, items, s)
                     : BN == 128 ? launch_gemm_bn<128>(ctx, tmX, tmW, tmX, tmW, tmW, g, items, s)
                                 : launch_gemm_bn<64>(ctx, tmX, tmW, tmX, tmW, tmW, g, items, s);
     return ok ? 1 : -1;
