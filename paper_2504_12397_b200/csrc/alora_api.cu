@@ -28,7 +28,7 @@ int launch_mlp_expand(alora_ctx *, void *, int, int, const void *, int, const vo
 int launch_mlp_shrink(alora_ctx *, const void *, const void *, int, int, int, void *, float *, size_t, int32_t *, int,
                       cudaStream_t);
 bool build_layer_maps(alora_ctx *ctx, int layer);
-bool project_is_few_row(const alora_ctx *ctx, int layer, int T);   // gemm_tcgen05.cu
+bool project_is_few_row(const alora_ctx *ctx, int layer, int T, int R);   // gemm_tcgen05.cu
 int launch_attend_tc(alora_ctx *, const void *, const BatchArgs &, const void *, void *, cudaStream_t);
 
 // bf16 runs on the tensor cores; the fp32 data type (tiny exact-precision configurations) on CUDA cores.
@@ -80,7 +80,7 @@ static alora_status run_layer(alora_ctx *ctx, int layer, const void *hidden, con
     if (!ctx->layers[layer].wqkv) return ALORA_ERR_NO_WEIGHTS;
     BatchArgs b = b_in;
     b.layer = layer;
-    b.few_row = project_is_few_row(ctx, layer, b.T) ? 1 : 0;   // (n_layers > 1 only where all of them take that route)
+    b.few_row = project_is_few_row(ctx, layer, b.T, b.R) ? 1 : 0;   // (n_layers > 1 only where all of them take that route)
     int n = 0, k;
     // The per-token arrays and the projection's lists first; the attention work lists are built beside the
     // projection (the few-row projection launches them between its two kernels, the other routes right after).
@@ -236,6 +236,7 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
         {
             // few-row projection: one 128 x 256 fp32 partial per work item (at most one item per SM, or one per column
             // tile of the widest matrix), and the partial shrink results of the q/k/v projection's K slices
+            few_cluster_init(ctx);
             const int widest = std::max(std::max(d.N, d.H), 2 * d.I);
             ctx->skinny_max_items = std::max(ctx->sm_count, (widest + 255) / 256);
             ctx->skinny_p_cap = std::min(std::max(c.max_adapters, 0), 128);
@@ -243,7 +244,8 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
             const int ksplit = std::max(1, std::min(kb, ctx->sm_count / std::max(n_tiles, 1)));
             alloc((void **)&ctx->d_skinny_part, (size_t)ctx->skinny_max_items * 128 * 256 * 4);
             alloc((void **)&ctx->d_skinny_t, (size_t)ksplit * 128 * std::max(ctx->skinny_p_cap, 1) * 192 * 4);
-            alloc(&ctx->d_skinny_meta, (size_t)c.n_layers * sizeof(FewRowMeta));
+            ctx->few_tiles = std::min(kFewTiles, std::max(1, (c.max_tokens + kFewRowMax - 1) / kFewRowMax));
+            alloc((void **)&ctx->d_skinny_meta, (size_t)c.n_layers * ctx->few_tiles * sizeof(FewRowMeta));
         }
         const size_t na = (size_t)std::max(1, c.max_adapters);
         ctx->tc_a_all.assign(c.n_layers, nullptr);
@@ -527,7 +529,7 @@ alora_status alora_project_qkv(alora_ctx *ctx, int layer, int mode, const void *
     const int32_t *d_block_tables = nullptr; const int max_blocks = 0, num_pages = 0;
     ALORA_BATCH(mode);
     b.layer = layer;
-    b.few_row = project_is_few_row(ctx, layer, T) ? 1 : 0;
+    b.few_row = project_is_few_row(ctx, layer, T, R) ? 1 : 0;
     int n = launch_metadata(ctx, b, s, kMetaProjection), k;
     if (n < 0) return ALORA_ERR_UNSUPPORTED;
     if ((k = launch_project(ctx, layer, d_hidden, T, R, d_qkv, s, nullptr, 0, nullptr)) < 0) return ALORA_ERR_UNSUPPORTED;
@@ -675,7 +677,7 @@ alora_status alora_forward_stack(alora_ctx *ctx, int mode, const void *d_hidden_
     // facts of all layers.  (They were rebuilt by every layer: 63 of 240 us of a layer's decode step of 40 requests in
     // prefix groups.)  Only where the layers' projections take different routes does each build its own.
     int n_few = 0;
-    for (int l = 0; l < ctx->cfg.n_layers; ++l) n_few += project_is_few_row(ctx, l, T) ? 1 : 0;
+    for (int l = 0; l < ctx->cfg.n_layers; ++l) n_few += project_is_few_row(ctx, l, T, R) ? 1 : 0;
     const bool one_route = n_few == 0 || n_few == ctx->cfg.n_layers;
     b.n_layers = one_route ? ctx->cfg.n_layers : 1;
     for (int l = 0; l < ctx->cfg.n_layers; ++l) {

@@ -87,10 +87,11 @@ constexpr int32_t kSplitOwnKeys = 0x40000000;
 constexpr int kSplitScratch = 8;       // per-request integers that the builder of the few-row list needs
 constexpr int kSplitItemsPerSm = 16;   // target number of (row tile, key range) pairs per SM
 
-// Few-row projection (batches of at most kFewRowMax rows): what its two kernels need to know about the batch's
+// Few-row projection: what it needs to know about a tile of at most kFewRowMax rows of the batch, the tile's
 // adapters, written by the batch-metadata step: the adapters that occur among the rows' applied adapters
 // (ascending ids), per slot the padded rank and the scale, and per row the slot of its adapter.
 constexpr int kFewRowMax = 128;
+constexpr int kFewTiles = 8;   // row tiles of a batch on that route
 struct FewRowMeta {
     int32_t n_present;
     int32_t pad_[3];
@@ -191,7 +192,8 @@ struct alora_ctx {
     // few-row projection (batches of <= 128 rows): K-slice partial products and partial shrink results
     float *d_skinny_part = nullptr;   // [skinny_max_items][128][256] fp32
     float *d_skinny_t = nullptr;      // [slices of the q/k/v projection][128][skinny_p_cap][192] fp32
-    void *d_skinny_meta = nullptr;    // [n_layers] FewRowMeta of the current batch
+    alora::FewRowMeta *d_skinny_meta = nullptr;   // [n_layers][few_tiles] of the current batch
+    int few_tiles = 1;
     const alora::BatchArgs *pending_attn_meta = nullptr;   // run_layer: attention lists still to be built for this batch
     int skinny_max_items = 0, skinny_p_cap = 0;
     void *d_qkv = nullptr;        // [max_tokens][N]
@@ -206,6 +208,7 @@ struct alora_ctx {
     int64_t launches = 0;
     std::string cuda_err;
     int sm_count = 148;
+    int few_clusters[9] = {};   // [size] clusters of the few-row projection that fit on the device at once (0: route closed)
 };
 
 namespace alora {
@@ -268,6 +271,7 @@ struct BatchArgs {
 // the attention lists alone is a programmatic dependent launch: it may run beside the projection kernel that
 // precedes it in the stream.  `timed`: bracket it with profiling events of the metadata family.
 constexpr int kMetaProjection = 1, kMetaAttention = 2;
+void few_cluster_init(alora_ctx *ctx);   // gemm_few_cluster.cu: what that route needs to know about the device
 int launch_metadata(alora_ctx *ctx, const BatchArgs &b, cudaStream_t s, int phases = kMetaProjection | kMetaAttention,
                     bool timed = true);
 int launch_repack_adapter(alora_ctx *ctx, int rank, const void *Aq, const void *Bq, const void *Ak,

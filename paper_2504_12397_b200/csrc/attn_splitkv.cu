@@ -63,7 +63,9 @@ struct SkSmem {
     static constexpr int kMlOff = kOOff + kOBytes;
     static constexpr int kMlBytes = 4 * 16 * 2 * 4;
     static constexpr int kBarOff = kMlOff + kMlBytes;
-    static constexpr int kTotal = kBarOff + 256 + 1024;
+    // (one block per SM also for head dim 64, whose blocks would fit twice: started beside a projection that leaves some
+    // SMs free, they would all settle on those, two to an SM, and the other SMs would stay empty)
+    static constexpr int kTotal = kBarOff + 256 + 1024 > 116 * 1024 ? kBarOff + 256 + 1024 : 116 * 1024;
 };
 
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3) {

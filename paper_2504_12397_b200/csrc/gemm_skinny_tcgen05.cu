@@ -1,5 +1,6 @@
-// Projection of a batch of at most 128 rows (decode steps, short invocation suffixes): out = x W^T with the
-// aLoRA delta of Eq. 5 on the rows whose gate is open.  With so few rows the weights are read once and never
+// Projection of a batch of at most 128 rows for contexts whose adapters do not fit the one-launch kernel of
+// gemm_few_cluster.cu (more than 256 padded rank columns, q / k / v blocks that 256 does not divide): out = x W^T with
+// the aLoRA delta of Eq. 5 on the rows whose gate is open.  With so few rows the weights are read once and never
 // reused: the step is bound by streaming W out of HBM, so the work is cut to put every SM on that stream.
 //
 // Kernel 1 (tensor cores, one work item per block): item = (256-column tile of W, slice of K).  The K dimension is
@@ -509,7 +510,7 @@ int launch_skinny_tc(alora_ctx *ctx, const void *x, const CUtensorMap &tmW, cons
     if (a.n_stages < 2) return -1;
     a.part = ctx->d_skinny_part; a.t_part = ctx->d_skinny_t; a.p_cap = p_cap;
     a.row_adapter = lora ? ctx->d_row_adapter : nullptr;
-    a.meta = lora ? (const FewRowMeta *)ctx->d_skinny_meta + layer : nullptr;
+    a.meta = lora ? ctx->d_skinny_meta + (size_t)layer * ctx->few_tiles : nullptr;
     a.max_adapters = ctx->cfg.max_adapters; a.status = ctx->d_status;
     const size_t smem = (size_t)a.n_stages * a.stage_bytes + 1024 + 256;
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {

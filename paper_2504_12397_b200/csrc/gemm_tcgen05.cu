@@ -508,12 +508,30 @@ int launch_skinny_tc(alora_ctx *ctx, const void *x, const CUtensorMap &tmW, cons
                      const AdapterDev *adapters, const void *b_all, int T, int K, int N, int Nq, int Nkv, void *out,
                      const void *residual, void *kv_pool, int num_pages, int layer, cudaStream_t s);
 
+bool few_cluster_route(const alora_ctx *ctx, int T, int R, int N, int K, bool lora, int Nq, int Nkv);   // gemm_few_cluster.cu
+int launch_few_cluster(alora_ctx *ctx, const void *x, const void *W, const CUtensorMap *tmA16, const FewRowMeta *meta,
+                       const void *b_all, int T, int R, int K, int N, int Nq, int Nkv, void *out, const void *residual, void *kv_pool,
+                       int num_pages, cudaStream_t s);
+
+// The weight-streaming routes for few rows: in one launch, or (at most 128 rows, more adapters than that takes) in two.
+static bool few_row_linear(const alora_ctx *ctx, int T, int N, int K) {
+    return few_cluster_route(ctx, T, 0, N, K, false, N, 0) || skinny_route(ctx, T, N, K, false, N, 0);
+}
+// Whether the q/k/v projection takes the one-launch route: with more than 128 rows only in a context without adapters on
+// the MLP block (those need the (row tile, adapter) pairs, which that route's metadata step does not build).
+static bool project_few_cluster(const alora_ctx *ctx, int layer, int T, int R) {
+    const Dims &d = ctx->d;
+    if (T > kFewRowMax)
+        for (int n : ctx->mlp_n_adapters) if (n > 0) return false;
+    return few_cluster_route(ctx, T, R, d.N, d.H, ctx->layer_has_adapter[layer] != 0, d.Nq, d.Nkv);
+}
+
 // Whether the q/k/v projection of a batch of T rows on this layer takes the few-row route (the batch-metadata step
 // then prepares that route's adapter facts instead of row tiles).
-bool project_is_few_row(const alora_ctx *ctx, int layer, int T) {
+bool project_is_few_row(const alora_ctx *ctx, int layer, int T, int R) {
     if (ctx->cfg.dtype != ALORA_DTYPE_BF16 || layer < 0 || layer >= ctx->cfg.n_layers) return false;
     const Dims &d = ctx->d;
-    return skinny_route(ctx, T, d.N, d.H, ctx->layer_has_adapter[layer] != 0, d.Nq, d.Nkv);
+    return project_few_cluster(ctx, layer, T, R) || skinny_route(ctx, T, d.N, d.H, ctx->layer_has_adapter[layer] != 0, d.Nq, d.Nkv);
 }
 
 int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int R, void *qkv, cudaStream_t s, void *kv_pool,
@@ -521,7 +539,13 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
     if (T == 0) return 0;
     const Dims &d = ctx->d;
     const bool have_adapters = ctx->layer_has_adapter[layer];
-    if (skinny_route(ctx, T, d.N, d.H, have_adapters, d.Nq, d.Nkv)) {   // at most 128 rows: weight-streaming route
+    if (project_few_cluster(ctx, layer, T, R)) {
+        ProfScope prof(ctx, KK_PROJECT, s);
+        return launch_few_cluster(ctx, hidden, ctx->layers[layer].wqkv, &ctx->tc_maps[layer].a_all16,
+                                  have_adapters ? ctx->d_skinny_meta + (size_t)layer * ctx->few_tiles : nullptr, ctx->tc_b_all[layer], T, R,
+                                  d.H, d.N, d.Nq, d.Nkv, qkv, nullptr, kv_pool, num_pages, s);
+    }
+    if (skinny_route(ctx, T, d.N, d.H, have_adapters, d.Nq, d.Nkv)) {
         ProfScope prof(ctx, KK_PROJECT, s);
         const TcLayerMaps &lm = ctx->tc_maps[layer];
         const AdapterDev *ads = ctx->d_adapters + (size_t)layer * ctx->cfg.max_adapters;
@@ -591,7 +615,9 @@ int launch_linear256_tc(alora_ctx *ctx, const void *x, const void *W, int T, int
 bool build_pair_maps(alora_ctx *ctx, int layer);                 // gemm_pair_tcgen05.cu
 
 // Whether launch_linear_tc can add a gated delta to a projection of this shape (not on the few-row route).
-bool linear_takes_delta(const alora_ctx *ctx, int T, int K, int N) { return !skinny_route(ctx, T, N, K, false, N, 0); }
+bool linear_takes_delta(const alora_ctx *ctx, int T, int K, int N) {
+    return T > kFewRowMax || !few_row_linear(ctx, T, N, K);
+}
 
 // Dense projection y = x W^T (+ residual) for o_proj and the MLP matrices, with the gated delta of the MLP adapters where
 // `delta` is given.
@@ -601,6 +627,8 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
     if (K % 8 != 0 || N % 8 != 0) return -1;
     if (delta != nullptr && (!linear_takes_delta(ctx, T, K, N) || (N / delta->n_blk) % 256 != 0)) return -1;
     ProfScope prof(ctx, KK_LINEAR, s);
+    if (delta == nullptr && few_cluster_route(ctx, T, 0, N, K, false, N, 0))
+        return launch_few_cluster(ctx, x, W, nullptr, nullptr, nullptr, T, 0, K, N, N, 0, y, residual, nullptr, 0, s);
     if (skinny_route(ctx, T, N, K, false, N, 0)) {
         CUtensorMap tmW256;
         if (!make_tensor_map_bf16(&tmW256, W, N, K, K, 256)) return -1;

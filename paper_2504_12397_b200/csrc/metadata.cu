@@ -614,7 +614,7 @@ __device__ __forceinline__ void metadata_split_items(const int32_t *__restrict__
     }
 }
 
-// FewRowMeta of a batch of at most kFewRowMax rows, thread t's applied adapter being k_mine (-1: none, or no such
+// FewRowMeta of a tile of at most kFewRowMax rows, thread t's applied adapter being k_mine (-1: none, or no such
 // row): the adapters that occur, ascending, each one's padded rank and scale, and every row's slot.  Called by all
 // kFewRowMax threads of a block.
 __device__ __forceinline__ void metadata_few_row(int k_mine, const AdapterDev *__restrict__ adapters, int max_adapters,
@@ -729,11 +729,11 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
     if (!proj) tc::grid_dep_wait();
 }
 
-// The projection phase for a batch on the few-row route (at most kFewRowMax tokens): per-token arrays and the adapter
-// facts, nothing else.  A kernel of its own because every step of a decode loop waits for it: what it costs is mostly
-// the fetch of its instructions, and this one is short.  Block l writes the facts of layer l of the call (a stack call
-// builds those of all layers in one launch: with a launch per layer each layer waited 10 us for it), block 0 also the
-// per-token arrays.  row_adapter holds the adapter of every row whose gate is open; whether it is registered on a layer
+// The projection phase for a batch on the few-row route (at most kFewTiles tiles of kFewRowMax tokens): per-token arrays and
+// the adapter facts, nothing else.  A kernel of its own because every step of a decode loop waits for it: what it costs is mostly
+// the fetch of its instructions, and this one is short.  Block (tile, l) writes the tile's facts of layer l of the call (a stack call
+// builds those of all layers in one launch: with a launch per layer each layer waited 10 us for it), those of layer 0 also
+// the per-token arrays.  row_adapter holds the adapter of every row whose gate is open; whether it is registered on a layer
 // (else: base output and a finding) goes into that layer's facts.
 __global__ void __launch_bounds__(kFewRowMax)
 metadata_few_row_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, const int32_t *adapter_ids,
@@ -741,7 +741,7 @@ metadata_few_row_kernel(const int32_t *__restrict__ positions, const int32_t *a_
                         int max_blocks, int num_pages, int page_size, int max_adapters, int T, int R, int mode,
                         int32_t *__restrict__ token_req, int32_t *__restrict__ row_adapter,
                         int32_t *__restrict__ slot_map, const AdapterDev *__restrict__ adapters,
-                        FewRowMeta *__restrict__ few_row_meta, int32_t *status) {
+                        FewRowMeta *__restrict__ few_row_meta, int few_tiles, int32_t *status) {
     __shared__ int32_t s_req[4 * kFewRowMax + 1];
     tc::grid_dep_launch();
     if (R <= kFewRowMax) {   // the per-request inputs are read several times (binary search): stage them
@@ -757,14 +757,14 @@ metadata_few_row_kernel(const int32_t *__restrict__ positions, const int32_t *a_
         if (adapter_ids) adapter_ids = s_ids;
         if (a_req) a_req = s_areq;
     }
-    const bool first = blockIdx.x == 0;
-    int k = metadata_token((int)threadIdx.x, positions, a_req, adapter_ids, qsl, seq_lens, first ? block_tables : nullptr,
+    const bool first = blockIdx.y == 0;
+    int k = metadata_token((int)(blockIdx.x * kFewRowMax + threadIdx.x), positions, a_req, adapter_ids, qsl, seq_lens, first ? block_tables : nullptr,
                            max_blocks, num_pages, page_size, max_adapters, T, R, mode, first ? token_req : nullptr,
                            first ? row_adapter : nullptr, first ? slot_map : nullptr, status);
     if (few_row_meta != nullptr) {
-        const AdapterDev *ads = adapters + (size_t)blockIdx.x * max_adapters;
+        const AdapterDev *ads = adapters + (size_t)blockIdx.y * max_adapters;
         if (k >= 0 && ads[k].rank == 0) { report(status, ALORA_ERR_NO_WEIGHTS); k = -1; }
-        metadata_few_row(k, ads, max_adapters, few_row_meta + blockIdx.x);
+        metadata_few_row(k, ads, max_adapters, few_row_meta + (size_t)blockIdx.y * few_tiles + blockIdx.x);
     }
 }
 
@@ -784,12 +784,12 @@ int launch_metadata(alora_ctx *ctx, const BatchArgs &b, cudaStream_t s, int phas
     constexpr int kSplitBuilders = 8;
     const int grid = attn_only ? (14 * b.R + 5 <= kMetaSmemInts ? 1 + kSplitBuilders : 2) : std::max((phases & kMetaAttention) ? 3 : 1, (b.T + threads - 1) / threads);
     const AdapterDev *ads = b.layer >= 0 ? ctx->d_adapters + (size_t)b.layer * ctx->cfg.max_adapters : nullptr;
-    if (phases == kMetaProjection && b.few_row && b.T <= kFewRowMax) {
-        FewRowMeta *few = ads != nullptr ? (FewRowMeta *)ctx->d_skinny_meta + b.layer : nullptr;
-        metadata_few_row_kernel<<<b.n_layers, kFewRowMax, 0, s>>>(
+    if (phases == kMetaProjection && b.few_row) {
+        FewRowMeta *few = ads != nullptr ? ctx->d_skinny_meta + (size_t)b.layer * ctx->few_tiles : nullptr;
+        metadata_few_row_kernel<<<dim3((b.T + kFewRowMax - 1) / kFewRowMax, b.n_layers), kFewRowMax, 0, s>>>(
             b.positions, b.activation_offsets, b.adapter_ids, b.query_start_loc, b.seq_lens, b.block_tables, b.max_blocks,
             b.num_pages, ctx->d.page, ctx->cfg.max_adapters, b.T, b.R, b.mode, ctx->d_token_req, ctx->d_row_adapter,
-            ctx->d_slot, ads, few, ctx->d_status);
+            ctx->d_slot, ads, few, ctx->few_tiles, ctx->d_status);
         return 1;
     }
     const cudaError_t e = launch_kernel(metadata_kernel, dim3(grid), dim3(threads), 0, s, attn_only,

@@ -301,6 +301,20 @@ def test_projection_few_row_route_mixed_adapters(oracle64, T):
     _check_projection(oracle64, MID, w, ads, b)
 
 
+@pytest.mark.parametrize("T,n_ad,rank", [(16, 1, 64), (17, 2, 24), (32, 16, 16), (127, 3, 40), (40, 17, 16), (129, 3, 40), (385, 2, 64)])
+def test_projection_few_row_route_row_boxes_and_adapter_limits(oracle64, T, n_ad, rank):
+    """Row counts at the edges of the 16 / 32 / 64 / 128-row boxes, ranks that padding rounds up, the most rank columns that
+    the one-launch kernel takes (16 adapters of rank 16) and one adapter more (the two-kernel route); several row tiles, the
+    last of one row."""
+    rng = np.random.default_rng(300 + T)
+    w = wl.make_wqkv(MID, rng)
+    ads = _boosted_adapters(MID, rng, tuple((max(1, rank - i % 5), 0.5 + 0.25 * (i % 3)) for i in range(n_ad)))
+    P = [int(x) for x in rng.integers(0, 300, T)]
+    ids = [(i * 7) % (n_ad + 1) - 1 for i in range(T)]
+    b = wl.make_batch(MID, P, [1] * T, ids, rng, activation_offsets=[p + (i % 6 == 1) for i, p in enumerate(P)])
+    _check_projection(oracle64, MID, w, ads, b)
+
+
 def test_projection_few_row_route_short_suffixes_one_adapter(oracle64):
     """8 requests x 16 new tokens (128 rows), one adapter, gates opening inside the chunk."""
     rng = np.random.default_rng(49)
