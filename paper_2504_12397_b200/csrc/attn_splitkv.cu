@@ -210,15 +210,16 @@ attn_splitkv_kernel(const __grid_constant__ CUtensorMap tmKV, const SplitArgs a)
         const int units_per_stage = kSkStageKeys / a.box_rows;
         uint32_t kt = 0, n_it = 0;
         bool ok = true;
-        // items are handed out in list order to whichever block is free; the claim of the item after the current
-        // one is issued before the current item's loads, so its latency is hidden behind them
-        int it_next = 0;
-        if (lane == 0) it_next = atomicAdd(a.work_counter, 1);
+        // block b begins with item b; the rest are handed out in list order to whichever block is free, the claim of the
+        // item after the current one being issued before the current item's loads, so that its latency is hidden behind
+        // them.  (With the first item claimed too, early blocks claimed their second one before late blocks came: where
+        // there is an item per block, some did two while others did none; 2 requests of 4745 keys, head dim 64: 38 -> 32 us.)
+        int it_next = blockIdx.x;
         while (ok) {
             int it = -1;
             if (lane == 0) {
                 it = it_next < n_items ? it_next : -1;
-                if (it >= 0) it_next = atomicAdd(a.work_counter, 1);
+                if (it >= 0) it_next = (int)gridDim.x + atomicAdd(a.work_counter, 1);
                 const int slot = n_it % kSkItemSlots;
                 ok = tc::mbar_wait(item_empty(slot), ((n_it / kSkItemSlots) & 1) ^ 1, abort_flag);
                 if (ok) {
