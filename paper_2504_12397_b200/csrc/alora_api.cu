@@ -14,7 +14,7 @@ alora_status cuda_fail(alora_ctx *ctx, cudaError_t e, const char *what) {
     return ALORA_ERR_CUDA;
 }
 
-int launch_project_simt(alora_ctx *, int, const void *, int, void *, cudaStream_t);
+int launch_project_simt(alora_ctx *, int, const void *, int, void *, cudaStream_t, void *, int);
 int launch_linear_simt(alora_ctx *, const void *, const void *, int, int, int, void *, const void *, cudaStream_t);
 int launch_attend_simt(alora_ctx *, const void *, const BatchArgs &, const void *, void *, cudaStream_t);
 
@@ -32,17 +32,15 @@ bool project_is_few_row(const alora_ctx *ctx, int layer, int T, int R);   // gem
 int launch_attend_tc(alora_ctx *, const void *, const BatchArgs &, const void *, void *, cudaStream_t);
 
 // bf16 runs on the tensor cores; the fp32 data type (tiny exact-precision configurations) on CUDA cores.
-// With a page pool given, the bf16 projection also writes the k / v columns of every row to the row's cache slot
+// With a page pool given, the projection also writes the k / v columns of every row to the row's cache slot
 // (the KV append fused into its epilogue) and sets *kv_appended.
 int launch_project(alora_ctx *ctx, int layer, const void *hidden, int T, int R, void *qkv, cudaStream_t s, void *kv_pool,
                    int num_pages, bool *kv_appended) {
     if (kv_appended) *kv_appended = false;
-    if (ctx->cfg.dtype == ALORA_DTYPE_BF16) {
-        const int n = launch_project_tc(ctx, layer, hidden, T, R, qkv, s, kv_pool, num_pages);
-        if (kv_appended && n >= 0 && kv_pool != nullptr) *kv_appended = true;
-        return n;
-    }
-    return launch_project_simt(ctx, layer, hidden, T, qkv, s);
+    const int n = ctx->cfg.dtype == ALORA_DTYPE_BF16 ? launch_project_tc(ctx, layer, hidden, T, R, qkv, s, kv_pool, num_pages)
+                                                     : launch_project_simt(ctx, layer, hidden, T, qkv, s, kv_pool, num_pages);
+    if (kv_appended && n >= 0 && kv_pool != nullptr) *kv_appended = true;
+    return n;
 }
 int launch_linear(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
                   const void *residual, cudaStream_t s, const LinearDelta *delta) {
@@ -90,7 +88,7 @@ static alora_status run_layer(alora_ctx *ctx, int layer, const void *hidden, con
     }
     bool kv_appended = false;
     const bool rope = ctx->d_rope_inv_freq != nullptr;   // the rotation comes between projection and append
-    ctx->pending_attn_meta = (b.facts_ready & kMetaAttention) ? nullptr : &b;
+    ctx->pending_attn_meta = (b.facts_ready & kMetaAttention) || (ctx->d_attn_items == nullptr && ctx->d_split_items == nullptr) ? nullptr : &b;   // (no lists in fp32)
     k = launch_project(ctx, layer, hidden, b.T, b.R, ctx->d_qkv, s, rope ? nullptr : pool, b.num_pages, &kv_appended);
     const bool attn_meta_pending = ctx->pending_attn_meta != nullptr;
     ctx->pending_attn_meta = nullptr;

@@ -60,89 +60,124 @@ int launch_repack_adapter(alora_ctx *ctx, int rank, const void *Aq, const void *
 }
 
 // ---------------------------------------------------------------------------------------------
-// CUDA-core shrink: t[row][blk][i] = scale * sum_h A[blk][i][h] x[row][h] for rows with an applied
-// adapter (Eq. 5, inner product of the low-rank delta).  One block per row, one warp per output.
+// CUDA-core shrink (fp32): t[row][blk][i] = scale * sum_h A[blk][i][h] x[row][h] for rows with an applied
+// adapter (Eq. 5, inner product of the low-rank delta).  One block per (row, q/k/v block), one warp per output.
 // ---------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void shrink_simt_kernel(const T *__restrict__ x, const int32_t *__restrict__ row_adapter,
-                                  const AdapterDev *__restrict__ adapters, int H, int RP,
-                                  float *__restrict__ t) {
-    const int row = blockIdx.x;
+__global__ void __launch_bounds__(256)
+shrink_simt_kernel(const float *__restrict__ x, const int32_t *__restrict__ row_adapter, const AdapterDev *__restrict__ adapters,
+                   int H, int RP, float *__restrict__ t) {
+    tc::grid_dep_launch();
+    const int row = blockIdx.x, blk = blockIdx.y;
     const int k = row_adapter[row];
     if (k < 0) return;
     const AdapterDev ad = adapters[k];
-    const T *A = (const T *)ad.A;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    for (int o = warp; o < 3 * RP; o += nwarps) {
-        const int i = o % RP;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const float4 *xv = reinterpret_cast<const float4 *>(x + (size_t)row * H);
+    for (int i = warp; i < RP; i += 8) {
         float acc = 0.f;
         if (i < ad.rank) {
-            const T *a = A + (size_t)o * H;
-            for (int h = lane; h < H; h += 32) acc += ldf(a + h) * ldf(x + (size_t)row * H + h);
+            const float4 *av = reinterpret_cast<const float4 *>((const float *)ad.A + (size_t)(blk * RP + i) * H);
+#pragma unroll 4
+            for (int h = lane; h < H / 4; h += 32) {
+                const float4 a = av[h], b = xv[h];
+                acc += a.x * b.x; acc += a.y * b.y; acc += a.z * b.z; acc += a.w * b.w;
+            }
             for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
         }
-        if (lane == 0) t[(size_t)row * 3 * RP + o] = acc * ad.scale;
+        if (lane == 0) t[((size_t)row * 3 + blk) * RP + i] = acc * ad.scale;
     }
 }
 
 // ---------------------------------------------------------------------------------------------
-// CUDA-core projection y[row][n] = sum_h W[n][h] x[row][h]  (+ sum_i B[n][i] t[row][blk(n)][i] when the
-// row has an applied adapter).  64x64 output tile per block, 16x16 threads, 4x4 outputs each,
-// K staged through shared memory 16 columns at a time.  The base sum of a row is formed by the
-// same instruction sequence whether or not the delta follows, so gated-off rows equal a base-only
-// call bit for bit.  Optional residual: y += residual[row][n] (used by o_proj / down_proj).
+// CUDA-core projection (fp32) y[row][n] = sum_h W[n][h] x[row][h]  (+ sum_i B[n][i] t[row][blk(n)][i] when the
+// row has an applied adapter).  The sizes that run here (the exact-precision layers of the tests: 16 rows, K 256, N 512) are
+// bound by latency: 32 tiles of 64 x 64 walked K through shared memory in 16 steps on 8 SMs and took 35 us.  So tiles are
+// 16 x 32 and the 8 warps of a block share K (warp w takes every eighth vector of four), each straight from global
+// memory, the loads of two steps in flight; their sums are added in warp order: 10 us.  The split of K does not
+// depend on the row count and the base sum of a row is formed by the same instruction sequence whether or not the
+// delta follows, so gated-off rows equal a base-only call bit for bit.  Optional residual: y += residual[row][n]
+// (used by o_proj / down_proj); with a page pool the k and v columns also go to the rows' cache slots.
+// `base_first`: x was complete before the preceding kernel of the stream began, so that the base sums do not wait for it.
 // ---------------------------------------------------------------------------------------------
-template <typename T>
 __global__ void __launch_bounds__(256)
-linear_simt_kernel(const T *__restrict__ x, const T *__restrict__ W, int Tn, int K, int N,
-                  const int32_t *__restrict__ row_adapter, const AdapterDev *__restrict__ adapters,
-                  const float *__restrict__ t, int RP, int Nq, int Nkv, const T *residual /* may alias y */,
-                   T *y) {
-    __shared__ float xs[16][64 + 1], ws[16][64 + 1];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int row0 = blockIdx.y * 64, col0 = blockIdx.x * 64;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        for (int i = threadIdx.x; i < 64 * 16; i += 256) {
-            int rr = i >> 4, kk = i & 15;
-            int gr = row0 + rr, gc = col0 + rr, gk = k0 + kk;
-            xs[kk][rr] = (gr < Tn && gk < K) ? ldf(x + (size_t)gr * K + gk) : 0.f;
-            ws[kk][rr] = (gc < N && gk < K) ? ldf(W + (size_t)gc * K + gk) : 0.f;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { a[i] = xs[kk][ty * 4 + i]; b[i] = ws[kk][tx * 4 + i]; }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] += a[i] * b[j];
-        }
-        __syncthreads();
-    }
+linear_simt_kernel(const float *__restrict__ x, const float *__restrict__ W, int Tn, int K, int N,
+                   const int32_t *__restrict__ row_adapter, const AdapterDev *__restrict__ adapters,
+                   const float *__restrict__ t, int RP, int Nq, int Nkv, const float *residual /* may alias y */, float *y,
+                   float *__restrict__ pool, const int32_t *__restrict__ slot_map, int hd, int Hkv, int page_size,
+                   int num_pages, int base_first, int32_t *status) {
+    __shared__ float part[8][16][32 + 1];
+    tc::grid_dep_launch();
+    if (!base_first) tc::grid_dep_wait();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tx = lane & 7, ty = lane >> 3;
+    const int row0 = blockIdx.y * 16, col0 = blockIdx.x * 32;
+    float acc[4][4] = {};   // rows row0 + ty + 4 i, columns col0 + tx + 8 j (beyond the edge: the last one again, not stored)
+    const float *xr[4], *wr[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const int row = row0 + ty * 4 + i;
-        if (row >= Tn) continue;
-        const int k = row_adapter ? row_adapter[row] : -1;
+        xr[i] = x + (size_t)min(row0 + ty + 4 * i, Tn - 1) * K;
+        wr[i] = W + (size_t)min(col0 + tx + 8 * i, N - 1) * K;
+    }
+    auto step = [&](const float4 (&a)[4], const float4 (&b)[4]) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = col0 + tx * 4 + j;
-            if (n >= N) continue;
-            float v = acc[i][j];
-            if (k >= 0) {
-                const AdapterDev ad = adapters[k];
-                const T *B = (const T *)ad.B + (size_t)n * RP;
-                const int blk = n < Nq ? 0 : (n < Nq + Nkv ? 1 : 2);
-                const float *tr = t + ((size_t)row * 3 + blk) * RP;
-                float dlt = 0.f;
-                for (int r = 0; r < ad.rank; ++r) dlt += ldf(B + r) * tr[r];
-                v += dlt;
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                acc[i][j] += a[i].x * b[j].x; acc[i][j] += a[i].y * b[j].y;
+                acc[i][j] += a[i].z * b[j].z; acc[i][j] += a[i].w * b[j].w;
             }
-            if (residual) v += ldf(residual + (size_t)row * N + n);
-            stf(y + (size_t)row * N + n, v);
+    };
+    if (K % 4 == 0) {
+#pragma unroll 2
+        for (int k = warp * 4; k < K; k += 32) {
+            float4 a[4], b[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { a[i] = *reinterpret_cast<const float4 *>(xr[i] + k); b[i] = *reinterpret_cast<const float4 *>(wr[i] + k); }
+            step(a, b);
+        }
+    } else {
+        for (int k = warp * 4; k < K; k += 32) {
+            float4 a[4], b[4];
+            auto four = [&](const float *r) {
+                return make_float4(r[k], k + 1 < K ? r[k + 1] : 0.f, k + 2 < K ? r[k + 2] : 0.f, k + 3 < K ? r[k + 3] : 0.f);
+            };
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { a[i] = four(xr[i]); b[i] = four(wr[i]); }
+            step(a, b);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) part[warp][ty + 4 * i][tx + 8 * j] = acc[i][j];
+    __syncthreads();
+    if (base_first) tc::grid_dep_wait();   // t
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int row = row0 + (int)(threadIdx.x >> 5) + 8 * h, n = col0 + lane;
+        if (row >= Tn || n >= N) continue;
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) v += part[w][row - row0][lane];
+        const int k = row_adapter ? row_adapter[row] : -1;
+        const int blk = n < Nq ? 0 : (n < Nq + Nkv ? 1 : 2);
+        if (k >= 0) {
+            const AdapterDev ad = adapters[k];
+            const float *B = (const float *)ad.B + (size_t)n * RP;
+            const float *tr = t + ((size_t)row * 3 + blk) * RP;
+            float dlt = 0.f;
+#pragma unroll 8
+            for (int r = 0; r < ad.rank; ++r) dlt += B[r] * tr[r];
+            v += dlt;
+        }
+        if (residual) v += residual[(size_t)row * N + n];
+        y[(size_t)row * N + n] = v;
+        if (pool != nullptr && blk > 0) {
+            const int slot = slot_map[row];
+            if (slot < 0) continue;
+            const int page = slot / page_size;
+            if (page >= num_pages) { report(status, ALORA_ERR_PAGE_RANGE); continue; }
+            const int c = n - Nq - (blk - 1) * Nkv;
+            pool[((((size_t)page * 2 + blk - 1) * Hkv + c / hd) * page_size + slot % page_size) * hd + c % hd] = v;
         }
     }
 }
@@ -341,77 +376,129 @@ int launch_rope(alora_ctx *ctx, void *qkv, const int32_t *positions, int T, void
 }
 
 // ---------------------------------------------------------------------------------------------
-// CUDA-core attention (Eq. 1 / Eq. 3): one warp per (token, query head); the block holds the G query
-// heads that share a KV head.  Keys are taken 32 at a time: lane j scores key j0 + j against the
-// query kept in shared memory, the warp combines the 32 scores with shuffles (running maximum and
-// sum: online softmax), then every lane accumulates its slice of the head dimension over the 32
-// value rows.
+// CUDA-core attention (fp32; Eq. 1 / Eq. 3): a block per (token, KV head, HC of the query heads that share it).  Bound by the
+// latency of a key's loads and sums at the lengths that run here: its 32 groups of 8 lanes are streams of their own, stream g
+// taking keys g, g + 32, ... with its own running maximum and sum (online softmax), a lane an eighth of the head
+// dimension, the keys and values of U of the stream's keys in flight; the streams are put together at the end.  (A warp per
+// head that scored a key per lane, element by element, and went over the values one key after the other took 24 us for 16
+// tokens on 64 cached ones, 27 with its launch: 4 us.)
 // ---------------------------------------------------------------------------------------------
-template <typename T, int HD>
-__global__ void attn_simt_kernel(const T *__restrict__ qkv, const int32_t *__restrict__ positions,
-                                const int32_t *__restrict__ token_req, const int32_t *__restrict__ slot_map,
-                                const int32_t *__restrict__ block_tables, int max_blocks, int num_pages, int page_size, int N, int Nq, int Hkv, int G,
-                                float scale, const T *__restrict__ pool, T *__restrict__ out,
-                                 int32_t *status) {
-    extern __shared__ float q_s[];  // [G][HD]
-    constexpr int DPL = HD / 32;    // head-dim elements per lane
-    const int t = blockIdx.x, kvh = blockIdx.y;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int h = kvh * G + warp;
-    const int r = token_req[t];
-    const int p = positions[t];
+template <int HD, int HC>
+__global__ void __launch_bounds__(256)
+attn_simt_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ positions, const int32_t *__restrict__ token_req,
+                 const int32_t *__restrict__ slot_map, const int32_t *__restrict__ block_tables, int max_blocks, int num_pages,
+                 int page_size, int N, int Nq, int Hkv, int G, float scale, const float *__restrict__ pool,
+                 float *__restrict__ out, int32_t *status) {
+    constexpr int V = HD / 32, U = HD == 128 ? 2 : 4;   // 16-byte vectors of a lane; keys of a stream in flight
+    __shared__ float o_s[8][HC][HD], m_s[8][HC], l_s[8][HC];
+    tc::grid_dep_launch();
+    tc::grid_dep_wait();
+    const int t = blockIdx.x, kvh = blockIdx.y, h0 = (int)blockIdx.z * HC, nh = min(HC, G - h0);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, stream = warp * 4 + (lane >> 3), d0 = (lane & 7) * 4;
+    const int r = token_req[t], p = positions[t];
+    float *orow = out + (size_t)t * Nq + (size_t)(kvh * G + h0) * HD;
     if (slot_map[t] < 0) {  // token rejected by the metadata step: defined output, no cache access
-        for (int d = lane; d < HD; d += 32) stf(out + (size_t)t * Nq + (size_t)h * HD + d, 0.f);
+        for (int d = threadIdx.x; d < nh * HD; d += 256) orow[d] = 0.f;
         return;
     }
-    float *qs = q_s + warp * HD;
-    for (int d = lane; d < HD; d += 32) qs[d] = ldf(qkv + (size_t)t * N + (size_t)h * HD + d) * scale;
-    __syncwarp();
-    float m = -INFINITY, l = 0.f, acc[DPL];
+    float4 q[HC][V], acc[HC][V];
+    float m[HC], l[HC];
 #pragma unroll
-    for (int i = 0; i < DPL; ++i) acc[i] = 0.f;
-    const size_t plane_stride = (size_t)Hkv * page_size * HD;
-    for (int j0 = 0; j0 <= p; j0 += 32) {
-        const int j = j0 + lane;
-        float s = -INFINITY;
-        const T *krow = nullptr;
-        if (j <= p) {
-            const int page = block_tables[(size_t)r * max_blocks + j / page_size];
-            if (page >= 0 && page < num_pages) {
-                krow = pool + ((size_t)page * 2 * Hkv + kvh) * page_size * HD + (size_t)(j % page_size) * HD;
-                float dot = 0.f;
-#pragma unroll 8
-                for (int d = 0; d < HD; ++d) dot += qs[d] * ldf(krow + d);
-                s = dot;
-            } else {
-                report(status, ALORA_ERR_PAGE_RANGE);
+    for (int c = 0; c < HC; ++c) {
+        m[c] = -INFINITY; l[c] = 0.f;
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            const float4 a = *reinterpret_cast<const float4 *>(qkv + (size_t)t * N + (size_t)(kvh * G + min(h0 + c, G - 1)) * HD + d0 + 32 * v);
+            q[c][v] = make_float4(a.x * scale, a.y * scale, a.z * scale, a.w * scale);
+            acc[c][v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+    const size_t plane = (size_t)Hkv * page_size * HD;
+    const int32_t *table = block_tables + (size_t)r * max_blocks;
+    for (int j0 = stream; j0 - stream <= p; j0 += 32 * U) {
+        float4 kv[U][V], vv[U][V];
+        bool on[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int j = j0 + 32 * u, page = j <= p ? table[j / page_size] : -1;
+            on[u] = page >= 0 && page < num_pages;
+            if (j <= p && !on[u]) report(status, ALORA_ERR_PAGE_RANGE);
+            const float *kr = pool + ((size_t)(on[u] ? page : 0) * 2 * Hkv + kvh) * page_size * HD + (size_t)(j % page_size) * HD + d0;
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                kv[u][v] = on[u] ? *reinterpret_cast<const float4 *>(kr + 32 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
+                vv[u][v] = on[u] ? *reinterpret_cast<const float4 *>(kr + plane + 32 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
-        float mx = s;
-        for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-        const float m_new = fmaxf(m, mx);
-        if (m_new == -INFINITY) continue;  // nothing visible in this group (only on bad pages)
-        const float w = (s == -INFINITY) ? 0.f : __expf(s - m_new);
-        float wsum = w;
-        for (int off = 16; off; off >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, off);
-        const float corr = (m == -INFINITY) ? 0.f : __expf(m - m_new);
-        l = l * corr + wsum;
 #pragma unroll
-        for (int i = 0; i < DPL; ++i) acc[i] *= corr;
-        const int nvis = min(32, p - j0 + 1);
-        for (int jj = 0; jj < nvis; ++jj) {
-            const float wj = __shfl_sync(0xffffffffu, w, jj);
-            const unsigned long long kp = __shfl_sync(0xffffffffu, (unsigned long long)krow, jj);
-            if (kp == 0ull) continue;
-            const T *vrow = (const T *)kp + plane_stride;
+        for (int c = 0; c < HC; ++c) {
+            float s[U], mx = m[c];
 #pragma unroll
-            for (int i = 0; i < DPL; ++i) acc[i] += wj * ldf(vrow + lane + 32 * i);
+            for (int u = 0; u < U; ++u) {
+                float dot = 0.f;
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    dot += q[c][v].x * kv[u][v].x; dot += q[c][v].y * kv[u][v].y;
+                    dot += q[c][v].z * kv[u][v].z; dot += q[c][v].w * kv[u][v].w;
+                }
+                for (int off = 1; off < 8; off <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+                s[u] = on[u] ? dot : -INFINITY;
+                mx = fmaxf(mx, s[u]);
+            }
+            if (mx != -INFINITY) {   // (else nothing visible yet to this stream; its 8 lanes agree)
+                const float corr = m[c] == -INFINITY ? 0.f : __expf(m[c] - mx);
+                m[c] = mx; l[c] *= corr;
+#pragma unroll
+                for (int v = 0; v < V; ++v) { acc[c][v].x *= corr; acc[c][v].y *= corr; acc[c][v].z *= corr; acc[c][v].w *= corr; }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const float w = on[u] ? __expf(s[u] - mx) : 0.f;
+                    l[c] += w;
+#pragma unroll
+                    for (int v = 0; v < V; ++v) {
+                        acc[c][v].x += w * vv[u][v].x; acc[c][v].y += w * vv[u][v].y;
+                        acc[c][v].z += w * vv[u][v].z; acc[c][v].w += w * vv[u][v].w;
+                    }
+                }
+            }
         }
-        m = m_new;
     }
-    const float inv = l > 0.f ? 1.f / l : 0.f;
+    __syncwarp();
+    // the four streams of a warp, then the eight warps
 #pragma unroll
-    for (int i = 0; i < DPL; ++i) stf(out + (size_t)t * Nq + (size_t)h * HD + lane + 32 * i, acc[i] * inv);
+    for (int c = 0; c < HC; ++c) {
+        for (int off = 8; off < 32; off <<= 1) {
+            const float m2 = __shfl_xor_sync(0xffffffffu, m[c], off), l2 = __shfl_xor_sync(0xffffffffu, l[c], off);
+            const float mx = fmaxf(m[c], m2);
+            const float w1 = m[c] == -INFINITY ? 0.f : __expf(m[c] - mx), w2 = m2 == -INFINITY ? 0.f : __expf(m2 - mx);
+            m[c] = mx; l[c] = l[c] * w1 + l2 * w2;
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                acc[c][v].x = acc[c][v].x * w1 + __shfl_xor_sync(0xffffffffu, acc[c][v].x, off) * w2;
+                acc[c][v].y = acc[c][v].y * w1 + __shfl_xor_sync(0xffffffffu, acc[c][v].y, off) * w2;
+                acc[c][v].z = acc[c][v].z * w1 + __shfl_xor_sync(0xffffffffu, acc[c][v].z, off) * w2;
+                acc[c][v].w = acc[c][v].w * w1 + __shfl_xor_sync(0xffffffffu, acc[c][v].w, off) * w2;
+            }
+        }
+        if (lane < 8) {
+#pragma unroll
+            for (int v = 0; v < V; ++v) *reinterpret_cast<float4 *>(&o_s[warp][c][d0 + 32 * v]) = acc[c][v];
+            if (lane == 0) { m_s[warp][c] = m[c]; l_s[warp][c] = l[c]; }
+        }
+    }
+    __syncthreads();
+    for (int d = threadIdx.x; d < nh * HD; d += 256) {
+        const int c = d / HD;
+        float mx = -INFINITY, lsum = 0.f, o = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) mx = fmaxf(mx, m_s[w][c]);
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            const float e = m_s[w][c] == -INFINITY ? 0.f : __expf(m_s[w][c] - mx);
+            lsum += l_s[w][c] * e; o += o_s[w][c][d % HD] * e;
+        }
+        orow[d] = lsum > 0.f ? o / lsum : 0.f;
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -561,70 +648,49 @@ int launch_swiglu(alora_ctx *ctx, const void *gate_up, int T, void *y, cudaStrea
     return 1;
 }
 
-// ---- launchers of the CUDA-core projection / attention, by data type -------------------------------
-template <typename T>
-static int project_simt(alora_ctx *ctx, int layer, const void *hidden, int Tn, void *qkv, cudaStream_t s) {
+// ---- launchers of the fp32 projection / attention ------------------------------------------------------------------
+int launch_project_simt(alora_ctx *ctx, int layer, const void *hidden, int T, void *qkv, cudaStream_t s, void *kv_pool,
+                        int num_pages) {
+    if (T == 0) return 0;
     const Dims &d = ctx->d;
     const AdapterDev *ads = ctx->d_adapters + (size_t)layer * ctx->cfg.max_adapters;
-    {
+    {   // (an ordinary launch: x is complete before it begins, and so before the projection's base sums)
         ProfScope prof(ctx, KK_SHRINK, s);
-        shrink_simt_kernel<T><<<Tn, 256, 0, s>>>((const T *)hidden, ctx->d_row_adapter, ads, d.H, d.RP, (float *)ctx->d_t);
+        shrink_simt_kernel<<<dim3(T, 3), 256, 0, s>>>((const float *)hidden, ctx->d_row_adapter, ads, d.H, d.RP, (float *)ctx->d_t);
     }
     ProfScope prof(ctx, KK_PROJECT, s);
-    dim3 grid((d.N + 63) / 64, (Tn + 63) / 64);
-    linear_simt_kernel<T><<<grid, 256, 0, s>>>((const T *)hidden, (const T *)ctx->layers[layer].wqkv, Tn, d.H, d.N,
-                                               ctx->d_row_adapter, ads, (const float *)ctx->d_t, d.RP, d.Nq, d.Nkv,
-                                               nullptr, (T *)qkv);
-    return 2;
-}
-
-int launch_project_simt(alora_ctx *ctx, int layer, const void *hidden, int T, void *qkv, cudaStream_t s) {
-    if (T == 0) return 0;
-    return ctx->cfg.dtype == ALORA_DTYPE_FP32 ? project_simt<float>(ctx, layer, hidden, T, qkv, s)
-                                              : project_simt<__nv_bfloat16>(ctx, layer, hidden, T, qkv, s);
+    const cudaError_t e = launch_kernel(linear_simt_kernel, dim3((d.N + 31) / 32, (T + 15) / 16), dim3(256), 0, s, true,
+        (const float *)hidden, (const float *)ctx->layers[layer].wqkv, T, d.H, d.N, (const int32_t *)ctx->d_row_adapter, ads,
+        (const float *)ctx->d_t, d.RP, d.Nq, d.Nkv, (const float *)nullptr, (float *)qkv, (float *)kv_pool, (const int32_t *)ctx->d_slot,
+        d.hd, d.Hkv, d.page, num_pages, 1, ctx->d_status);
+    return e == cudaSuccess ? 2 : -1;
 }
 
 int launch_linear_simt(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
                        const void *residual, cudaStream_t s) {
     if (T == 0) return 0;
     ProfScope prof(ctx, KK_LINEAR, s);
-    dim3 grid((N + 63) / 64, (T + 63) / 64);
-    if (ctx->cfg.dtype == ALORA_DTYPE_FP32)
-        linear_simt_kernel<float><<<grid, 256, 0, s>>>((const float *)x, (const float *)W, T, K, N, nullptr, nullptr,
-                                                       nullptr, 0, 0, 0, (const float *)residual, (float *)y);
-    else
-        linear_simt_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>((const __nv_bfloat16 *)x, (const __nv_bfloat16 *)W, T, K,
-                                                               N, nullptr, nullptr, nullptr, 0, 0, 0,
-                                                               (const __nv_bfloat16 *)residual, (__nv_bfloat16 *)y);
-    return 1;
-}
-
-template <typename T>
-static int attend_simt(alora_ctx *ctx, const void *qkv, const BatchArgs &b, const void *pool, void *out,
-                       cudaStream_t s) {
-    const Dims &d = ctx->d;
-    ProfScope prof(ctx, KK_ATTENTION, s);
-    dim3 grid(b.T, d.Hkv);
-    const int threads = 32 * d.G;
-    const size_t smem = (size_t)d.G * d.hd * sizeof(float);
-#define ALORA_ATTN_SIMT(HD)                                                                              \
-    attn_simt_kernel<T, HD><<<grid, threads, smem, s>>>((const T *)qkv, b.positions, ctx->d_token_req,   \
-                                                        ctx->d_slot, b.block_tables, b.max_blocks, b.num_pages, d.page, \
-                                                        d.N, d.Nq, d.Hkv, d.G, d.softmax_scale,           \
-                                                        (const T *)pool, (T *)out, ctx->d_status)
-    if (d.hd == 32) ALORA_ATTN_SIMT(32);
-    else if (d.hd == 64) ALORA_ATTN_SIMT(64);
-    else if (d.hd == 128) ALORA_ATTN_SIMT(128);
-    else return -1;
-#undef ALORA_ATTN_SIMT
-    return 1;
+    const cudaError_t e = launch_kernel(linear_simt_kernel, dim3((N + 31) / 32, (T + 15) / 16), dim3(256), 0, s, true, (const float *)x,
+        (const float *)W, T, K, N, (const int32_t *)nullptr, (const AdapterDev *)nullptr, (const float *)nullptr, 0, 0, 0,
+        (const float *)residual, (float *)y, (float *)nullptr, (const int32_t *)nullptr, 0, 0, 0, 0, 0, ctx->d_status);
+    return e == cudaSuccess ? 1 : -1;
 }
 
 int launch_attend_simt(alora_ctx *ctx, const void *qkv, const BatchArgs &b, const void *pool, void *out,
                        cudaStream_t s) {
     if (b.T == 0) return 0;
-    return ctx->cfg.dtype == ALORA_DTYPE_FP32 ? attend_simt<float>(ctx, qkv, b, pool, out, s)
-                                              : attend_simt<__nv_bfloat16>(ctx, qkv, b, pool, out, s);
+    const Dims &d = ctx->d;
+    ProfScope prof(ctx, KK_ATTENTION, s);
+    auto go = [&](auto kernel, int hc) {
+        return launch_kernel(kernel, dim3(b.T, d.Hkv, (d.G + hc - 1) / hc), dim3(256), 0, s, true, (const float *)qkv, b.positions,
+                             (const int32_t *)ctx->d_token_req, (const int32_t *)ctx->d_slot, b.block_tables, b.max_blocks, b.num_pages,
+                             d.page, d.N, d.Nq, d.Hkv, d.G, d.softmax_scale, (const float *)pool, (float *)out, ctx->d_status);
+    };
+    const bool two = d.G > 1;
+    const cudaError_t e = d.hd == 32 ? (two ? go(attn_simt_kernel<32, 2>, 2) : go(attn_simt_kernel<32, 1>, 1))
+                          : d.hd == 64 ? (two ? go(attn_simt_kernel<64, 2>, 2) : go(attn_simt_kernel<64, 1>, 1))
+                                       : (two ? go(attn_simt_kernel<128, 2>, 2) : go(attn_simt_kernel<128, 1>, 1));
+    return e == cudaSuccess ? 1 : -1;
 }
 
 }  // namespace alora

@@ -114,6 +114,35 @@ def test_config1_tiny_fp32_layer(oracle64):
         g.close()
 
 
+@pytest.mark.parametrize("hidden,heads,kv_heads,hd,new", [(36, 3, 1, 32, (1, 16)), (100, 4, 4, 128, (33, 5)), (64, 5, 1, 64, (17, 130))])
+def test_fp32_layer_tile_and_head_edges(oracle64, hidden, heads, kv_heads, hd, new):
+    """Rows, widths and K that do not fill the fp32 tiles, one and several query heads per KV head (an odd number too), every
+    head dimension, gates opening inside a request, keys from none but the token's own to more than a block's streams."""
+    shape = wl.LayerShape(hidden=hidden, n_q_heads=heads, n_kv_heads=kv_heads, head_dim=hd, page_size=16, dtype="fp32", intermediate=64)
+    rng = np.random.default_rng(hidden)
+    w = wl.make_wqkv(shape, rng)
+    ads = [wl.make_adapter(shape, 3, rng), wl.make_adapter(shape, 8, rng, scale=2.0)]
+    b = wl.make_batch(shape, [0, 70], list(new), [1, 0], rng, activation_offsets=[0, 73], shuffle_pages=True, with_prefix_hidden=True)
+    g = hp.GpuLayers(shape, [dict(wqkv=w)], [ads], 256, 4)
+    try:
+        pool = g.new_pool(b.num_pages)
+        _run_base_prefill(g, shape, b, pool)
+        d = hp.DevBatch(b, shape.dtype)
+        out = g.empty(b.T, shape.Nq)
+        ab.alora_prefill_layer(g.ctx, 0, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, pool, d.bt,
+                               d.max_blocks, b.num_pages, d.T, d.R, out)
+        assert g.status() == 0
+        Ks, Vs = hp.oracle_base_prefix(oracle64, shape, w, b)
+        want = hp.oracle_block(oracle64, shape, w, ads, b, Ks, Vs)
+        hp.assert_close(hp.to_host(out), want["out"], 1e-5, "")   # the bound of the other fp32 layer test
+        got = _gather_pool(oracle64, shape, hp.to_host(pool), b)
+        for r in range(b.R):
+            hp.assert_close(got[r][0], want["K"][r], 1e-5, "")
+            hp.assert_close(got[r][1], want["V"][r], 1e-5, "")
+    finally:
+        g.close()
+
+
 def test_ragged_multi_adapter_layer_bf16(oracle64):
     """Projection, append and attention on a ragged multi-adapter batch with mid-chunk activation."""
     w, ads, b = _mid_workload()
