@@ -110,11 +110,15 @@ struct ProfEvent {
     int kind;
 };
 
+// All adapters' A rows [max_adapters * 192][H] in boxes of 16, 32, 48 and 64 rows: box[r / 16 - 1] fetches the rows of one q / k /
+// v block of an adapter of padded rank r in one copy (a copy takes 75 ns however few rows it brings).
+struct RankMaps { CUtensorMap box[4]; };
+
 // Tensor maps of one layer that depend only on registered weights (bf16 tensor-core path).
 struct TcLayerMaps {
     CUtensorMap wqkv[3];      // W_qkv [N][H], boxes of 128 / 256 / 64 rows
     CUtensorMap a_all;        // all adapters' A rows [max_adapters*192][H], box 192 rows
-    CUtensorMap a_all16;      // the same rows in boxes of 16 (shrink chunks of the few-row projection)
+    RankMaps a_rank;
     CUtensorMap b_all_bn[3];  // all adapters' B rows [max_adapters*N][64], boxes of 128 / 256 / 64 rows
     // for the 256 x 192 tiles of gemm_pair_tcgen05.cu: W in boxes of 192 rows; per q / k / v block the B rows of all
     // adapters as (rank column, row inside the block, adapter), boxes of 192 rows

@@ -81,9 +81,9 @@ __device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t (&r)[16])
 
 __global__ void __launch_bounds__(kFcThreads, 1)
 gemm_few_cluster_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
-                        const __grid_constant__ CUtensorMap tmA, const FewArgs a) {
+                        const __grid_constant__ RankMaps tmA, const FewArgs a) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ int kv_slot_s[kFewRowMax], slot_s[kFewRowMax], id_s[kFewRowMax], rpad_s[kFewRowMax], first_chunk[kFewRowMax], b_start[kFewRowMax], chunk_row[kFcMaxChunks];
+    __shared__ int kv_slot_s[kFewRowMax], slot_s[kFewRowMax], id_s[kFewRowMax], rpad_s[kFewRowMax], first_chunk[kFewRowMax], b_start[kFewRowMax];
     __shared__ float scale_s[kFewRowMax];
     __shared__ int n_present_s, n_chunk_s, max_rank_s;
     const uint32_t smem_base = (tc::smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -141,13 +141,13 @@ gemm_few_cluster_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
         }
         if (threadIdx.x == kFcThreads - 1) n_present_s = meta->n_present;
         __syncthreads();
-        if (threadIdx.x == 0) {   // the A rows that this column tile needs, in chunks of 16
+        if (threadIdx.x == 0) {   // where each adapter's A rows lie in a ring stage, in chunks of 16 (at most kFcMaxChunks: few_plan())
             int n = 0, mx = 0;
             for (int p = 0; p < n_present_s; ++p) {
                 first_chunk[p] = n;
                 b_start[p] = n * share * 32 + 16 * p;   // 16 bytes between the adapters: rows of different ones in different banks
                 mx = max(mx, rpad_s[p]);
-                for (int c = 0; c < rpad_s[p] && n < kFcMaxChunks; c += 16) chunk_row[n++] = id_s[p] * 3 * kFcRank + blk * kFcRank + c;
+                n += rpad_s[p] / 16;
             }
             n_chunk_s = n;
             max_rank_s = mx;
@@ -179,7 +179,8 @@ gemm_few_cluster_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                     tc::tma_load_2d(sw, &tmW, full_bar(s), k, col0);
                 }
                 tc::tma_load_2d(sx, &tmX, full_bar(s), k, row0);
-                for (int i = 0; i < n_chunk; ++i) tc::tma_load_2d(sc + i * kFcChunkBytes, &tmA, full_bar(s), k, chunk_row[i]);
+                for (int p = 0; p < n_present; ++p)
+                    tc::tma_load_2d(sc + first_chunk[p] * kFcChunkBytes, &tmA.box[rpad_s[p] / 16 - 1], full_bar(s), k, id_s[p] * 3 * kFcRank + blk * kFcRank);
             }
             if (!ok) {
                 // copies already in flight must land before the shared memory is reused or released
@@ -405,7 +406,7 @@ gemm_few_cluster_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
 constexpr int kFcDynMax = 227 * 1024 - 4096;
 
 cudaError_t launch_cluster(dim3 grid, int cluster, size_t smem, cudaStream_t s, const CUtensorMap &x, const CUtensorMap &w,
-                           const CUtensorMap &am, const FewArgs &a) {
+                           const RankMaps &am, const FewArgs &a) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = dim3(kFcThreads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
     cudaLaunchAttribute attr[2];
@@ -487,9 +488,9 @@ bool few_cluster_route(const alora_ctx *ctx, int T, int R, int N, int K, bool lo
     return few_plan(ctx, T, R, N, K, lora, Nq, Nkv, a);
 }
 
-// Returns kernels launched, or -1.  `meta`: the batch's adapter facts of the layer (with the layer's A rows as a tensor
-// map of 16-row boxes and its B slab), or nullptr for a plain dense projection.
-int launch_few_cluster(alora_ctx *ctx, const void *x, const void *W, const CUtensorMap *tmA16, const FewRowMeta *meta,
+// Returns kernels launched, or -1.  `meta`: the batch's adapter facts of the layer (with the layer's A rows as tensor
+// maps and its B slab), or nullptr for a plain dense projection.
+int launch_few_cluster(alora_ctx *ctx, const void *x, const void *W, const RankMaps *tmA, const FewRowMeta *meta,
                        const void *b_all, int T, int R, int K, int N, int Nq, int Nkv, void *out, const void *residual, void *kv_pool,
                        int num_pages, cudaStream_t s) {
     FewArgs a{};
@@ -505,7 +506,7 @@ int launch_few_cluster(alora_ctx *ctx, const void *x, const void *W, const CUten
         a.kv_page_size = ctx->d.page; a.kv_num_pages = num_pages;
     }
     const int n_tiles = (N + a.bn - 1) / a.bn * a.n_rt;
-    if (launch_cluster(dim3(n_tiles * a.ksplit), a.ksplit, (size_t)a.bar_off + 256 + 1024, s, tmX, tmW, meta ? *tmA16 : tmW, a) != cudaSuccess)
+    if (launch_cluster(dim3(n_tiles * a.ksplit), a.ksplit, (size_t)a.bar_off + 256 + 1024, s, tmX, tmW, meta ? *tmA : RankMaps{}, a) != cudaSuccess)
         return -1;
     // the attention work lists of this batch are built now, beside the weight stream (a dependent launch that reads
     // nothing this kernel writes; its blocks wait for this kernel before they exit)

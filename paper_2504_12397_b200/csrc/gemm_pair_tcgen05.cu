@@ -496,7 +496,7 @@ static bool pair_kernel_ready(alora_ctx *ctx) {
     return attr_set[dev];
 }
 
-bool launch_shrink_tc(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap &tmA, const AdapterDev *adapters,
+bool launch_shrink_tc(alora_ctx *ctx, const CUtensorMap &tmX, const RankMaps &tmA, const AdapterDev *adapters,
                       int T, int K, int max_pairs, int t_parts, cudaStream_t s);  // shrink_tcgen05.cu
 bool shrink_apart(const alora_ctx *ctx, int T, int R, int items);                  // gemm_tcgen05.cu
 
@@ -541,7 +541,7 @@ int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T,
     }
     g.status = ctx->d_status;
     const int grid = std::max(1, std::min(G, items + (apart ? 0 : max_pairs)));
-    if (apart && !launch_shrink_tc(ctx, tmX, lm.a_all, ads, T, d.H, max_pairs, 1, s)) return -1;
+    if (apart && !launch_shrink_tc(ctx, tmX, lm.a_rank, ads, T, d.H, max_pairs, 1, s)) return -1;
     if (launch_kernel(gemm_pair_tcgen05_kernel<kBNqkv, true>, dim3(grid), dim3(kThreadsP), PairSmem<kBNqkv>::kTotal, s, true, tmX,
                       lm.wqkv192, tmT, lm.a_all, lm.b_blk[0], lm.b_blk[1], lm.b_blk[2], g) != cudaSuccess)
         return -1;

@@ -473,7 +473,7 @@ static bool launch_gemm_bn(alora_ctx *ctx, const CUtensorMap &tmA, const CUtenso
     return true;
 }
 
-bool launch_shrink_tc(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap &tmA, const AdapterDev *adapters,
+bool launch_shrink_tc(alora_ctx *ctx, const CUtensorMap &tmX, const RankMaps &tmA, const AdapterDev *adapters,
                       int T, int K, int max_pairs, int t_parts, cudaStream_t s);  // shrink_tcgen05.cu
 
 // Picks the column-tile width: 256 when the q/k/v block boundaries allow it, else 128; 64 for batches of at most
@@ -509,7 +509,7 @@ int launch_skinny_tc(alora_ctx *ctx, const void *x, const CUtensorMap &tmW, cons
                      const void *residual, void *kv_pool, int num_pages, int layer, cudaStream_t s);
 
 bool few_cluster_route(const alora_ctx *ctx, int T, int R, int N, int K, bool lora, int Nq, int Nkv);   // gemm_few_cluster.cu
-int launch_few_cluster(alora_ctx *ctx, const void *x, const void *W, const CUtensorMap *tmA16, const FewRowMeta *meta,
+int launch_few_cluster(alora_ctx *ctx, const void *x, const void *W, const RankMaps *tmA, const FewRowMeta *meta,
                        const void *b_all, int T, int R, int K, int N, int Nq, int Nkv, void *out, const void *residual, void *kv_pool,
                        int num_pages, cudaStream_t s);
 
@@ -541,7 +541,7 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
     const bool have_adapters = ctx->layer_has_adapter[layer];
     if (project_few_cluster(ctx, layer, T, R)) {
         ProfScope prof(ctx, KK_PROJECT, s);
-        return launch_few_cluster(ctx, hidden, ctx->layers[layer].wqkv, &ctx->tc_maps[layer].a_all16,
+        return launch_few_cluster(ctx, hidden, ctx->layers[layer].wqkv, &ctx->tc_maps[layer].a_rank,
                                   have_adapters ? ctx->d_skinny_meta + (size_t)layer * ctx->few_tiles : nullptr, ctx->tc_b_all[layer], T, R,
                                   d.H, d.N, d.Nq, d.Nkv, qkv, nullptr, kv_pool, num_pages, s);
     }
@@ -549,7 +549,7 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
         ProfScope prof(ctx, KK_PROJECT, s);
         const TcLayerMaps &lm = ctx->tc_maps[layer];
         const AdapterDev *ads = ctx->d_adapters + (size_t)layer * ctx->cfg.max_adapters;
-        return launch_skinny_tc(ctx, hidden, lm.wqkv[1], have_adapters ? &lm.a_all16 : nullptr,
+        return launch_skinny_tc(ctx, hidden, lm.wqkv[1], have_adapters ? &lm.a_rank.box[0] : nullptr,
                                 have_adapters ? ads : nullptr, ctx->tc_b_all[layer], T, d.H, d.N, d.Nq, d.Nkv, qkv, nullptr,
                                 kv_pool, num_pages, layer, s);
     }
@@ -573,7 +573,7 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
     int n = 0;
     if (have_adapters && !fuse_shrink) {
         ProfScope prof(ctx, KK_SHRINK, s);
-        if (!launch_shrink_tc(ctx, tmX, lm.a_all, ads, T, d.H, max_pairs, t_parts, s)) return -1;
+        if (!launch_shrink_tc(ctx, tmX, lm.a_rank, ads, T, d.H, max_pairs, t_parts, s)) return -1;
         ++n;
     }
     {
@@ -680,7 +680,7 @@ bool build_layer_maps(alora_ctx *ctx, int layer) {
     }
     const size_t na = (size_t)std::max(1, ctx->cfg.max_adapters);
     ok &= make_tensor_map_bf16(&lm.a_all, ctx->tc_a_all[layer], na * 3 * kTensorRP, d.H, d.H, 3 * kTensorRP);
-    ok &= make_tensor_map_bf16(&lm.a_all16, ctx->tc_a_all[layer], na * 3 * kTensorRP, d.H, d.H, 16);
+    for (int i = 0; i < 4; ++i) ok &= make_tensor_map_bf16(&lm.a_rank.box[i], ctx->tc_a_all[layer], na * 3 * kTensorRP, d.H, d.H, 16 * (i + 1));
     ok &= make_tensor_map_bf16(&lm.b_all_bn[0], ctx->tc_b_all[layer], na * d.N, kTensorRP, kTensorRP, 128);
     ok &= make_tensor_map_bf16(&lm.b_all_bn[1], ctx->tc_b_all[layer], na * d.N, kTensorRP, kTensorRP, 256);
     ok &= make_tensor_map_bf16(&lm.b_all_bn[2], ctx->tc_b_all[layer], na * d.N, kTensorRP, kTensorRP, 64);

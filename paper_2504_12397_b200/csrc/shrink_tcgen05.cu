@@ -1,13 +1,16 @@
 // Rank-r shrink t = s A_k x on the tensor cores (the inner product of the low-rank delta of Eq. 5),
 // split along the hidden dimension over a thread-block cluster.
 //
-// The shrink has few output tiles (one 128 x 192 tile per (row tile, adapter) pair: 3 blocks q/k/v of 64 padded rank
-// columns) but a long contraction (the hidden dimension), so each pair is given to a cluster of
-// kShrinkSplits blocks.  Block c of the cluster contracts hidden columns of its own K range with
-// tcgen05.mma into tensor memory, copies its fp32 partial tile into its shared memory, and after a
-// cluster barrier reduces a 24-column slice of the tile over all blocks' shared memory (distributed
-// shared memory loads) in the fixed order 0, 1, ..., 7.  The order does not depend on timing, so the
-// result is run-to-run deterministic.
+// The shrink has few output tiles (one of 128 rows x 3 blocks q / k / v of the adapter's padded rank per (row tile,
+// adapter) pair) but a long contraction (the hidden dimension), so each pair is given to a cluster of 8 or 4 blocks.
+// Block c of the cluster contracts hidden columns of its own K range with tcgen05.mma into tensor memory, copies its fp32
+// partial tile into its shared memory, and after a cluster barrier reduces its share of the tile's columns over all
+// blocks' shared memory (distributed shared memory loads) in the fixed order 0, 1, ....  The order does not depend on
+// timing, so the result is run-to-run deterministic.
+// Bound by what a block takes in (75 bytes / ns of operands, 20 of other blocks' shared memory) and by the rounds of clusters:
+// only the padded rank's rows of A are loaded, multiplied and reduced, and where more pairs are possible than clusters
+// of 8 fit on the device (15), clusters are of 4 (33 fit).  48 requests over four adapters of rank 8 .. 64, 24 pairs at
+// hidden 4096: 32 -> 18 us against 192 rows of A for each and 8 blocks.
 #include <algorithm>
 
 #include "alora_internal.h"
@@ -15,13 +18,12 @@
 
 namespace alora {
 
-constexpr int kShrinkSplits = 8;        // blocks per cluster = K ranges per row tile
+constexpr int kShrinkMaxSplits = 8;     // blocks per cluster = K ranges per row tile
 constexpr int kShrinkBM = 128;          // rows per tile
-constexpr int kShrinkBN = 192;          // 3 blocks x 64 padded rank columns
+constexpr int kShrinkBN = 192;          // 3 blocks x 64 rows of A stored per adapter
 constexpr int kShrinkBK = 64;
 constexpr int kShrinkStages = 4;
 constexpr int kShrinkThreads = 192;     // warp 0 TMA, warp 1 MMA, warps 2-5 epilogue / reduction
-constexpr int kShrinkSlice = kShrinkBN / kShrinkSplits;  // 24 columns reduced by each block
 
 struct ShrinkArgs {
     const TilePair *pairs;
@@ -29,7 +31,7 @@ struct ShrinkArgs {
     const int32_t *row_adapter;   // [T] applied adapter per row
     const AdapterDev *adapters;
     __nv_bfloat16 *t;   // [pair][t_parts][128][192]
-    int t_parts, T;
+    int t_parts, T, splits;
     int K;              // hidden
     int32_t *status;
 };
@@ -61,8 +63,8 @@ __device__ __forceinline__ float ld_dsmem_f32(uint32_t local_addr, uint32_t rank
     return v;
 }
 
-__global__ void __cluster_dims__(kShrinkSplits, 1, 1) __launch_bounds__(kShrinkThreads, 1)
-shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmA,
+__global__ void __launch_bounds__(kShrinkThreads, 1)
+shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ RankMaps tmA,
                       const ShrinkArgs a) {
     using S = ShrinkSmem;
     tc::grid_dep_launch();
@@ -70,6 +72,8 @@ shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     // the whole cluster takes the same decision: blockIdx.y selects the pair
     if ((int)blockIdx.y >= *a.n_pairs) return;
     const TilePair pair = a.pairs[blockIdx.y];
+    const int rpad = a.adapters[pair.adapter].rpad, cols = 3 * rpad;
+    if (cols == 0) return;   // not registered on this layer (a finding of the metadata step): its t is not used
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (tc::smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -101,22 +105,24 @@ shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     // this block's K range, in 64-column blocks
     const uint32_t crank = cluster_ctarank();
     const int kb_all = (a.K + kShrinkBK - 1) / kShrinkBK;
-    const int kb_per = (kb_all + kShrinkSplits - 1) / kShrinkSplits;
+    const int kb_per = (kb_all + a.splits - 1) / a.splits;
     const int kb0 = (int)crank * kb_per;
     const int nkb = max(0, min(kb_per, kb_all - kb0));
 
     if (warp == 0) {
         if (lane == 0) {
-            tc::tma_prefetch_desc(&tmX); tc::tma_prefetch_desc(&tmA);
+            tc::tma_prefetch_desc(&tmX); tc::tma_prefetch_desc(&tmA.box[rpad / 16 - 1]);
             bool ok = true;
             int kc = 0;
             for (; kc < nkb; ++kc) {
                 const int s = kc % kShrinkStages;
                 if (!tc::mbar_wait(empty_bar(s), ((kc / kShrinkStages) & 1) ^ 1, abort_flag)) { ok = false; break; }
                 const uint32_t sa = smem_base + s * S::kStageBytes, sb = sa + S::kABytes;
-                tc::mbar_arrive_expect_tx(full_bar(s), S::kStageBytes);
+                tc::mbar_arrive_expect_tx(full_bar(s), S::kABytes + cols * kShrinkBK * 2);
                 tc::tma_load_2d(sa, &tmX, full_bar(s), (kb0 + kc) * kShrinkBK, pair.tile * kShrinkBM);
-                tc::tma_load_2d(sb, &tmA, full_bar(s), (kb0 + kc) * kShrinkBK, pair.adapter * kShrinkBN);
+                for (int blk = 0; blk < 3; ++blk)
+                    tc::tma_load_2d(sb + blk * rpad * kShrinkBK * 2, &tmA.box[rpad / 16 - 1], full_bar(s), (kb0 + kc) * kShrinkBK,
+                                    pair.adapter * kShrinkBN + blk * kRankPadMax);
             }
             if (!ok) {
                 // copies already in flight must land before the shared memory is reused or released
@@ -129,7 +135,7 @@ shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         }
     } else if (warp == 1) {
         if (lane == 0 && nkb > 0) {
-            constexpr uint32_t idesc = tc::idesc_bf16_f32(kShrinkBM, kShrinkBN);
+            const uint32_t idesc = tc::idesc_bf16_f32(kShrinkBM, cols);
             for (int kc = 0; kc < nkb; ++kc) {
                 const int s = kc % kShrinkStages;
                 if (!tc::mbar_wait(full_bar(s), (kc / kShrinkStages) & 1, abort_flag)) break;
@@ -151,7 +157,7 @@ shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         if (have) have = tc::mbar_wait(acc_bar, 0, abort_flag);
         tc::tc_fence_after();
 #pragma unroll 1
-        for (int c = 0; c < kShrinkBN; c += 32) {
+        for (int c = 0; c < cols; c += 32) {   // (16 columns of a last half are not read by anyone)
             uint32_t v[32];
             if (have) {
                 tc::tmem_ld_32x32(tmem_base + c + ((uint32_t)(q * 32) << 16), v);
@@ -173,20 +179,28 @@ shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         const int q = warp & 3;
         const int r = q * 32 + lane;
         const float scale = a.adapters[pair.adapter].scale;
-        const int c0 = (int)crank * kShrinkSlice;
-        float acc[kShrinkSlice];
-#pragma unroll
-        for (int j = 0; j < kShrinkSlice; ++j) acc[j] = 0.f;
-#pragma unroll 1
-        for (uint32_t src = 0; src < (uint32_t)kShrinkSplits; ++src) {  // fixed order: deterministic sum
-#pragma unroll
-            for (int j = 0; j < kShrinkSlice; ++j)
-                acc[j] += ld_dsmem_f32(tc::smem_u32(partial + (c0 + j) * kShrinkBM + r), src);
-        }
         const int row = pair.tile * kShrinkBM + r;
-        __nv_bfloat16 *orow = a.t + ((size_t)blockIdx.y * a.t_parts * kShrinkBM + r) * kShrinkBN + c0;
-        tc::store_t<kShrinkSlice>(acc, scale, row < a.T && a.row_adapter[row] == pair.adapter, orow,
-                                  a.t_parts > 1 ? orow + (size_t)kShrinkBM * kShrinkBN : nullptr);
+        const bool use = row < a.T && a.row_adapter[row] == pair.adapter;
+        for (int u = (int)crank * (cols / 8) / a.splits; u < ((int)crank + 1) * (cols / 8) / a.splits; ++u) {   // 8 columns
+            float part[kShrinkMaxSplits][8], acc[8];
+#pragma unroll
+            for (int src = 0; src < kShrinkMaxSplits; ++src)
+                if (src < a.splits) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) part[src][j] = ld_dsmem_f32(tc::smem_u32(partial + (u * 8 + j) * kShrinkBM + r), (uint32_t)src);
+                }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[j] = 0.f;
+#pragma unroll
+            for (int src = 0; src < kShrinkMaxSplits; ++src)   // fixed order: deterministic sum
+                if (src < a.splits) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) acc[j] += part[src][j];
+                }
+            const int blk = u * 8 / rpad;
+            __nv_bfloat16 *orow = a.t + ((size_t)blockIdx.y * a.t_parts * kShrinkBM + r) * kShrinkBN + blk * kRankPadMax + u * 8 - blk * rpad;
+            tc::store_t<8>(acc, scale, use, orow, a.t_parts > 1 ? orow + (size_t)kShrinkBM * kShrinkBN : nullptr);
+        }
     }
 
     cluster_sync_all();  // no block may release its shared memory while another still reads it
@@ -199,7 +213,7 @@ shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
 
 // t = s A x of the (row tile, adapter) pairs of the current batch, of which there are at most max_pairs.  Returns false
 // if the launch could not be set up.
-bool launch_shrink_tc(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap &tmA, const AdapterDev *adapters,
+bool launch_shrink_tc(alora_ctx *ctx, const CUtensorMap &tmX, const RankMaps &tmA, const AdapterDev *adapters,
                       int T, int K, int max_pairs, int t_parts, cudaStream_t s) {
     static bool attr_set[64] = {};
     const int dev = ctx->cfg.device;
@@ -209,9 +223,18 @@ bool launch_shrink_tc(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap 
             return false;
         attr_set[dev] = true;
     }
-    ShrinkArgs a{ctx->d_pairs, ctx->d_counts + 2, ctx->d_row_adapter, adapters, (__nv_bfloat16 *)ctx->d_t, t_parts, T, K, ctx->d_status};
-    return launch_kernel(shrink_tcgen05_kernel, dim3(kShrinkSplits, std::max(1, max_pairs)), dim3(kShrinkThreads),
-                         ShrinkSmem::kTotal, s, true, tmX, tmA, a) == cudaSuccess;
+    ShrinkArgs a{ctx->d_pairs, ctx->d_counts + 2, ctx->d_row_adapter, adapters, (__nv_bfloat16 *)ctx->d_t, t_parts, T,
+                 max_pairs <= ctx->few_clusters[8] ? 8 : 4, K, ctx->d_status};
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(a.splits, std::max(1, max_pairs)); cfg.blockDim = dim3(kShrinkThreads);
+    cfg.dynamicSmemBytes = ShrinkSmem::kTotal; cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)a.splits; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, shrink_tcgen05_kernel, tmX, tmA, a) == cudaSuccess;
 }
 
 }  // namespace alora
