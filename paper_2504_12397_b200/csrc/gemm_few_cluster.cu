@@ -440,7 +440,9 @@ static bool few_plan(const alora_ctx *ctx, int T, int R, int N, int K, bool lora
         if (Nkv > 0 && bn < kFcBNMax && (Nq % bn != 0 || Nkv % bn != 0)) continue;   // a tile lies in one of q, k, v
         const int n_tiles = (N + bn - 1) / bn * a.n_rt;
         int ks = std::max(1, std::min(std::min(kFcMaxCluster, kb_total), ctx->sm_count / n_tiles));
-        while (ks > 1 && ctx->few_clusters[ks] < n_tiles) --ks;   // all clusters at once
+        // all clusters at once; with two places to spare where blocks do not pair up, since what still runs of the kernel
+        // before breaks up the free SMs (26 clusters of 5 where 26 fit: the last one ran alone, 42 us instead of 25)
+        while (ks > 1 && ctx->few_clusters[ks] - (ks % 2 ? 2 : 0) < n_tiles) --ks;
         const long cost = (long)((n_tiles * ks + ctx->sm_count - 1) / ctx->sm_count) * (bn + rs / 2) * ((kb_total + ks - 1) / ks);
         if (a.bn == 0 || cost < best) { best = cost; a.bn = bn; a.ksplit = ks; }
     }
