@@ -210,16 +210,16 @@ attn_splitkv_kernel(const __grid_constant__ CUtensorMap tmKV, const SplitArgs a)
         const int units_per_stage = kSkStageKeys / a.box_rows;
         uint32_t kt = 0, n_it = 0;
         bool ok = true;
-        // block b begins with item b; the rest are handed out in list order to whichever block is free, the claim of the
-        // item after the current one being issued before the current item's loads, so that its latency is hidden behind
-        // them.  (With the first item claimed too, early blocks claimed their second one before late blocks came: where
-        // there is an item per block, some did two while others did none; 2 requests of 4745 keys, head dim 64: 38 -> 32 us.)
+        // block b begins with item b; the rest are handed out in list order to whichever block is free.  A block claims
+        // its next item three stages before the end of the one it loads, which hides the claim's latency.  (Claimed at the
+        // beginning of an item instead, the list's last, short items went to blocks that still had their long one to do:
+        // 40 decode rows in 8 prefix groups, 128 ranges of 34 units and 64 of 5: 61 -> 55 us a layer.  With the first item claimed
+        // too, early blocks took a second one before late blocks had any: 2 requests at head dim 64, 38 -> 32 us.)
         int it_next = blockIdx.x;
         while (ok) {
             int it = -1;
             if (lane == 0) {
                 it = it_next < n_items ? it_next : -1;
-                if (it >= 0) it_next = (int)gridDim.x + atomicAdd(a.work_counter, 1);
                 const int slot = n_it % kSkItemSlots;
                 ok = tc::mbar_wait(item_empty(slot), ((n_it / kSkItemSlots) & 1) ^ 1, abort_flag);
                 if (ok) {
@@ -232,7 +232,8 @@ attn_splitkv_kernel(const __grid_constant__ CUtensorMap tmKV, const SplitArgs a)
             ++n_it;
             if (!ok || it < 0) break;
             const AttnSplitWork w = a.items[it];
-            const int n_st = (w.kv_end - w.kv_start + kSkStageKeys - 1) / kSkStageKeys;
+            const int n_st = (w.kv_end - w.kv_start + kSkStageKeys - 1) / kSkStageKeys, claim_at = max(0, n_st - 3);
+            if (lane == 0 && n_st <= 0) it_next = (int)gridDim.x + atomicAdd(a.work_counter, 1);   // (an empty share of the own keys)
             // Window of the request's block-table row: lane l holds entry win0 + l (win0 a multiple of 32; 32 entries
             // cover a whole number of 64-key stages, and key ranges start at multiples of 64).  A table entry is a
             // dependent load from global memory that would otherwise sit in front of every stage's copies; the
@@ -241,6 +242,7 @@ attn_splitkv_kernel(const __grid_constant__ CUtensorMap tmKV, const SplitArgs a)
                 // the own keys of a prefix group's members: every stage has its own request (table row) and positions
                 const int n_mem = w.pad_ & 0xffff;
                 for (int j = 0; j < n_st && ok; ++j, ++kt) {
+                    if (lane == 0 && j == claim_at) it_next = (int)gridDim.x + atomicAdd(a.work_counter, 1);
                     const int st = kt % kSkStages;
                     int member, kbase;
                     own_key_stage(a.seq_lens, w.req, n_mem, w.pos0, w.kv_start / kSkStageKeys + j, member, kbase);
@@ -270,6 +272,7 @@ attn_splitkv_kernel(const __grid_constant__ CUtensorMap tmKV, const SplitArgs a)
             int win0 = (w.kv_start / a.page_size) & ~31;
             int win = load_window(win0), win_next = load_window(win0 + 32);
             for (int j = 0; j < n_st && ok; ++j, ++kt) {
+                if (lane == 0 && j == claim_at) it_next = (int)gridDim.x + atomicAdd(a.work_counter, 1);
                 const int st = kt % kSkStages;
                 const int kbase = w.kv_start + j * kSkStageKeys;
                 if (kbase / a.page_size >= win0 + 32) {
