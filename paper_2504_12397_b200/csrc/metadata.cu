@@ -26,17 +26,17 @@ __device__ __forceinline__ int find_request(const int32_t *qsl, int R, int t) {
 // page * page_size + position % page_size.  Findings (inconsistent positions, page id out of
 // range, adapter id out of range) go to the status word; the row then gets adapter -1 / slot -1 so that later kernels
 // skip it.  (Whether the adapter is registered on a layer is not looked at here: one that is not has rank 0 there.)
-__device__ __forceinline__ int metadata_token(int t, const int32_t *__restrict__ positions,
+template <typename Hook>
+__device__ __forceinline__ int metadata_token(int t, int p,
                                       const int32_t *__restrict__ a_req,
                                       const int32_t *__restrict__ adapter_ids,
                                       const int32_t *__restrict__ qsl, const int32_t *__restrict__ seq_lens,
                                       const int32_t *__restrict__ block_tables, int max_blocks,
                                       int num_pages, int page_size, int max_adapters, int T, int R, int mode,
                                       int32_t *__restrict__ token_req, int32_t *__restrict__ row_adapter,
-                                      int32_t *__restrict__ slot_map, int32_t *status) {
+                                      int32_t *__restrict__ slot_map, int32_t *status, Hook &&with_adapter) {
     if (t >= T) return -1;
     int r = find_request(qsl, R, t);
-    int p = positions[t];
     // positions of a request are consecutive and end at seq_len - 1
     int expect = seq_lens[r] - (qsl[r + 1] - t);
     bool ok = (p == expect) && p >= 0;
@@ -49,6 +49,7 @@ __device__ __forceinline__ int metadata_token(int t, const int32_t *__restrict__
     }
     if (token_req) token_req[t] = r;
     k = ok ? k : -1;
+    with_adapter(k);
     if (row_adapter) row_adapter[t] = k;
     if (slot_map) {
         int slot = -1;
@@ -615,43 +616,33 @@ __device__ __forceinline__ void metadata_split_items(const int32_t *__restrict__
 }
 
 // FewRowMeta of a tile of at most kFewRowMax rows, thread t's applied adapter being k_mine (-1: none, or no such
-// row): the adapters that occur, ascending, each one's padded rank and scale, and every row's slot.  Called by all
-// kFewRowMax threads of a block.
-__device__ __forceinline__ void metadata_few_row(int k_mine, const AdapterDev *__restrict__ adapters, int max_adapters,
-                                                 FewRowMeta *__restrict__ meta) {
-    __shared__ uint32_t bits[32];
-    __shared__ int16_t ids[kFewRowMax];
-    __shared__ int n_present;
+// row) and `ad` that adapter: the adapters that occur, ascending, each one's padded rank and scale, and every row's slot.
+// Called by all kFewRowMax threads of a block.
+__device__ __forceinline__ void metadata_few_row(int k_mine, const AdapterDev &ad, int max_adapters, FewRowMeta *__restrict__ meta) {
+    __shared__ uint32_t bits[32], below[32];   // adapters present, 32 to a word; how many there are in the words before
     if (threadIdx.x < 32) bits[threadIdx.x] = 0u;
     __syncthreads();
     if (k_mine >= 0 && k_mine < max_adapters && k_mine < 1024) atomicOr(&bits[k_mine >> 5], 1u << (k_mine & 31));
     else k_mine = -1;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int n = 0;
-        for (int w = 0; w < 32; ++w) {
-            uint32_t b = bits[w];
-            while (b && n < kFewRowMax) {
-                const int i = __ffs(b) - 1;
-                b &= b - 1;
-                ids[n++] = (int16_t)(w * 32 + i);
-            }
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x, n = __popc(bits[lane]);
+        int sum = n;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, sum, off);
+            if (lane >= off) sum += v;
         }
-        n_present = n;
-        meta->n_present = n;
+        below[lane] = (uint32_t)(sum - n);
+        if (lane == 31) meta->n_present = sum;
     }
     __syncthreads();
-    const int n = n_present;
-    if ((int)threadIdx.x < n) {
-        const AdapterDev ad = adapters[ids[threadIdx.x]];
-        meta->id[threadIdx.x] = ids[threadIdx.x]; meta->rpad[threadIdx.x] = ad.rpad; meta->scale[threadIdx.x] = ad.scale;
+    int slot = -1;
+    if (k_mine >= 0) {   // (the rows of an adapter all write the same)
+        slot = (int)below[k_mine >> 5] + __popc(bits[k_mine >> 5] & ((1u << (k_mine & 31)) - 1u));
+        meta->id[slot] = k_mine; meta->rpad[slot] = ad.rpad; meta->scale[slot] = ad.scale;
     }
-    if ((int)threadIdx.x < kFewRowMax) {
-        int slot = -1;
-        if (k_mine >= 0)
-            for (int p = 0; p < n; ++p) if (ids[p] == k_mine) slot = p;
-        meta->slot_of_row[threadIdx.x] = slot;
-    }
+    if ((int)threadIdx.x < kFewRowMax) meta->slot_of_row[threadIdx.x] = slot;
 }
 
 // The metadata step.  Phase bit 0: every block handles 256 tokens (request, applied adapter, slot); block 0 then
@@ -677,6 +668,8 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
     // in shared memory, so that the later steps do not each pay a round trip to global memory.
     __shared__ int32_t s_req[4 * kMetaStageR + 1];
     tc::grid_dep_launch();   // the next kernel's blocks may start their set-up; they wait for this kernel's results
+    const int tok = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    const int my_pos = (phases & kMetaProjection) && tok < T ? positions[tok] : 0;   // (in flight with the per-request inputs)
     if (R <= kMetaStageR) {
         int32_t *s_qsl = s_req, *s_len = s_req + R + 1, *s_ids = s_len + R, *s_areq = s_ids + R;
         for (int i = threadIdx.x; i <= R; i += blockDim.x) s_qsl[i] = qsl[i];
@@ -691,8 +684,8 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
         if (a_req) a_req = s_areq;
     }
     if (phases & kMetaProjection)
-        metadata_token((int)(blockIdx.x * blockDim.x + threadIdx.x), positions, a_req, adapter_ids, qsl, seq_lens, block_tables,
-                       max_blocks, num_pages, page_size, max_adapters, T, R, mode, token_req, row_adapter, slot_map, status);
+        metadata_token(tok, my_pos, a_req, adapter_ids, qsl, seq_lens, block_tables,
+                       max_blocks, num_pages, page_size, max_adapters, T, R, mode, token_req, row_adapter, slot_map, status, [](int) {});
     // The three list builders are independent of one another: blocks 0, 1 and 2 take one each (a launch of both
     // phases has at least three blocks, one of the attention phase alone two).
     const int nb = (int)gridDim.x;
@@ -744,6 +737,7 @@ metadata_few_row_kernel(const int32_t *__restrict__ positions, const int32_t *a_
                         FewRowMeta *__restrict__ few_row_meta, int few_tiles, int32_t *status) {
     __shared__ int32_t s_req[4 * kFewRowMax + 1];
     tc::grid_dep_launch();
+    const int tok = (int)(blockIdx.x * kFewRowMax + threadIdx.x), my_pos = tok < T ? positions[tok] : 0;   // (in flight with the per-request inputs)
     if (R <= kFewRowMax) {   // the per-request inputs are read several times (binary search): stage them
         int32_t *s_qsl = s_req, *s_len = s_req + R + 1, *s_ids = s_len + R, *s_areq = s_ids + R;
         for (int i = threadIdx.x; i <= R; i += blockDim.x) s_qsl[i] = qsl[i];
@@ -757,14 +751,16 @@ metadata_few_row_kernel(const int32_t *__restrict__ positions, const int32_t *a_
         if (adapter_ids) adapter_ids = s_ids;
         if (a_req) a_req = s_areq;
     }
+    // (the adapter is fetched beside the block-table entry: neither waits for the other)
     const bool first = blockIdx.y == 0;
-    int k = metadata_token((int)(blockIdx.x * kFewRowMax + threadIdx.x), positions, a_req, adapter_ids, qsl, seq_lens, first ? block_tables : nullptr,
+    AdapterDev ad{};
+    int k = metadata_token(tok, my_pos, a_req, adapter_ids, qsl, seq_lens, first ? block_tables : nullptr,
                            max_blocks, num_pages, page_size, max_adapters, T, R, mode, first ? token_req : nullptr,
-                           first ? row_adapter : nullptr, first ? slot_map : nullptr, status);
+                           first ? row_adapter : nullptr, first ? slot_map : nullptr, status,
+                           [&](int applied) { if (few_row_meta != nullptr && applied >= 0) ad = adapters[(size_t)blockIdx.y * max_adapters + applied]; });
     if (few_row_meta != nullptr) {
-        const AdapterDev *ads = adapters + (size_t)blockIdx.y * max_adapters;
-        if (k >= 0 && ads[k].rank == 0) { report(status, ALORA_ERR_NO_WEIGHTS); k = -1; }
-        metadata_few_row(k, ads, max_adapters, few_row_meta + (size_t)blockIdx.y * few_tiles + blockIdx.x);
+        if (k >= 0 && ad.rank == 0) { report(status, ALORA_ERR_NO_WEIGHTS); k = -1; }
+        metadata_few_row(k, ad, max_adapters, few_row_meta + (size_t)blockIdx.y * few_tiles + blockIdx.x);
     }
 }
 
