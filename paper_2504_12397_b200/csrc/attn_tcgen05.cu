@@ -70,47 +70,52 @@ __device__ __forceinline__ int whole_item(int round) {
     return round * n + ((round & 1) ? n - 1 - b : b);
 }
 
+// partial-result slot of part `part` of an item whose first part is held by block c_first: a block holds at
+// most one part > 0 (the piece its run starts with) and at most one part 0 of a cut item (the piece it ends with)
+__host__ __device__ __forceinline__ int part_slot(int c_first, int part) { return 2 * (c_first + part) + (part == 0 ? 1 : 0); }
+
 // A block's work: whole items (one of each round of `blocks` items) below n_whole, then the pieces of its run (tiles
 // [blockIdx * len, +len) of the concatenated key tiles of the items from n_whole on).  One piece = tiles [t0, t1)
-// of one item.  An item cut by run boundaries is worked on by n_parts consecutive blocks (this block holds part
-// `part`, the first of them is block c_first); each writes its partial result to a slot and a merge kernel adds
-// the parts up afterwards.
+// of one item.  An item cut by run boundaries is worked on by consecutive blocks; each writes
+// its partial result to a slot and a merge kernel adds the parts up afterwards.
 struct RunPiece {
     AttnWork w;
-    int item, t0, t1, n_parts, part, c_first;
+    int t0, t1, slot;   // slot of the partial result, -1: the whole item
 };
+// (What the iterator needs of the split is read again for every piece: kept in registers across the softmax it made the
+// batches that may be cut up to 10 % slower than those that cannot be; 4 x 1024 on 32768: 2 x 2080 -> 2 x 2020 us.)
+__device__ __forceinline__ int ld_again(const int32_t *p) {
+    int v;
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
 struct RunIter {
-    int gt, gt_end, it, len, off, n_whole, round = 0;
-    __device__ explicit RunIter(const AttnArgs &a) {
-        const int total = a.run_counts[0];
-        len = a.run_counts[1];
-        n_whole = a.run_counts[2];
-        off = a.run_counts[3];
-        gt = min(total, (int)blockIdx.x * len);
-        gt_end = min(total, gt + len);
-        it = gt < gt_end ? a.cta_start[blockIdx.x] : 0;
-    }
+    int gt = -1, it = 0, round = 0;   // next tile of this block's run (-1: not begun), its item; rounds of whole items done
+    __device__ explicit RunIter(const AttnArgs &) {}
     __device__ bool next(const AttnArgs &a, RunPiece &p) {
         const int whole = whole_item(round);
-        if (whole < n_whole) {
+        if (whole < ld_again(a.run_counts + 2)) {
             ++round;
-            p.item = whole;
-            p.w = a.items[p.item];
+            p.w = a.items[whole];
             p.t0 = 0;
             p.t1 = (p.w.kv_end + kKeysPerTile - 1) / kKeysPerTile;
-            p.c_first = 0; p.n_parts = 1; p.part = 0;
+            p.slot = -1;
             return true;
         }
-        if (gt >= gt_end) return false;
-        p.item = it;
+        const int total = ld_again(a.run_counts), len = ld_again(a.run_counts + 1), off = ld_again(a.run_counts + 3);
+        const int begin = min(total, (int)blockIdx.x * len), end = min(total, begin + len);
+        if (gt < 0) {
+            gt = begin;
+            if (begin < end) it = ld_again(a.cta_start + blockIdx.x);
+        }
+        if (gt >= end) return false;
         p.w = a.items[it];
         const int n_tiles = (p.w.kv_end + kKeysPerTile - 1) / kKeysPerTile;
         const int first = p.w.split - off;    // the item's first tile in the concatenation
         p.t0 = gt - first;
-        p.t1 = min(n_tiles, gt_end - first);
-        p.c_first = first / len;
-        p.n_parts = (first + n_tiles - 1) / len - p.c_first + 1;
-        p.part = (int)blockIdx.x - p.c_first;
+        p.t1 = min(n_tiles, end - first);
+        const int c_first = first / len, n_parts = (first + n_tiles - 1) / len - c_first + 1;
+        p.slot = n_parts == 1 ? -1 : part_slot(c_first, (int)blockIdx.x - c_first);
         gt = first + p.t1;
         ++it;
         return true;
@@ -125,17 +130,13 @@ struct WholeIter {
         const int whole = whole_item(round);
         if (whole >= n_items) return false;
         ++round;
-        p.item = whole;
-        p.w = a.items[p.item];
+        p.w = a.items[whole];
         p.t0 = 0;
         p.t1 = (p.w.kv_end + kKeysPerTile - 1) / kKeysPerTile;
-        p.c_first = 0; p.n_parts = 1; p.part = 0;
+        p.slot = -1;
         return true;
     }
 };
-// partial-result slot of part `part` of an item whose first part is held by block c_first: a block holds at
-// most one part > 0 (the piece its run starts with) and at most one part 0 of a cut item (the piece it ends with)
-__host__ __device__ __forceinline__ int part_slot(int c_first, int part) { return 2 * (c_first + part) + (part == 0 ? 1 : 0); }
 
 template <int HD>
 struct AttnSmem {
@@ -718,13 +719,13 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 const float w_own = m_ref == -INFINITY ? 0.f : fast_exp2((m_ref - m_all) * a.scale_log2);
                 const float w_oth = m_oth == -INFINITY ? 0.f : fast_exp2((m_oth - m_all) * a.scale_log2);
                 const float l_all = fmaf(l_run, w_own, l_oth * w_oth);
-                const bool whole = !kRuns || pc.n_parts == 1;
+                const bool whole = !kRuns || pc.slot < 0;
                 const float inv = whole ? 1.f / l_all : 1.f;
                 // part of a cut item: the merged, unnormalised rows go to the part's slot as rows of group 0
                 float *po = a.part_o, *pml = a.part_ml;
                 if (kRuns && !whole) {
-                    po += (size_t)part_slot(pc.c_first, pc.part) * HD * 256 + row;
-                    pml += (size_t)part_slot(pc.c_first, pc.part) * 512 + row;
+                    po += (size_t)pc.slot * HD * 256 + row;
+                    pml += (size_t)pc.slot * 512 + row;
                 }
 #pragma unroll 1
                 for (int c = g * (HD / 2); c < (g + 1) * (HD / 2); c += 32) {
@@ -754,7 +755,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 // P V: the other group must have read both before this group goes on
                 if (!tc::mbar_wait(merge_done, (n_merge - 1) & 1, abort_flag)) { ok = false; break; }
                 tc::tc_fence_after();
-            } else if (!kRuns || pc.n_parts == 1) {
+            } else if (!kRuns || pc.slot < 0) {
                 const float inv = 1.f / l_run;
 #pragma unroll 1
                 for (int c = 0; c < HD; c += 32) {
@@ -770,8 +771,8 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             } else {
                 // part of a cut item: unnormalised rows, exponent references and sums go to the part's slot
                 const int grow = g * 128 + row;
-                float *po = a.part_o + (size_t)part_slot(pc.c_first, pc.part) * HD * 256 + grow;
-                float *pml = a.part_ml + (size_t)part_slot(pc.c_first, pc.part) * 512 + grow;
+                float *po = a.part_o + (size_t)pc.slot * HD * 256 + grow;
+                float *pml = a.part_ml + (size_t)pc.slot * 512 + grow;
 #pragma unroll 1
                 for (int c = 0; c < HD; c += 32) {
                     uint32_t v[32];
