@@ -517,12 +517,17 @@ int launch_few_cluster(alora_ctx *ctx, const void *x, const void *W, const RankM
 static bool few_row_linear(const alora_ctx *ctx, int T, int N, int K) {
     return few_cluster_route(ctx, T, 0, N, K, false, N, 0) || skinny_route(ctx, T, N, K, false, N, 0);
 }
-// Whether the q/k/v projection takes the one-launch route: with more than 128 rows only in a context without adapters on
-// the MLP block (those need the (row tile, adapter) pairs, which that route's metadata step does not build).
-static bool project_few_cluster(const alora_ctx *ctx, int layer, int T, int R) {
-    const Dims &d = ctx->d;
+// More than 128 rows take the one-launch route only in a context without adapters on the MLP block: those need the (row tile,
+// adapter) pairs, which that route's metadata step does not build, and a call in which none of them applies has to take the
+// route of the others (rows without a delta keep their bits).
+static bool few_cluster_rows(const alora_ctx *ctx, int T) {
     if (T > kFewRowMax)
         for (int n : ctx->mlp_n_adapters) if (n > 0) return false;
+    return true;
+}
+static bool project_few_cluster(const alora_ctx *ctx, int layer, int T, int R) {
+    const Dims &d = ctx->d;
+    if (!few_cluster_rows(ctx, T)) return false;
     return few_cluster_route(ctx, T, R, d.N, d.H, ctx->layer_has_adapter[layer] != 0, d.Nq, d.Nkv);
 }
 
@@ -627,7 +632,7 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
     if (K % 8 != 0 || N % 8 != 0) return -1;
     if (delta != nullptr && (!linear_takes_delta(ctx, T, K, N) || (N / delta->n_blk) % 256 != 0)) return -1;
     ProfScope prof(ctx, KK_LINEAR, s);
-    if (delta == nullptr && few_cluster_route(ctx, T, 0, N, K, false, N, 0))
+    if (delta == nullptr && few_cluster_rows(ctx, T) && few_cluster_route(ctx, T, 0, N, K, false, N, 0))
         return launch_few_cluster(ctx, x, W, nullptr, nullptr, nullptr, T, 0, K, N, N, 0, y, residual, nullptr, 0, s);
     if (skinny_route(ctx, T, N, K, false, N, 0)) {
         CUtensorMap tmW256;
