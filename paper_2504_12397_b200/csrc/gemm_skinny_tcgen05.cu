@@ -15,7 +15,7 @@
 // Kernel 2 (CUDA cores): per output element the K-slice partials are added in slice order; a row with an applied
 //   adapter k adds s B_k t_k (t_k = the slice partials of ITS adapter's shrink, added in slice order, fp32); rows
 //   without one add nothing, so they go through exactly the arithmetic of a base-only call (Prop. 1: gated-off rows
-//   are bit-identical).  Optional residual add; bf16 store; the k / v columns also go to the row's cache slot.
+//   are bit-identical).  bf16 store; the k / v columns also go to the row's cache slot.
 // No atomics in the arithmetic, fixed summation orders: results are run-to-run deterministic.  The route is chosen
 // by the row count alone, never by the mode or the adapters.
 #include <algorithm>
@@ -266,14 +266,13 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
     }
 }
 
-// ---- kernel 2: add the slice partials, the delta of gated rows, the residual; store; append k / v ----
+// ---- kernel 2: add the slice partials, the delta of gated rows; store; append k / v ----
 struct SkinnyFinArgs {
     int T, N, n_tiles, ksplit, p_cap;
     const float *part, *t_part;
     const FewRowMeta *meta;           // nullptr: no adapters in this launch
     const __nv_bfloat16 *b_all;       // the layer's B rows of all adapters, [adapter][N][64]
     int Nq, Nkv;
-    const __nv_bfloat16 *residual;
     __nv_bfloat16 *out;
     int ldo;
     __nv_bfloat16 *kv_pool;
@@ -431,16 +430,6 @@ skinny_finish_kernel(const SkinnyFinArgs a) {
         }
     }
     if (!mine) return;
-    if (a.residual) {
-        const uint4 rv4 = *reinterpret_cast<const uint4 *>(a.residual + (size_t)row * a.ldo + col);
-        const uint32_t rw[4] = {rv4.x, rv4.y, rv4.z, rv4.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const __nv_bfloat162 b2 = *reinterpret_cast<const __nv_bfloat162 *>(&rw[e]);
-            f[2 * e] += __low2float(b2);
-            f[2 * e + 1] += __high2float(b2);
-        }
-    }
     uint4 o;
     o.x = tc::pack_bf16(f[0], f[1]); o.y = tc::pack_bf16(f[2], f[3]);
     o.z = tc::pack_bf16(f[4], f[5]); o.w = tc::pack_bf16(f[6], f[7]);
@@ -485,7 +474,7 @@ bool skinny_route(const alora_ctx *ctx, int T, int N, int K, bool lora, int Nq, 
 // 16 rows) and `layer`, whose adapter facts are used, or nullptr for a plain dense projection.  Returns kernels launched, or -1.
 int launch_skinny_tc(alora_ctx *ctx, const void *x, const CUtensorMap &tmW, const CUtensorMap *tmA16,
                      const AdapterDev *adapters, const void *b_all, int T, int K, int N, int Nq, int Nkv, void *out,
-                     const void *residual, void *kv_pool, int num_pages, int layer, cudaStream_t s) {
+                     void *kv_pool, int num_pages, int layer, cudaStream_t s) {
     static bool attr_set[64] = {};
     const int dev = ctx->cfg.device;
     int extra_launches = 0;
@@ -534,7 +523,7 @@ int launch_skinny_tc(alora_ctx *ctx, const void *x, const CUtensorMap &tmW, cons
     f.T = T; f.N = N; f.n_tiles = n_tiles; f.ksplit = ksplit; f.p_cap = p_cap;
     f.part = ctx->d_skinny_part; f.t_part = ctx->d_skinny_t;
     f.meta = a.meta; f.b_all = (const __nv_bfloat16 *)b_all;
-    f.Nq = Nq; f.Nkv = Nkv; f.residual = (const __nv_bfloat16 *)residual; f.out = (__nv_bfloat16 *)out; f.ldo = N;
+    f.Nq = Nq; f.Nkv = Nkv; f.out = (__nv_bfloat16 *)out; f.ldo = N;
     f.status = ctx->d_status;
     if (kv_pool != nullptr) {
         int shift = 0;

@@ -503,20 +503,17 @@ bool shrink_apart(const alora_ctx *ctx, int T, int R, int items) {
     return rounds <= 2 && (items + n + G - 1) / G > rounds && n * 8 <= 4 * G;
 }
 
-bool skinny_route(const alora_ctx *ctx, int T, int N, int K, bool lora, int Nq, int Nkv);   // gemm_skinny_tcgen05.cu
+bool skinny_route(const alora_ctx *ctx, int T, int N, int K, bool lora, int Nq, int Nkv);   // gemm_skinny_tcgen05.cu: at most 128
+                                  // rows, more adapters than the one-launch kernel takes
 int launch_skinny_tc(alora_ctx *ctx, const void *x, const CUtensorMap &tmW, const CUtensorMap *tmA16,
                      const AdapterDev *adapters, const void *b_all, int T, int K, int N, int Nq, int Nkv, void *out,
-                     const void *residual, void *kv_pool, int num_pages, int layer, cudaStream_t s);
+                     void *kv_pool, int num_pages, int layer, cudaStream_t s);
 
 bool few_cluster_route(const alora_ctx *ctx, int T, int R, int N, int K, bool lora, int Nq, int Nkv);   // gemm_few_cluster.cu
 int launch_few_cluster(alora_ctx *ctx, const void *x, const void *W, const RankMaps *tmA, const FewRowMeta *meta,
                        const void *b_all, int T, int R, int K, int N, int Nq, int Nkv, void *out, const void *residual, void *kv_pool,
                        int num_pages, cudaStream_t s);
 
-// The weight-streaming routes for few rows: in one launch, or (at most 128 rows, more adapters than that takes) in two.
-static bool few_row_linear(const alora_ctx *ctx, int T, int N, int K) {
-    return few_cluster_route(ctx, T, 0, N, K, false, N, 0) || skinny_route(ctx, T, N, K, false, N, 0);
-}
 // More than 128 rows take the one-launch route only in a context without adapters on the MLP block: those need the (row tile,
 // adapter) pairs, which that route's metadata step does not build, and a call in which none of them applies has to take the
 // route of the others (rows without a delta keep their bits).
@@ -555,7 +552,7 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
         const TcLayerMaps &lm = ctx->tc_maps[layer];
         const AdapterDev *ads = ctx->d_adapters + (size_t)layer * ctx->cfg.max_adapters;
         return launch_skinny_tc(ctx, hidden, lm.wqkv[1], have_adapters ? &lm.a_rank.box[0] : nullptr,
-                                have_adapters ? ads : nullptr, ctx->tc_b_all[layer], T, d.H, d.N, d.Nq, d.Nkv, qkv, nullptr,
+                                have_adapters ? ads : nullptr, ctx->tc_b_all[layer], T, d.H, d.N, d.Nq, d.Nkv, qkv,
                                 kv_pool, num_pages, layer, s);
     }
     if (ctx->tc_maps[layer].pair_ok) {   // many rows: two row tiles per block, 192-wide column tiles
@@ -621,7 +618,7 @@ bool build_pair_maps(alora_ctx *ctx, int layer);                 // gemm_pair_tc
 
 // Whether launch_linear_tc can add a gated delta to a projection of this shape (not on the few-row route).
 bool linear_takes_delta(const alora_ctx *ctx, int T, int K, int N) {
-    return T > kFewRowMax || !few_row_linear(ctx, T, N, K);
+    return T > kFewRowMax || !few_cluster_route(ctx, T, 0, N, K, false, N, 0);
 }
 
 // Dense projection y = x W^T (+ residual) for o_proj and the MLP matrices, with the gated delta of the MLP adapters where
@@ -634,11 +631,6 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
     ProfScope prof(ctx, KK_LINEAR, s);
     if (delta == nullptr && few_cluster_rows(ctx, T) && few_cluster_route(ctx, T, 0, N, K, false, N, 0))
         return launch_few_cluster(ctx, x, W, nullptr, nullptr, nullptr, T, 0, K, N, N, 0, y, residual, nullptr, 0, s);
-    if (skinny_route(ctx, T, N, K, false, N, 0)) {
-        CUtensorMap tmW256;
-        if (!make_tensor_map_bf16(&tmW256, W, N, K, K, 256)) return -1;
-        return launch_skinny_tc(ctx, x, tmW256, nullptr, nullptr, nullptr, T, K, N, N, 0, y, residual, nullptr, 0, 0, s);
-    }
     {
         const int r = launch_linear256_tc(ctx, x, W, T, K, N, y, residual, delta, s);   // many rows: 256 x 256 tiles
         if (r != 0) return r;
