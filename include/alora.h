@@ -129,7 +129,8 @@ alora_status alora_set_layer_weights(alora_ctx *ctx, int layer, const void *d_wq
  * blk in {q, k, v} (Eq. 4 / Eq. 5).  d_Aq/d_Ak/d_Av are [rank][H], d_Bq is [Nq][rank], d_Bk and
  * d_Bv are [Nkv][rank].  The matrices are COPIED into context-owned, rank-padded storage on the
  * given stream; the caller's buffers may be released once that stream has passed this point.
- * 1 <= rank <= max_rank.
+ * 1 <= rank <= max_rank.  The values have to be finite: on the row-tile routes a row that does not use an
+ * adapter of its tile adds zero times that adapter's B.
  */
 alora_status alora_register_adapter(alora_ctx *ctx, int adapter_id, int layer, int rank, float scale,
                                     const void *d_Aq, const void *d_Bq, const void *d_Ak,
@@ -392,9 +393,9 @@ alora_status alora_selftest_claim_order(int grid, int n_shrink, int n_row_tiles,
  * alora_profile_enable(ctx, 1) clears what was accumulated and starts, (ctx, 0) stops.
  * alora_profile_read synchronises the device and adds up, per family, the elapsed milliseconds and
  * the number of bracketed launch groups; both arrays have ALORA_PROFILE_KINDS entries.
- * Families: 0 batch metadata, 1 rank-r shrink (t = A x) when it is a launch of its own, or the per-row
- * low-rank delta of small batches, 2 q/k/v projection (on the bf16 layer paths it also appends the new k / v rows
- * to the cache), 3 KV append as a launch of its own (alora_kv_append, fp32 layers), 4 attention on the tensor-core
+ * Families: 0 batch metadata, 1 rank-r shrink (t = A x) when it is a launch of its own, 2 q/k/v projection (on the
+ * layer paths it also appends the new k / v rows to the cache), 3 KV append as a launch of its own
+ * (alora_kv_append), 4 attention on the tensor-core
  * kernel (with the merge of cut work items) and the fp32 kernel, 5 attention on the few-row split-KV kernel (decode
  * steps, shortest suffixes, prefix groups), 6 other dense projections (o_proj, MLP), 7 norm / activation
  * glue.
