@@ -200,6 +200,7 @@ struct alora_ctx {
     int few_tiles = 1;
     const alora::BatchArgs *pending_attn_meta = nullptr;   // run_layer: attention lists still to be built for this batch
     int skinny_max_items = 0, skinny_p_cap = 0;
+    bool x_before_facts = false;   // the projection's input was complete before the batch-facts launch that precedes it
     void *d_qkv = nullptr;        // [max_tokens][N]
     void *d_act[4] = {nullptr, nullptr, nullptr, nullptr};  // stack activations
     double *d_rope_inv_freq = nullptr;   // [hd / 2] theta^(-2i/hd), only with a rotary base configured

@@ -512,7 +512,7 @@ int launch_skinny_tc(alora_ctx *ctx, const void *x, const CUtensorMap &tmW, cons
 bool few_cluster_route(const alora_ctx *ctx, int T, int R, int N, int K, bool lora, int Nq, int Nkv);   // gemm_few_cluster.cu
 int launch_few_cluster(alora_ctx *ctx, const void *x, const void *W, const RankMaps *tmA, const FewRowMeta *meta,
                        const void *b_all, int T, int R, int K, int N, int Nq, int Nkv, void *out, const void *residual, void *kv_pool,
-                       int num_pages, cudaStream_t s);
+                       int num_pages, bool x_early, cudaStream_t s);
 
 // More than 128 rows take the one-launch route only in a context without adapters on the MLP block: those need the (row tile,
 // adapter) pairs, which that route's metadata step does not build, and a call in which none of them applies has to take the
@@ -545,7 +545,7 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
         ProfScope prof(ctx, KK_PROJECT, s);
         return launch_few_cluster(ctx, hidden, ctx->layers[layer].wqkv, &ctx->tc_maps[layer].a_rank,
                                   have_adapters ? ctx->d_skinny_meta + (size_t)layer * ctx->few_tiles : nullptr, ctx->tc_b_all[layer], T, R,
-                                  d.H, d.N, d.Nq, d.Nkv, qkv, nullptr, kv_pool, num_pages, s);
+                                  d.H, d.N, d.Nq, d.Nkv, qkv, nullptr, kv_pool, num_pages, ctx->x_before_facts, s);
     }
     if (skinny_route(ctx, T, d.N, d.H, have_adapters, d.Nq, d.Nkv)) {
         ProfScope prof(ctx, KK_PROJECT, s);
@@ -630,7 +630,7 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
     if (delta != nullptr && (!linear_takes_delta(ctx, T, K, N) || (N / delta->n_blk) % 256 != 0)) return -1;
     ProfScope prof(ctx, KK_LINEAR, s);
     if (delta == nullptr && few_cluster_rows(ctx, T) && few_cluster_route(ctx, T, 0, N, K, false, N, 0))
-        return launch_few_cluster(ctx, x, W, nullptr, nullptr, nullptr, T, 0, K, N, N, 0, y, residual, nullptr, 0, s);
+        return launch_few_cluster(ctx, x, W, nullptr, nullptr, nullptr, T, 0, K, N, N, 0, y, residual, nullptr, 0, false, s);
     {
         const int r = launch_linear256_tc(ctx, x, W, T, K, N, y, residual, delta, s);   // many rows: 256 x 256 tiles
         if (r != 0) return r;

@@ -344,6 +344,35 @@ def test_projection_few_row_route_row_boxes_and_adapter_limits(oracle64, T, n_ad
     _check_projection(oracle64, MID, w, ads, b)
 
 
+@pytest.mark.parametrize("T,n_ad,rank", [(1, 1, 64), (33, 3, 24), (128, 16, 16), (300, 0, 8)])
+def test_few_row_layer_call_equals_its_sub_steps(T, n_ad, rank):
+    """In a layer call W x starts before the batch's adapter facts are there and A x takes a second pass over x; the
+    projection alone does both in one pass.  The new K / V rows and the attention rows have to be the same bits."""
+    rng = np.random.default_rng(400 + T)
+    w = wl.make_wqkv(MID, rng)
+    ads = _boosted_adapters(MID, rng, tuple((rank, 1.0) for _ in range(n_ad)))
+    P = [int(x) for x in rng.integers(0, 300, T)]
+    ids = [(i * 7) % (n_ad + 1) - 1 if T > 1 else 0 for i in range(T)]
+    b = wl.make_batch(MID, P, [1] * T, ids, rng, activation_offsets=[p + (i % 6 == 1) for i, p in enumerate(P)])
+    g = hp.GpuLayers(MID, [dict(wqkv=w)], [ads], 512, 512)
+    try:
+        fill = wl.random_kv_pool(MID, b.num_pages, rng)
+        d = hp.DevBatch(b, MID.dtype)
+        pool1, pool2 = g.new_pool(b.num_pages, fill), g.new_pool(b.num_pages, fill)
+        out1, out2, qkv = g.empty(b.T, MID.Nq), g.empty(b.T, MID.Nq), g.empty(b.T, MID.N)
+        ab.alora_prefill_layer(g.ctx, 0, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, pool1, d.bt,
+                               d.max_blocks, b.num_pages, d.T, d.R, out1)
+        ab.alora_project_qkv(g.ctx, 0, ab.MODE_ALORA, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens,
+                             d.T, d.R, qkv)
+        ab.alora_kv_append(g.ctx, qkv, d.positions, d.qsl, d.seq_lens, d.bt, d.max_blocks, b.num_pages, d.T, d.R, pool2)
+        ab.alora_attend(g.ctx, qkv, d.positions, d.qsl, d.seq_lens, pool2, d.bt, d.max_blocks, b.num_pages, d.T, d.R, out2)
+        assert g.status() == 0
+        assert np.array_equal(hp.to_host(pool1).view(np.uint32), hp.to_host(pool2).view(np.uint32))
+        assert np.array_equal(hp.to_host(out1).view(np.uint32), hp.to_host(out2).view(np.uint32))
+    finally:
+        g.close()
+
+
 def test_projection_few_row_route_short_suffixes_one_adapter(oracle64):
     """8 requests x 16 new tokens (128 rows), one adapter, gates opening inside the chunk."""
     rng = np.random.default_rng(49)
