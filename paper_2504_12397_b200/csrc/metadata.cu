@@ -645,9 +645,9 @@ __device__ __forceinline__ void metadata_few_row(int k_mine, const AdapterDev &a
     if ((int)threadIdx.x < kFewRowMax) meta->slot_of_row[threadIdx.x] = slot;
 }
 
-// The metadata step.  Phase bit 0: every block handles 256 tokens (request, applied adapter, slot); block 0 then
+// The metadata step.  Phase bit 0: every block handles 256 tokens (request, applied adapter, slot); one block more
 // builds the projection's (row tile, adapter) pairs.  Phase bit 1: the two attention
-// work lists, one block each (their serial parts are O(R)).  Both phases in one launch: blocks 0, 1, 2 take one
+// work lists, one block each (their serial parts are O(R)).  Both phases in one launch: the last block, 1 and 2 take one
 // builder each.  The attention phase alone is launched as a programmatic dependent of the projection kernel, beside
 // which it runs (it reads nothing that kernel writes); its blocks wait for that kernel before they exit, so that
 // whatever follows in the stream still sees the projection complete.
@@ -683,14 +683,14 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
         if (adapter_ids) adapter_ids = s_ids;
         if (a_req) a_req = s_areq;
     }
-    if (phases & kMetaProjection)
+    if ((phases & kMetaProjection) && tok < T)
         metadata_token(tok, my_pos, a_req, adapter_ids, qsl, seq_lens, block_tables,
                        max_blocks, num_pages, page_size, max_adapters, T, R, mode, token_req, row_adapter, slot_map, status, [](int) {});
-    // The three list builders are independent of one another: blocks 0, 1 and 2 take one each (a launch of both
-    // phases has at least three blocks, one of the attention phase alone two).
+    // The three list builders are independent of one another: the last block, 1 and 2 take one each (a launch of both
+    // phases has at least four blocks, one of the attention phase alone two).
     const int nb = (int)gridDim.x;
     const bool proj = (phases & kMetaProjection) != 0, attn = (phases & kMetaAttention) != 0;
-    const int b_pairs = proj && pairs != nullptr ? 0 : -1;
+    const int b_pairs = proj && pairs != nullptr ? nb - 1 : -1;   // (a block without tokens of its own: the projection waits for it)
     const int b_attn = !attn ? -1 : (proj ? (nb > 1 ? 1 : 0) : 0);
     const int b_split = !attn ? -1 : (proj ? (nb > 2 ? 2 : 0) : (nb > 1 ? 1 : 0));
     // the attention phase alone: block 0 builds the tensor-core kernel's list, all the others share the few-row list
@@ -778,7 +778,7 @@ int launch_metadata(alora_ctx *ctx, const BatchArgs &b, cudaStream_t s, int phas
     // (attention phase alone: one block for the tensor-core list, kSplitBuilders for the few-row list; they need the
     // shared-memory scratch, i.e. batches of at most 511 requests, else one block builds it in the global scratch)
     constexpr int kSplitBuilders = 8;
-    const int grid = attn_only ? (14 * b.R + 5 <= kMetaSmemInts ? 1 + kSplitBuilders : 2) : std::max((phases & kMetaAttention) ? 3 : 1, (b.T + threads - 1) / threads);
+    const int grid = attn_only ? (14 * b.R + 5 <= kMetaSmemInts ? 1 + kSplitBuilders : 2) : 1 + std::max((phases & kMetaAttention) ? 3 : 1, (b.T + threads - 1) / threads);
     const AdapterDev *ads = b.layer >= 0 ? ctx->d_adapters + (size_t)b.layer * ctx->cfg.max_adapters : nullptr;
     if (phases == kMetaProjection && b.few_row) {
         FewRowMeta *few = ads != nullptr ? ctx->d_skinny_meta + (size_t)b.layer * ctx->few_tiles : nullptr;
