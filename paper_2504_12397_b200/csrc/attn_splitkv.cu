@@ -202,6 +202,9 @@ attn_splitkv_kernel(const __grid_constant__ CUtensorMap tmKV, const SplitArgs a)
     __syncthreads();
     tc::grid_dep_launch();
     tc::grid_dep_wait();   // work list, q/k/v rows and the cache rows of the new tokens come from earlier kernels
+    // (the producer fetches its first item beside the length of the list, in which it may not be)
+    AttnSplitWork first{};
+    if (warp == kSkConsumerWarps) first = a.items[blockIdx.x];
     const int n_items = *a.n_items;
 
     if (warp == kSkConsumerWarps) {
@@ -231,7 +234,7 @@ attn_splitkv_kernel(const __grid_constant__ CUtensorMap tmKV, const SplitArgs a)
             ok = __shfl_sync(0xffffffffu, ok, 0);
             ++n_it;
             if (!ok || it < 0) break;
-            const AttnSplitWork w = a.items[it];
+            const AttnSplitWork w = it == (int)blockIdx.x ? first : a.items[it];
             const int n_st = (w.kv_end - w.kv_start + kSkStageKeys - 1) / kSkStageKeys, claim_at = max(0, n_st - 3);
             if (lane == 0 && n_st <= 0) it_next = (int)gridDim.x + atomicAdd(a.work_counter, 1);   // (an empty share of the own keys)
             // Window of the request's block-table row: lane l holds entry win0 + l (win0 a multiple of 32; 32 entries
