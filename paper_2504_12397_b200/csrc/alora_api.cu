@@ -677,11 +677,12 @@ alora_status alora_forward_stack(alora_ctx *ctx, int mode, const void *d_hidden_
     } while (0)
     // The batch's lists depend on the batch alone: the first layer builds them for all, with the few-row route's adapter
     // facts of all layers.  (They were rebuilt by every layer: 63 of 240 us of a layer's decode step of 40 requests in
-    // prefix groups.)  Only where the layers' projections take different routes does each build its own.
+    // prefix groups.)  Only the projection's facts are built by each layer where the layers' projections take different routes.
     int n_few = 0;
     for (int l = 0; l < ctx->cfg.n_layers; ++l) n_few += project_is_few_row(ctx, l, T, R) ? 1 : 0;
     const bool one_route = n_few == 0 || n_few == ctx->cfg.n_layers;
     b.n_layers = one_route ? ctx->cfg.n_layers : 1;
+    b.lists_shared = ctx->cfg.n_layers > 1;   // (whatever the projections' routes)
     for (int l = 0; l < ctx->cfg.n_layers; ++l) {
         const LayerWeights &lw = ctx->layers[l];
         if (l > 0) b.facts_ready = kMetaAttention | (one_route ? kMetaProjection : 0);

@@ -624,7 +624,8 @@ int launch_attend_splitkv(alora_ctx *ctx, const void *qkv, const BatchArgs &b, c
     a.max_blocks = b.max_blocks; a.num_pages = b.num_pages; a.Hkv = d.Hkv; a.G = d.G; a.page_size = d.page;
     a.box_rows = box_rows; a.N = d.N; a.Nq = d.Nq; a.scale_log2 = d.softmax_scale * 1.4426950408889634f;
     a.qkv = (const __nv_bfloat16 *)qkv; a.out = (__nv_bfloat16 *)out; a.part_o = ctx->d_part_o;
-    a.part_ml = ctx->d_part_ml; a.work_counter = ctx->d_counts + 4; a.blocks_done = b.n_layers > 1 || b.facts_ready ? ctx->d_counts + 12 : nullptr; a.group_done = ctx->d_group_done;
+    a.part_ml = ctx->d_part_ml; a.work_counter = ctx->d_counts + 4; a.group_done = ctx->d_group_done;
+    a.blocks_done = b.lists_shared ? ctx->d_counts + 12 : nullptr;
     a.status = ctx->d_status;
     static bool attr_set[2][64] = {};
     const int dev = ctx->cfg.device, hi = d.hd == 128;

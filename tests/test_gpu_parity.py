@@ -776,3 +776,38 @@ def test_decode_steps_through_the_stack_match_the_prefill_rows(oracle64):
         hp.assert_close(hp.to_host(hout), x[keep], 2e-2, "prefilled rows")
     finally:
         g.close()
+
+
+def test_stack_layers_on_different_projection_routes_share_the_attention_list(oracle64):
+    """Three decoder layers of which only the first has adapters, more of them than the few-row projection takes (5 x 64 rank
+    columns): its q/k/v go through the row tiles, those of the other layers through the few-row kernel, while the attention
+    list of the 200 decode rows (800 streams, more than there are blocks, the long ones cut into key ranges) is built once.
+    Every layer has to see all of it."""
+    shape = wl.LayerShape(hidden=512, n_q_heads=8, n_kv_heads=4, head_dim=64, page_size=16, dtype="bf16", intermediate=512)
+    rng = np.random.default_rng(61)
+    n, R = 3, 200
+    layers = [wl.make_stack_weights(shape, rng) for _ in range(n)]
+    ads = [_boosted_adapters(shape, rng, [(64, 1.0)] * 5), [], []]
+    P = [int(p) for p in rng.integers(1, 300, R)]
+    P[7], P[150] = 2900, 2111
+    b = wl.make_batch(shape, P, [1] * R, [-1] * R, rng, shuffle_pages=True)   # (the route is chosen by what is registered)
+    pools_np = [wl.random_kv_pool(shape, b.num_pages, rng) for _ in range(n)]
+    g = hp.GpuLayers(shape, layers, ads, R, R)
+    try:
+        d = hp.DevBatch(b, shape.dtype)
+        hout = g.empty(R, shape.hidden)
+        for _ in range(2):   # (a second call finds what the first one left)
+            pools = [g.new_pool(b.num_pages, fill=p) for p in pools_np]
+            ab.alora_decode_stack(g.ctx, d.hidden, d.positions, d.a_req, d.ids, d.seq_lens, pools, d.bt, d.max_blocks,
+                                  b.num_pages, R, hout)
+            assert g.status() == 0
+            x = b.hidden.astype(np.float64)
+            for l in range(n):
+                kv = [oracle64.paged_gather(pools_np[l], b.block_tables[r], P[r], shape.n_kv_heads, shape.page_size,
+                                            shape.head_dim) for r in range(R)]
+                x, _ = oracle64.decoder_layer(x, layers[l], shape.Nq, shape.Nkv, shape.n_q_heads, shape.n_kv_heads,
+                                              shape.head_dim, 1e-5, b.positions, b.query_start_loc, b.activation_offsets,
+                                              b.adapter_ids, [], [k for k, _ in kv], [v for _, v in kv])
+            hp.assert_close(hp.to_host(hout), x, 2e-2, "decode step through layers on different routes", block=shape.head_dim)
+    finally:
+        g.close()
