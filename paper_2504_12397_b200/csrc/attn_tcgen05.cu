@@ -224,10 +224,12 @@ __device__ __forceinline__ void add2(float &d0, float &d1, float a0, float a1) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(D), "l"(A));
     asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(d));
 }
-// 2^x of two x <= 0 on the FMA pipe: x = n + f with n the nearest integer, a cubic for 2^f on [-0.5, 0.5] (relative
-// error 7.5e-5, below the bf16 rounding of the probabilities), n added to the exponent field; two values per instruction
+// 2^x of two x on the FMA pipe: x = n + f with n the nearest integer, a cubic for 2^f on [-0.5, 0.5] (relative
+// error 7.5e-5, below the bf16 rounding of the probabilities), n added to the exponent field; two values per instruction.
+// x is not known to be <= 0 here: beyond 126 (and for a NaN) the result is 2^126, which no sum in the safe range can hold;
+// without that limit the exponent field ran over into the sign.
 __device__ __forceinline__ void exp2_poly2(float &p0, float &p1, float x0, float x1) {
-    x0 = fmaxf(x0, -125.f); x1 = fmaxf(x1, -125.f);
+    x0 = fmaxf(fminf(x0, 126.f), -125.f); x1 = fmaxf(fminf(x1, 126.f), -125.f);
     uint64_t x, xr, f, p, k;
     asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(x0), "f"(x1));
     auto pair = [](float c) { uint64_t r; asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(c)); return r; };

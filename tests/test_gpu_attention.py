@@ -100,3 +100,58 @@ def test_shapes_group_sizes_and_page_sizes(oracle64, hq, hkv, hd, page):
     S = [1, 5, 16, 150, 2]
     err, _, _ = _attend_case(oracle64, shape, P, S, seed=500 + hq + hd + page)
     assert err <= 2e-2
+
+
+def _attend_values(shape, b, pool_np, qkv_np):
+    """Append + attend on the GPU with the given cache and q/k/v rows; the output rows."""
+    import torch
+    g = hp.GpuLayers(shape, [dict(wqkv=np.zeros((shape.N, shape.hidden), np.float32))], [[]], b.T, b.R)
+    try:
+        pool, qkv, d = hp.to_dev(pool_np, "bf16"), hp.to_dev(qkv_np, "bf16"), hp.DevBatch(b, "bf16")
+        out = torch.full((b.T, shape.Nq), float("nan"), dtype=torch.bfloat16, device="cuda")
+        ab.alora_kv_append(g.ctx, qkv, d.positions, d.qsl, d.seq_lens, d.bt, d.max_blocks, b.num_pages, b.T, b.R, pool)
+        ab.alora_attend(g.ctx, qkv, d.positions, d.qsl, d.seq_lens, pool, d.bt, d.max_blocks, b.num_pages, b.T, b.R, out)
+        assert g.status() == 0
+        return hp.to_host(out)
+    finally:
+        g.close()
+
+
+def _oracle_values(oracle, shape, b, pool_np, qkv_np):
+    Ks, Vs, kvl = [], [], [0]
+    for r in range(b.R):
+        K0, V0 = oracle.paged_gather(pool_np, b.block_tables[r], int(b.prefix_lens[r]), shape.n_kv_heads, shape.page_size,
+                                     shape.head_dim)
+        rows = slice(b.query_start_loc[r], b.query_start_loc[r + 1])
+        Ks.append(np.concatenate([K0, qkv_np[rows, shape.Nq:shape.Nq + shape.Nkv]]))
+        Vs.append(np.concatenate([V0, qkv_np[rows, shape.Nq + shape.Nkv:]]))
+        kvl.append(kvl[-1] + len(Ks[-1]))
+    return oracle.attention(qkv_np[:, :shape.Nq], np.concatenate(Ks), np.concatenate(Vs), kvl, b.positions, b.query_start_loc,
+                            shape.n_q_heads, shape.n_kv_heads, shape.head_dim)[0]
+
+
+def _write_keys(shape, b, pool_np, r, first, keys):
+    """Puts `keys` [n, head_dim] (for every KV head) into request r's cached positions first, first + 1, ..."""
+    for i, k in enumerate(keys):
+        pool_np[b.block_tables[r, (first + i) // shape.page_size], 0, :, (first + i) % shape.page_size] = k
+
+
+@pytest.mark.parametrize("page", [8, 16, 64])
+@pytest.mark.parametrize("S", [20, 40])
+@pytest.mark.parametrize("nats", [60, 100, 200])
+def test_one_late_key_far_above_the_reference(oracle64, page, S, nats):
+    """A key in the middle of the context whose score lies `nats` above all others, at each of 32 neighbouring positions in
+    turn (one request each): the softmax works on a running reference, and whatever unit takes this key's exponential, the
+    row has to become that key's value."""
+    shape = wl.LayerShape(hidden=256, n_q_heads=8, n_kv_heads=2, head_dim=128, page_size=page, dtype="bf16")
+    rng = np.random.default_rng(700 + page + S + nats)
+    R = 32
+    b = wl.make_batch(shape, [1000] * R, [S] * R, [-1] * R, rng, shuffle_pages=True, with_hidden=False)
+    pool = wl.random_kv_pool(shape, b.num_pages, rng)
+    qkv = wl.bf16_round(rng.standard_normal((b.T, shape.N), dtype=np.float32))
+    u = rng.choice([-1.0, 1.0], shape.head_dim).astype(np.float32)
+    qkv[:, :shape.Nq] = np.tile(u, shape.n_q_heads)
+    for r in range(R):
+        _write_keys(shape, b, pool, r, 640 + r, wl.bf16_round(u * np.float32(nats / shape.head_dim ** 0.5))[None])
+    got, want = _attend_values(shape, b, pool, qkv), _oracle_values(oracle64, shape, b, pool, qkv)
+    hp.assert_close(got, want, 2e-2, f"a key {nats} nats above the others", block=shape.head_dim)
