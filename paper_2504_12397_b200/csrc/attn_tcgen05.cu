@@ -572,8 +572,9 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 if (lane == 0) tc::mbar_arrive(s_free(g));
                 const bool masked = __any_sync(0xffffffffu, tbase + kKeysPerTile - 1 > pos);   // crosses some row's causal limit
                 uint32_t pk[kHalfKeys / 2];   // probabilities (bf16 pairs)
-                // probabilities of the scores against the current reference; returns their sum in fp32
-                auto exponentials = [&](auto poly) {
+                // probabilities of the scores against the current reference; returns their sum in fp32.  fast: one pair in
+                // eight on the FMA pipe; else only in the rows with `poly`, of which there are none unless `mixed`
+                auto exponentials = [&](auto fast, bool mixed, bool poly) {
                     // (a piece that starts at an item's last tile can hold rows that see none of its keys so far)
                     const float mb = m_ref == -INFINITY ? 0.f : m_ref * a.scale_log2;
                     float l0 = 0.f, l1 = 0.f;
@@ -581,8 +582,17 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     for (int e = 0; e < kHalfKeys; e += 2) {
                         float x0, x1, p0, p1;
                         fma2(x0, x1, __uint_as_float(sv[e]), __uint_as_float(sv[e + 1]), a.scale_log2, -mb);
-                        if (decltype(poly)::value && ((kPolyPairs >> ((e >> 1) & 7)) & 1)) exp2_poly2(p0, p1, x0, x1);
-                        else { p0 = fast_exp2(x0); p1 = fast_exp2(x1); }
+                        const bool poly_pair = (kPolyPairs >> ((e >> 1) & 7)) & 1;
+                        if (decltype(fast)::value && poly_pair) {
+                            exp2_poly2(p0, p1, x0, x1);
+                        } else {
+                            p0 = fast_exp2(x0); p1 = fast_exp2(x1);
+                            if (!decltype(fast)::value && poly_pair && mixed) {
+                                float q0, q1;
+                                exp2_poly2(q0, q1, x0, x1);
+                                p0 = poly ? q0 : p0; p1 = poly ? q1 : p1;
+                            }
+                        }
                         add2(l0, l1, p0, p1);
                         pk[e >> 1] = pack_cvt(p0, p1);
                     }
@@ -597,13 +607,18 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 };
                 // No pass over the scores for their maximum: the exponentials are taken against the current
                 // reference, and only if their sum says that one of them may have left the safe range
-                // (> 2^14; also catches inf / NaN) is the true maximum taken and the half tile redone.  Half tiles
-                // that cross a causal limit and the first one of an item take their maximum first.  The two paths share
-                // no code: merging the registers of the probabilities would cost a move each.
-                bool fast = !masked && i != 0;
+                // (> 2^14; also catches inf / NaN) does the row take its true maximum and redo the half tile.  In half
+                // tiles that cross a causal limit, and in the first one of an item, every row takes its maximum first.
+                // Which way a row goes depends on its own scores and on positions alone, never on the rows that share
+                // its warp: a row before its activation offset keeps the bits of the base model's call.  The other rows of
+                // a warp with a row to redo repeat what they had, so that the two paths share no code: merging the
+                // registers of the probabilities instead costs a move each (2 % of the calls that attention dominates).
+                const bool plain = masked || i == 0;
+                bool fast = !plain, redo = plain;
                 if (fast) {
-                    const float l = exponentials(std::true_type());
-                    if (__any_sync(0xffffffffu, !(l <= 16384.f))) {
+                    const float l = exponentials(std::true_type(), false, true);
+                    redo = !(l <= 16384.f);
+                    if (__any_sync(0xffffffffu, redo)) {
                         fast = false;
                     } else {
                         l_run += l;
@@ -626,11 +641,11 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     }
                     const float m_tile = fmaxf(m0, m1);
                     float alpha = 1.f;   // factor of O_g and the row sum when the reference moves
-                    if ((m_tile - m_ref) * a.scale_log2 > 8.f) {
+                    if (redo && (m_tile - m_ref) * a.scale_log2 > 8.f) {
                         alpha = fast_exp2((m_ref - m_tile) * a.scale_log2);
                         m_ref = m_tile;
                     }
-                    l_run = fmaf(l_run, alpha, exponentials(std::false_type()));
+                    l_run = fmaf(l_run, alpha, exponentials(std::false_type(), !plain, !redo));
                     if (!pv_wait()) { ok = false; break; }
                     if (i != 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
                         // O_g holds the earlier products relative to the old reference: scale the rows that moved

@@ -155,3 +155,22 @@ def test_one_late_key_far_above_the_reference(oracle64, page, S, nats):
         _write_keys(shape, b, pool, r, 640 + r, wl.bf16_round(u * np.float32(nats / shape.head_dim ** 0.5))[None])
     got, want = _attend_values(shape, b, pool, qkv), _oracle_values(oracle64, shape, b, pool, qkv)
     hp.assert_close(got, want, 2e-2, f"a key {nats} nats above the others", block=shape.head_dim)
+
+
+@pytest.mark.parametrize("S", [24, 48])
+def test_a_row_does_not_depend_on_the_rows_beside_it(S):
+    """Every third token of a request gets queries whose scores jump by tens of nats from tile to tile, so that its rows
+    take their maximum again and again; the other tokens (which share their warps) keep the bits that they have without
+    that, as rows before an activation offset have to."""
+    shape = wl.LayerShape(hidden=256, n_q_heads=8, n_kv_heads=2, head_dim=128, page_size=16, dtype="bf16")
+    rng = np.random.default_rng(800 + S)
+    R = 8
+    b = wl.make_batch(shape, [1500 + 61 * r for r in range(R)], [S] * R, [-1] * R, rng, shuffle_pages=True, with_hidden=False)
+    pool = wl.random_kv_pool(shape, b.num_pages, rng)
+    qkv = wl.bf16_round(rng.standard_normal((b.T, shape.N), dtype=np.float32))
+    jumpy = qkv.copy()
+    loud = np.arange(b.T) % 3 == 1
+    jumpy[loud, :shape.Nq] = wl.bf16_round(jumpy[loud, :shape.Nq] * 30)
+    calm_rows, jumpy_rows = _attend_values(shape, b, pool, qkv), _attend_values(shape, b, pool, jumpy)
+    assert np.array_equal(calm_rows[~loud].view(np.uint32), jumpy_rows[~loud].view(np.uint32))
+    assert hp.rel_err(jumpy_rows[loud], calm_rows[loud]) > 0.1
