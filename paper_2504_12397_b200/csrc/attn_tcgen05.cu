@@ -575,8 +575,10 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 // probabilities of the scores against the current reference; returns their sum in fp32.  fast: one pair in
                 // eight on the FMA pipe; else only in the rows with `poly`, of which there are none unless `mixed`
                 auto exponentials = [&](auto fast, bool mixed, bool poly) {
-                    // (a piece that starts at an item's last tile can hold rows that see none of its keys so far)
-                    const float mb = m_ref == -INFINITY ? 0.f : m_ref * a.scale_log2;
+                    // A row without a reference (nothing but -inf so far): on the fast path mb = -inf makes the sum fail its
+                    // test, and the row takes its maximum; if that is -inf too, mb is 0 (a piece that starts at an item's
+                    // last tile can hold rows that see none of its keys)
+                    const float mb = !decltype(fast)::value && m_ref == -INFINITY ? 0.f : m_ref * a.scale_log2;
                     float l0 = 0.f, l1 = 0.f;
 #pragma unroll
                     for (int e = 0; e < kHalfKeys; e += 2) {

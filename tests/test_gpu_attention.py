@@ -174,3 +174,29 @@ def test_a_row_does_not_depend_on_the_rows_beside_it(S):
     calm_rows, jumpy_rows = _attend_values(shape, b, pool, qkv), _attend_values(shape, b, pool, jumpy)
     assert np.array_equal(calm_rows[~loud].view(np.uint32), jumpy_rows[~loud].view(np.uint32))
     assert hp.rel_err(jumpy_rows[loud], calm_rows[loud]) > 0.1
+
+
+@pytest.mark.parametrize("S", [20, 40])
+@pytest.mark.parametrize("dead", [64, 128, 300])
+def test_leading_keys_with_scores_of_minus_infinity(oracle64, S, dead):
+    """The first keys of a context give every query a score of -inf, the others scores far below zero: the row has no
+    reference when it meets the first finite score, and takes that score's maximum however low it is."""
+    shape = wl.LayerShape(hidden=256, n_q_heads=8, n_kv_heads=2, head_dim=128, page_size=16, dtype="bf16")
+    rng = np.random.default_rng(900 + S + dead)
+    P = [1000, 77 + dead, 2000]
+    b = wl.make_batch(shape, P, [S] * 3, [-1] * 3, rng, shuffle_pages=True, with_hidden=False)
+    pool = wl.random_kv_pool(shape, b.num_pages, rng)
+    qkv = wl.bf16_round(rng.standard_normal((b.T, shape.N), dtype=np.float32))
+    qkv[:, :shape.Nq] = np.abs(qkv[:, :shape.Nq]) + 0.5
+    qkv[:, :shape.Nq] = wl.bf16_round(qkv[:, :shape.Nq])
+    new_k = slice(shape.Nq, shape.Nq + shape.Nkv)
+    qkv[:, new_k] -= 13   # scores of about -13 * sum(q) / sqrt(128): -190
+    qkv[:, new_k] = wl.bf16_round(qkv[:, new_k])
+    pool[:, 0] = wl.bf16_round(pool[:, 0] - 13)
+    for r in range(3):
+        keys = wl.bf16_round(rng.standard_normal((dead, shape.head_dim), dtype=np.float32))
+        keys[:, 5] = -np.inf
+        _write_keys(shape, b, pool, r, 0, keys)
+    got = _attend_values(shape, b, pool, qkv)
+    want = _oracle_values(oracle64, shape, b, np.where(np.isinf(pool), np.float32(-1e30), pool), qkv)
+    hp.assert_close(got, want, 2e-2, "keys of -inf in front", block=shape.head_dim)
