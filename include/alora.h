@@ -129,8 +129,7 @@ alora_status alora_set_layer_weights(alora_ctx *ctx, int layer, const void *d_wq
  * blk in {q, k, v} (Eq. 4 / Eq. 5).  d_Aq/d_Ak/d_Av are [rank][H], d_Bq is [Nq][rank], d_Bk and
  * d_Bv are [Nkv][rank].  The matrices are COPIED into context-owned, rank-padded storage on the
  * given stream; the caller's buffers may be released once that stream has passed this point.
- * 1 <= rank <= max_rank.  The values have to be finite: on the row-tile routes a row that does not use an
- * adapter of its tile adds zero times that adapter's B.
+ * 1 <= rank <= max_rank.  Values that are not finite reach the rows that use the adapter and no others.
  */
 alora_status alora_register_adapter(alora_ctx *ctx, int adapter_id, int layer, int rank, float scale,
                                     const void *d_Aq, const void *d_Bq, const void *d_Ak,

@@ -22,7 +22,7 @@ int launch_project_tc(alora_ctx *, int, const void *, int, int, void *, cudaStre
 int launch_linear_tc(alora_ctx *, const void *, const void *, int, int, int, void *, const void *, const LinearDelta *,
                      cudaStream_t);
 int launch_repack_mlp(const void *, const void *, const void *, const void *, int, int, int, int, int, void *, void *,
-                      cudaStream_t);   // mlp_adapter.cu
+                      int32_t *, int32_t *, cudaStream_t);   // mlp_adapter.cu
 int launch_mlp_expand(alora_ctx *, void *, int, int, const void *, int, const void *, int, int, int, const int32_t *,
                       const MlpAdapterDev *, int, cudaStream_t);
 int launch_mlp_shrink(alora_ctx *, const void *, const void *, int, int, int, void *, float *, size_t, int32_t *, int,
@@ -364,14 +364,13 @@ alora_status alora_register_adapter(alora_ctx *ctx, int adapter_id, int layer, i
         A = ctx->adapter_storage[2 * idx]; B = ctx->adapter_storage[2 * idx + 1];
     }
     ctx->layer_has_adapter[layer] = 1;
-    int n = launch_repack_adapter(ctx, rank, d_Aq, d_Bq, d_Ak, d_Bk, d_Av, d_Bv, A, B, s);
     AdapterDev rec{A, B, rank, (rank + 15) / 16 * 16, scale, 0};
     ctx->h_adapters[idx] = rec;
     // the table entry is a kernel argument of later launches on this stream: order the update after
     // earlier work by copying on the same stream (source is context-owned host memory).
     ALORA_CUDA(ctx, cudaMemcpyAsync(ctx->d_adapters + idx, &ctx->h_adapters[idx], sizeof(AdapterDev),
                                     cudaMemcpyHostToDevice, s));
-    return finish(ctx, n);
+    return finish(ctx, launch_repack_adapter(ctx, rank, d_Aq, d_Bq, d_Ak, d_Bk, d_Av, d_Bv, A, B, &ctx->d_adapters[idx].b_odd, s));
 }
 
 // Rows of the down projection's A slab: every adapter's RP rows, rounded up to whole 128-row GEMM tiles.
@@ -399,7 +398,7 @@ alora_status alora_register_mlp_adapter(alora_ctx *ctx, int adapter_id, int laye
         ctx->mlp_a_gu.assign(ctx->cfg.n_layers, nullptr); ctx->mlp_b_gu.assign(ctx->cfg.n_layers, nullptr);
         ctx->mlp_a_dn.assign(ctx->cfg.n_layers, nullptr); ctx->mlp_b_dn.assign(ctx->cfg.n_layers, nullptr);
         ctx->mlp_n_adapters.assign(ctx->cfg.n_layers, 0);
-        ctx->h_mlp_adapters.assign((size_t)ctx->cfg.n_layers * na, MlpAdapterDev{0, 0.f});
+        ctx->h_mlp_adapters.assign((size_t)ctx->cfg.n_layers * na, MlpAdapterDev{0, 0.f, 0});
     }
     if (!ctx->d_mlp_adapters) {
         const size_t bytes = ctx->h_mlp_adapters.size() * sizeof(MlpAdapterDev);
@@ -428,22 +427,23 @@ alora_status alora_register_mlp_adapter(alora_ctx *ctx, int adapter_id, int laye
             ALORA_CUDA(ctx, cudaMemsetAsync(*sl.p, 0, sl.bytes, s));
         }
     }
+    const size_t idx = (size_t)layer * na + adapter_id;
+    ctx->h_mlp_adapters[idx] = MlpAdapterDev{(rank + 15) / 16 * 16, scale, 0};
+    ctx->mlp_n_adapters[layer] = std::max(ctx->mlp_n_adapters[layer], adapter_id + 1);
+    ALORA_CUDA(ctx, cudaMemcpyAsync(ctx->d_mlp_adapters + idx, &ctx->h_mlp_adapters[idx], sizeof(MlpAdapterDev),
+                                    cudaMemcpyHostToDevice, s));
+    int32_t *b_odd = &ctx->d_mlp_adapters[idx].b_odd, *any_odd = ctx->d_counts + kOddAdapters;
     int n = 0, k;
     k = launch_repack_mlp(d_Agate, d_Aup, d_Bgate, d_Bup, 2, rank, d.RP, d.H, d.I,
                           (char *)ctx->mlp_a_gu[layer] + (size_t)adapter_id * a_gu,
-                          (char *)ctx->mlp_b_gu[layer] + (size_t)adapter_id * b_gu, s);
+                          (char *)ctx->mlp_b_gu[layer] + (size_t)adapter_id * b_gu, b_odd, any_odd, s);
     if (k < 0) return cuda_fail(ctx, cudaGetLastError(), "repack_mlp_kernel");
     n += k;
     k = launch_repack_mlp(d_Adown, nullptr, d_Bdown, nullptr, 1, rank, d.RP, d.I, d.H,
                           (char *)ctx->mlp_a_dn[layer] + (size_t)adapter_id * a_dn,
-                          (char *)ctx->mlp_b_dn[layer] + (size_t)adapter_id * b_dn, s);
+                          (char *)ctx->mlp_b_dn[layer] + (size_t)adapter_id * b_dn, b_odd, any_odd, s);
     if (k < 0) return cuda_fail(ctx, cudaGetLastError(), "repack_mlp_kernel");
     n += k;
-    const size_t idx = (size_t)layer * na + adapter_id;
-    ctx->h_mlp_adapters[idx] = MlpAdapterDev{(rank + 15) / 16 * 16, scale};
-    ctx->mlp_n_adapters[layer] = std::max(ctx->mlp_n_adapters[layer], adapter_id + 1);
-    ALORA_CUDA(ctx, cudaMemcpyAsync(ctx->d_mlp_adapters + idx, &ctx->h_mlp_adapters[idx], sizeof(MlpAdapterDev),
-                                    cudaMemcpyHostToDevice, s));
     return finish(ctx, n);
 }
 

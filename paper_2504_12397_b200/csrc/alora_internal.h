@@ -25,13 +25,14 @@ struct AdapterDev {
     int32_t rank;   // 0 = not registered
     int32_t rpad;   // rank rounded up to 16
     float scale;
-    int32_t pad_;
+    int32_t b_odd;  // B holds an Inf or NaN: its delta may not go through a row tile's matrix product (TilePair)
 };
 
 // One adapter's part on the MLP block of one layer (gate, up and down projections share rank and scale).
 struct MlpAdapterDev {
     int32_t rpad;   // rank rounded up to 16; 0 = no MLP part registered
     float scale;
+    int32_t b_odd;  // a B matrix holds an Inf or NaN (as in AdapterDev)
 };
 
 struct LayerWeights {
@@ -42,7 +43,9 @@ struct LayerWeights {
 // The projection works on dense tiles of kTileRows rows.  A row tile meets the adapters applied to its rows (gate open)
 // one after another: one TilePair per (row tile, adapter that occurs in it).  The pair's t = s A x is kept for the whole
 // tile with the rows of other adapters and the rows with a closed gate set to zero, so the expand step t B^T adds
-// nothing to them.
+// nothing to them.  That takes a finite B (0 x Inf is a NaN in every row of the tile): where registration has met an Inf or
+// NaN, the pair's matrix product is left out and the epilogue adds the delta to the adapter's own rows on the CUDA cores
+// (tc::OddRow).
 constexpr int kTileRows = 128;
 struct TilePair {
     int32_t tile, adapter;
@@ -171,7 +174,8 @@ struct alora_ctx {
                                   // [3] few-row attention items, [4] next unclaimed few-row item,
                                   // [6] key tiles of the attention items that are cut into runs, [7] tiles per run,
                                   // [8] attention items taken whole (the first ones), [9] key tiles of those,
-                                  // [10], [11] next unclaimed projection item and blocks done, [12] few-row attention blocks done
+                                  // [10], [11] next unclaimed projection item and blocks done, [12] few-row attention blocks done,
+                                  // [13] an adapter with a non-finite B has been registered (kOddAdapters)
     int32_t *d_seg_scratch = nullptr;  // [14*max_requests+5] per-request values and merged row runs of the current batch
     int32_t *d_t_ready = nullptr;      // [max_pairs] per pair: epilogue warps that have published t (zero between launches)
     int32_t *d_iota = nullptr;         // 0..max_requests: query_start_loc of a decode batch
@@ -277,12 +281,13 @@ struct BatchArgs {
 // the attention lists alone is a programmatic dependent launch: it may run beside the projection kernel that
 // precedes it in the stream.  `timed`: bracket it with profiling events of the metadata family.
 constexpr int kMetaProjection = 1, kMetaAttention = 2;
+constexpr int kOddAdapters = 13;   // index into d_counts
 void few_cluster_init(alora_ctx *ctx);   // gemm_few_cluster.cu: what that route needs to know about the device
 int launch_metadata(alora_ctx *ctx, const BatchArgs &b, cudaStream_t s, int phases = kMetaProjection | kMetaAttention,
                     bool timed = true);
 int launch_repack_adapter(alora_ctx *ctx, int rank, const void *Aq, const void *Bq, const void *Ak,
                           const void *Bk, const void *Av, const void *Bv, void *A_dst, void *B_dst,
-                          cudaStream_t s);
+                          int32_t *b_odd, cudaStream_t s);
 int launch_project(alora_ctx *ctx, int layer, const void *hidden, int T, int R, void *qkv, cudaStream_t s, void *kv_pool,
                    int num_pages, bool *kv_appended);
 // Most (row tile, adapter) pairs that a batch of T rows and R requests can have.

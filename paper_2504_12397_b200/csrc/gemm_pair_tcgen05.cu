@@ -53,7 +53,7 @@ struct PairArgs {
     int tile0;                      // row tile of the batch that holds this launch's first row
     int shrink;                     // the launch has shrink items, one per pair of its row tiles (0: t is there already)
     int t_cols;                     // columns of t: 64 padded rank columns per adapted matrix
-    const int32_t *adapters;        // per adapter `ad_stride` words, the first two: padded rank, scale (float)
+    const int32_t *adapters;        // per adapter `ad_stride` words, the first three: padded rank, scale (float), b_odd
     int ad_stride;
     int M, N, K, Nq, Nkv;           // Nq, Nkv: the q/k/v blocks of the fused row
     int blk_cols;                   // other launches: columns per adapted matrix
@@ -61,8 +61,10 @@ struct PairArgs {
     int ldo;
     const __nv_bfloat16 *residual;  // optional, same layout as out, may alias it
     const int32_t *row_adapter;     // [M] applied adapter per row (shrink items: which rows of t are kept)
+    const int32_t *any_odd;         // not 0: an adapter of the context may have b_odd set
+    const __nv_bfloat16 *b_all;     // the launch's B rows of all adapters, [adapter][N][64] (read for rows of those)
     int32_t *t_ready;               // [pair] epilogue warps that have published their part of t
-    __nv_bfloat16 *t_out;           // [pair][128][t_cols]
+    __nv_bfloat16 *t;               // [pair][128][t_cols]
     // KV append fused into the epilogue (nullptr: off), as in gemm_tcgen05.cu
     __nv_bfloat16 *kv_pool;
     const int32_t *slot_map;
@@ -84,7 +86,12 @@ __device__ __forceinline__ void tma_load_3d_p(uint32_t smem_dst, const CUtensorM
         : "memory");
 }
 
-__device__ __forceinline__ int rank_steps(const PairArgs &a, int adapter) { return a.adapters[adapter * a.ad_stride] / 16; }
+// (none for a B with an Inf or NaN: see TilePair)
+__device__ __forceinline__ int rank_steps(const PairArgs &a, int adapter) {
+    const int32_t *ad = a.adapters + adapter * a.ad_stride;
+    const int rpad = ad[0], odd = ad[2];
+    return odd ? 0 : rpad / 16;
+}
 
 // One work item: a shrink item (pair p0[0], row tile m[0]) or two row tiles (m[1] = -1: none) x one column tile.
 struct PairItem {
@@ -341,6 +348,7 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
         // ------------------------------ epilogue (warps 2..5: first row tile, warps 6..9: second) ------------------------------
         const int q = warp & 3;           // tensor-memory lane quarter this warp may read
         const int my_h = (warp - 2) >> 2; // the half of tensor memory (row tile of the pair) this warp drains
+        const bool any_odd = a.pairs != nullptr && *a.any_odd != 0;
         uint32_t it = 0;
         bool ok = true;
         for (;; ++it) {
@@ -361,7 +369,7 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                 const int row = g.m[0] * 128 + r;
                 const bool use = row < a.M && a.row_adapter[row] == g.adapter;
                 const float scale = __int_as_float(a.adapters[g.adapter * a.ad_stride + 1]);
-                __nv_bfloat16 *trow = a.t_out + ((size_t)g.p0[0] * 128 + r) * a.t_cols;
+                __nv_bfloat16 *trow = a.t + ((size_t)g.p0[0] * 128 + r) * a.t_cols;
 #pragma unroll 1
                 for (int c = 0; c < a.t_cols; c += 32) {
                     uint32_t v[32];
@@ -385,6 +393,18 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                 if (g.m[h] >= 0) {
                     const int row = g.m[h] * 128 + r;
                     const bool row_ok = row < a.M;
+                    tc::OddRow odd;
+                    if (any_odd && row_ok) {
+                        const int k = a.row_adapter[row], p1 = g.p1[h];
+                        int p = k >= 0 && a.adapters[k * a.ad_stride + 2] ? g.p0[h] : p1;
+                        while (p < p1 && a.pairs[p].adapter != k) ++p;
+                        if (p < p1) {
+                            if (a.shrink) ld_acquire_p(a.t_ready + p);   // (complete since the tile's K blocks were loaded; orders the reads)
+                            odd.t = a.t + ((size_t)p * 128 + r) * a.t_cols;
+                            odd.b = a.b_all + (size_t)k * a.N * kTensorRP;
+                            odd.n = a.adapters[k * a.ad_stride];
+                        }
+                    }
                     __nv_bfloat16 *orow = a.out + (size_t)row * a.ldo + g.n0;
                     const __nv_bfloat16 *rrow = a.residual ? a.residual + (size_t)row * a.ldo + g.n0 : nullptr;
                     // fused KV append: where this row's k / v columns go in the page pool
@@ -409,6 +429,10 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                                 float f[8];
 #pragma unroll
                                 for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[8 * j + e]);
+                                if (odd.n) {
+                                    const int col = g.n0 + c + 8 * j;
+                                    odd.add8(f, col, !kQkv ? col / a.blk_cols : col < a.Nq ? 0 : (col < a.Nq + a.Nkv ? 1 : 2));
+                                }
                                 if (!kQkv && rrow) {
                                     const uint4 rv = *reinterpret_cast<const uint4 *>(rrow + c + 8 * j);
                                     const uint32_t rw[4] = {rv.x, rv.y, rv.z, rv.w};
@@ -527,11 +551,12 @@ int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T,
     const bool have_adapters = ctx->layer_has_adapter[layer] != 0;
     const bool apart = have_adapters && shrink_apart(ctx, T, R, items);
     const int max_pairs = have_adapters ? pair_bound(ctx, T, R) : 0;
-    if (have_adapters) { g.pairs = ctx->d_pairs; g.pair_off = ctx->d_pair_off; }
-    if (have_adapters && !apart) {
-        g.shrink = 1; g.row_adapter = ctx->d_row_adapter;
-        g.t_ready = ctx->d_t_ready; g.t_out = (__nv_bfloat16 *)ctx->d_t;
+    if (have_adapters) {
+        g.pairs = ctx->d_pairs; g.pair_off = ctx->d_pair_off; g.t = (__nv_bfloat16 *)ctx->d_t;
+        g.row_adapter = ctx->d_row_adapter; g.any_odd = ctx->d_counts + kOddAdapters;
+        g.b_all = (const __nv_bfloat16 *)ctx->tc_b_all[layer];
     }
+    if (have_adapters && !apart) { g.shrink = 1; g.t_ready = ctx->d_t_ready; }
     g.item_counters = ctx->d_counts + 10;
     if (kv_pool != nullptr) {
         int shift = 0;
@@ -575,7 +600,8 @@ int launch_linear256_tc(alora_ctx *ctx, const void *x, const void *W, int T, int
         if (!make_tensor_map_bf16(&tmB, delta->B, na * N, kTensorRP, kTensorRP, BN)) return -1;
         g.pairs = ctx->d_pairs; g.pair_off = ctx->d_pair_off; g.tile0 = delta->tile0; g.shrink = 1;
         g.adapters = &delta->table->rpad; g.ad_stride = sizeof(MlpAdapterDev) / 4;
-        g.row_adapter = delta->row_adapter; g.t_ready = ctx->d_t_ready; g.t_out = (__nv_bfloat16 *)delta->t;
+        g.row_adapter = delta->row_adapter; g.t_ready = ctx->d_t_ready; g.t = (__nv_bfloat16 *)delta->t;
+        g.any_odd = ctx->d_counts + kOddAdapters; g.b_all = (const __nv_bfloat16 *)delta->B;
     }
     if (!pair_kernel_ready<BN, false>(ctx)) return -1;
     const int grid = std::max(1, std::min(G, items + (delta != nullptr ? ctx->max_pairs : 0)));

@@ -50,7 +50,7 @@ struct GemmArgs {
     int tile0;                      // row tile of the batch that holds this launch's first row
     int shrink;                     // the launch has shrink items, one per pair of its row tiles (0: t is there already)
     int t_cols;                     // columns of t: 64 padded rank columns per adapted matrix
-    const int32_t *adapters;        // per adapter `ad_stride` words, the first two: padded rank, scale (float)
+    const int32_t *adapters;        // per adapter `ad_stride` words, the first three: padded rank, scale (float), b_odd
     int ad_stride;
     int M, N, K;
     __nv_bfloat16 *out;
@@ -59,8 +59,10 @@ struct GemmArgs {
     int Nq, Nkv;                    // block boundaries of the fused output row (expand; gate | up: Nq = Nkv = half)
     int total_adapter_rows;         // rows per adapter in the B_all map (= N of the layer)
     const int32_t *row_adapter;     // [M] applied adapter per row (shrink items: which rows of t are kept)
+    const int32_t *any_odd;         // not 0: an adapter of the context may have b_odd set
+    const __nv_bfloat16 *b_all;     // the launch's B rows of all adapters, [adapter][N][64] (read for rows of those)
     int32_t *t_ready;               // [pair] epilogue warps that have published their part of t
-    __nv_bfloat16 *t_out;           // [pair][t_parts][128][t_cols]
+    __nv_bfloat16 *t;               // [pair][t_parts][128][t_cols]
     int t_parts;                    // t is the sum of this many bf16 values (1 or 2)
     // KV append fused into the epilogue (nullptr: off): columns Nq .. N of row t also go to the paged cache,
     // pool[page][plane][head][row in page][:] with page * page_size + row = slot_map[t] (-1: token rejected, skipped)
@@ -84,7 +86,12 @@ struct GemmSmem {
     static constexpr int kTotal = kItemRingOffset + 128 + 1024;  // barriers, item ring, slack for 1024-byte alignment
 };
 
-__device__ __forceinline__ int rank_steps(const GemmArgs &a, int adapter) { return a.adapters[adapter * a.ad_stride] / 16; }
+// (none for a B with an Inf or NaN: see TilePair)
+__device__ __forceinline__ int rank_steps(const GemmArgs &a, int adapter) {
+    const int32_t *ad = a.adapters + adapter * a.ad_stride;
+    const int rpad = ad[0], odd = ad[2];
+    return odd ? 0 : rpad / 16;
+}
 
 // Work item `item` of a launch: shrink items first (one per pair), then the projection's
 // (row tile, column tile) pairs.
@@ -318,6 +325,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     } else {
         // ------------------------------ epilogue (warps 2..5) ------------------------------
         const int q = warp & 3;  // tensor-memory lane quarter this warp may read
+        const bool any_odd = a.pairs != nullptr && *a.any_odd != 0;
         uint32_t it = 0;
         bool ok = true;
         while (ok) {
@@ -333,7 +341,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 // t = s A x of this pair, zero in the rows that do not use the adapter
                 const float scale = __int_as_float(a.adapters[g.adapter * a.ad_stride + 1]);
                 const bool use = row_ok && a.row_adapter[row] == g.adapter;
-                __nv_bfloat16 *trow = a.t_out + ((size_t)g.p0 * a.t_parts * kBM + q * 32 + lane) * a.t_cols;
+                __nv_bfloat16 *trow = a.t + ((size_t)g.p0 * a.t_parts * kBM + q * 32 + lane) * a.t_cols;
                 __nv_bfloat16 *tlow = a.t_parts > 1 ? trow + (size_t)kBM * a.t_cols : nullptr;
 #pragma unroll 1
                 for (int c = 0; c < a.t_cols && c < BN; c += 32) {
@@ -353,6 +361,19 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 }
                 ++it;
                 continue;
+            }
+            tc::OddRow odd;
+            if (any_odd && row_ok) {
+                const int k = a.row_adapter[row];
+                int p = k >= 0 && a.adapters[k * a.ad_stride + 2] ? g.p0 : g.p1;
+                while (p < g.p1 && a.pairs[p].adapter != k) ++p;
+                if (p < g.p1) {
+                    if (a.shrink) ld_acquire(a.t_ready + p);   // (complete since the tile's K blocks were loaded; orders the reads)
+                    odd.t = a.t + ((size_t)p * a.t_parts * kBM + q * 32 + lane) * a.t_cols;
+                    odd.b = a.b_all + (size_t)k * a.N * kTensorRP;
+                    odd.n = a.adapters[k * a.ad_stride];
+                    odd.low = a.t_parts > 1 ? kBM * a.t_cols : 0;
+                }
             }
             __nv_bfloat16 *orow = a.out + (size_t)row * a.ldo + n0;
             const __nv_bfloat16 *rrow = a.residual ? a.residual + (size_t)row * a.ldo + n0 : nullptr;
@@ -378,6 +399,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         float f[8];
 #pragma unroll
                         for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[8 * j + e]);
+                        if (odd.n) odd.add8(f, n0 + c + 8 * j, n0 < a.Nq ? 0 : (n0 < a.Nq + a.Nkv ? 1 : 2));
                         if (rrow) {
                             const uint4 rv = *reinterpret_cast<const uint4 *>(rrow + c + 8 * j);
                             const uint32_t rw[4] = {rv.x, rv.y, rv.z, rv.w};
@@ -589,17 +611,18 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
         g.ad_stride = sizeof(AdapterDev) / 4; g.t_cols = 3 * kTensorRP;
         g.Nq = d.Nq; g.Nkv = d.Nkv; g.total_adapter_rows = d.N; g.status = ctx->d_status;
         g.item_counters = ctx->d_counts + 10;
-        if (have_adapters) { g.pairs = ctx->d_pairs; g.pair_off = ctx->d_pair_off; g.t_parts = t_parts; }
+        if (have_adapters) {
+            g.pairs = ctx->d_pairs; g.pair_off = ctx->d_pair_off; g.t = (__nv_bfloat16 *)ctx->d_t; g.t_parts = t_parts;
+            g.row_adapter = ctx->d_row_adapter; g.any_odd = ctx->d_counts + kOddAdapters;
+            g.b_all = (const __nv_bfloat16 *)ctx->tc_b_all[layer];
+        }
         if (kv_pool != nullptr) {
             int shift = 0;
             while ((1 << shift) < d.hd) ++shift;
             g.kv_pool = (__nv_bfloat16 *)kv_pool; g.slot_map = ctx->d_slot; g.kv_hd_shift = shift; g.kv_heads = d.Hkv;
             g.kv_page_size = d.page; g.kv_num_pages = num_pages;
         }
-        if (fuse_shrink) {
-            g.shrink = 1; g.row_adapter = ctx->d_row_adapter;
-            g.t_ready = ctx->d_t_ready; g.t_out = (__nv_bfloat16 *)ctx->d_t;
-        }
+        if (fuse_shrink) { g.shrink = 1; g.t_ready = ctx->d_t_ready; }
         const int items = proj_items + (fuse_shrink ? max_pairs : 0);
         const bool ok = BN == 256
                             ? launch_gemm_bn<256>(ctx, tmXg, lm.wqkv[1], tmTt, lm.b_all_bn[1], lm.a_all, g, items, s)
@@ -655,7 +678,8 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
         if (!make_tensor_map_bf16(&tmB, delta->B, na * N, kTensorRP, kTensorRP, BN)) return -1;
         g.pairs = ctx->d_pairs; g.pair_off = ctx->d_pair_off; g.tile0 = delta->tile0; g.shrink = 1;
         g.adapters = &delta->table->rpad; g.ad_stride = sizeof(MlpAdapterDev) / 4;
-        g.row_adapter = delta->row_adapter; g.t_ready = ctx->d_t_ready; g.t_out = (__nv_bfloat16 *)delta->t;
+        g.row_adapter = delta->row_adapter; g.t_ready = ctx->d_t_ready; g.t = (__nv_bfloat16 *)delta->t;
+        g.any_odd = ctx->d_counts + kOddAdapters; g.b_all = (const __nv_bfloat16 *)delta->B;
     }
     const int items = ((T + kBM - 1) / kBM) * ((N + BN - 1) / BN) + (delta != nullptr ? ctx->max_pairs : 0);
     const bool ok = BN == 256 ? launch_gemm_bn<256>(ctx, tmX, tmW, tmT, tmB, tmA, g, items, s)

@@ -16,11 +16,12 @@
 namespace alora {
 
 // A rows of every adapter, rank-padded: dst[(k * nblk + blk) * RP + i][K] <- src_blk[i][K] (zero rows beyond the rank).
-// B rows: dst[k][blk * width + c][RP] <- src_blk[c][rank] (zero columns beyond the rank).
+// B rows: dst[k][blk * width + c][RP] <- src_blk[c][rank] (zero columns beyond the rank); an Inf or NaN among them sets
+// *b_odd (the adapter's record, written before this launch) and *any_odd.
 __global__ void repack_mlp_kernel(const __nv_bfloat16 *__restrict__ a0, const __nv_bfloat16 *__restrict__ a1,
                                   const __nv_bfloat16 *__restrict__ b0, const __nv_bfloat16 *__restrict__ b1, int nblk,
                                   int rank, int RP, int K, int width, __nv_bfloat16 *__restrict__ A_dst,
-                                  __nv_bfloat16 *__restrict__ B_dst) {
+                                  __nv_bfloat16 *__restrict__ B_dst, int32_t *b_odd, int32_t *any_odd) {
     const size_t nA = (size_t)nblk * RP * K, nB = (size_t)nblk * width * RP;
     const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nA + nB; i += (size_t)gridDim.x * blockDim.x) {
@@ -35,16 +36,18 @@ __global__ void repack_mlp_kernel(const __nv_bfloat16 *__restrict__ a0, const __
             const int col = (int)(j / RP), c = (int)(j % RP);
             const int blk = col / width, n = col % width;
             const __nv_bfloat16 *src = blk == 0 ? b0 : b1;
-            B_dst[j] = c < rank ? src[(size_t)n * rank + c] : zero;
+            const __nv_bfloat16 v = c < rank ? src[(size_t)n * rank + c] : zero;
+            if (!isfinite(__bfloat162float(v))) { *b_odd = 1; *any_odd = 1; }
+            B_dst[j] = v;
         }
     }
 }
 
 int launch_repack_mlp(const void *a0, const void *a1, const void *b0, const void *b1, int nblk, int rank, int RP, int K,
-                      int width, void *A_dst, void *B_dst, cudaStream_t s) {
+                      int width, void *A_dst, void *B_dst, int32_t *b_odd, int32_t *any_odd, cudaStream_t s) {
     repack_mlp_kernel<<<256, 256, 0, s>>>((const __nv_bfloat16 *)a0, (const __nv_bfloat16 *)a1, (const __nv_bfloat16 *)b0,
                                          (const __nv_bfloat16 *)b1, nblk, rank, RP, K, width, (__nv_bfloat16 *)A_dst,
-                                         (__nv_bfloat16 *)B_dst);
+                                         (__nv_bfloat16 *)B_dst, b_odd, any_odd);
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
@@ -341,9 +344,15 @@ __global__ void __launch_bounds__(kMxThreads, 4) mlp_expand_add_kernel(const Mlp
                         if (rb <= mt * 16 || ra >= mt * 16 + 16) continue;   // the run has no row in this tile
                         uint32_t af[4];
                         ldmatrix_x4(af, sT + (mt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8) * kMxLd + ks + (lane >> 4) * 8);
+                        // (a tile with rows of other runs: those keep what they have, whatever 0 x B is)
+                        const bool lo = mt * 16 + g >= ra && mt * 16 + g < rb, hi = mt * 16 + 8 + g >= ra && mt * 16 + 8 + g < rb;
 #pragma unroll
-                        for (int nt = 0; nt < 4; ++nt)
-                            mma_bf16_16816(acc[mt][nt], af, bf[nt >> 1][(nt & 1) * 2], bf[nt >> 1][(nt & 1) * 2 + 1]);
+                        for (int nt = 0; nt < 4; ++nt) {
+                            float c[4] = {acc[mt][nt][0], acc[mt][nt][1], acc[mt][nt][2], acc[mt][nt][3]};
+                            mma_bf16_16816(c, af, bf[nt >> 1][(nt & 1) * 2], bf[nt >> 1][(nt & 1) * 2 + 1]);
+                            if (lo) { acc[mt][nt][0] = c[0]; acc[mt][nt][1] = c[1]; }
+                            if (hi) { acc[mt][nt][2] = c[2]; acc[mt][nt][3] = c[3]; }
+                        }
                     }
                 }
             }

@@ -15,12 +15,13 @@ template <> __device__ __forceinline__ void stf<__nv_bfloat16>(__nv_bfloat16 *p,
 
 // ---------------------------------------------------------------------------------------------
 // Adapter repack: A_dst[3][RP][H] <- (Aq, Ak, Av)[r][H] with zero rows r..RP-1;
-// B_dst[N][RP] <- rows of (Bq | Bk | Bv)[.][r] with zero columns r..RP-1.
+// B_dst[N][RP] <- rows of (Bq | Bk | Bv)[.][r] with zero columns r..RP-1.  An Inf or NaN among the B values sets *b_odd (the
+// adapter's record, written before this launch) and *any_odd.
 // ---------------------------------------------------------------------------------------------
 template <typename T>
 __global__ void repack_adapter_kernel(const T *Aq, const T *Ak, const T *Av, const T *Bq, const T *Bk,
                                       const T *Bv, int rank, int RP, int H, int Nq, int Nkv, T *A_dst,
-                                      T *B_dst) {
+                                      T *B_dst, int32_t *b_odd, int32_t *any_odd) {
     const size_t nA = (size_t)3 * RP * H, nB = (size_t)(Nq + 2 * Nkv) * RP;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nA + nB;
          i += (size_t)gridDim.x * blockDim.x) {
@@ -37,6 +38,7 @@ __global__ void repack_adapter_kernel(const T *Aq, const T *Ak, const T *Av, con
                 if (n < Nq) v = Bq[(size_t)n * rank + c];
                 else if (n < Nq + Nkv) v = Bk[(size_t)(n - Nq) * rank + c];
                 else v = Bv[(size_t)(n - Nq - Nkv) * rank + c];
+                if (!isfinite(ldf(&v))) { *b_odd = 1; *any_odd = 1; }
             }
             B_dst[j] = v;
         }
@@ -45,17 +47,19 @@ __global__ void repack_adapter_kernel(const T *Aq, const T *Ak, const T *Av, con
 
 int launch_repack_adapter(alora_ctx *ctx, int rank, const void *Aq, const void *Bq, const void *Ak,
                           const void *Bk, const void *Av, const void *Bv, void *A_dst, void *B_dst,
-                          cudaStream_t s) {
+                          int32_t *b_odd, cudaStream_t s) {
     const Dims &d = ctx->d;
+    int32_t *any_odd = ctx->d_counts + kOddAdapters;
     if (ctx->cfg.dtype == ALORA_DTYPE_FP32)
         repack_adapter_kernel<float><<<256, 256, 0, s>>>((const float *)Aq, (const float *)Ak, (const float *)Av,
                                                          (const float *)Bq, (const float *)Bk, (const float *)Bv,
-                                                         rank, d.RP, d.H, d.Nq, d.Nkv, (float *)A_dst, (float *)B_dst);
+                                                         rank, d.RP, d.H, d.Nq, d.Nkv, (float *)A_dst, (float *)B_dst,
+                                                         b_odd, any_odd);
     else
         repack_adapter_kernel<__nv_bfloat16><<<256, 256, 0, s>>>(
             (const __nv_bfloat16 *)Aq, (const __nv_bfloat16 *)Ak, (const __nv_bfloat16 *)Av,
             (const __nv_bfloat16 *)Bq, (const __nv_bfloat16 *)Bk, (const __nv_bfloat16 *)Bv, rank, d.RP, d.H,
-            d.Nq, d.Nkv, (__nv_bfloat16 *)A_dst, (__nv_bfloat16 *)B_dst);
+            d.Nq, d.Nkv, (__nv_bfloat16 *)A_dst, (__nv_bfloat16 *)B_dst, b_odd, any_odd);
     return 1;
 }
 

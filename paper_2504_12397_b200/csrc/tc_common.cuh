@@ -233,6 +233,23 @@ __device__ __forceinline__ void store_t(const float (&v)[n], float scale, bool u
     }
 }
 
+// Delta of one row whose adapter's B holds an Inf or NaN (TilePair), on the CUDA cores.  The matrix products of a row tile
+// leave such a pair out: the zeros of the other rows would meet the Inf.  `t` is the row's part of the pair (two summands
+// `low` elements apart, 0: one), `b` the adapter's B row of output column 0 of the launch, `cols` the columns of t per block.
+struct OddRow {
+    const __nv_bfloat16 *t = nullptr, *b = nullptr;
+    int n = 0, low = 0;   // padded rank, 0: nothing to do for this row
+    __device__ __forceinline__ void add8(float (&f)[8], int col, int blk) const {   // output columns col .. col + 7 of block blk
+        const __nv_bfloat16 *tb = t + blk * kRankPadMax, *bc = b + (size_t)col * kRankPadMax;
+#pragma unroll 1
+        for (int i = 0; i < n; ++i) {
+            const float ti = __bfloat162float(__ldcg(tb + i)) + (low ? __bfloat162float(__ldcg(tb + low + i)) : 0.f);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) f[e] = fmaf(ti, __bfloat162float(bc[e * kRankPadMax + i]), f[e]);
+        }
+    }
+};
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t *>(&v);

@@ -272,3 +272,32 @@ def test_mlp_adapter_registration_errors():
         assert reg(g.ctx, 0, 0, m.rank) == 0
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("each", [9, 30])
+def test_non_finite_mlp_adapter_values_stay_in_the_rows_that_use_them(each):
+    """One of two MLP adapters has Inf and NaN among its B values, in turn in the gate, up and down part: the rows of the
+    other one and of the base model keep their bits, on the few-row route (separate expand step) and on the row tiles."""
+    rng = np.random.default_rng(48)
+    layers, ads, mlps = _weights(rng, 1)
+    R = 9
+    ids = [(r % 3) - 1 for r in range(R)]
+    b = wl.make_batch(SHAPE, [0] * R, [each] * R, ids, rng, activation_offsets=[0] * R, shuffle_pages=True)
+    own = np.repeat(np.array(ids), each) == 1
+
+    def run():
+        g = hp.GpuLayers(SHAPE, layers, ads, 512, R, mlp_adapters_per_layer=mlps)
+        try:
+            return _run_stack(g, b)[0]
+        finally:
+            g.close()
+
+    finite = run()
+    for n, v in (("Bg", np.inf), ("Bu", np.nan), ("Bd", -np.inf)):
+        m = getattr(mlps[0][1], n)
+        kept = m[200, 5]
+        m[200, 5] = v
+        odd = run()
+        m[200, 5] = kept
+        assert np.array_equal(odd[~own].view(np.uint32), finite[~own].view(np.uint32)), n
+        assert not np.isfinite(odd[own]).all(), n

@@ -811,3 +811,44 @@ def test_stack_layers_on_different_projection_routes_share_the_attention_list(or
             hp.assert_close(hp.to_host(hout), x, 2e-2, "decode step through layers on different routes", block=shape.head_dim)
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("n_req,each,kv_heads,slots", [(9, 12, 2, 3), (9, 12, 2, 5), (20, 30, 2, 3), (20, 30, 2, 5), (47, 17, 2, 5),
+                                                       (30, 45, 2, 3), (11, 50, 1, 5)])
+def test_non_finite_adapter_values_stay_in_the_rows_that_use_them(oracle64, n_req, each, kv_heads, slots):
+    """One of three adapters has Inf, -Inf and NaN among its B values.  On every projection route (few rows in one launch or,
+    with five adapter slots, in two; one row tile per block, two, 128-wide column tiles) the rows of the other adapters and of the base model, which share its row tiles, keep
+    the bits they have beside a finite adapter; its own rows are non-finite in those columns and right in all others."""
+    shape = wl.LayerShape(hidden=512, n_q_heads=4, n_kv_heads=kv_heads, head_dim=128, page_size=16, dtype="bf16")
+    rng = np.random.default_rng(71 + n_req)
+    w = wl.make_wqkv(shape, rng)
+    ads = _boosted_adapters(shape, rng, [(16, 1.0), (24, 0.5), (64, 1.0)])
+    ids = [(r % 4) - 1 for r in range(n_req)]
+    b = wl.make_batch(shape, [40] * n_req, [each] * n_req, ids, rng, activation_offsets=[40 + (3 if r % 3 == 0 else 0) for r in range(n_req)])
+    want, gate = oracle64.project_qkv(b.hidden, w, shape.Nq, shape.Nkv, b.positions, b.query_start_loc, b.activation_offsets,
+                                      b.adapter_ids, hp.oracle_adapters(ads))
+    odd_cols = [(0, 5, np.inf), (0, 300, -np.inf), (1, 17, np.nan), (2, 100, np.inf), (2, 101, np.nan)]   # block, row of B, value
+
+    def project():
+        g = hp.GpuLayers(shape, [dict(wqkv=w)], [ads], b.T, b.R, n_adapters=slots)
+        try:
+            d = hp.DevBatch(b, shape.dtype)
+            out = g.empty(b.T, shape.N)
+            ab.alora_project_qkv(g.ctx, 0, ab.MODE_ALORA, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, d.T, d.R, out)
+            assert g.status() == 0
+            return hp.to_host(out)
+        finally:
+            g.close()
+
+    finite = project()
+    for blk, row, v in odd_cols:
+        m = getattr(ads[1], ("Bq", "Bk", "Bv")[blk])
+        m[row, 3] = v
+    odd = project()
+    own = (np.repeat(np.array(ids), each) == 1) & (gate != 0)
+    cols = [(0, shape.Nq, shape.Nq + shape.Nkv)[blk] + row for blk, row, _ in odd_cols]
+    assert own.any() and (~own).any()
+    assert np.array_equal(odd[~own].view(np.uint32), finite[~own].view(np.uint32))
+    assert not np.isfinite(odd[own][:, cols]).any()
+    others = np.setdiff1d(np.arange(shape.N), cols)
+    hp.assert_close(odd[own][:, others], want[own][:, others], 2e-2, "the adapter's own rows")
