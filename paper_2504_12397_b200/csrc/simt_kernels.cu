@@ -113,7 +113,7 @@ linear_simt_kernel(const float *__restrict__ x, const float *__restrict__ W, int
     tc::grid_dep_launch();
     if (!base_first) tc::grid_dep_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tx = lane & 7, ty = lane >> 3;
-    const int row0 = blockIdx.y * 16, col0 = blockIdx.x * 32;
+    const int n_col = (N + 31) / 32, row0 = (int)blockIdx.x / n_col * 16, col0 = (int)blockIdx.x % n_col * 32;   // (any number of rows)
     float acc[4][4] = {};   // rows row0 + ty + 4 i, columns col0 + tx + 8 j (beyond the edge: the last one again, not stored)
     const float *xr[4], *wr[4];
 #pragma unroll
@@ -663,7 +663,7 @@ int launch_project_simt(alora_ctx *ctx, int layer, const void *hidden, int T, vo
         shrink_simt_kernel<<<dim3(T, 3), 256, 0, s>>>((const float *)hidden, ctx->d_row_adapter, ads, d.H, d.RP, (float *)ctx->d_t);
     }
     ProfScope prof(ctx, KK_PROJECT, s);
-    const cudaError_t e = launch_kernel(linear_simt_kernel, dim3((d.N + 31) / 32, (T + 15) / 16), dim3(256), 0, s, true,
+    const cudaError_t e = launch_kernel(linear_simt_kernel, dim3((d.N + 31) / 32 * ((T + 15) / 16)), dim3(256), 0, s, true,
         (const float *)hidden, (const float *)ctx->layers[layer].wqkv, T, d.H, d.N, (const int32_t *)ctx->d_row_adapter, ads,
         (const float *)ctx->d_t, d.RP, d.Nq, d.Nkv, (const float *)nullptr, (float *)qkv, (float *)kv_pool, (const int32_t *)ctx->d_slot,
         d.hd, d.Hkv, d.page, num_pages, 1, ctx->d_status);
@@ -674,7 +674,7 @@ int launch_linear_simt(alora_ctx *ctx, const void *x, const void *W, int T, int 
                        const void *residual, cudaStream_t s) {
     if (T == 0) return 0;
     ProfScope prof(ctx, KK_LINEAR, s);
-    const cudaError_t e = launch_kernel(linear_simt_kernel, dim3((N + 31) / 32, (T + 15) / 16), dim3(256), 0, s, true, (const float *)x,
+    const cudaError_t e = launch_kernel(linear_simt_kernel, dim3((N + 31) / 32 * ((T + 15) / 16)), dim3(256), 0, s, true, (const float *)x,
         (const float *)W, T, K, N, (const int32_t *)nullptr, (const AdapterDev *)nullptr, (const float *)nullptr, 0, 0, 0,
         (const float *)residual, (float *)y, (float *)nullptr, (const int32_t *)nullptr, 0, 0, 0, 0, 0, ctx->d_status);
     return e == cudaSuccess ? 1 : -1;

@@ -852,3 +852,27 @@ def test_non_finite_adapter_values_stay_in_the_rows_that_use_them(oracle64, n_re
     assert not np.isfinite(odd[own][:, cols]).any()
     others = np.setdiff1d(np.arange(shape.N), cols)
     hp.assert_close(odd[own][:, others], want[own][:, others], 2e-2, "the adapter's own rows")
+
+
+def test_fp32_projection_of_more_rows_than_one_grid_dimension_holds_tiles(oracle64):
+    """The fp32 projection takes 16 rows a tile; 65536 tiles and one row more, a sample of rows against the oracle."""
+    import torch
+    shape = wl.LayerShape(hidden=32, n_q_heads=1, n_kv_heads=1, head_dim=32, page_size=16, dtype="fp32")
+    rng = np.random.default_rng(81)
+    T = 16 * 65536 + 1
+    w = wl.make_wqkv(shape, rng)
+    g = hp.GpuLayers(shape, [dict(wqkv=w)], [[]], T, 1)
+    try:
+        gen = torch.Generator(device="cuda"); gen.manual_seed(81)
+        x = torch.randn(T, shape.hidden, device="cuda", generator=gen)
+        out = torch.full((T, shape.N), float("nan"), device="cuda")
+        ab.alora_project_qkv(g.ctx, 0, ab.MODE_BASE, x, torch.arange(T, dtype=torch.int32, device="cuda"), None, None,
+                             hp.idev([0, T]), hp.idev([T]), T, 1, out)
+        assert g.status() == 0
+        rows = np.unique(np.concatenate([rng.integers(0, T, 200), [0, T - 17, T - 2, T - 1]]))
+        idx = torch.from_numpy(rows).cuda()
+        want = oracle64.linear(hp.to_host(x[idx]).astype(np.float64), w)
+        hp.assert_close(hp.to_host(out[idx]), want, hp.tol(shape), "rows of a million-row fp32 projection")
+        assert bool(torch.isfinite(out).all())
+    finally:
+        g.close()
