@@ -699,7 +699,7 @@ alora_status alora_forward_stack(alora_ctx *ctx, int mode, const void *d_hidden_
             // the layer's A rows (one launch) and an expand step that adds each open-gate row's delta in place
             const int n_mlp = (mode != ALORA_MODE_BASE && !ctx->mlp_n_adapters.empty()) ? ctx->mlp_n_adapters[l] : 0;
             const MlpAdapterDev *mlp_tab = n_mlp ? ctx->d_mlp_adapters + (size_t)l * std::max(1, ctx->cfg.max_adapters) : nullptr;
-            const bool fused = n_mlp && linear_takes_delta(ctx, tc, d.H, 2 * d.I) && linear_takes_delta(ctx, tc, d.I, d.H);
+            const bool fused = n_mlp && tc > kFewRowMax;   // (fewer rows: the batch's pairs may not have been built)
             LinearDelta gu{}, dn{};
             if (fused) {
                 gu = LinearDelta{ctx->mlp_a_gu[l], ctx->mlp_b_gu[l], 2, mlp_tab, t0 / kTileRows, ctx->d_row_adapter + t0, ctx->d_mlp_t};

@@ -317,7 +317,6 @@ struct LinearDelta {
 };
 int launch_linear(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
                   const void *residual, cudaStream_t s, const LinearDelta *delta = nullptr);
-bool linear_takes_delta(const alora_ctx *ctx, int T, int K, int N);   // gemm_tcgen05.cu
 int launch_rmsnorm(alora_ctx *ctx, const void *x, const void *w, int T, void *y, cudaStream_t s);
 int launch_swiglu(alora_ctx *ctx, const void *gate_up, int T, void *y, cudaStream_t s);
 

@@ -498,16 +498,13 @@ static bool launch_gemm_bn(alora_ctx *ctx, const CUtensorMap &tmA, const CUtenso
 bool launch_shrink_tc(alora_ctx *ctx, const CUtensorMap &tmX, const RankMaps &tmA, const AdapterDev *adapters,
                       int T, int K, int max_pairs, int t_parts, cudaStream_t s);  // shrink_tcgen05.cu
 
-// Picks the column-tile width: 256 when the q/k/v block boundaries allow it, else 128; 64 for batches of at most
-// 128 rows, where the kernel streams the weights once and more, narrower tiles put more SMs to work.
-static int pick_bn(int N, int Nq, int Nkv, bool lora, int T) {
+// Picks the column-tile width of the q/k/v projection: 256 when the block boundaries allow it, else 128; 64 for batches of
+// at most 128 rows, where the kernel streams the weights once and more, narrower tiles put more SMs to work.
+static int pick_bn(int N, int Nq, int Nkv, int T) {
     if (T <= kBM && N >= 64 * 48 && Nq % 64 == 0 && Nkv % 64 == 0) return 64;
-    if (lora) {
-        if (Nq % 256 == 0 && Nkv % 256 == 0) return 256;
-        if (Nq % 128 == 0 && Nkv % 128 == 0) return 128;
-        return 0;
-    }
-    return (N % 256 == 0 || N > 1024) ? 256 : 128;
+    if (Nq % 256 == 0 && Nkv % 256 == 0) return 256;
+    if (Nq % 128 == 0 && Nkv % 128 == 0) return 128;
+    return 0;
 }
 
 // q/k/v projection of one layer on the tensor cores: shrink (t = s A x of the (row tile, adapter) pairs), then the
@@ -582,7 +579,7 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
         const int r = launch_project_pair_tc(ctx, layer, hidden, T, R, qkv, s, kv_pool, num_pages);
         if (r != 0) return r;
     }
-    const int BN = pick_bn(d.N, d.Nq, d.Nkv, true, T);
+    const int BN = pick_bn(d.N, d.Nq, d.Nkv, T);
     if (BN == 0 || d.H % 8 != 0) return -1;
     CUtensorMap tmX, tmTt, tmX64;
     if (!make_tensor_map_bf16(&tmX, hidden, T, d.H, d.H, kBM)) return -1;
@@ -639,18 +636,13 @@ int launch_linear256_tc(alora_ctx *ctx, const void *x, const void *W, int T, int
                         const void *residual, const LinearDelta *delta, cudaStream_t s);  // gemm_pair_tcgen05.cu
 bool build_pair_maps(alora_ctx *ctx, int layer);                 // gemm_pair_tcgen05.cu
 
-// Whether launch_linear_tc can add a gated delta to a projection of this shape (not on the few-row route).
-bool linear_takes_delta(const alora_ctx *ctx, int T, int K, int N) {
-    return T > kFewRowMax || !few_cluster_route(ctx, T, 0, N, K, false, N, 0);
-}
-
 // Dense projection y = x W^T (+ residual) for o_proj and the MLP matrices, with the gated delta of the MLP adapters where
-// `delta` is given.
+// `delta` is given (more than kFewRowMax rows: a smaller batch may be on the few-row route, which builds no pairs).
 int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
                      const void *residual, const LinearDelta *delta, cudaStream_t s) {
     if (T == 0) return 0;
     if (K % 8 != 0 || N % 8 != 0) return -1;
-    if (delta != nullptr && (!linear_takes_delta(ctx, T, K, N) || (N / delta->n_blk) % 256 != 0)) return -1;
+    if (delta != nullptr && (T <= kFewRowMax || (N / delta->n_blk) % 256 != 0)) return -1;
     ProfScope prof(ctx, KK_LINEAR, s);
     if (delta == nullptr && few_cluster_rows(ctx, T) && few_cluster_route(ctx, T, 0, N, K, false, N, 0))
         return launch_few_cluster(ctx, x, W, nullptr, nullptr, nullptr, T, 0, K, N, N, 0, y, residual, nullptr, 0, false, s);
@@ -658,13 +650,11 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
         const int r = launch_linear256_tc(ctx, x, W, T, K, N, y, residual, delta, s);   // many rows: 256 x 256 tiles
         if (r != 0) return r;
     }
-    const int BN = delta != nullptr ? 256 : pick_bn(N, N, 0, false, T);
+    const int BN = N % 256 == 0 || N > 1024 ? 256 : 128;
     CUtensorMap tmX, tmW;
-    const bool half_box = T <= kBM / 2;   // see GemmArgs::a_tile_bytes
-    if (!make_tensor_map_bf16(&tmX, x, T, K, K, half_box ? kBM / 2 : kBM)) return -1;
+    if (!make_tensor_map_bf16(&tmX, x, T, K, K, kBM)) return -1;
     if (!make_tensor_map_bf16(&tmW, W, N, K, K, BN)) return -1;
     GemmArgs g{};
-    g.a_tile_bytes = half_box ? (kBM / 2) * kBK * 2 : 0;
     g.M = T; g.N = N; g.K = K; g.out = (__nv_bfloat16 *)y; g.ldo = N;
     g.residual = (const __nv_bfloat16 *)residual; g.Nq = N; g.Nkv = 0; g.t_cols = kTensorRP;
     g.total_adapter_rows = N; g.status = ctx->d_status; g.item_counters = ctx->d_counts + 10;
@@ -683,8 +673,7 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
     }
     const int items = ((T + kBM - 1) / kBM) * ((N + BN - 1) / BN) + (delta != nullptr ? ctx->max_pairs : 0);
     const bool ok = BN == 256 ? launch_gemm_bn<256>(ctx, tmX, tmW, tmT, tmB, tmA, g, items, s)
-                    : BN == 128 ? launch_gemm_bn<128>(ctx, tmX, tmW, tmX, tmW, tmW, g, items, s)
-                                : launch_gemm_bn<64>(ctx, tmX, tmW, tmX, tmW, tmW, g, items, s);
+                              : launch_gemm_bn<128>(ctx, tmX, tmW, tmX, tmW, tmW, g, items, s);
     return ok ? 1 : -1;
 }
 
