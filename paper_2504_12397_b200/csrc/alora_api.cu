@@ -188,7 +188,7 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
     const size_t Tm = (size_t)c.max_tokens;
     ctx->max_pairs = pair_bound(ctx, c.max_tokens, c.max_requests);
     if (c.dtype == ALORA_DTYPE_BF16)
-        ctx->t_slots = std::max(ctx->max_pairs, 2 * pair_bound(ctx, std::min(c.max_tokens, kSplitTTokens), c.max_requests));
+        ctx->t_slots = std::max(ctx->max_pairs, 3 * pair_bound(ctx, std::min(c.max_tokens, kSplitTTokens), c.max_requests));
     alloc((void **)&ctx->d_adapters, n_ad * sizeof(AdapterDev));
     alloc((void **)&ctx->d_token_req, Tm * 4);
     alloc((void **)&ctx->d_row_adapter, Tm * 4);

@@ -50,8 +50,8 @@ constexpr int kTileRows = 128;
 struct TilePair {
     int32_t tile, adapter;
 };
-// Batches of at most this many rows carry t as the sum of two bf16 values (16 significant bits, for the few rows of a
-// handful of requests), larger ones as one.
+// Batches of at most this many rows carry t as the sum of three bf16 values (all 24 bits of its fp32 value, for the few rows
+// of a handful of requests), larger ones as one.
 constexpr int kSplitTTokens = 1024;
 
 // One unit of attention work: query tokens [q_start, q_start + q_count) of request `req` (flat
@@ -196,7 +196,7 @@ struct alora_ctx {
     float *d_part_o = nullptr, *d_part_ml = nullptr;
     int32_t *d_group_done = nullptr;    // [max_split_rows / 16] finished key ranges per (stream, KV head), at its first partial row / 16
     int32_t max_split_items = 0, max_split_rows = 0, small_max_tokens = 0;
-    void *d_t = nullptr;          // rank-r intermediate: fp32 [max_tokens][3][RP]; bf16 [pair][1 or 2 summands][128][3][RP]
+    void *d_t = nullptr;          // rank-r intermediate: fp32 [max_tokens][3][RP]; bf16 [pair][1 or 3 summands][128][3][RP]
     // few-row projection (batches of <= 128 rows): K-slice partial products and partial shrink results
     float *d_skinny_part = nullptr;   // [skinny_max_items][128][256] fp32
     float *d_skinny_t = nullptr;      // [slices of the q/k/v projection][128][skinny_p_cap][192] fp32

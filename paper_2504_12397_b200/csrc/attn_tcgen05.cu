@@ -245,23 +245,6 @@ __device__ __forceinline__ void exp2_poly2(float &p0, float &p1, float x0, float
     p0 = __uint_as_float(r0 + (n0 << 23));
     p1 = __uint_as_float(r1 + (n1 << 23));
 }
-// 4 x 4 transpose of 16-byte units across the 4 lanes of a quad (l = lane & 3): on entry u[0..3] are the units of
-// this lane's own row; on return u[j] is unit l of the row held by quad lane j.  Every lane of the warp takes part.
-__device__ __forceinline__ void quad_transpose(uint4 (&u)[4], int l) {
-#pragma unroll
-    for (int s = 2; s >= 1; s >>= 1) {
-        const bool up = (l & s) != 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (i & s) continue;
-            const uint4 send = up ? u[i] : u[i ^ s];
-            uint4 recv;
-            recv.x = __shfl_xor_sync(0xffffffffu, send.x, s); recv.y = __shfl_xor_sync(0xffffffffu, send.y, s);
-            recv.z = __shfl_xor_sync(0xffffffffu, send.z, s); recv.w = __shfl_xor_sync(0xffffffffu, send.w, s);
-            if (up) u[i] = recv; else u[i ^ s] = recv;
-        }
-    }
-}
 __device__ __forceinline__ float fast_exp2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -713,7 +696,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                     u[x].x = tc::pack_bf16(o[8 * x], o[8 * x + 1]); u[x].y = tc::pack_bf16(o[8 * x + 2], o[8 * x + 3]);
                     u[x].z = tc::pack_bf16(o[8 * x + 4], o[8 * x + 5]); u[x].w = tc::pack_bf16(o[8 * x + 6], o[8 * x + 7]);
                 }
-                quad_transpose(u, ql);
+                tc::quad_transpose(u, ql);
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
                     if (dst_quad[j]) *reinterpret_cast<uint4 *>(dst_quad[j] + c) = u[j];

@@ -370,12 +370,14 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
                 const bool use = row < a.M && a.row_adapter[row] == g.adapter;
                 const float scale = __int_as_float(a.adapters[g.adapter * a.ad_stride + 1]);
                 __nv_bfloat16 *trow = a.t + ((size_t)g.p0[0] * 128 + r) * a.t_cols;
+                const int rpad = a.adapters[g.adapter * a.ad_stride];
 #pragma unroll 1
                 for (int c = 0; c < a.t_cols; c += 32) {
+                    if ((c & (kTensorRP - 1)) >= rpad) continue;   // (columns that no MMA step reads)
                     uint32_t v[32];
                     tc::tmem_ld_32x32(tmem_base + c + ((uint32_t)(q * 32) << 16), v);
                     tc::tmem_ld_wait();
-                    tc::store_t<32>(reinterpret_cast<float(&)[32]>(v), scale, use, trow + c, nullptr);
+                    tc::store_t_warp(reinterpret_cast<float(&)[32]>(v), scale, use, trow + c, a.t_cols, 1, 0);
                 }
                 tc::tc_fence_before();
                 // publish: the rows are read by other blocks through TMA (async proxy)

@@ -63,7 +63,7 @@ struct GemmArgs {
     const __nv_bfloat16 *b_all;     // the launch's B rows of all adapters, [adapter][N][64] (read for rows of those)
     int32_t *t_ready;               // [pair] epilogue warps that have published their part of t
     __nv_bfloat16 *t;               // [pair][t_parts][128][t_cols]
-    int t_parts;                    // t is the sum of this many bf16 values (1 or 2)
+    int t_parts;                    // t is the sum of this many bf16 values (1 or 3)
     // KV append fused into the epilogue (nullptr: off): columns Nq .. N of row t also go to the paged cache,
     // pool[page][plane][head][row in page][:] with page * page_size + row = slot_map[t] (-1: token rejected, skipped)
     __nv_bfloat16 *kv_pool;
@@ -81,6 +81,7 @@ struct GemmSmem {
     static constexpr int kABytes = kBM * kBK * 2;
     static constexpr int kBBytes = BN * kBK * 2;
     static constexpr int kStageBytes = kABytes + kBBytes;
+    static constexpr int kSummandsPerSlot = kBBytes >= kABytes ? 2 : 1;   // t blocks in a slot without B
     static constexpr int kBarOffset = kStages * kStageBytes;
     static constexpr int kItemRingOffset = kBarOffset + 256;
     static constexpr int kTotal = kItemRingOffset + 128 + 1024;  // barriers, item ring, slack for 1024-byte alignment
@@ -176,11 +177,13 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const int n_shrink = (BN == 256 && a.shrink) ? a.pair_off[a.tile0 + n_m] - p_base : 0;
     const int total = n_shrink + n_m * n_n;
     const int kb_main = (a.K + kBK - 1) / kBK;
+    const int t_slots = a.t_parts > 1 ? 1 + (a.t_parts - 1) / S::kSummandsPerSlot : 1;   // ring slots of a pair
 
     if (warp == 0) {
         if (lane == 0) {
             // ------------------------------ TMA producer ------------------------------
             tc::tma_prefetch_desc(&tmA); tc::tma_prefetch_desc(&tmB);
+            if (a.pairs != nullptr) { tc::tma_prefetch_desc(&tmT); tc::tma_prefetch_desc(&tmL); }
             const uint32_t a_bytes = a.a_tile_bytes ? (uint32_t)a.a_tile_bytes : (uint32_t)S::kABytes;
             uint32_t kc = 0;        // ring slots filled so far
             bool ok = true;
@@ -222,7 +225,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     if (g.shrink) tc::tma_load_2d(sb, &tmS, full_bar(s), kb * kBK, g.adapter * a.t_cols);
                     else tc::tma_load_2d(sb, &tmB, full_bar(s), kb * kBK, n0);
                 }
-                // expand: per adapter of the row tile one K block for each summand of t
+                // expand: per adapter of the row tile a ring slot with the first summand of t and B, and one with the
+                // other two summands, which meet the same B
                 int next_ad = g.p0 < g.p1 ? a.pairs[g.p0].adapter : -1;
                 for (int p = g.p0; p < g.p1 && ok; ++p) {
                     const int adapter = next_ad;
@@ -239,13 +243,16 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         fence_proxy_async_global();
                     }
                     const int blk = n0 < a.Nq ? 0 : (n0 < a.Nq + a.Nkv ? 1 : 2);
-                    for (int part = 0; part < a.t_parts; ++part, ++kc) {
+                    for (int slot = 0; slot < t_slots; ++slot, ++kc) {
                         const int s = kc % kStages;
                         if (!tc::mbar_wait(empty_bar(s), ((kc / kStages) & 1) ^ 1, abort_flag)) { ok = false; break; }
                         const uint32_t sa = smem_base + s * S::kStageBytes, sb = sa + S::kABytes;
-                        tc::mbar_arrive_expect_tx(full_bar(s), S::kStageBytes);
+                        const int part = slot * (slot > 0 ? S::kSummandsPerSlot : 1) - (slot > 0 ? S::kSummandsPerSlot - 1 : 0);
+                        const bool two = slot > 0 && S::kSummandsPerSlot == 2;
+                        tc::mbar_arrive_expect_tx(full_bar(s), slot == 0 ? S::kStageBytes : (two ? 2 : 1) * S::kABytes);
                         tc::tma_load_2d(sa, &tmT, full_bar(s), blk * kTensorRP, (p * a.t_parts + part) * kBM);
-                        tc::tma_load_2d(sb, &tmL, full_bar(s), 0, adapter * a.total_adapter_rows + n0);
+                        if (slot == 0) tc::tma_load_2d(sb, &tmL, full_bar(s), 0, adapter * a.total_adapter_rows + n0);
+                        else if (two) tc::tma_load_2d(sb, &tmT, full_bar(s), blk * kTensorRP, (p * a.t_parts + part + 1) * kBM);
                     }
                 }
             }
@@ -300,17 +307,23 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 for (int p = g.p0; p < g.p1 && ok; ++p) {
                     const int at = p - g.p0;
                     const int steps = at < 32 ? __shfl_sync(0xffffffffu, my_steps, at) : rank_steps(a, a.pairs[p].adapter);
-                    for (int part = 0; part < a.t_parts; ++part, ++kc) {
-                        const int s = kc % kStages;
-                        if (!wait_all(full_bar(s), (kc / kStages) & 1)) { ok = false; break; }
+                    uint64_t db = 0;
+                    for (int slot = 0; slot < t_slots; ++slot) {
+                        const int s = (kc + slot) % kStages;
+                        if (!wait_all(full_bar(s), ((kc + slot) / kStages) & 1)) { ok = false; break; }
                         tc::tc_fence_after();
                         const uint32_t sa = smem_base + s * S::kStageBytes, sb = sa + S::kABytes;
-                        const uint64_t da = tc::smem_desc_k_sw128(sa), db = tc::smem_desc_k_sw128(sb);
+                        const uint64_t da = tc::smem_desc_k_sw128(sa), db2 = tc::smem_desc_k_sw128(sb);
+                        if (slot == 0) db = db2;
                         if (leader) {
                             for (int k = 0; k < steps; ++k) tc::mma_bf16(d_tmem, da + 2 * k, db + 2 * k, idesc, 1u);
-                            tc::mma_commit(empty_bar(s));
+                            if (slot > 0 && S::kSummandsPerSlot == 2)   // (the third summand lies where B lies in the first slot)
+                                for (int k = 0; k < steps; ++k) tc::mma_bf16(d_tmem, db2 + 2 * k, db + 2 * k, idesc, 1u);
                         }
                     }
+                    if (!ok) break;
+                    for (int slot = 0; slot < t_slots; ++slot, ++kc)   // B is read up to the last summand
+                        if (leader) tc::mma_commit(empty_bar(kc % kStages));
                 }
                 if (!ok) break;
                 if (leader) tc::mma_commit(accf_bar(acc));      // accumulator complete
@@ -342,13 +355,14 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 const float scale = __int_as_float(a.adapters[g.adapter * a.ad_stride + 1]);
                 const bool use = row_ok && a.row_adapter[row] == g.adapter;
                 __nv_bfloat16 *trow = a.t + ((size_t)g.p0 * a.t_parts * kBM + q * 32 + lane) * a.t_cols;
-                __nv_bfloat16 *tlow = a.t_parts > 1 ? trow + (size_t)kBM * a.t_cols : nullptr;
+                const int rpad = a.adapters[g.adapter * a.ad_stride];
 #pragma unroll 1
                 for (int c = 0; c < a.t_cols && c < BN; c += 32) {
+                    if ((c & (kTensorRP - 1)) >= rpad) continue;   // (columns that no MMA step reads)
                     uint32_t v[32];
                     tc::tmem_ld_32x32(tmem_base + acc * BN + c + ((uint32_t)(q * 32) << 16), v);
                     tc::tmem_ld_wait();
-                    tc::store_t<32>(reinterpret_cast<float(&)[32]>(v), scale, use, trow + c, tlow ? tlow + c : nullptr);
+                    tc::store_t_warp(reinterpret_cast<float(&)[32]>(v), scale, use, trow + c, a.t_cols, a.t_parts, kBM * a.t_cols);
                 }
                 tc::tc_fence_before();
                 // publish: the rows are read by other blocks through TMA (async proxy)
@@ -372,7 +386,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     odd.t = a.t + ((size_t)p * a.t_parts * kBM + q * 32 + lane) * a.t_cols;
                     odd.b = a.b_all + (size_t)k * a.N * kTensorRP;
                     odd.n = a.adapters[k * a.ad_stride];
-                    odd.low = a.t_parts > 1 ? kBM * a.t_cols : 0;
+                    odd.parts = a.t_parts; odd.part_stride = kBM * a.t_cols;
                 }
             }
             __nv_bfloat16 *orow = a.out + (size_t)row * a.ldo + n0;
@@ -588,7 +602,7 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
     if (!make_tensor_map_bf16(&tmTt, ctx->d_t, (uint64_t)ctx->t_slots * kBM, 3 * kTensorRP, 3 * kTensorRP, kBM)) return -1;
     const TcLayerMaps &lm = ctx->tc_maps[layer];
     const AdapterDev *ads = ctx->d_adapters + (size_t)layer * ctx->cfg.max_adapters;
-    const int t_parts = T <= kSplitTTokens ? 2 : 1, max_pairs = have_adapters ? pair_bound(ctx, T, R) : 0;
+    const int t_parts = T <= kSplitTTokens ? 3 : 1, max_pairs = have_adapters ? pair_bound(ctx, T, R) : 0;
     const int proj_items = ((T + kBM - 1) / kBM) * ((d.N + BN - 1) / BN);
     const bool fuse_shrink = have_adapters && BN == 256 && !shrink_apart(ctx, T, R, proj_items);
     int n = 0;

@@ -199,7 +199,7 @@ shrink_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                 }
             const int blk = u * 8 / rpad;
             __nv_bfloat16 *orow = a.t + ((size_t)blockIdx.y * a.t_parts * kShrinkBM + r) * kShrinkBN + blk * kRankPadMax + u * 8 - blk * rpad;
-            tc::store_t<8>(acc, scale, use, orow, a.t_parts > 1 ? orow + (size_t)kShrinkBM * kShrinkBN : nullptr);
+            tc::store_t8(acc, scale, use, orow, a.t_parts, kShrinkBM * kShrinkBN);
         }
     }
 

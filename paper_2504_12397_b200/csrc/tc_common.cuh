@@ -212,38 +212,74 @@ __device__ __forceinline__ void item_counter_release(int32_t *counters, int32_t 
     }
 }
 
-// t of a (row tile, adapter) pair as the operand of the expand step: `n` (a multiple of 8) fp32 columns of one row, times
-// the adapter's scale, rounded to bf16; with `lo` also what the rounding left, rounded again (their sum has 16
-// significant bits).  A row that does not use the adapter gets zeros.
-template <int n>
-__device__ __forceinline__ void store_t(const float (&v)[n], float scale, bool use, __nv_bfloat16 *hi, __nv_bfloat16 *lo) {
+// t of a (row tile, adapter) pair as the operand of the expand step: fp32 sums times the adapter's scale, as one bf16 value or as the
+// sum of three (24 significant bits: nothing of the fp32 value is lost).  A row that does not use the adapter gets zeros.
+// Summand `part` of 8 values; takes it off them.
+__device__ __forceinline__ uint4 take_summand8(float (&v)[8]) {
+    uint32_t h[4];
 #pragma unroll
-    for (int j = 0; j < n; j += 8) {
-        uint32_t h[4], l[4];
+    for (int e = 0; e < 4; ++e) {
+        const __nv_bfloat162 r = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
+        h[e] = *reinterpret_cast<const uint32_t *>(&r);
+        v[2 * e] -= __low2float(r); v[2 * e + 1] -= __high2float(r);
+    }
+    return make_uint4(h[0], h[1], h[2], h[3]);
+}
+// 8 columns of one row; the summands lie `part_stride` elements apart.
+__device__ __forceinline__ void store_t8(float (&v)[8], float scale, bool use, __nv_bfloat16 *dst, int parts, int part_stride) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float a = use ? v[j + 2 * e] * scale : 0.f, b = use ? v[j + 2 * e + 1] * scale : 0.f;
-            const __nv_bfloat162 r = __floats2bfloat162_rn(a, b);
-            const __nv_bfloat162 q = __floats2bfloat162_rn(a - __low2float(r), b - __high2float(r));
-            h[e] = *reinterpret_cast<const uint32_t *>(&r);
-            l[e] = *reinterpret_cast<const uint32_t *>(&q);
+    for (int e = 0; e < 8; ++e) v[e] = use ? v[e] * scale : 0.f;
+    for (int p = 0; p < parts; ++p) *reinterpret_cast<uint4 *>(dst + (size_t)p * part_stride) = take_summand8(v);
+}
+// 4 x 4 transpose of 16-byte units across the 4 lanes of a quad (l = lane & 3): on entry u[0..3] are the units of
+// this lane's own row; on return u[j] is unit l of the row held by quad lane j.  Every lane of the warp takes part.
+__device__ __forceinline__ void quad_transpose(uint4 (&u)[4], int l) {
+#pragma unroll
+    for (int s = 2; s >= 1; s >>= 1) {
+        const bool up = (l & s) != 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (i & s) continue;
+            const uint4 send = up ? u[i] : u[i ^ s];
+            uint4 recv;
+            recv.x = __shfl_xor_sync(0xffffffffu, send.x, s); recv.y = __shfl_xor_sync(0xffffffffu, send.y, s);
+            recv.z = __shfl_xor_sync(0xffffffffu, send.z, s); recv.w = __shfl_xor_sync(0xffffffffu, send.w, s);
+            if (up) u[i] = recv; else u[i ^ s] = recv;
         }
-        *reinterpret_cast<uint4 *>(hi + j) = make_uint4(h[0], h[1], h[2], h[3]);
-        if (lo) *reinterpret_cast<uint4 *>(lo + j) = make_uint4(l[0], l[1], l[2], l[3]);
+    }
+}
+// 32 columns of the 32 rows of a warp, a row per lane (`dst`: this lane's row, `pitch` elements to the next one).  Every other
+// block of the launch that meets the pair waits for these stores: transposed in quads they are 64 contiguous bytes a
+// row and instruction (two summands of 192 columns as 16 bytes a row took 6.2 us).
+__device__ __forceinline__ void store_t_warp(float (&v)[32], float scale, bool use, __nv_bfloat16 *dst, int pitch, int parts,
+                                             int part_stride) {
+    const int l = threadIdx.x & 3;
+#pragma unroll
+    for (int e = 0; e < 32; ++e) v[e] = use ? v[e] * scale : 0.f;
+    __nv_bfloat16 *quad = dst - l * pitch + l * 8;
+#pragma unroll 1
+    for (int p = 0; p < parts; ++p) {
+        uint4 u[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) u[j] = take_summand8(reinterpret_cast<float(&)[8]>(v[8 * j]));
+        quad_transpose(u, l);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4 *>(quad + (size_t)p * part_stride + j * pitch) = u[j];
     }
 }
 
 // Delta of one row whose adapter's B holds an Inf or NaN (TilePair), on the CUDA cores.  The matrix products of a row tile
-// leave such a pair out: the zeros of the other rows would meet the Inf.  `t` is the row's part of the pair (two summands
-// `low` elements apart, 0: one), `b` the adapter's B row of output column 0 of the launch, `cols` the columns of t per block.
+// leave such a pair out: the zeros of the other rows would meet the Inf.  `t` is the row's part of the pair (its summands
+// `part_stride` elements apart), `b` the adapter's B row of output column 0 of the launch.
 struct OddRow {
     const __nv_bfloat16 *t = nullptr, *b = nullptr;
-    int n = 0, low = 0;   // padded rank, 0: nothing to do for this row
+    int n = 0, parts = 1, part_stride = 0;   // n: padded rank, 0: nothing to do for this row
     __device__ __forceinline__ void add8(float (&f)[8], int col, int blk) const {   // output columns col .. col + 7 of block blk
         const __nv_bfloat16 *tb = t + blk * kRankPadMax, *bc = b + (size_t)col * kRankPadMax;
 #pragma unroll 1
         for (int i = 0; i < n; ++i) {
-            const float ti = __bfloat162float(__ldcg(tb + i)) + (low ? __bfloat162float(__ldcg(tb + low + i)) : 0.f);
+            float ti = 0.f;
+            for (int p = parts - 1; p >= 0; --p) ti += __bfloat162float(__ldcg(tb + (size_t)p * part_stride + i));
 #pragma unroll
             for (int e = 0; e < 8; ++e) f[e] = fmaf(ti, __bfloat162float(bc[e * kRankPadMax + i]), f[e]);
         }

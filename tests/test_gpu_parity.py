@@ -876,3 +876,43 @@ def test_fp32_projection_of_more_rows_than_one_grid_dimension_holds_tiles(oracle
         assert bool(torch.isfinite(out).all())
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("n_req,each,heads,kv_heads,slots", [(9, 12, 4, 2, 3), (9, 12, 4, 2, 5), (100, 1, 16, 4, 200), (20, 30, 4, 2, 3),
+                                                             (20, 30, 4, 2, 5), (47, 17, 4, 2, 5), (11, 50, 4, 1, 5)])
+def test_projection_of_at_most_1024_rows_loses_nothing_of_t(n_req, each, heads, kv_heads, slots):
+    """Whole numbers for which every product and sum is exact in 32 bits, t = A x taking up to 22 of them; the adapters
+    subtract one, two and three times rows of the base product.  On every route of few rows (one launch, two, row tiles of
+    64, 256 and 128 columns) the result is the exact one, rounded once: t as one or two bf16 values is off by whole numbers
+    where the difference is zero."""
+    shape = wl.LayerShape(hidden=512, n_q_heads=heads, n_kv_heads=kv_heads, head_dim=128, page_size=16, dtype="bf16")
+    rng = np.random.default_rng(91 + n_req)
+    whole = lambda *d: rng.integers(-255, 256, d).astype(np.float32)  # noqa: E731
+    w = whole(shape.N, shape.hidden)
+    starts = (0, shape.Nq, shape.Nq + shape.Nkv)
+    ads = []
+    for times in (1, 2, 3):
+        a = wl.make_adapter(shape, 64, rng)
+        for name, s in zip("qkv", starts):
+            b_m = np.zeros_like(getattr(a, "B" + name))
+            b_m[:64] = -times * np.eye(64, dtype=np.float32)
+            setattr(a, "B" + name, b_m)
+            setattr(a, "A" + name, w[s:s + 64].copy())
+        ads.append(a)
+    ids = [(r % 4) - 1 for r in range(n_req)]
+    b = wl.make_batch(shape, [40] * n_req, [each] * n_req, ids, rng)
+    b.hidden[:] = whole(b.T, shape.hidden)
+    y = b.hidden.astype(np.int64) @ w.astype(np.int64).T
+    assert np.abs(y).max() * 4 < 2 ** 24
+    for s in starts:
+        y[:, s:s + 64] *= (1 - (np.repeat(np.array(ids), each) + 1))[:, None]
+    g = hp.GpuLayers(shape, [dict(wqkv=w)], [ads], b.T, b.R, n_adapters=slots)
+    try:
+        d = hp.DevBatch(b, shape.dtype)
+        out = g.empty(b.T, shape.N)
+        ab.alora_project_qkv(g.ctx, 0, ab.MODE_ALORA, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, d.T, d.R, out)
+        assert g.status() == 0
+        got = hp.to_host(out)
+    finally:
+        g.close()
+    assert np.array_equal(got, wl.bf16_round(y.astype(np.float32)))
