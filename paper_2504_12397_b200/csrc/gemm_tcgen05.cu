@@ -376,19 +376,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 ++it;
                 continue;
             }
-            tc::OddRow odd;
-            if (any_odd && row_ok) {
-                const int k = a.row_adapter[row];
-                int p = k >= 0 && a.adapters[k * a.ad_stride + 2] ? g.p0 : g.p1;
-                while (p < g.p1 && a.pairs[p].adapter != k) ++p;
-                if (p < g.p1) {
-                    if (a.shrink) ld_acquire(a.t_ready + p);   // (complete since the tile's K blocks were loaded; orders the reads)
-                    odd.t = a.t + ((size_t)p * a.t_parts * kBM + q * 32 + lane) * a.t_cols;
-                    odd.b = a.b_all + (size_t)k * a.N * kTensorRP;
-                    odd.n = a.adapters[k * a.ad_stride];
-                    odd.parts = a.t_parts; odd.part_stride = kBM * a.t_cols;
-                }
-            }
             __nv_bfloat16 *orow = a.out + (size_t)row * a.ldo + n0;
             const __nv_bfloat16 *rrow = a.residual ? a.residual + (size_t)row * a.ldo + n0 : nullptr;
             // fused KV append: where this row's k / v columns go in the page pool
@@ -401,42 +388,70 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     if (kv_page >= a.kv_num_pages) { report(a.status, ALORA_ERR_PAGE_RANGE); kv_page = -1; }
                 }
             }
+            const uint32_t acc_addr = tmem_base + acc * BN + ((uint32_t)(q * 32) << 16);
+            auto put8 = [&](int c, float (&f)[8]) {   // columns c .. c + 7 of the tile
+                if (rrow) {
+                    const uint4 rv = *reinterpret_cast<const uint4 *>(rrow + c);
+                    const uint32_t rw[4] = {rv.x, rv.y, rv.z, rv.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const __nv_bfloat162 b2 = *reinterpret_cast<const __nv_bfloat162 *>(&rw[e]);
+                        f[2 * e] += __low2float(b2);
+                        f[2 * e + 1] += __high2float(b2);
+                    }
+                }
+                uint4 o;
+                o.x = tc::pack_bf16(f[0], f[1]); o.y = tc::pack_bf16(f[2], f[3]);
+                o.z = tc::pack_bf16(f[4], f[5]); o.w = tc::pack_bf16(f[6], f[7]);
+                *reinterpret_cast<uint4 *>(orow + c) = o;
+                const int kc = n0 + c - a.Nq;   // column inside [k | v]
+                if (kv_page >= 0 && kc >= 0) {
+                    const int plane = kc >= a.Nkv ? 1 : 0, c2 = kc - plane * a.Nkv;
+                    const int head = c2 >> a.kv_hd_shift, dd = c2 & ((1 << a.kv_hd_shift) - 1);
+                    __nv_bfloat16 *dst = a.kv_pool +
+                        ((((size_t)kv_page * 2 + plane) * a.kv_heads + head) * a.kv_page_size + kv_row << a.kv_hd_shift) + dd;
+                    *reinterpret_cast<uint4 *>(dst) = o;
+                }
+            };
+            bool own_pass = false;   // the row's adapter has a B with an Inf or NaN
+            if (any_odd && row_ok && g.p0 < g.p1) {
+                const int k = a.row_adapter[row];
+                own_pass = k >= 0 && a.adapters[k * a.ad_stride + 2] != 0;
+            }
 #pragma unroll 1
             for (int c = 0; c < BN; c += 32) {
                 uint32_t v[32];
-                tc::tmem_ld_32x32(tmem_base + acc * BN + c + ((uint32_t)(q * 32) << 16), v);
+                tc::tmem_ld_32x32(acc_addr + c, v);
                 tc::tmem_ld_wait();
-                if (row_ok) {
+                if (row_ok && !own_pass) {
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         if (n0 + c + 8 * j >= a.N) break;
-                        float f[8];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[8 * j + e]);
-                        if (odd.n) odd.add8(f, n0 + c + 8 * j, n0 < a.Nq ? 0 : (n0 < a.Nq + a.Nkv ? 1 : 2));
-                        if (rrow) {
-                            const uint4 rv = *reinterpret_cast<const uint4 *>(rrow + c + 8 * j);
-                            const uint32_t rw[4] = {rv.x, rv.y, rv.z, rv.w};
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const __nv_bfloat162 b2 = *reinterpret_cast<const __nv_bfloat162 *>(&rw[e]);
-                                f[2 * e] += __low2float(b2);
-                                f[2 * e + 1] += __high2float(b2);
-                            }
-                        }
-                        uint4 o;
-                        o.x = tc::pack_bf16(f[0], f[1]); o.y = tc::pack_bf16(f[2], f[3]);
-                        o.z = tc::pack_bf16(f[4], f[5]); o.w = tc::pack_bf16(f[6], f[7]);
-                        *reinterpret_cast<uint4 *>(orow + c + 8 * j) = o;
-                        const int kc = n0 + c + 8 * j - a.Nq;   // column inside [k | v]
-                        if (kv_page >= 0 && kc >= 0) {
-                            const int plane = kc >= a.Nkv ? 1 : 0, c2 = kc - plane * a.Nkv;
-                            const int head = c2 >> a.kv_hd_shift, dd = c2 & ((1 << a.kv_hd_shift) - 1);
-                            __nv_bfloat16 *dst = a.kv_pool +
-                                ((((size_t)kv_page * 2 + plane) * a.kv_heads + head) * a.kv_page_size + kv_row << a.kv_hd_shift) + dd;
-                            *reinterpret_cast<uint4 *>(dst) = o;
-                        }
+                        put8(c + 8 * j, reinterpret_cast<float(&)[8]>(v[8 * j]));
                     }
+                }
+            }
+            if (__any_sync(0xffffffffu, own_pass)) {
+                tc::OddRow odd;
+                if (own_pass) {
+                    const int k = a.row_adapter[row];
+                    int p = g.p0;
+                    while (p + 1 < g.p1 && a.pairs[p].adapter != k) ++p;
+                    if (a.shrink) ld_acquire(a.t_ready + p);   // (complete since the tile's K blocks were loaded; orders the reads)
+                    odd.t = a.t + ((size_t)p * a.t_parts * kBM + q * 32 + lane) * a.t_cols;
+                    odd.b = a.b_all + (size_t)k * a.N * kTensorRP;
+                    odd.n = a.adapters[k * a.ad_stride];
+                    odd.parts = a.t_parts; odd.part_stride = kBM * a.t_cols;
+                }
+                const int blk = n0 < a.Nq ? 0 : (n0 < a.Nq + a.Nkv ? 1 : 2);
+#pragma unroll 1
+                for (int c = 0; c < BN && n0 + c < a.N; c += 8) {
+                    uint32_t v[8];
+                    tc::tmem_ld_32x8(acc_addr + c, v);
+                    tc::tmem_ld_wait();
+                    if (!own_pass) continue;
+                    odd.add8(reinterpret_cast<float(&)[8]>(v), n0 + c, blk);
+                    put8(c, reinterpret_cast<float(&)[8]>(v));
                 }
             }
             tc::tc_fence_before();
