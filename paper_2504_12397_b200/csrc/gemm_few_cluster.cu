@@ -509,11 +509,16 @@ static bool few_plan(const alora_ctx *ctx, int T, int R, int N, int K, bool lora
         const long cost = (long)((n_tiles * ks + ctx->sm_count - 1) / ctx->sm_count) * (bn + rs / 2) * ((kb_total + ks - 1) / ks);
         if (a.bn == 0 || cost < best) { best = cost; a.bn = bn; a.ksplit = ks; }
     }
-    // several row tiles only where that still splits K: each block takes in 48 KB per K block at 75 bytes / ns, so that one
-    // block per 128 x 256 tile takes 40 us at K = 4096 however few tiles there are (194 rows: 44 us on the dense route, 31
-    // here), and with all SMs busy the dense route's kernel is as fast
+    // several row tiles only where that still splits K: one block per 128 x 256 tile takes 24 us at K = 4096 when there are 48
+    // of them and 31 when there are 144 (base prefill of 192 rows: a call 57.5 us on the row tiles, 47.5 here), and with all SMs
+    // busy the row tiles' kernel is as fast
     if (a.n_rt > 1 && a.ksplit < 2) return false;
     const int p_cap = lora ? std::min(std::min(ctx->cfg.max_adapters, T), R) : 0, rank = (ctx->cfg.max_rank + 15) / 16 * 16;
+    // ... and, with adapters, where the delta is small: a block's share of the columns x rank multiply-adds a row on the CUDA
+    // cores, while more row tiles fill the other route's SMs.  Layer calls here / on the row tiles, us, by columns x rank x
+    // row tiles: 51 x 64 x 2 44 .. 47 / 49 .. 53; 64 x 32 x 3 48 / 51; 128 x 32 x 2 (hidden 4096) 65.4 / 66.0; 128 x 16 x 4 51.4 / 51.4;
+    // 128 x 16 x 5 52 / 51; 64 x 64 x 3 54.2 / 53.3; 128 x 32 x 3 71 / 69; 128 x 64 x 2 74 .. 78 / 66 .. 70; 128 x 64 x 4 66 / 53.
+    if (a.n_rt > 1 && lora && a.bn / a.ksplit * rank * a.n_rt > 8192) return false;
     const int chunk_cap = p_cap * (rank / 16);
     if (lora && (Nq % a.bn != 0 || Nkv % a.bn != 0 || ctx->cfg.max_adapters > 1024 || chunk_cap > kFcMaxChunks)) return false;
     // shared memory: the ring, over it later the partial products, t and B; then the barriers
@@ -521,8 +526,8 @@ static bool few_plan(const alora_ctx *ctx, int T, int R, int N, int K, bool lora
     const int b_bytes = lora ? (a.bn / 8 + a.ksplit - 1) / a.ksplit * 8 * chunk_cap * 32 + 16 * p_cap : 0;
     // (a second pass over x brings the A rows where W was)
     const int w_bytes = a.bn * kFcBK * 2, a_bytes = chunk_cap * kFcChunkBytes, nkb = (kb_total + a.ksplit - 1) / a.ksplit;
-    // (128 rows with 13 K blocks a slice: 83.2 -> 80.1 us for the call; with 32 K blocks the second pass costs 4 us more than the
-    // wait it saves)
+    // (what the second pass costs against the wait it saves, by the bytes of x in a slice: up to 208 KB 0 .. 3 % of the call
+    // saved, 1 .. 128 rows, 13 K blocks; 256 KB, 384 rows of a narrow layer 3 .. 5 % lost; 512 KB, 140 .. 384 rows 3 .. 4 % lost)
     a.x_early = x_early && (!lora || (long)rs * kFcBK * 2 * nkb <= 224 * 1024) ? 1 : 0;
     const bool second_pass = a.x_early && lora;
     a.stage_bytes = rs * kFcBK * 2 + (second_pass ? std::max(w_bytes, a_bytes) : w_bytes + a_bytes);
