@@ -594,9 +594,13 @@ int launch_linear256_tc(alora_ctx *ctx, const void *x, const void *W, int T, int
     constexpr int BN = 256;
     const int n_n = (N + BN - 1) / BN, G = ctx->sm_count;
     const int items = ((T + 255) / 256) * n_n, items128 = ((T + 127) / 128) * n_n;
-    // Rounds over the blocks x cycles of a tile's K block: 1230 here (0.83 of the tensor pipe), 790 for the 128 x 256 tile
-    // (shared-memory fill rate).
-    const long long here = (long long)((items + G - 1) / G) * 1230, other = (long long)((items128 + G - 1) / G) * 790;
+    // Rounds over the blocks x cycles of a tile's K block: 1230 here (0.83 of the tensor pipe), 790 for the 128 x 256 tile.  That
+    // kernel walks the column tiles of a row tile first, so a W that L2 does not hold is streamed from HBM (3400 bytes a cycle)
+    // in every round.  Dense matrices of two 8B layers, us, 128-row tiles for all / for o_proj and down only: 384 rows 427 / 388,
+    // 640 rows 650 / 577, 896 rows 803 / 687; this kernel for all / for gate and up only: 1152 rows 820 / 703, 1280 rows 862 / 937.
+    const long long rounds128 = (items128 + G - 1) / G;
+    const long long w_cycles = (long long)N * K * 2 > (64ll << 20) ? (n_n >= G ? (T + 127) / 128 : rounds128) * N * (2 * kBKp) / 3400 : 0;
+    const long long here = (long long)((items + G - 1) / G) * 1230, other = std::max(rounds128 * 790, w_cycles);
     if (T <= 256 || K % 8 != 0 || N % 8 != 0 || here > other) return 0;
     CUtensorMap tmX, tmW, tmT, tmA, tmB;
     if (!make_tensor_map_bf16(&tmX, x, T, K, K, 128)) return -1;
