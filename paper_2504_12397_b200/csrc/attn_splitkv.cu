@@ -236,7 +236,7 @@ attn_splitkv_kernel(const __grid_constant__ CUtensorMap tmKV, const SplitArgs a)
             if (!ok || it < 0) break;
             const AttnSplitWork w = it == (int)blockIdx.x ? first : a.items[it];
             const int n_st = (w.kv_end - w.kv_start + kSkStageKeys - 1) / kSkStageKeys, claim_at = max(0, n_st - 3);
-            if (lane == 0 && n_st <= 0) it_next = (int)gridDim.x + atomicAdd(a.work_counter, 1);   // (an empty share of the own keys)
+            if (lane == 0 && n_st <= 0) it_next = (int)gridDim.x + atomicAdd(a.work_counter, 1);   // (the list has no empty ranges; one would otherwise be taken for ever)
             // Window of the request's block-table row: lane l holds entry win0 + l (win0 a multiple of 32; 32 entries
             // cover a whole number of 64-key stages, and key ranges start at multiples of 64).  A table entry is a
             // dependent load from global memory that would otherwise sit in front of every stage's copies; the

@@ -17,7 +17,8 @@
 //   without one add nothing, so they go through exactly the arithmetic of a base-only call (Prop. 1: gated-off rows
 //   are bit-identical).  bf16 store; the k / v columns also go to the row's cache slot.
 // No atomics in the arithmetic, fixed summation orders: results are run-to-run deterministic.  The route is chosen
-// by the row count alone, never by the mode or the adapters.
+// by the row count and by what the context may register, never by the mode.  (Layers without adapters come here only on a
+// device where the cluster kernel cannot run.)
 #include <algorithm>
 
 #include "alora_internal.h"

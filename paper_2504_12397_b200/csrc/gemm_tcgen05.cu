@@ -542,7 +542,7 @@ int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T,
                            void *kv_pool, int num_pages);  // gemm_pair_tcgen05.cu
 
 // Whether the shrink of a launch of `items` projection items is a kernel of its own.  As leading items of the projection
-// it is free unless it makes another round over the blocks of a launch of one or two rounds (a round is 27 us at
+// it is free unless it makes another round over the blocks of a launch of one or two rounds (a round is 24 .. 31 us at
 // hidden 4096, a kernel for a few pairs 8 us); a kernel for many pairs takes rounds of its own.  The number of pairs is
 // an upper bound from the row and request counts, so that the choice does not depend on the mode.
 bool shrink_apart(const alora_ctx *ctx, int T, int R, int items) {

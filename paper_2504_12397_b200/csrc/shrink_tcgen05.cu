@@ -7,7 +7,7 @@
 // partial tile into its shared memory, and after a cluster barrier reduces its share of the tile's columns over all
 // blocks' shared memory (distributed shared memory loads) in the fixed order 0, 1, ....  The order does not depend on
 // timing, so the result is run-to-run deterministic.
-// Bound by what a block takes in (75 bytes / ns of operands, 20 of other blocks' shared memory) and by the rounds of clusters:
+// Bound by what a block takes in (operands by TMA, 20 bytes / ns of other blocks' shared memory) and by the rounds of clusters:
 // only the padded rank's rows of A are loaded, multiplied and reduced, and where more pairs are possible than clusters
 // of 8 fit on the device (15), clusters are of 4 (33 fit).  48 requests over four adapters of rank 8 .. 64, 24 pairs at
 // hidden 4096: 32 -> 18 us against 192 rows of A for each and 8 blocks.

@@ -52,14 +52,15 @@ def _run_stack(g, b, mode=ab.MODE_ALORA):
     return hp.to_host(hout), pools
 
 
-def test_two_layer_stack_with_mlp_adapters(oracle64):
+@pytest.mark.parametrize("S,a0", [([70, 33, 20, 45], 41), ([30, 23, 20, 35], 11)])
+def test_two_layer_stack_with_mlp_adapters(oracle64, S, a0):
     """Two decoder layers, four requests on two adapters (ranks 16 / 8 on q/k/v, 16 / 32 with scales 1 / 0.5 on the
-    MLP) and the base model; one gate opens in the middle of its request's new tokens, and the 64-row tiles of the
-    expand step hold rows of several requests.  Hidden states out of the stack and both layers' caches against the
-    oracle; the oracle WITHOUT the MLP adapters is far outside the tolerance, so the comparison sees them."""
+    MLP) and the base model; one gate opens in the middle of its request's new tokens, and the row tiles (of the dense
+    kernels, or at 108 rows the 64-row tiles of the separate expand step) hold rows of several requests.  Hidden states
+    out of the stack and both layers' caches against the oracle; the oracle WITHOUT the MLP adapters is far outside the tolerance, so the comparison sees them."""
     rng = np.random.default_rng(41)
     layers, ads, mlps = _weights(rng, 2)
-    S, ids, a_req = [70, 33, 20, 45], [0, -1, 1, 0], [41, 0, 0, 0]
+    ids, a_req = [0, -1, 1, 0], [a0, 0, 0, 0]
     b = wl.make_batch(SHAPE, [0] * 4, S, ids, rng, activation_offsets=a_req, shuffle_pages=True)
     g = hp.GpuLayers(SHAPE, layers, ads, 512, 8, mlp_adapters_per_layer=mlps)
     try:
@@ -73,7 +74,7 @@ def test_two_layer_stack_with_mlp_adapters(oracle64):
                 hp.assert_close(kv[r][0], blks[l]["K"][r], 2e-2, f"layer {l} keys of request {r}", block=SHAPE.head_dim)
                 hp.assert_close(kv[r][1], blks[l]["V"][r], 2e-2, f"layer {l} values of request {r}", block=SHAPE.head_dim)
         plain, _ = _oracle_stack(oracle64, layers, ads, mlps, b, with_mlp=False)
-        open_rows = np.concatenate([np.arange(41, 70), np.arange(103, 123), np.arange(123, 168)])
+        open_rows = np.concatenate([np.arange(a0, S[0]), np.arange(S[0] + S[1], b.T)])
         assert hp.rel_err(got[open_rows], plain[open_rows]) > 0.1
     finally:
         g.close()
@@ -81,8 +82,8 @@ def test_two_layer_stack_with_mlp_adapters(oracle64):
 
 def test_closed_gate_rows_keep_the_bits_of_the_base_mlp(oracle64):
     """One layer: the rows before the activation offset, and the rows of a base-model request, come out of the stack
-    with exactly the bits of an ALORA_MODE_BASE call on the same inputs (the expand step neither reads nor writes
-    them); the open rows differ."""
+    with exactly the bits of an ALORA_MODE_BASE call on the same inputs (the adapters of their row tile add exact zeros
+    to them); the open rows differ."""
     rng = np.random.default_rng(42)
     layers, ads, mlps = _weights(rng, 1)
     S, ids, a_req = [90, 50, 40], [0, -1, 1], [37, 0, 40]          # request 2's gate never opens
@@ -116,7 +117,7 @@ def test_full_lora_mode_opens_the_mlp_gate_everywhere(oracle64):
 
 def test_decode_steps_with_mlp_adapters_match_the_prefill_rows(oracle64):
     """Two layers: a prefill of all but the last two tokens, then two decode steps through alora_decode_stack (few
-    rows: the shrink runs on the weight-streaming GEMM pair); the produced rows equal the oracle's rows of the whole
+    rows: shrink and expand are kernels of their own); the produced rows equal the oracle's rows of the whole
     sequences.  Adapter 1 has no MLP part on layer 1: its rows there get the q/k/v deltas only."""
     rng = np.random.default_rng(44)
     layers, ads, mlps = _weights(rng, 2)

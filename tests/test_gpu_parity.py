@@ -279,8 +279,8 @@ def test_projection_of_many_rows_two_row_tiles_per_block(oracle64):
 
 
 def test_projection_row_wise_route_many_short_requests(oracle64):
-    """Many requests of 1..9 new tokens over different adapters and the base model, some gated off: the row
-    tiles would hold a few rows each, so the batch takes the row-wise delta route."""
+    """Many requests of 1..9 new tokens over different adapters and the base model, some gated off: every row tile
+    holds rows of all four adapters, a few each."""
     rng = np.random.default_rng(44)
     w = wl.make_wqkv(MID, rng)
     ads = _boosted_adapters(MID, rng, ((8, 1.0), (64, 0.5), (32, 2.0), (16, 1.0)))
@@ -296,7 +296,7 @@ def test_projection_row_wise_route_many_short_requests(oracle64):
 @pytest.mark.parametrize("n_req,each", [(129, 1), (140, 1), (33, 5), (257, 4)])
 def test_projection_row_tiles_with_many_adapters(oracle64, n_req, each):
     """More requests and more adapters in a row tile than a warp has lanes, a last tile of one row, requests across the
-    tile boundary, with t in two summands (up to 1024 rows) and in one (257 x 4 rows)."""
+    tile boundary, with t in three summands (up to 1024 rows) and in one (257 x 4 rows)."""
     rng = np.random.default_rng(49)
     w = wl.make_wqkv(MID, rng)
     ads = _boosted_adapters(MID, rng, tuple((8, 0.5 + 0.1 * (i % 7)) for i in range(36)))
@@ -386,8 +386,8 @@ def test_projection_few_row_route_short_suffixes_one_adapter(oracle64):
 
 def test_decode_sized_stack_takes_the_few_row_projections(oracle64):
     """Two decoder layers on a batch of 40 rows (requests of 1 .. 6 new tokens on cached prefixes made by a base
-    prefill through the same stack): q/k/v, o_proj, gate/up and down all run on the few-row route, the last three
-    with the residual added in its second kernel."""
+    prefill through the same stack): q/k/v, o_proj, gate/up and down all run on the few-row route, two of the
+    last three with the residual added."""
     shape = wl.LayerShape(hidden=512, n_q_heads=4, n_kv_heads=2, head_dim=128, page_size=16, dtype="bf16",
                           intermediate=1024)
     rng = np.random.default_rng(33)
