@@ -21,6 +21,7 @@ int launch_attend_simt(alora_ctx *, const void *, const BatchArgs &, const void 
 int launch_project_tc(alora_ctx *, int, const void *, int, int, void *, cudaStream_t, void *, int);
 int launch_linear_tc(alora_ctx *, const void *, const void *, int, int, int, void *, const void *, const LinearDelta *,
                      cudaStream_t);
+int launch_glu_tc(alora_ctx *, const void *, const void *, int, int, int, void *, cudaStream_t, const LinearDelta *);   // gemm_tcgen05.cu
 int launch_repack_mlp(const void *, const void *, const void *, const void *, int, int, int, int, int, void *, void *,
                       int32_t *, int32_t *, cudaStream_t);   // mlp_adapter.cu
 int launch_mlp_expand(alora_ctx *, void *, int, int, const void *, int, const void *, int, int, int, const int32_t *,
@@ -46,6 +47,9 @@ int launch_linear(alora_ctx *ctx, const void *x, const void *W, int T, int K, in
                   const void *residual, cudaStream_t s, const LinearDelta *delta) {
     if (ctx->cfg.dtype == ALORA_DTYPE_BF16) return launch_linear_tc(ctx, x, W, T, K, N, y, residual, delta, s);
     return launch_linear_simt(ctx, x, W, T, K, N, y, residual, s);
+}
+int launch_glu(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y, cudaStream_t s, const LinearDelta *delta) {
+    return ctx->cfg.dtype == ALORA_DTYPE_BF16 ? launch_glu_tc(ctx, x, W, T, K, N, y, s, delta) : 0;
 }
 int launch_attend(alora_ctx *ctx, const void *qkv, const BatchArgs &b, const void *pool, void *out,
                   cudaStream_t s) {
@@ -187,8 +191,14 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
     if (cudaGetDeviceProperties(&prop, c.device) == cudaSuccess) ctx->sm_count = prop.multiProcessorCount;
     const size_t Tm = (size_t)c.max_tokens;
     ctx->max_pairs = pair_bound(ctx, c.max_tokens, c.max_requests);
-    if (c.dtype == ALORA_DTYPE_BF16)
+    ctx->max_quads = quad_bound(ctx, c.max_tokens, c.max_requests);
+    if (c.dtype == ALORA_DTYPE_BF16) {
         ctx->t_slots = std::max(ctx->max_pairs, 3 * pair_bound(ctx, std::min(c.max_tokens, kSplitTTokens), c.max_requests));
+        if (c.max_tokens > kSplitTTokens) ctx->t_slots = std::max(ctx->t_slots, 4 * ctx->max_quads);
+        alloc((void **)&ctx->d_quads, (size_t)ctx->max_quads * sizeof(TilePair));
+        alloc((void **)&ctx->d_quad_off, (Tm / kQuadRows + 2) * 4);
+        alloc((void **)&ctx->d_quad_ready, (size_t)ctx->max_quads * 4);
+    }
     alloc((void **)&ctx->d_adapters, n_ad * sizeof(AdapterDev));
     alloc((void **)&ctx->d_token_req, Tm * 4);
     alloc((void **)&ctx->d_row_adapter, Tm * 4);
@@ -281,6 +291,7 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
         if (e == cudaSuccess) e = cudaMemset(ctx->d_adapters, 0, n_ad * sizeof(AdapterDev));
         if (e == cudaSuccess) e = cudaMemset(ctx->d_counts, 0, 64);
         if (e == cudaSuccess) e = cudaMemset(ctx->d_t_ready, 0, (size_t)ctx->max_pairs * 4);
+        if (e == cudaSuccess && ctx->d_quad_ready) e = cudaMemset(ctx->d_quad_ready, 0, (size_t)ctx->max_quads * 4);
         if (e == cudaSuccess && ctx->d_rope_inv_freq) {
             std::vector<double> f((size_t)c.head_dim / 2);
             for (size_t i = 0; i < f.size(); ++i) f[i] = pow((double)c.rope_theta, -2.0 * (double)i / (double)c.head_dim);
@@ -311,7 +322,7 @@ alora_status alora_destroy(alora_ctx *ctx) {
     if (ctx->d_mlp_part) cudaFree(ctx->d_mlp_part);
     if (ctx->d_mlp_done) cudaFree(ctx->d_mlp_done);
     void *ptrs[] = {ctx->d_adapters, ctx->d_token_req, ctx->d_row_adapter, ctx->d_slot, ctx->d_pairs, ctx->d_pair_off, ctx->d_counts,
-                    ctx->d_seg_scratch, ctx->d_t_ready, ctx->d_t, ctx->d_qkv, ctx->d_status, ctx->d_act[0], ctx->d_act[1],
+                    ctx->d_quads, ctx->d_quad_off, ctx->d_quad_ready, ctx->d_seg_scratch, ctx->d_t_ready, ctx->d_t, ctx->d_qkv, ctx->d_status, ctx->d_act[0], ctx->d_act[1],
                     ctx->d_act[2], ctx->d_act[3], ctx->d_iota, ctx->d_attn_items, ctx->d_attn_off, ctx->d_split_items,
                     ctx->d_req_scratch, ctx->d_part_o, ctx->d_part_ml, ctx->d_group_done,
                     ctx->d_skinny_part, ctx->d_skinny_t, ctx->d_skinny_meta, ctx->d_rope_inv_freq, ctx->d_prefix_groups,
@@ -409,7 +420,8 @@ alora_status alora_register_mlp_adapter(alora_ctx *ctx, int adapter_id, int laye
         // (shrink kernel and its partials: only for the projections of at most kFewRowMax rows)
         const size_t rows = (size_t)std::min(std::max(ctx->cfg.max_tokens, 1), kFewRowMax);
         const size_t rows_pad = (rows + 63) / 64 * 64;
-        ALORA_CUDA(ctx, cudaMalloc(&ctx->d_mlp_t, std::max(rows * na, (size_t)ctx->max_pairs * kTileRows) * 2 * d.RP * es));
+        const size_t t_rows = std::max((size_t)ctx->max_pairs * kTileRows, (size_t)ctx->max_quads * kQuadRows);
+        ALORA_CUDA(ctx, cudaMalloc(&ctx->d_mlp_t, std::max(rows * na, t_rows) * 2 * d.RP * es));
         // K-slice partials of the shrink kernel: room for four slices of the widest result, at most 64 MB (the
         // kernel takes fewer slices when a batch's partials would not fit)
         ctx->mlp_part_floats = std::min<size_t>(4 * rows_pad * na * 2 * d.RP, (size_t)16 << 20);
@@ -705,7 +717,13 @@ alora_status alora_forward_stack(alora_ctx *ctx, int mode, const void *d_hidden_
                 gu = LinearDelta{ctx->mlp_a_gu[l], ctx->mlp_b_gu[l], 2, mlp_tab, t0 / kTileRows, ctx->d_row_adapter + t0, ctx->d_mlp_t};
                 dn = LinearDelta{ctx->mlp_a_dn[l], ctx->mlp_b_dn[l], 1, mlp_tab, t0 / kTileRows, ctx->d_row_adapter + t0, ctx->d_mlp_t};
             }
-            ALORA_STEP(launch_linear(ctx, xm, lw.wgate_up, tc, d.H, 2 * d.I, ctx->d_act[2], nullptr, s, fused ? &gu : nullptr));
+            // many rows: SwiGLU in the epilogue of the gate / up projection
+            int glu = 0;
+            if (!n_mlp || fused) {
+                glu = launch_glu(ctx, xm, lw.wgate_up, tc, d.H, 2 * d.I, ctx->d_act[3], s, fused ? &gu : nullptr);
+                ALORA_STEP(glu);
+            }
+            if (!glu) ALORA_STEP(launch_linear(ctx, xm, lw.wgate_up, tc, d.H, 2 * d.I, ctx->d_act[2], nullptr, s, fused ? &gu : nullptr));
             if (n_mlp && !fused) {
                 const int tw = n_mlp * 2 * d.RP;
                 ALORA_STEP(launch_mlp_shrink(ctx, xm, ctx->mlp_a_gu[l], tc, d.H, tw, ctx->d_mlp_t, ctx->d_mlp_part,
@@ -713,7 +731,7 @@ alora_status alora_forward_stack(alora_ctx *ctx, int mode, const void *d_hidden_
                 ALORA_STEP(launch_mlp_expand(ctx, ctx->d_act[2], 2 * d.I, tc, ctx->d_mlp_t, tw, ctx->mlp_b_gu[l], 2 * d.I,
                                              d.I, 2, ctx->d_row_adapter + t0, mlp_tab, n_mlp, s));
             }
-            ALORA_STEP(launch_swiglu(ctx, ctx->d_act[2], tc, ctx->d_act[3], s));
+            if (!glu) ALORA_STEP(launch_swiglu(ctx, ctx->d_act[2], tc, ctx->d_act[3], s));
             ALORA_STEP(launch_linear(ctx, ctx->d_act[3], lw.wdown, tc, d.I, d.H, hc, hc, s, fused ? &dn : nullptr));  // h += down(...)
             if (n_mlp && !fused) {
                 const int tw = n_mlp * d.RP;

@@ -50,6 +50,8 @@ constexpr int kTileRows = 128;
 struct TilePair {
     int32_t tile, adapter;
 };
+// The same for the kernel that works on four row tiles at once (gemm_duo_tcgen05.cu): one entry per (quad, adapter), `tile` the quad.
+constexpr int kQuadRows = 4 * kTileRows;
 // Batches of at most this many rows carry t as the sum of three bf16 values (all 24 bits of its fp32 value, for the few rows
 // of a handful of requests), larger ones as one.
 constexpr int kSplitTTokens = 1024;
@@ -123,11 +125,6 @@ struct TcLayerMaps {
     CUtensorMap a_all;        // all adapters' A rows [max_adapters*192][H], box 192 rows
     RankMaps a_rank;
     CUtensorMap b_all_bn[3];  // all adapters' B rows [max_adapters*N][64], boxes of 128 / 256 / 64 rows
-    // for the 256 x 192 tiles of gemm_pair_tcgen05.cu: W in boxes of 192 rows; per q / k / v block the B rows of all
-    // adapters as (rank column, row inside the block, adapter), boxes of 192 rows
-    CUtensorMap wqkv192;
-    CUtensorMap b_blk[3];
-    bool pair_ok = false;
 };
 
 struct Dims {
@@ -159,8 +156,8 @@ struct alora_ctx {
     std::vector<int> mlp_n_adapters;                 // [layer] highest registered MLP adapter id + 1
     std::vector<alora::MlpAdapterDev> h_mlp_adapters;   // [layer * max_adapters + id], mirrors d_mlp_adapters
     alora::MlpAdapterDev *d_mlp_adapters = nullptr;
-    void *d_mlp_t = nullptr;                         // t of the MLP adapters: [max_pairs][128][2 * RP], or (few-row route)
-                                                     // [kFewRowMax][max_adapters * 2 * RP]
+    void *d_mlp_t = nullptr;                         // t of the MLP adapters: [max_pairs][128][2 * RP], [max_quads][512][2 * RP], or
+                                                     // (few-row route) [kFewRowMax][max_adapters * 2 * RP]
     float *d_mlp_part = nullptr;                     // K-slice partials of the shrink kernel
     size_t mlp_part_floats = 0;
     int32_t *d_mlp_done = nullptr;                   // per 64 x 64 tile of the shrink result: slices stored (zero between launches)
@@ -170,12 +167,17 @@ struct alora_ctx {
     int32_t *d_token_req = nullptr, *d_row_adapter = nullptr, *d_slot = nullptr;
     alora::TilePair *d_pairs = nullptr;       // [max_pairs] (row tile, adapter) pairs of the batch, tile after tile
     int32_t *d_pair_off = nullptr;            // [row tiles + 1] first pair of each row tile
+    alora::TilePair *d_quads = nullptr;       // [max_quads] (quad, adapter) entries of the batch (bf16), quad after quad
+    int32_t *d_quad_off = nullptr;            // [quads + 1] first entry of each quad
+    int32_t *d_quad_ready = nullptr;          // [max_quads] per entry: epilogue warps that have published t (zero between launches)
+    int32_t max_quads = 0;
     int32_t *d_counts = nullptr;  // [1] attention work items, [2] (row tile, adapter) pairs,
                                   // [3] few-row attention items, [4] next unclaimed few-row item,
                                   // [6] key tiles of the attention items that are cut into runs, [7] tiles per run,
                                   // [8] attention items taken whole (the first ones), [9] key tiles of those,
                                   // [10], [11] next unclaimed projection item and blocks done, [12] few-row attention blocks done,
-                                  // [13] an adapter with a non-finite B has been registered (kOddAdapters)
+                                  // [13] an adapter with a non-finite B has been registered (kOddAdapters),
+                                  // [14] (quad, adapter) entries
     int32_t *d_seg_scratch = nullptr;  // [14*max_requests+5] per-request values and merged row runs of the current batch
     int32_t *d_t_ready = nullptr;      // [max_pairs] per pair: epilogue warps that have published t (zero between launches)
     int32_t *d_iota = nullptr;         // 0..max_requests: query_start_loc of a decode batch
@@ -196,7 +198,8 @@ struct alora_ctx {
     float *d_part_o = nullptr, *d_part_ml = nullptr;
     int32_t *d_group_done = nullptr;    // [max_split_rows / 16] finished key ranges per (stream, KV head), at its first partial row / 16
     int32_t max_split_items = 0, max_split_rows = 0, small_max_tokens = 0;
-    void *d_t = nullptr;          // rank-r intermediate: fp32 [max_tokens][3][RP]; bf16 [pair][1 or 3 summands][128][3][RP]
+    void *d_t = nullptr;          // rank-r intermediate: fp32 [max_tokens][3][RP]; bf16 [pair][1 or 3 summands][128][3][RP], or
+                                  // [(quad, adapter) entry][512][3][RP]
     // few-row projection (batches of <= 128 rows): K-slice partial products and partial shrink results
     float *d_skinny_part = nullptr;   // [skinny_max_items][128][256] fp32
     float *d_skinny_t = nullptr;      // [slices of the q/k/v projection][128][skinny_p_cap][192] fp32
@@ -298,6 +301,14 @@ inline int pair_bound(const alora_ctx *ctx, int T, int R) {
     if (n > n_m * na) n = n_m * na;
     return (int)n;
 }
+// Most (quad, adapter) entries.
+inline int quad_bound(const alora_ctx *ctx, int T, int R) {
+    const long long n_q = (T + kQuadRows - 1) / kQuadRows, na = ctx->cfg.max_adapters > 0 ? ctx->cfg.max_adapters : 1;
+    long long n = n_q + R;
+    if (n > T) n = T;
+    if (n > n_q * na) n = n_q * na;
+    return (int)n;
+}
 int launch_kv_append(alora_ctx *ctx, const void *qkv, int T, int num_pages, void *pool, cudaStream_t s);
 int launch_cow_tail_pages(alora_ctx *ctx, const int32_t *qsl, const int32_t *seq_lens, int32_t *block_tables, int max_blocks,
                           int num_pages, int R, const int32_t *fresh_pages, void *pool, cudaStream_t s);
@@ -317,6 +328,8 @@ struct LinearDelta {
 };
 int launch_linear(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
                   const void *residual, cudaStream_t s, const LinearDelta *delta = nullptr);
+// y = silu(x Wg^T) * (x Wu^T), W = [Wg; Wu], in one launch; 0: not for this shape (nothing launched).
+int launch_glu(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y, cudaStream_t s, const LinearDelta *delta);
 int launch_rmsnorm(alora_ctx *ctx, const void *x, const void *w, int T, void *y, cudaStream_t s);
 int launch_swiglu(alora_ctx *ctx, const void *gate_up, int T, void *y, cudaStream_t s);
 

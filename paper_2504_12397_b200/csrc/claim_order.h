@@ -7,7 +7,7 @@
 //   2. a block starts on its projection items only after the counter has passed n_shrink, i.e. after every shrink
 //      item has been claimed by a running block.  Projection items are dealt by block index as if the shrink items
 //      occupied list positions 0 .. n_shrink-1, so that in the usual case every block keeps the items it always had.
-// The two decisions below are shared by the kernels (gemm_tcgen05.cu, gemm_pair_tcgen05.cu) and by the host-side
+// The two decisions below are shared by the kernels (gemm_tcgen05.cu, gemm_duo_tcgen05.cu) and by the host-side
 // model that the tests run against small grids with few resident blocks (alora_selftest_claim_order).
 #pragma once
 

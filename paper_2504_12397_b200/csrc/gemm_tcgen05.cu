@@ -538,8 +538,8 @@ static int pick_bn(int N, int Nq, int Nkv, int T) {
 
 // q/k/v projection of one layer on the tensor cores: shrink (t = s A x of the (row tile, adapter) pairs), then the
 // base GEMM with the expand step fused.  Returns kernels launched, or -1 when the shape is unsupported.
-int launch_project_pair_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int R, void *qkv, cudaStream_t s,
-                           void *kv_pool, int num_pages);  // gemm_pair_tcgen05.cu
+int launch_project_duo_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int R, void *qkv, cudaStream_t s,
+                           void *kv_pool, int num_pages);  // gemm_duo_tcgen05.cu
 
 // Whether the shrink of a launch of `items` projection items is a kernel of its own.  As leading items of the projection
 // it is free unless it makes another round over the blocks of a launch of one or two rounds (a round is 24 .. 31 us at
@@ -603,9 +603,9 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
                                 have_adapters ? ads : nullptr, ctx->tc_b_all[layer], T, d.H, d.N, d.Nq, d.Nkv, qkv,
                                 kv_pool, num_pages, layer, s);
     }
-    if (ctx->tc_maps[layer].pair_ok) {   // many rows: two row tiles per block, 192-wide column tiles
+    {   // many rows: pairs of SMs
         ProfScope prof(ctx, KK_PROJECT, s);
-        const int r = launch_project_pair_tc(ctx, layer, hidden, T, R, qkv, s, kv_pool, num_pages);
+        const int r = launch_project_duo_tc(ctx, layer, hidden, T, R, qkv, s, kv_pool, num_pages);
         if (r != 0) return r;
     }
     const int BN = pick_bn(d.N, d.Nq, d.Nkv, T);
@@ -661,9 +661,8 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
     return n;
 }
 
-int launch_linear256_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
-                        const void *residual, const LinearDelta *delta, cudaStream_t s);  // gemm_pair_tcgen05.cu
-bool build_pair_maps(alora_ctx *ctx, int layer);                 // gemm_pair_tcgen05.cu
+int launch_linear_duo_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
+                         const void *residual, const LinearDelta *delta, bool glu, cudaStream_t s);  // gemm_duo_tcgen05.cu
 
 // Dense projection y = x W^T (+ residual) for o_proj and the MLP matrices, with the gated delta of the MLP adapters where
 // `delta` is given (more than kFewRowMax rows: a smaller batch may be on the few-row route, which builds no pairs).
@@ -676,7 +675,7 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
     if (delta == nullptr && few_cluster_rows(ctx, T) && few_cluster_route(ctx, T, 0, N, K, false, N, 0))
         return launch_few_cluster(ctx, x, W, nullptr, nullptr, nullptr, T, 0, K, N, N, 0, y, residual, nullptr, 0, false, s);
     {
-        const int r = launch_linear256_tc(ctx, x, W, T, K, N, y, residual, delta, s);   // many rows: 256 x 256 tiles
+        const int r = launch_linear_duo_tc(ctx, x, W, T, K, N, y, residual, delta, false, s);   // many rows: pairs of SMs
         if (r != 0) return r;
     }
     const int BN = N % 256 == 0 || N > 1024 ? 256 : 128;
@@ -706,6 +705,13 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
     return ok ? 1 : -1;
 }
 
+// Gate and up projection with SwiGLU in the epilogue, for the batches that the pairs of SMs serve; 0: nothing launched.
+int launch_glu_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y, cudaStream_t s, const LinearDelta *delta) {
+    if (T == 0 || (delta == nullptr && few_cluster_rows(ctx, T) && few_cluster_route(ctx, T, 0, N, K, false, N, 0))) return 0;
+    ProfScope prof(ctx, KK_LINEAR, s);
+    return launch_linear_duo_tc(ctx, x, W, T, K, N, y, nullptr, delta, true, s);
+}
+
 // Tensor maps that depend only on registered weights; (re)built when weights or adapters are set.
 bool build_layer_maps(alora_ctx *ctx, int layer) {
     const Dims &d = ctx->d;
@@ -723,7 +729,6 @@ bool build_layer_maps(alora_ctx *ctx, int layer) {
     ok &= make_tensor_map_bf16(&lm.b_all_bn[0], ctx->tc_b_all[layer], na * d.N, kTensorRP, kTensorRP, 128);
     ok &= make_tensor_map_bf16(&lm.b_all_bn[1], ctx->tc_b_all[layer], na * d.N, kTensorRP, kTensorRP, 256);
     ok &= make_tensor_map_bf16(&lm.b_all_bn[2], ctx->tc_b_all[layer], na * d.N, kTensorRP, kTensorRP, 64);
-    lm.pair_ok = lw.wqkv != nullptr && build_pair_maps(ctx, layer);   // optional: the 128-row kernel serves every shape
     return ok;
 }
 

@@ -69,13 +69,14 @@ __device__ __forceinline__ int metadata_token(int t, int p,
 }
 
 // The (row tile, adapter) pairs of the projection: for every tile of kTileRows rows the adapters whose gate is open on
-// some row of it, in the order of their first request, each once.  One block; a warp per tile, a lane per request.  Also
-// reports a request whose open rows name an adapter that some layer of the call has not registered.
+// some row of it, in the order of their first request, each once; or the same for tiles of `tile_rows` rows.  One block; a
+// warp per tile, a lane per request.  With `adapters` it also reports a request whose open rows name an adapter that some
+// layer of the call has not registered.
 __device__ __forceinline__ void metadata_pairs(const int32_t *__restrict__ a_req, const int32_t *__restrict__ adapter_ids,
                                                const int32_t *__restrict__ qsl, const int32_t *__restrict__ seq_lens,
-                                               int R, int mode, int max_adapters, int T, int max_pairs,
+                                               int R, int mode, int max_adapters, int T, int tile_rows, int max_pairs,
                                                TilePair *__restrict__ pairs, int32_t *__restrict__ pair_off,
-                                               int32_t *__restrict__ counts, int32_t *scratch /* [3R] */,
+                                               int32_t *__restrict__ n_pairs, int32_t *scratch /* [3R] */,
                                                const AdapterDev *__restrict__ adapters, int n_layers, int32_t *status) {
     constexpr int kBatch = 128;   // tiles per round
     __shared__ int r_lo[kBatch], r_hi[kBatch], cnt[kBatch], off_s[kBatch];
@@ -99,16 +100,16 @@ __device__ __forceinline__ void metadata_pairs(const int32_t *__restrict__ a_req
                 if (adapters[(size_t)l * max_adapters + k].rank == 0) report(status, ALORA_ERR_NO_WEIGHTS);
     }
     any = __syncthreads_or(any);
-    const int n_tiles = (T + kTileRows - 1) / kTileRows;
+    const int n_tiles = (T + tile_rows - 1) / tile_rows;
     if (!any) {   // base model only
         for (int i = threadIdx.x; i <= n_tiles; i += blockDim.x) pair_off[i] = 0;
-        if (threadIdx.x == 0) counts[2] = 0;
+        if (threadIdx.x == 0) *n_pairs = 0;
         return;
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = (int)blockDim.x >> 5;
     // adapters of tile `t` (requests lo .. hi): counted, or written from pairs[at] on; called by whole warps
     auto walk = [&](int t, int lo, int hi, bool write, int at) {
-        const int row0 = t * kTileRows, row1 = min(row0 + kTileRows, T);
+        const int row0 = t * tile_rows, row1 = min(row0 + tile_rows, T);
         int n = 0;
         for (int base = lo; base <= hi; base += 32) {
             const int r = base + lane;
@@ -130,8 +131,8 @@ __device__ __forceinline__ void metadata_pairs(const int32_t *__restrict__ a_req
     for (int t0 = 0; t0 < n_tiles; t0 += kBatch) {
         const int nb = min(kBatch, n_tiles - t0);
         for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-            r_lo[i] = find_request(qsl, R, (t0 + i) * kTileRows);
-            r_hi[i] = find_request(qsl, R, min((t0 + i + 1) * kTileRows, T) - 1);
+            r_lo[i] = find_request(qsl, R, (t0 + i) * tile_rows);
+            r_hi[i] = find_request(qsl, R, min((t0 + i + 1) * tile_rows, T) - 1);
         }
         __syncthreads();
         for (int i = warp; i < nb; i += n_warps) {
@@ -161,7 +162,7 @@ __device__ __forceinline__ void metadata_pairs(const int32_t *__restrict__ a_req
     if (threadIdx.x == 0) {
         if (carry > max_pairs) report(status, ALORA_ERR_CAPACITY);
         pair_off[n_tiles] = min(carry, max_pairs);
-        counts[2] = min(carry, max_pairs);
+        *n_pairs = min(carry, max_pairs);
     }
 }
 
@@ -645,8 +646,8 @@ __device__ __forceinline__ void metadata_few_row(int k_mine, const AdapterDev &a
     if ((int)threadIdx.x < kFewRowMax) meta->slot_of_row[threadIdx.x] = slot;
 }
 
-// The metadata step.  Phase bit 0: every block handles 256 tokens (request, applied adapter, slot); one block more
-// builds the projection's (row tile, adapter) pairs.  Phase bit 1: the two attention
+// The metadata step.  Phase bit 0: every block handles 256 tokens (request, applied adapter, slot); two blocks more
+// build the projection's (row tile, adapter) pairs and (quad, adapter) entries.  Phase bit 1: the two attention
 // work lists, one block each (their serial parts are O(R)).  Both phases in one launch: the last block, 1 and 2 take one
 // builder each.  The attention phase alone is launched as a programmatic dependent of the projection kernel, beside
 // which it runs (it reads nothing that kernel writes); its blocks wait for that kernel before they exit, so that
@@ -656,8 +657,8 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
                 const int32_t *qsl, const int32_t *seq_lens, const int32_t *__restrict__ block_tables, int max_blocks,
                 int num_pages, int page_size, int max_adapters, int T, int R, int mode,
                 int32_t *__restrict__ token_req, int32_t *__restrict__ row_adapter, int32_t *__restrict__ slot_map,
-                int max_pairs, TilePair *__restrict__ pairs, int32_t *__restrict__ pair_off, int32_t *__restrict__ counts,
-                int32_t *seg_scratch,
+                int max_pairs, TilePair *__restrict__ pairs, int32_t *__restrict__ pair_off, int max_quads,
+                TilePair *__restrict__ quads, int32_t *__restrict__ quad_off, int32_t *__restrict__ counts, int32_t *seg_scratch,
                 int Hkv, int q_block, int max_items, AttnWork *__restrict__ items, int32_t *blk_off,
                 int G, int n_sm, int small_max, int max_split_items, int max_split_rows,
                 AttnSplitWork *__restrict__ split_items,
@@ -686,17 +687,18 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
     if ((phases & kMetaProjection) && tok < T)
         metadata_token(tok, my_pos, a_req, adapter_ids, qsl, seq_lens, block_tables,
                        max_blocks, num_pages, page_size, max_adapters, T, R, mode, token_req, row_adapter, slot_map, status, [](int) {});
-    // The three list builders are independent of one another: the last block, 1 and 2 take one each (a launch of both
-    // phases has at least four blocks, one of the attention phase alone two).
+    // The list builders are independent of one another: the last two blocks, 1 and 2 take one each (a launch of both
+    // phases has at least five blocks, one of the attention phase alone two).
     const int nb = (int)gridDim.x;
     const bool proj = (phases & kMetaProjection) != 0, attn = (phases & kMetaAttention) != 0;
     const int b_pairs = proj && pairs != nullptr ? nb - 1 : -1;   // (a block without tokens of its own: the projection waits for it)
+    const int b_quads = proj && quads != nullptr ? nb - 2 : -1;
     const int b_attn = !attn ? -1 : (proj ? (nb > 1 ? 1 : 0) : 0);
     const int b_split = !attn ? -1 : (proj ? (nb > 2 ? 2 : 0) : (nb > 1 ? 1 : 0));
     // the attention phase alone: block 0 builds the tensor-core kernel's list, all the others share the few-row list
     const int split_parts = (!proj && attn && nb > 1) ? nb - 1 : 1;
     const bool split_helper = !proj && attn && (int)blockIdx.x > b_split;
-    if ((int)blockIdx.x != b_pairs && (int)blockIdx.x != b_attn && (int)blockIdx.x != b_split && !split_helper) {
+    if ((int)blockIdx.x != b_pairs && (int)blockIdx.x != b_quads && (int)blockIdx.x != b_attn && (int)blockIdx.x != b_split && !split_helper) {
         if (!proj) tc::grid_dep_wait();
         return;
     }
@@ -706,9 +708,12 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
     if (14 * R + 5 <= kMetaSmemInts) seg_scratch = blk_off = req_scratch = smem_scratch;
     __syncthreads();
     if ((int)blockIdx.x == b_pairs) {
-        metadata_pairs(a_req, adapter_ids, qsl, seq_lens, R, mode, max_adapters, T, max_pairs, pairs, pair_off, counts,
+        metadata_pairs(a_req, adapter_ids, qsl, seq_lens, R, mode, max_adapters, T, kTileRows, max_pairs, pairs, pair_off, counts + 2,
                        seg_scratch, adapters, n_layers, status);
         __syncthreads();  // a builder that follows in this block reuses the scratch
+    } else if ((int)blockIdx.x == b_quads) {
+        metadata_pairs(a_req, adapter_ids, qsl, seq_lens, R, mode, max_adapters, T, kQuadRows, max_quads, quads, quad_off, counts + 14,
+                       seg_scratch == smem_scratch ? smem_scratch : seg_scratch + 3 * R, nullptr, 0, status);
     }
     if ((int)blockIdx.x == b_attn && items != nullptr && block_tables != nullptr) {
         metadata_attn_items(qsl, seq_lens, R, Hkv, q_block, small_max, max_items, items, counts, blk_off,
@@ -778,7 +783,7 @@ int launch_metadata(alora_ctx *ctx, const BatchArgs &b, cudaStream_t s, int phas
     // (attention phase alone: one block for the tensor-core list, kSplitBuilders for the few-row list; they need the
     // shared-memory scratch, i.e. batches of at most 511 requests, else one block builds it in the global scratch)
     constexpr int kSplitBuilders = 8;
-    const int grid = attn_only ? (14 * b.R + 5 <= kMetaSmemInts ? 1 + kSplitBuilders : 2) : 1 + std::max((phases & kMetaAttention) ? 3 : 1, (b.T + threads - 1) / threads);
+    const int grid = attn_only ? (14 * b.R + 5 <= kMetaSmemInts ? 1 + kSplitBuilders : 2) : 2 + std::max((phases & kMetaAttention) ? 3 : 1, (b.T + threads - 1) / threads);
     const AdapterDev *ads = b.layer >= 0 ? ctx->d_adapters + (size_t)b.layer * ctx->cfg.max_adapters : nullptr;
     if (phases == kMetaProjection && b.few_row) {
         FewRowMeta *few = ads != nullptr ? ctx->d_skinny_meta + (size_t)b.layer * ctx->few_tiles : nullptr;
@@ -791,7 +796,7 @@ int launch_metadata(alora_ctx *ctx, const BatchArgs &b, cudaStream_t s, int phas
     const cudaError_t e = launch_kernel(metadata_kernel, dim3(grid), dim3(threads), 0, s, attn_only,
         b.positions, b.activation_offsets, b.adapter_ids, b.query_start_loc, b.seq_lens, b.block_tables,
         b.max_blocks, b.num_pages, ctx->d.page, ctx->cfg.max_adapters, b.T, b.R, b.mode, ctx->d_token_req,
-        ctx->d_row_adapter, ctx->d_slot, ctx->max_pairs, ctx->d_pairs, ctx->d_pair_off, ctx->d_counts, ctx->d_seg_scratch,
+        ctx->d_row_adapter, ctx->d_slot, ctx->max_pairs, ctx->d_pairs, ctx->d_pair_off, ctx->max_quads, ctx->d_quads, ctx->d_quad_off, ctx->d_counts, ctx->d_seg_scratch,
         ctx->d.Hkv, ctx->attn_q_block, ctx->max_attn_items, ctx->d_attn_items, ctx->d_attn_off, ctx->d.G,
         ctx->sm_count, ctx->small_max_tokens, ctx->max_split_items, ctx->max_split_rows, ctx->d_split_items,
         ctx->d_req_scratch, ctx->d_group_done,

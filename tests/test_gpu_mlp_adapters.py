@@ -302,3 +302,51 @@ def test_non_finite_mlp_adapter_values_stay_in_the_rows_that_use_them(each):
         m[200, 5] = kept
         assert np.array_equal(odd[~own].view(np.uint32), finite[~own].view(np.uint32)), n
         assert not np.isfinite(odd[own]).all(), n
+
+
+def test_dense_matrices_on_pairs_of_sms(oracle64):
+    """One layer of 4900 rows (three row tiles in the last quad, the last one partial): o_proj, gate / up with SwiGLU in the
+    epilogue (column tiles of 96, the last one cut off) and down on pairs of SMs, with MLP adapters; closed rows keep the bits of
+    the base-mode call, and a non-finite B reaches only the rows that use it."""
+    shape = wl.LayerShape(hidden=1024, n_q_heads=8, n_kv_heads=2, head_dim=128, page_size=16, dtype="bf16", intermediate=1280)
+    rng = np.random.default_rng(52)
+    layers = [wl.make_stack_weights(shape, rng)]
+    ads = [[wl.make_adapter(shape, r, rng) for r in (32, 8)]]
+    mlps = [[wl.make_mlp_adapter(shape, r, rng, scale=s) for r, s in ((16, 1.0), (64, 0.5))]]
+    for m in mlps[0]:
+        for n in ("Bg", "Bu", "Bd"):
+            setattr(m, n, wl.bf16_round(getattr(m, n) * 8))
+    S, ids = [700] * 7, [0, -1, 1, 0, 1, -1, 0]
+    a_req = [333, 0, 0, 0, 77, 0, 650]
+    b = wl.make_batch(shape, [0] * 7, S, ids, rng, activation_offsets=a_req, shuffle_pages=True)
+
+    def run(mode=ab.MODE_ALORA):
+        g = hp.GpuLayers(shape, layers, ads, b.T, b.R, mlp_adapters_per_layer=mlps)
+        try:
+            d = hp.DevBatch(b, shape.dtype)
+            pools, hout = [g.new_pool(b.num_pages)], g.empty(b.T, shape.hidden)
+            ab.alora_forward_stack(g.ctx, mode, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, pools, d.bt,
+                                   d.max_blocks, b.num_pages, d.T, d.R, hout)
+            assert g.status() == 0
+            return hp.to_host(hout)
+        finally:
+            g.close()
+
+    got, base = run(), run(ab.MODE_BASE)
+    x, _ = oracle64.decoder_layer(b.hidden.astype(np.float64), layers[0], shape.Nq, shape.Nkv, shape.n_q_heads, shape.n_kv_heads,
+                                  shape.head_dim, 1e-5, b.positions, b.query_start_loc, b.activation_offsets, b.adapter_ids,
+                                  hp.oracle_adapters(ads[0]), [None] * b.R, [None] * b.R, mlp_adapters=hp.oracle_mlp_adapters(mlps[0]))
+    hp.assert_close(got, x, 2e-2, "4900 rows with MLP adapters", block=shape.head_dim)
+    owner = np.repeat(np.array(ids), S)
+    closed = (owner < 0) | (b.positions < np.repeat(np.array(a_req), S))
+    assert np.array_equal(got[closed].view(np.uint32), base[closed].view(np.uint32))
+    assert hp.rel_err(got[~closed], base[~closed]) > 0.02
+    for n, v in (("Bg", np.inf), ("Bu", np.nan), ("Bd", -np.inf)):
+        m = getattr(mlps[0][1], n)
+        kept = m[200, 5]
+        m[200, 5] = v
+        odd = run()
+        m[200, 5] = kept
+        own = (owner == 1) & ~closed
+        assert np.array_equal(odd[~own].view(np.uint32), got[~own].view(np.uint32)), n
+        assert not np.isfinite(odd[own]).all(), n

@@ -916,3 +916,46 @@ def test_projection_of_at_most_1024_rows_loses_nothing_of_t(n_req, each, heads, 
     finally:
         g.close()
     assert np.array_equal(got, wl.bf16_round(y.astype(np.float32)))
+
+
+@pytest.mark.parametrize("S", [[1500, 900, 600, 201], [900, 1200, 700, 600], [700, 1313, 880, 692, 1]])
+def test_projection_on_pairs_of_sms(oracle64, S):
+    """Batches that the kernel on pairs of SMs serves, four row tiles an item: two, three and one row tiles in the last quad, a
+    last tile of one row; column tiles that straddle the q | k | v boundaries, gates that open inside requests.  The cache rows
+    of a layer call are those of its sub-steps, and a non-finite B reaches only the rows that use it."""
+    shape = wl.LayerShape(hidden=1024, n_q_heads=8, n_kv_heads=2, head_dim=128, page_size=16, dtype="bf16")
+    rng = np.random.default_rng(101)
+    w = wl.make_wqkv(shape, rng)
+    ads = _boosted_adapters(shape, rng, ((8, 1.0), (64, 0.5), (32, 2.0)))
+    R = len(S)
+    ids = ([1, 0, -1, 2, 1])[:R]
+    b = wl.make_batch(shape, [20] * R, S, ids, rng, activation_offsets=[150, 20, 20, 220, 20][:R])
+    assert (b.T + 127) // 128 in (26, 27, 29)
+    _check_projection(oracle64, shape, w, ads, b)
+
+    def run():
+        g = hp.GpuLayers(shape, [dict(wqkv=w)], [ads], b.T, b.R)
+        try:
+            d = hp.DevBatch(b, shape.dtype)
+            fill = np.zeros((b.num_pages, 2, shape.n_kv_heads, shape.page_size, shape.head_dim), np.float32)
+            pool, pool2, out, qkv = g.new_pool(b.num_pages, fill), g.new_pool(b.num_pages, fill), g.empty(b.T, shape.Nq), g.empty(b.T, shape.N)
+            ab.alora_prefill_layer(g.ctx, 0, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, pool, d.bt, d.max_blocks,
+                                   b.num_pages, d.T, d.R, out)
+            ab.alora_project_qkv(g.ctx, 0, ab.MODE_ALORA, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, d.T, d.R, qkv)
+            ab.alora_kv_append(g.ctx, qkv, d.positions, d.qsl, d.seq_lens, d.bt, d.max_blocks, b.num_pages, d.T, d.R, pool2)
+            assert g.status() == 0
+            return hp.to_host(pool), hp.to_host(pool2), hp.to_host(qkv)
+        finally:
+            g.close()
+
+    pool, pool2, finite = run()
+    assert np.array_equal(pool.view(np.uint32), pool2.view(np.uint32))
+    ads[0].Bq[7, 3] = np.inf
+    ads[0].Bk[100, 2] = np.nan
+    pool, pool2, odd = run()
+    assert np.array_equal(pool.view(np.uint32), pool2.view(np.uint32))
+    own = np.repeat(np.array(ids), S) == 0
+    assert np.array_equal(odd[~own].view(np.uint32), finite[~own].view(np.uint32))
+    assert not np.isfinite(odd[own][:, [7, shape.Nq + 100]]).any()
+    others = np.setdiff1d(np.arange(shape.N), [7, shape.Nq + 100])
+    hp.assert_close(odd[own][:, others], finite[own][:, others], 2e-2, "the adapter's own rows")
