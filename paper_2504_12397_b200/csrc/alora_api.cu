@@ -16,6 +16,8 @@ alora_status cuda_fail(alora_ctx *ctx, cudaError_t e, const char *what) {
 
 int launch_project_simt(alora_ctx *, int, const void *, int, void *, cudaStream_t, void *, int);
 int launch_linear_simt(alora_ctx *, const void *, const void *, int, int, int, void *, const void *, cudaStream_t);
+bool simt_small_layer(const alora_ctx *, int);
+int launch_project_small_simt(alora_ctx *, int, const void *, const BatchArgs &, void *, void *, cudaStream_t);
 int launch_attend_simt(alora_ctx *, const void *, const BatchArgs &, const void *, void *, cudaStream_t);
 
 int launch_project_tc(alora_ctx *, int, const void *, int, int, void *, cudaStream_t, void *, int);
@@ -84,6 +86,17 @@ static alora_status run_layer(alora_ctx *ctx, int layer, const void *hidden, con
     b.layer = layer;
     b.few_row = project_is_few_row(ctx, layer, b.T, b.R) ? 1 : 0;   // (n_layers > 1 only where all of them take that route)
     int n = 0, k;
+    if (simt_small_layer(ctx, b.T)) {   // few fp32 rows: facts, shrink, projection and append in one launch
+        const bool rotate = ctx->d_rope_inv_freq != nullptr;
+        if ((k = launch_project_small_simt(ctx, layer, hidden, b, ctx->d_qkv, rotate ? nullptr : pool, s)) < 0) return ALORA_ERR_UNSUPPORTED;
+        n += k;
+        if (rotate) {
+            if ((k = launch_rope(ctx, ctx->d_qkv, b.positions, b.T, pool, b.num_pages, s)) < 0) return ALORA_ERR_UNSUPPORTED;
+            n += k;
+        }
+        if ((k = launch_attend(ctx, ctx->d_qkv, b, pool, attn_out, s)) < 0) return ALORA_ERR_UNSUPPORTED;
+        return finish(ctx, n + k);
+    }
     // The per-token arrays and the projection's lists first; the attention work lists are built beside the
     // projection (the few-row projection launches them between its two kernels, the other routes right after).
     if (!(b.facts_ready & kMetaProjection)) {

@@ -187,6 +187,145 @@ linear_simt_kernel(const float *__restrict__ x, const float *__restrict__ W, int
 }
 
 // ---------------------------------------------------------------------------------------------
+// What a new token's row needs to know, from the caller's arrays (the same findings as the batch-metadata step): request, position,
+// applied adapter (the gate of Eq. 5; -1: none) and cache slot (-1: rejected).  Called by whole warps.
+// ---------------------------------------------------------------------------------------------
+struct RowFacts { int req, pos, adapter, slot; };
+__device__ __forceinline__ RowFacts row_facts(int t, const int32_t *__restrict__ positions, const int32_t *__restrict__ a_req,
+                                              const int32_t *__restrict__ adapter_ids, const int32_t *__restrict__ qsl,
+                                              const int32_t *__restrict__ seq_lens, const int32_t *__restrict__ block_tables,
+                                              int max_blocks, int num_pages, int page_size, int max_adapters, int R, int mode, int32_t *status) {
+    const int lane = threadIdx.x & 31;
+    RowFacts f;
+    f.pos = positions[t];
+    int r = 0;   // the last request that starts at or before t (empty requests start where their successor does)
+    for (int i = 1; i < R; i += 32) r += __popc(__ballot_sync(0xffffffffu, i + lane < R && qsl[i + lane] <= t));
+    f.req = r;
+    const int len = seq_lens[r], next = qsl[r + 1], first_open = a_req != nullptr && mode == ALORA_MODE_ALORA ? a_req[r] : 0;
+    int k = mode != ALORA_MODE_BASE && adapter_ids != nullptr ? adapter_ids[r] : -1;
+    const bool ok = f.pos == len - (next - t) && f.pos >= 0;   // positions of a request are consecutive and end at seq_len - 1
+    if (!ok) report(status, ALORA_ERR_BAD_BATCH);
+    if (k >= max_adapters || k < -1) { report(status, ALORA_ERR_BAD_BATCH); k = -1; }
+    f.adapter = ok && f.pos >= first_open ? k : -1;
+    f.slot = -1;
+    if (ok) {
+        const int blk = f.pos / page_size, page = blk < max_blocks ? block_tables[(size_t)r * max_blocks + blk] : -1;
+        if (blk >= max_blocks) report(status, ALORA_ERR_BAD_BATCH);
+        else if (page < 0 || page >= num_pages) report(status, ALORA_ERR_PAGE_RANGE);
+        else f.slot = page * page_size + f.pos % page_size;
+    }
+    return f;
+}
+
+// ---------------------------------------------------------------------------------------------
+// The first half of a small fp32 layer call in one launch: facts, shrink, projection, KV append.  Warps 0..7 form the base sums of
+// a 16 x 32 tile as linear_simt_kernel does; beside them warp 8 + i finds row i's facts, its t = s A x and its delta
+// for the tile's 32 columns, which lie in one of the q / k / v blocks (a column a lane).  Batch metadata, shrink and projection
+// as launches of their own are chains of two to four fetches each, one after the other: 16 tokens at hidden 256 took 17 us
+// until the projection was done, of 22 for the call; here the chains run side by side (call: 13 us).  t is formed again
+// by every column tile, so this is for few rows and short rows of x (simt_small_layer()).
+// ---------------------------------------------------------------------------------------------
+constexpr int kSmallVecs = 8;   // 16-byte vectors of x a lane holds: hidden <= 1024
+__global__ void __launch_bounds__(768)
+project_small_simt_kernel(const float *__restrict__ x, const float *__restrict__ W, int Tn, int K, int N, int Nq, int Nkv, int RP,
+                          const AdapterDev *__restrict__ adapters, const int32_t *__restrict__ positions,
+                          const int32_t *__restrict__ a_req, const int32_t *__restrict__ adapter_ids, const int32_t *__restrict__ qsl,
+                          const int32_t *__restrict__ seq_lens, const int32_t *__restrict__ block_tables, int max_blocks, int num_pages,
+                          int page_size, int max_adapters, int R, int mode, int hd, int Hkv, float *__restrict__ pool,
+                          int32_t *__restrict__ token_req, int32_t *__restrict__ row_adapter, int32_t *__restrict__ slot_map,
+                          float *__restrict__ y, int32_t *status) {
+    __shared__ float part[8][16][32 + 1], delta_s[16][32 + 1];
+    __shared__ int adapter_s[16], slot_s[16];
+    tc::grid_dep_launch();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n_col = (N + 31) / 32, row0 = (int)blockIdx.x / n_col * 16, col0 = (int)blockIdx.x % n_col * 32;
+    if (warp < 8) {
+        const int tx = lane & 7, ty = lane >> 3;
+        float acc[4][4] = {};   // rows row0 + ty + 4 i, columns col0 + tx + 8 j (beyond the edge: the last one again, not stored)
+        const float *xr[4], *wr[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            xr[i] = x + (size_t)min(row0 + ty + 4 * i, Tn - 1) * K;
+            wr[i] = W + (size_t)min(col0 + tx + 8 * i, N - 1) * K;
+        }
+#pragma unroll 2
+        for (int k = warp * 4; k < K; k += 32) {
+            float4 a[4], b[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { a[i] = *reinterpret_cast<const float4 *>(xr[i] + k); b[i] = *reinterpret_cast<const float4 *>(wr[i] + k); }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    acc[i][j] += a[i].x * b[j].x; acc[i][j] += a[i].y * b[j].y;
+                    acc[i][j] += a[i].z * b[j].z; acc[i][j] += a[i].w * b[j].w;
+                }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) part[warp][ty + 4 * i][tx + 8 * j] = acc[i][j];
+    } else if (const int row = row0 + warp - 8; row < Tn) {
+        const int i_row = warp - 8, blk = col0 < Nq ? 0 : (col0 < Nq + Nkv ? 1 : 2);
+        float4 xv[kSmallVecs];
+#pragma unroll
+        for (int v = 0; v < kSmallVecs; ++v)
+            xv[v] = (lane + 32 * v) * 4 < K ? reinterpret_cast<const float4 *>(x + (size_t)row * K)[lane + 32 * v] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const RowFacts f = row_facts(row, positions, a_req, adapter_ids, qsl, seq_lens, block_tables, max_blocks, num_pages, page_size,
+                                     max_adapters, R, mode, status);
+        float dlt = 0.f;
+        if (f.adapter >= 0) {
+            const AdapterDev ad = adapters[f.adapter];
+            if (ad.rank == 0) report(status, ALORA_ERR_NO_WEIGHTS);
+            const float *A = (const float *)ad.A + (size_t)blk * RP * K, *B = (const float *)ad.B + (size_t)min(col0 + lane, N - 1) * RP;
+            for (int i0 = 0; i0 < ad.rank; i0 += 8) {   // (rows and columns of the padding are zero; RP is a multiple of 16)
+                float t[8];
+                float4 b[2];
+                b[0] = *reinterpret_cast<const float4 *>(B + i0); b[1] = *reinterpret_cast<const float4 *>(B + i0 + 4);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) t[i] = 0.f;
+#pragma unroll
+                for (int v = 0; v < kSmallVecs; ++v) {
+                    if (v * 128 >= K) break;
+                    const bool in = (lane + 32 * v) * 4 < K;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float4 a = in ? reinterpret_cast<const float4 *>(A + (size_t)(i0 + i) * K)[lane + 32 * v] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        t[i] += a.x * xv[v].x; t[i] += a.y * xv[v].y; t[i] += a.z * xv[v].z; t[i] += a.w * xv[v].w;
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    for (int off = 16; off; off >>= 1) t[i] += __shfl_xor_sync(0xffffffffu, t[i], off);
+                    t[i] *= ad.scale;
+                }
+                const float bb[8] = {b[0].x, b[0].y, b[0].z, b[0].w, b[1].x, b[1].y, b[1].z, b[1].w};
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (i0 + i < ad.rank) dlt += bb[i] * t[i];
+            }
+        }
+        delta_s[i_row][lane] = dlt;
+        if (lane == 0) {
+            adapter_s[i_row] = f.adapter; slot_s[i_row] = f.slot;
+            if (col0 == 0) { token_req[row] = f.req; row_adapter[row] = f.adapter; slot_map[row] = f.slot; }
+        }
+    }
+    __syncthreads();
+    const int row = row0 + warp, n = col0 + lane;
+    if (warp >= 16 || row >= Tn || n >= N) return;
+    float v = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) v += part[w][warp][lane];
+    if (adapter_s[warp] >= 0) v += delta_s[warp][lane];
+    y[(size_t)row * N + n] = v;
+    const int slot = slot_s[warp];
+    if (pool == nullptr || n < Nq || slot < 0) return;
+    const int plane = n < Nq + Nkv ? 0 : 1, c = n - Nq - plane * Nkv;
+    pool[((((size_t)(slot / page_size) * 2 + plane) * Hkv + c / hd) * page_size + slot % page_size) * hd + c % hd] = v;
+}
+
+// ---------------------------------------------------------------------------------------------
 // KV append (both data types): one 16-byte vector per thread.  Row t's k part
 // qkv[t][Nq .. Nq+Nkv) goes to pool[page][0][head][row][:], its v part to plane 1.  Tokens whose
 // slot is -1 (rejected by the metadata step) are skipped.
@@ -389,24 +528,51 @@ int launch_rope(alora_ctx *ctx, void *qkv, const int32_t *positions, int T, void
 // ---------------------------------------------------------------------------------------------
 template <int HD, int HC>
 __global__ void __launch_bounds__(256)
-attn_simt_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ positions, const int32_t *__restrict__ token_req,
-                 const int32_t *__restrict__ slot_map, const int32_t *__restrict__ block_tables, int max_blocks, int num_pages,
-                 int page_size, int N, int Nq, int Hkv, int G, float scale, const float *__restrict__ pool,
+attn_simt_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ positions, const int32_t *__restrict__ qsl,
+                 const int32_t *__restrict__ seq_lens, const int32_t *__restrict__ block_tables, int max_blocks, int num_pages,
+                 int page_size, int N, int Nq, int Hkv, int G, int R, float scale, const float *pool,
                  float *__restrict__ out, int32_t *status) {
     constexpr int V = HD / 32, U = HD == 128 ? 2 : 4;   // 16-byte vectors of a lane; keys of a stream in flight
     __shared__ float o_s[8][HC][HD], m_s[8][HC], l_s[8][HC];
     tc::grid_dep_launch();
-    tc::grid_dep_wait();
     const int t = blockIdx.x, kvh = blockIdx.y, h0 = (int)blockIdx.z * HC, nh = min(HC, G - h0);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, stream = warp * 4 + (lane >> 3), d0 = (lane & 7) * 4;
-    const int r = token_req[t], p = positions[t];
+    // The caller's arrays and the cached keys of earlier calls were complete before the preceding kernel of the stream (an
+    // ordinary launch) began: they are fetched beside it, the new rows after it.
+    const RowFacts f = row_facts(t, positions, nullptr, nullptr, qsl, seq_lens, block_tables, max_blocks, num_pages, page_size, 0, R,
+                                 ALORA_MODE_BASE, status);
+    const int r = f.req, p = f.pos, first_new = p - (t - qsl[r]);
     float *orow = out + (size_t)t * Nq + (size_t)(kvh * G + h0) * HD;
-    if (slot_map[t] < 0) {  // token rejected by the metadata step: defined output, no cache access
+    if (f.slot < 0) {  // a token that the metadata step rejects: defined output, no cache access
+        tc::grid_dep_wait();
         for (int d = threadIdx.x; d < nh * HD; d += 256) orow[d] = 0.f;
         return;
     }
     float4 q[HC][V], acc[HC][V];
     float m[HC], l[HC];
+    const size_t plane = (size_t)Hkv * page_size * HD;
+    const int32_t *table = block_tables + (size_t)r * max_blocks;
+    float4 kv[U][V], vv[U][V];
+    bool on[U];
+    // keys j0 + 32 u of a stream, either those in the cache before this call or the new ones
+    auto load = [&](int j0, bool cached) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int j = j0 + 32 * u;
+            if ((j < first_new) != cached) continue;
+            const int page = j <= p ? table[j / page_size] : -1;
+            on[u] = page >= 0 && page < num_pages;
+            if (j <= p && !on[u]) report(status, ALORA_ERR_PAGE_RANGE);
+            const float *kr = pool + ((size_t)(on[u] ? page : 0) * 2 * Hkv + kvh) * page_size * HD + (size_t)(j % page_size) * HD + d0;
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                kv[u][v] = on[u] ? *reinterpret_cast<const float4 *>(kr + 32 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
+                vv[u][v] = on[u] ? *reinterpret_cast<const float4 *>(kr + plane + 32 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+    };
+    load(stream, true);
+    tc::grid_dep_wait();
 #pragma unroll
     for (int c = 0; c < HC; ++c) {
         m[c] = -INFINITY; l[c] = 0.f;
@@ -417,23 +583,9 @@ attn_simt_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ posi
             acc[c][v] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
     }
-    const size_t plane = (size_t)Hkv * page_size * HD;
-    const int32_t *table = block_tables + (size_t)r * max_blocks;
     for (int j0 = stream; j0 - stream <= p; j0 += 32 * U) {
-        float4 kv[U][V], vv[U][V];
-        bool on[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int j = j0 + 32 * u, page = j <= p ? table[j / page_size] : -1;
-            on[u] = page >= 0 && page < num_pages;
-            if (j <= p && !on[u]) report(status, ALORA_ERR_PAGE_RANGE);
-            const float *kr = pool + ((size_t)(on[u] ? page : 0) * 2 * Hkv + kvh) * page_size * HD + (size_t)(j % page_size) * HD + d0;
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                kv[u][v] = on[u] ? *reinterpret_cast<const float4 *>(kr + 32 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
-                vv[u][v] = on[u] ? *reinterpret_cast<const float4 *>(kr + plane + 32 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-        }
+        if (j0 != stream) load(j0, true);
+        load(j0, false);
 #pragma unroll
         for (int c = 0; c < HC; ++c) {
             float s[U], mx = m[c];
@@ -670,6 +822,25 @@ int launch_project_simt(alora_ctx *ctx, int layer, const void *hidden, int T, vo
     return e == cudaSuccess ? 2 : -1;
 }
 
+// Whether a layer call takes project_small_simt_kernel: x rows that a warp holds in registers, and at most two blocks an SM (the t
+// that every column tile forms again costs as much as its base sums from rank 32 on).  A rule of sizes: all modes take the
+// same route.
+bool simt_small_layer(const alora_ctx *ctx, int T) {
+    const Dims &d = ctx->d;
+    return ctx->cfg.dtype == ALORA_DTYPE_FP32 && T > 0 && d.H % 4 == 0 && d.H <= 128 * kSmallVecs &&
+           (long long)((d.N + 31) / 32) * ((T + 15) / 16) <= 2ll * ctx->sm_count;
+}
+int launch_project_small_simt(alora_ctx *ctx, int layer, const void *hidden, const BatchArgs &b, void *qkv, void *kv_pool, cudaStream_t s) {
+    const Dims &d = ctx->d;
+    ProfScope prof(ctx, KK_PROJECT, s);
+    project_small_simt_kernel<<<(d.N + 31) / 32 * ((b.T + 15) / 16), 768, 0, s>>>(
+        (const float *)hidden, (const float *)ctx->layers[layer].wqkv, b.T, d.H, d.N, d.Nq, d.Nkv, d.RP,
+        ctx->d_adapters + (size_t)layer * ctx->cfg.max_adapters, b.positions, b.activation_offsets, b.adapter_ids, b.query_start_loc,
+        b.seq_lens, b.block_tables, b.max_blocks, b.num_pages, d.page, ctx->cfg.max_adapters, b.R, b.mode, d.hd, d.Hkv, (float *)kv_pool,
+        ctx->d_token_req, ctx->d_row_adapter, ctx->d_slot, (float *)qkv, ctx->d_status);
+    return 1;
+}
+
 int launch_linear_simt(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
                        const void *residual, cudaStream_t s) {
     if (T == 0) return 0;
@@ -687,8 +858,8 @@ int launch_attend_simt(alora_ctx *ctx, const void *qkv, const BatchArgs &b, cons
     ProfScope prof(ctx, KK_ATTENTION, s);
     auto go = [&](auto kernel, int hc) {
         return launch_kernel(kernel, dim3(b.T, d.Hkv, (d.G + hc - 1) / hc), dim3(256), 0, s, true, (const float *)qkv, b.positions,
-                             (const int32_t *)ctx->d_token_req, (const int32_t *)ctx->d_slot, b.block_tables, b.max_blocks, b.num_pages,
-                             d.page, d.N, d.Nq, d.Hkv, d.G, d.softmax_scale, (const float *)pool, (float *)out, ctx->d_status);
+                             b.query_start_loc, b.seq_lens, b.block_tables, b.max_blocks, b.num_pages,
+                             d.page, d.N, d.Nq, d.Hkv, d.G, b.R, d.softmax_scale, (const float *)pool, (float *)out, ctx->d_status);
     };
     const bool two = d.G > 1;
     const cudaError_t e = d.hd == 32 ? (two ? go(attn_simt_kernel<32, 2>, 2) : go(attn_simt_kernel<32, 1>, 1))
