@@ -668,6 +668,9 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
     // The per-request inputs are read many times (binary searches, list builders): one parallel pass stages them
     // in shared memory, so that the later steps do not each pay a round trip to global memory.
     __shared__ int32_t s_req[4 * kMetaStageR + 1];
+    // The first launch of a call is a dependent one too, but lets its successor start only when everything before the call
+    // has completed: later kernels rely on that for what they read of the caller's before their own wait.
+    if (phases & kMetaProjection) tc::grid_dep_wait();
     tc::grid_dep_launch();   // the next kernel's blocks may start their set-up; they wait for this kernel's results
     const int tok = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     const int my_pos = (phases & kMetaProjection) && tok < T ? positions[tok] : 0;   // (in flight with the per-request inputs)
@@ -741,6 +744,7 @@ metadata_few_row_kernel(const int32_t *__restrict__ positions, const int32_t *a_
                         int32_t *__restrict__ slot_map, const AdapterDev *__restrict__ adapters,
                         FewRowMeta *__restrict__ few_row_meta, int few_tiles, int32_t *status) {
     __shared__ int32_t s_req[4 * kFewRowMax + 1];
+    tc::grid_dep_wait();     // (in this order: see metadata_kernel)
     tc::grid_dep_launch();
     const int tok = (int)(blockIdx.x * kFewRowMax + threadIdx.x), my_pos = tok < T ? positions[tok] : 0;   // (in flight with the per-request inputs)
     if (R <= kFewRowMax) {   // the per-request inputs are read several times (binary search): stage them
@@ -787,13 +791,12 @@ int launch_metadata(alora_ctx *ctx, const BatchArgs &b, cudaStream_t s, int phas
     const AdapterDev *ads = b.layer >= 0 ? ctx->d_adapters + (size_t)b.layer * ctx->cfg.max_adapters : nullptr;
     if (phases == kMetaProjection && b.few_row) {
         FewRowMeta *few = ads != nullptr ? ctx->d_skinny_meta + (size_t)b.layer * ctx->few_tiles : nullptr;
-        metadata_few_row_kernel<<<dim3((b.T + kFewRowMax - 1) / kFewRowMax, b.n_layers), kFewRowMax, 0, s>>>(
+        return launch_kernel(metadata_few_row_kernel, dim3((b.T + kFewRowMax - 1) / kFewRowMax, b.n_layers), dim3(kFewRowMax), 0, s, true,
             b.positions, b.activation_offsets, b.adapter_ids, b.query_start_loc, b.seq_lens, b.block_tables, b.max_blocks,
             b.num_pages, ctx->d.page, ctx->cfg.max_adapters, b.T, b.R, b.mode, ctx->d_token_req, ctx->d_row_adapter,
-            ctx->d_slot, ads, few, ctx->few_tiles, ctx->d_status);
-        return 1;
+            ctx->d_slot, ads, few, ctx->few_tiles, ctx->d_status) == cudaSuccess ? 1 : -1;
     }
-    const cudaError_t e = launch_kernel(metadata_kernel, dim3(grid), dim3(threads), 0, s, attn_only,
+    const cudaError_t e = launch_kernel(metadata_kernel, dim3(grid), dim3(threads), 0, s, true,
         b.positions, b.activation_offsets, b.adapter_ids, b.query_start_loc, b.seq_lens, b.block_tables,
         b.max_blocks, b.num_pages, ctx->d.page, ctx->cfg.max_adapters, b.T, b.R, b.mode, ctx->d_token_req,
         ctx->d_row_adapter, ctx->d_slot, ctx->max_pairs, ctx->d_pairs, ctx->d_pair_off, ctx->max_quads, ctx->d_quads, ctx->d_quad_off, ctx->d_counts, ctx->d_seg_scratch,

@@ -236,6 +236,7 @@ project_small_simt_kernel(const float *__restrict__ x, const float *__restrict__
                           float *__restrict__ y, int32_t *status) {
     __shared__ float part[8][16][32 + 1], delta_s[16][32 + 1];
     __shared__ int adapter_s[16], slot_s[16];
+    tc::grid_dep_wait();     // (in this order: the attention kernel relies on it for what it reads before its own wait)
     tc::grid_dep_launch();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_col = (N + 31) / 32, row0 = (int)blockIdx.x / n_col * 16, col0 = (int)blockIdx.x % n_col * 32;
@@ -537,8 +538,8 @@ attn_simt_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ posi
     tc::grid_dep_launch();
     const int t = blockIdx.x, kvh = blockIdx.y, h0 = (int)blockIdx.z * HC, nh = min(HC, G - h0);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, stream = warp * 4 + (lane >> 3), d0 = (lane & 7) * 4;
-    // The caller's arrays and the cached keys of earlier calls were complete before the preceding kernel of the stream (an
-    // ordinary launch) began: they are fetched beside it, the new rows after it.
+    // The caller's arrays and the cached keys of earlier calls were complete before the preceding kernel of the call let this one
+    // start: they are fetched beside it, the new rows after it.
     const RowFacts f = row_facts(t, positions, nullptr, nullptr, qsl, seq_lens, block_tables, max_blocks, num_pages, page_size, 0, R,
                                  ALORA_MODE_BASE, status);
     const int r = f.req, p = f.pos, first_new = p - (t - qsl[r]);
@@ -833,12 +834,11 @@ bool simt_small_layer(const alora_ctx *ctx, int T) {
 int launch_project_small_simt(alora_ctx *ctx, int layer, const void *hidden, const BatchArgs &b, void *qkv, void *kv_pool, cudaStream_t s) {
     const Dims &d = ctx->d;
     ProfScope prof(ctx, KK_PROJECT, s);
-    project_small_simt_kernel<<<(d.N + 31) / 32 * ((b.T + 15) / 16), 768, 0, s>>>(
+    return launch_kernel(project_small_simt_kernel, dim3((d.N + 31) / 32 * ((b.T + 15) / 16)), dim3(768), 0, s, true,
         (const float *)hidden, (const float *)ctx->layers[layer].wqkv, b.T, d.H, d.N, d.Nq, d.Nkv, d.RP,
         ctx->d_adapters + (size_t)layer * ctx->cfg.max_adapters, b.positions, b.activation_offsets, b.adapter_ids, b.query_start_loc,
         b.seq_lens, b.block_tables, b.max_blocks, b.num_pages, d.page, ctx->cfg.max_adapters, b.R, b.mode, d.hd, d.Hkv, (float *)kv_pool,
-        ctx->d_token_req, ctx->d_row_adapter, ctx->d_slot, (float *)qkv, ctx->d_status);
-    return 1;
+        ctx->d_token_req, ctx->d_row_adapter, ctx->d_slot, (float *)qkv, ctx->d_status) == cudaSuccess ? 1 : -1;
 }
 
 int launch_linear_simt(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
