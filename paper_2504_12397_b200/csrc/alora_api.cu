@@ -218,7 +218,7 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
     alloc((void **)&ctx->d_slot, Tm * 4);
     alloc((void **)&ctx->d_pairs, (size_t)ctx->max_pairs * sizeof(TilePair));
     alloc((void **)&ctx->d_pair_off, (Tm / kTileRows + 2) * 4);
-    alloc((void **)&ctx->d_counts, 16 * 4);
+    alloc((void **)&ctx->d_counts, 32 * 4);
     alloc((void **)&ctx->d_seg_scratch, ((size_t)14 * c.max_requests + 5) * 4);
     alloc((void **)&ctx->d_t_ready, (size_t)ctx->max_pairs * 4);
     alloc(&ctx->d_t, c.dtype == ALORA_DTYPE_BF16 ? (size_t)ctx->t_slots * kTileRows * 3 * d.RP * 2 : Tm * 3 * d.RP * 4);
@@ -230,7 +230,7 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
     if (c.dtype == ALORA_DTYPE_BF16 && 128 % d.G == 0) {
         // tensor-core attention: one work item per (request, KV head, block of 2 * 128/G tokens)
         ctx->attn_q_block = 2 * (128 / d.G);
-        ctx->max_attn_items = (int)((Tm / ctx->attn_q_block + (size_t)c.max_requests) * d.Hkv);
+        ctx->max_attn_items = std::max((int)((Tm / ctx->attn_q_block + (size_t)c.max_requests) * d.Hkv), ctx->sm_count);
         alloc((void **)&ctx->d_attn_items, (size_t)ctx->max_attn_items * sizeof(AttnWork));
         alloc((void **)&ctx->d_attn_off, ((size_t)c.max_requests + 1) * 4);
         alloc((void **)&ctx->d_attn_cta_start, (size_t)ctx->sm_count * 4);
@@ -302,7 +302,7 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
     if (st == ALORA_OK) {
         e = cudaMemset(ctx->d_status, 0, 4);
         if (e == cudaSuccess) e = cudaMemset(ctx->d_adapters, 0, n_ad * sizeof(AdapterDev));
-        if (e == cudaSuccess) e = cudaMemset(ctx->d_counts, 0, 64);
+        if (e == cudaSuccess) e = cudaMemset(ctx->d_counts, 0, 32 * 4);
         if (e == cudaSuccess) e = cudaMemset(ctx->d_t_ready, 0, (size_t)ctx->max_pairs * 4);
         if (e == cudaSuccess && ctx->d_quad_ready) e = cudaMemset(ctx->d_quad_ready, 0, (size_t)ctx->max_quads * 4);
         if (e == cudaSuccess && ctx->d_rope_inv_freq) {

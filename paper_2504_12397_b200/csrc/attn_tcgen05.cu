@@ -58,23 +58,18 @@ struct AttnArgs {
     int32_t *status;
     // work split: items below n_whole are taken whole; the key tiles of the others are concatenated and cut into runs
     const int32_t *run_counts;  // [0] key tiles in the concatenation, [1] tiles per run, [2] n_whole, [3] tiles of the whole items
+    int32_t *claims;            // whole items claimed beyond the first round (zero at the launch)
+    int32_t *next_claims;       // the counter of the next layer's launch on the same list, cleared here
     const int32_t *cta_start;   // [blocks] item that holds the first tile of the block's run
     float *part_o;              // [2 * blocks][hd][256] unnormalised output of a part, column-major over the 256 rows
     float *part_ml;             // [2 * blocks][2][256] exponent reference and row sum of a part
 };
 
-// The item a block takes whole in its `round`: dealt back and forth, so that with the list longest first no block gets
-// the longer item of every round.
-__device__ __forceinline__ int whole_item(int round) {
-    const int n = (int)gridDim.x, b = (int)blockIdx.x;
-    return round * n + ((round & 1) ? n - 1 - b : b);
-}
-
 // partial-result slot of part `part` of an item whose first part is held by block c_first: a block holds at
 // most one part > 0 (the piece its run starts with) and at most one part 0 of a cut item (the piece it ends with)
 __host__ __device__ __forceinline__ int part_slot(int c_first, int part) { return 2 * (c_first + part) + (part == 0 ? 1 : 0); }
 
-// A block's work: whole items (one of each round of `blocks` items) below n_whole, then the pieces of its run (tiles
+// A block's work: whole items, then the pieces of its run (tiles
 // [blockIdx * len, +len) of the concatenated key tiles of the items from n_whole on).  One piece = tiles [t0, t1)
 // of one item.  An item cut by run boundaries is worked on by consecutive blocks; each writes
 // its partial result to a slot and a merge kernel adds the parts up afterwards.
@@ -82,26 +77,53 @@ struct RunPiece {
     AttnWork w;
     int t0, t1, slot;   // slot of the partial result, -1: the whole item
 };
-// (What the iterator needs of the split is read again for every piece: kept in registers across the softmax it made the
-// batches that may be cut up to 10 % slower than those that cannot be; 4 x 1024 on 32768: 2 x 2080 -> 2 x 2020 us.)
+// Whole items are claimed, in list order (longest first): block b begins with item b, its K producer takes every later one
+// from a counter and hands it to the block's other warps through a ring in shared memory.  (Dealt back and forth by block index,
+// 7 requests of 1395 .. 2791 tokens left the longest block 20 % more than the claims do, 32 of 16 .. 512 on 512 .. 16384 cached 5 %.)
+// What the iterator needs of the split is read again for every piece: kept in registers across the softmax it made the
+// batches that may be cut up to 10 % slower than those that cannot be; 4 x 1024 on 32768: 2 x 2080 -> 2 x 2020 us.
 __device__ __forceinline__ int ld_again(const int32_t *p) {
     int v;
     asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
-struct RunIter {
-    int gt = -1, it = 0, round = 0;   // next tile of this block's run (-1: not begun), its item; rounds of whole items done
-    __device__ explicit RunIter(const AttnArgs &) {}
-    __device__ bool next(const AttnArgs &a, RunPiece &p) {
-        const int whole = whole_item(round);
-        if (whole < ld_again(a.run_counts + 2)) {
-            ++round;
-            p.w = a.items[whole];
-            p.t0 = 0;
-            p.t1 = (p.w.kv_end + kKeysPerTile - 1) / kKeysPerTile;
-            p.slot = -1;
-            return true;
+template <bool kRuns>   // kRuns: items may be cut into runs
+struct PieceIter {
+    tc::ItemRing ring;
+    bool whole = true, begun = false;
+    int gt = -1, it = 0;   // next tile of this block's run (-1: not begun), its item
+    __device__ __forceinline__ explicit PieceIter(const tc::ItemRing &r) : ring(r) {}
+    // called by whole warps; kClaims: by the warp that claims
+    template <bool kClaims>
+    __device__ __forceinline__ bool next(const AttnArgs &a, RunPiece &p, volatile int *abort_flag, bool &ok) {
+        if (whole) {
+            int item;
+            if (!begun) {   // (the first item's entry is fetched beside the count: the list has room for an entry per block)
+                begun = true;
+                p.w = a.items[blockIdx.x];
+                item = (int)blockIdx.x < ld_again(kRuns ? a.run_counts + 2 : a.n_items) ? (int)blockIdx.x : -1;
+            } else if (kClaims) {
+                if ((threadIdx.x & 31) == 0) {
+                    item = (int)gridDim.x + atomicAdd(a.claims, 1);
+                    if (item >= ld_again(kRuns ? a.run_counts + 2 : a.n_items)) item = -1;
+                    if (!ring.put(item, abort_flag)) item = -2;
+                }
+                item = __shfl_sync(0xffffffffu, item, 0);
+                if ((threadIdx.x & 31) != 0) ++ring.n;
+            } else {
+                item = ring.take(abort_flag);
+            }
+            if (item >= 0) {
+                if (item != (int)blockIdx.x) p.w = a.items[item];
+                p.t0 = 0;
+                p.t1 = (p.w.kv_end + kKeysPerTile - 1) / kKeysPerTile;
+                p.slot = -1;
+                return true;
+            }
+            whole = false;
+            if (item == -2) { ok = false; return false; }
         }
+        if (!kRuns) return false;
         const int total = ld_again(a.run_counts), len = ld_again(a.run_counts + 1), off = ld_again(a.run_counts + 3);
         const int begin = min(total, (int)blockIdx.x * len), end = min(total, begin + len);
         if (gt < 0) {
@@ -121,22 +143,6 @@ struct RunIter {
         return true;
     }
 };
-// The same interface for batches whose items are all taken whole (what the host can tell in advance for short
-// batches).
-struct WholeIter {
-    int round = 0, n_items;
-    __device__ explicit WholeIter(const AttnArgs &a) : n_items(*a.n_items) {}
-    __device__ bool next(const AttnArgs &a, RunPiece &p) {
-        const int whole = whole_item(round);
-        if (whole >= n_items) return false;
-        ++round;
-        p.w = a.items[whole];
-        p.t0 = 0;
-        p.t1 = (p.w.kv_end + kKeysPerTile - 1) / kKeysPerTile;
-        p.slot = -1;
-        return true;
-    }
-};
 
 template <int HD>
 struct AttnSmem {
@@ -146,7 +152,8 @@ struct AttnSmem {
     static constexpr int kKOff = 2 * kQBytes;
     static constexpr int kVOff = kKOff + kKvStages * kKvBytes;
     static constexpr int kBarOff = kVOff + kKvStages * kKvBytes;
-    static constexpr int kTotal = kBarOff + 256 + 1024;
+    static constexpr int kItemRingOff = kBarOff + 256;
+    static constexpr int kTotal = kItemRingOff + 128 + 1024;
 };
 
 // V tile as the B operand of P V: N = head dim (contiguous in memory: "MN-major"), K = keys.
@@ -251,12 +258,12 @@ __device__ __forceinline__ float fast_exp2(float x) {
     return y;
 }
 
-template <int HD, bool kRuns>   // kRuns: items may be cut into runs (RunIter); else all items are whole (WholeIter)
+template <int HD, bool kRuns>   // kRuns: items may be cut into runs; else all items are whole
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKV,
                     const AttnArgs a) {
     using S = AttnSmem<HD>;
-    using Iter = typename std::conditional<kRuns, RunIter, WholeIter>::type;
+    using Iter = PieceIter<kRuns>;
     constexpr int kHalves = HD / 64;             // 64-wide column halves of the head dim
     constexpr int kHalfQ = 128 * 128;            // bytes of one 128-row x 64-col bf16 block
     extern __shared__ uint8_t smem_raw[];
@@ -281,8 +288,10 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem_al + S::kBarOff + 16 + 8 * 4 * kKvStages + 112);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem_al + S::kBarOff + 16 + 8 * 4 * kKvStages + 120);
 
+    const tc::ItemRing ring{smem_base + S::kItemRingOff, reinterpret_cast<volatile int *>(smem_al + S::kItemRingOff + 16 * tc::kItemSlots)};
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
+        ring.init(11);   // the V producer, the issuers and the softmax warps
         tc::mbar_init(q_full, 1); tc::mbar_init(q_free, 2);   // *_free: one commit per group's MMA issuer
         for (int s = 0; s < kKvStages; ++s) {
             tc::mbar_init(k_full(s), 1); tc::mbar_init(k_free(s), 2);
@@ -303,6 +312,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const uint32_t tmem_base = *tmem_slot;
     tc::grid_dep_launch();
     tc::grid_dep_wait();   // work list, q/k/v rows and the cache rows of the new tokens come from earlier kernels
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.next_claims = 0;
     // tensor-memory columns of group g (base g*256): S_g 0..63, P_g 64..95, the first 64 head-dim columns of Q_g as
     // bf16 pairs 96..127, O_g 128..255
     // A work item with more than 128 / G tokens gives each group its own 128 score rows, and each group takes both
@@ -334,9 +344,10 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         const int plane = warp == 8 ? 0 : 1;
         uint32_t n_item = 0, kt = 0;
         bool ok = true;
-        Iter run(a);
+        Iter run(ring);
         RunPiece pc;
-        for (; ok && run.next(a, pc); ++n_item) {
+        auto next = [&]() { return plane == 0 ? run.template next<true>(a, pc, abort_flag, ok) : run.template next<false>(a, pc, abort_flag, ok); };
+        for (; ok && next(); ++n_item) {
             const AttnWork &w = pc.w;
             if (plane == 0) {
                 if (lane == 0) {
@@ -430,9 +441,9 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         auto wait_all = [&](uint32_t bar, uint32_t parity) {
             return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort_flag));
         };
-        Iter run(a);
+        Iter run(ring);
         RunPiece pc;
-        for (; ok && run.next(a, pc); ++n_item) {
+        for (; ok && run.template next<false>(a, pc, abort_flag, ok); ++n_item) {
             const bool shared = pc.w.q_count <= tok_per_group;
             const int n_steps = (pc.t1 - pc.t0) << (shared ? 0 : 1);   // half tiles of this group in the piece
             if (!wait_all(q_full, n_item & 1)) { ok = false; break; }
@@ -498,7 +509,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         uint32_t n_s = 0, kt = 0;   // n_s: half tiles of this group so far (phase counter of its barriers)
         uint32_t n_merge = 0;       // shared items so far (phase counter of the merge barriers)
         bool ok = true;
-        Iter run(a);
+        Iter run(ring);
         RunPiece pc, pc_next;
         // first token of this group's rows inside an item (a shared item: both groups hold the same rows)
         auto tok_base = [&](const AttnWork &w) { return w.q_count <= tok_per_group ? 0 : g * tok_per_group; };
@@ -524,7 +535,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(q_ready(g));
         };
-        bool have = run.next(a, pc);
+        bool have = run.template next<false>(a, pc, abort_flag, ok);
         if (have) { load_q(pc.w); publish_q(); }
         while (ok && have) {
             const AttnWork &w = pc.w;
@@ -671,7 +682,8 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             if (!ok) break;
             // the next item's rows of Q go to tensor memory underneath this item's last P V, so that its first
             // Q K^T runs underneath this item's output
-            const bool have_next = run.next(a, pc_next);
+            const bool have_next = run.template next<false>(a, pc_next, abort_flag, ok);
+            if (!ok) break;
             if (have_next) { load_q(pc_next.w); publish_q(); }
             // the item's last P V, normalisation, store
             if (!tc::mbar_wait(pv_done(g), (n_s - 1) & 1, abort_flag)) { ok = false; break; }
@@ -922,7 +934,7 @@ static int launch_attend_long(alora_ctx *ctx, const void *qkv, const BatchArgs &
     a.N = d.N; a.Nq = d.Nq; a.qkv = (const __nv_bfloat16 *)qkv; a.scale_log2 = d.softmax_scale * 1.4426950408889634f;
     a.out = (__nv_bfloat16 *)out; a.status = ctx->d_status;
     a.run_counts = ctx->d_counts + 6; a.cta_start = ctx->d_attn_cta_start;
-    a.part_o = ctx->d_attn_part_o; a.part_ml = ctx->d_attn_part_ml;
+    a.part_o = ctx->d_attn_part_o; a.part_ml = ctx->d_attn_part_ml; a.claims = ctx->d_counts + 15 + (b.layer & 1); a.next_claims = ctx->d_counts + 15 + (~b.layer & 1);
     const int max_items = (b.T / ctx->attn_q_block + b.R) * d.Hkv;
     ProfScope prof(ctx, KK_ATTENTION, s);
     static bool attr_set[2][64] = {};
@@ -941,7 +953,7 @@ static int launch_attend_long(alora_ctx *ctx, const void *qkv, const BatchArgs &
     const bool few_items = max_items < n_sm && max_tiles >= (long long)kAttnMinRunTiles * n_sm &&
                            (long long)b.T > (long long)b.R * ctx->small_max_tokens;
     const bool runs = n_sm > 1 && (long_batch || few_items);
-    const int grid = runs ? n_sm : std::max(1, std::min(n_sm, max_items));
+    const int grid = runs ? n_sm : std::max(1, std::min(n_sm, 2 * max_items));   // (twice: the list may hold half-size items)
     if (dev >= 0 && dev < 64 && !attr_set[hi][dev]) {
         cudaError_t e = hi ? cudaFuncSetAttribute(attn_tcgen05_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<128>::kTotal)
                            : cudaFuncSetAttribute(attn_tcgen05_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<64>::kTotal);

@@ -192,8 +192,10 @@ __device__ __forceinline__ int few_row_limit(const int32_t *__restrict__ qsl, in
 // `q_block` tokens; one item per (request, KV head, block), blocks of the same KV stream adjacent so
 // that blocks running at the same time share their K/V pages in L2.  Keys 0 .. position of the
 // block's last token are visible to the block (causal limit); per-row limits are applied in the kernel.
-// Requests are taken longest first (`order`, where the scratch has room for it), a request's last block first: dealt to
-// the blocks back and forth (attn_tcgen05.cu), items of very different length then end at about the same time.
+// Requests are taken longest first (`order`, where the scratch has room for it), a request's last block first: the kernel's blocks
+// claim the items in this order and end at about the same time.
+// Where items of half the size still fit in one round over the n_blocks blocks of the kernel they are taken instead: a block of
+// q_block / 2 tokens takes half as long (both query groups of the kernel work on the same rows, each on half of the keys).
 __device__ __forceinline__ void metadata_attn_items(const int32_t *__restrict__ qsl, const int32_t *__restrict__ seq_lens,
                                            int R, int Hkv, int q_block, int small_max, int max_items,
                                            AttnWork *__restrict__ items, int32_t *__restrict__ counts,
@@ -205,6 +207,23 @@ __device__ __forceinline__ void metadata_attn_items(const int32_t *__restrict__ 
         const int n_new = qsl[r + 1] - qsl[r];
         return n_new > small_max ? (n_new + q_block - 1) / q_block : 0;
     };
+    {
+        __shared__ int n_half, n_tiles, longest;
+        if (threadIdx.x == 0) n_half = n_tiles = longest = 0;
+        __syncthreads();
+        for (int r = threadIdx.x; r < R; r += blockDim.x) {
+            const int n_new = qsl[r + 1] - qsl[r], n = blocks_of(r);
+            if (n == 0) continue;
+            atomicAdd(&n_half, (n_new + q_block / 2 - 1) / (q_block / 2));
+            const int t = (seq_lens[r] + kAttnKeysPerTile - 1) / kAttnKeysPerTile;
+            atomicAdd(&n_tiles, n * t);
+            atomicMax(&longest, t);
+        }
+        __syncthreads();
+        // (not where the items are long enough to be cut into runs, see below)
+        if (n_half * Hkv <= n_blocks && longest < n_tiles * Hkv / n_blocks + kAttnSpreadMinGain) q_block /= 2;
+        __syncthreads();
+    }
     if (order != nullptr) {
         int32_t *key = order + R;
         for (int r = threadIdx.x; r < R; r += blockDim.x) key[r] = blocks_of(r) > 0 ? seq_lens[r] : 0;
@@ -231,6 +250,7 @@ __device__ __forceinline__ void metadata_attn_items(const int32_t *__restrict__ 
         if (n > max_items) { report(status, ALORA_ERR_CAPACITY); n = 0; }
         total = n;
         counts[1] = n;
+        counts[15] = counts[16] = 0;   // (the kernel of layer l claims through the one and clears the other for layer l + 1)
     }
     __syncthreads();
     int sum = 0, tmin = INT_MAX, tmax = 0;   // key tiles of this thread's items
@@ -259,10 +279,10 @@ __device__ __forceinline__ void metadata_attn_items(const int32_t *__restrict__ 
         sum += n; tmin = min(tmin, n); tmax = max(tmax, n);
     }
     // Work split of the attention kernel over its n_blocks blocks (the launch uses that many whenever a cut is
-    // possible).  Normally every item is taken whole, round-robin.
+    // possible).  Normally every item is taken whole.
     // Long batches (at least kAttnCutMinTiles key tiles per block) of items of nearly equal length that make at
     // least kAttnCutMinWaves full rounds: the first n_whole = n_blocks * floor(items / n_blocks) items are taken
-    // whole, round-robin; the key tiles of the remaining items are concatenated and cut into runs of equal length,
+    // whole; the key tiles of the remaining items are concatenated and cut into runs of equal length,
     // one per block, so an item can be cut into parts that different blocks work on (a merge kernel adds the
     // parts up).
     //   items[i].split = tiles before item i;  counts[6] = tiles in the concatenation, counts[7] = run length,

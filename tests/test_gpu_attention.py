@@ -200,3 +200,12 @@ def test_leading_keys_with_scores_of_minus_infinity(oracle64, S, dead):
     got = _attend_values(shape, b, pool, qkv)
     want = _oracle_values(oracle64, shape, b, np.where(np.isinf(pool), np.float32(-1e30), pool), qkv)
     hp.assert_close(got, want, 2e-2, "keys of -inf in front", block=shape.head_dim)
+
+
+@pytest.mark.parametrize("S", [[33], [32, 64, 65, 31], [127, 128, 129], [33, 64] * 19, [40, 33] * 45])
+def test_blocks_of_half_size_and_claimed_items(oracle64, S):
+    """Few items: blocks of 32 tokens instead of 64, at the edges of both; 38 requests that fill the blocks exactly with
+    halves; 90 requests with more items than blocks, which the blocks claim."""
+    P = [(i * 613) % 1500 for i in range(len(S))]
+    err, _, _ = _attend_case(oracle64, SHAPE_G4, P, S, seed=700 + len(S))
+    assert err <= 2e-2
