@@ -19,8 +19,8 @@
 //   warp 1   MMA issuer (even block; the whole warp walks, an elected lane issues)
 //   warps 2-9  epilogue: tcgen05.ld one row per thread, bf16, through shared memory and TMA to the output, the new k and v
 //            rows to the page pool, or t for shrink items
-// The two row tiles of a block accumulate in the two halves of tensor memory; the epilogue drains one half while the
-// tensor cores still or already work on the other.
+// The two row tiles of a block accumulate in the two halves of tensor memory; the epilogue takes a half into registers while the
+// tensor cores still or already work on the other, and finishes it underneath the next item.
 // All waits are bounded; on expiry ALORA_ERR_TIMEOUT is recorded and the blocks leave normally.
 #include <algorithm>
 
@@ -141,19 +141,11 @@ __device__ __forceinline__ void mma2_commit(uint32_t bar) {
         ::"r"(bar), "h"((uint16_t)3)
         : "memory");
 }
-__device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-}
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, uint32_t src, int c0, int c1) {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];\n\tcp.async.bulk.commit_group;"
                  ::"l"((uint64_t)map), "r"(src), "r"(c0), "r"(c1) : "memory");
 }
-__device__ __forceinline__ float silu_mul(float g, float u) { return g / (1.f + __expf(-g)) * u; }
+__device__ __forceinline__ float silu_mul(float g, float u) { return __fdividef(g, 1.f + __expf(-g)) * u; }
 
 // (none for a B with an Inf or NaN: see TilePair)
 __device__ __forceinline__ int rank_steps(const DuoArgs &a, int adapter) {
@@ -171,7 +163,8 @@ struct DuoItem {
     __device__ __forceinline__ int tile(int h, uint32_t crank) const { return 4 * quad + 2 * (h0 + h) + (int)crank; }
 };
 // kDuoQkv: the column tiles of a quad are neighbours in the list; else the quads of a column tile (the clusters that
-// run together share a W tile).
+// run together share a W tile), beginning with another one in every column: a last quad of one or two row tiles takes half as
+// long, and would always fall to the same clusters.
 template <int kMode>
 __device__ __forceinline__ DuoItem decode_duo(const DuoArgs &a, int item, int n_shrink, int split, int e_base, int n_m, int n_q, int n_n) {
     DuoItem g;
@@ -184,7 +177,7 @@ __device__ __forceinline__ DuoItem decode_duo(const DuoArgs &a, int item, int n_
         g.adapter = p.adapter;
     } else {
         const int j = item - n_shrink;
-        g.quad = kMode == kDuoQkv ? j / n_n : j % n_q;
+        g.quad = kMode == kDuoQkv ? j / n_n : (j % n_q + j / n_q) % n_q;
         g.n0 = (kMode == kDuoQkv ? j % n_n : j / n_q) * (kMode == kDuoGlu ? a.bn / 2 : a.bn);
         if (a.quads) {
             g.e0 = a.quad_off[a.quad0 + g.quad];
@@ -547,14 +540,6 @@ gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                         else kv_at = ((long long)page * 2 * a.kv_heads * a.kv_page_size + slot % a.kv_page_size) << a.kv_hd_shift;
                     }
                 }
-                const bool mine = row_ok && !own_pass;
-                bool ok_j[4];   // the four rows of this lane's quad
-                long long kv_j[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    ok_j[j] = __shfl_sync(0xffffffffu, (int)mine, (lane & ~3) + j) != 0;
-                    kv_j[j] = kMode == kDuoQkv ? __shfl_sync(0xffffffffu, kv_at, (lane & ~3) + j) : -1;
-                }
                 const size_t row4 = (size_t)(row & ~3);
                 auto kv_put = [&](long long at, int col, uint4 o) {   // columns col .. col + 7 of the fused row
                     const int kcol = col - a.Nq;
@@ -583,84 +568,8 @@ gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                     else *reinterpret_cast<uint4 *>(a.out + (size_t)row * a.ldo + col) = o;
                 };
                 const bool any_own = __any_sync(0xffffffffu, own_pass);
-                // 32 columns from column `col` on of the warp's 32 rows, this lane's row in f
-                auto put32 = [&](int col, float (&f)[32]) {
-                    const int cu = col + ql * 8;   // the columns of the quad's four rows that this lane reads or writes
-                    uint4 u[4];
-                    if (kMode == kDuoLinear && a.residual) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            u[j] = ok_j[j] && cu < a.n_out ? *reinterpret_cast<const uint4 *>(a.residual + (row4 + j) * a.ldo + cu) : make_uint4(0, 0, 0, 0);
-                        tc::quad_transpose(u, ql);
-#pragma unroll
-                        for (int x = 0; x < 4; ++x) add_res8(reinterpret_cast<float(&)[8]>(f[8 * x]), u[x]);
-                    }
-#pragma unroll
-                    for (int x = 0; x < 4; ++x) u[x] = pack8(reinterpret_cast<const float(&)[8]>(f[8 * x]));
-                    const bool to_cache = kMode == kDuoQkv && a.kv_pool != nullptr && col >= a.Nq;
-                    if (!to_cache && !any_own) {
-                        // through shared memory and TMA, which cuts rows and columns off at the matrix's end (written from
-                        // registers, 64 bytes of a row per lane quad, a chunk took 1100 cycles, for which the tensor cores waited)
-                        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-                        __syncwarp();
-                        const int b = n_out_bufs++ & 1;
-#pragma unroll
-                        for (int x = 0; x < 4; ++x)   // 64-byte swizzle
-                            *reinterpret_cast<uint4 *>(out_row + b * S::kOutBytes + ((x ^ ((lane >> 1) & 3)) << 4)) = u[x];
-                        tc::fence_proxy_async();
-                        __syncwarp();
-                        if (lane == 0) tma_store_2d(&tmO, out_buf + b * S::kOutBytes, col, row);
-                        return;
-                    }
-                    // the cache rows, or rows of which some are left to the pass below
-                    tc::quad_transpose(u, ql);
-                    if (cu < a.n_out) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if (ok_j[j]) {
-                                if (to_cache) kv_put(kv_j[j], cu, u[j]);
-                                else *reinterpret_cast<uint4 *>(a.out + (row4 + j) * a.ldo + cu) = u[j];
-                            }
-                    }
-                };
-                const int c_mid = (out_bn / 2 + 31) & ~31, c_end = part == 0 ? c_mid : out_bn;
-                int c = part == 0 ? 0 : c_mid;
-#pragma unroll 1
-                for (; c + 32 <= c_end; c += 32) {
-                    uint32_t v[32], w[32];   // kDuoGlu: gate and up; else this chunk and the next
-                    const bool pair = kMode != kDuoGlu && c + 64 <= c_end;
-                    tc::tmem_ld_32x32(acc_addr + c, v);
-                    if (kMode == kDuoGlu) tc::tmem_ld_32x32(acc_addr + out_bn + c, w);
-                    else if (pair) tc::tmem_ld_32x32(acc_addr + c + 32, w);
-                    tc::tmem_ld_wait();
-                    if (kMode == kDuoGlu) {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(silu_mul(__uint_as_float(v[e]), __uint_as_float(w[e])));
-                    }
-                    if (g.n0 + c < a.n_out) put32(g.n0 + c, reinterpret_cast<float(&)[32]>(v));
-                    if (pair) {
-                        c += 32;
-                        if (g.n0 + c < a.n_out) put32(g.n0 + c, reinterpret_cast<float(&)[32]>(w));
-                    }
-                }
-                if (c < c_end) {   // 16 columns are left
-                    uint32_t v[16];
-                    tmem_ld_32x16(acc_addr + c, v);
-                    if (kMode == kDuoGlu) {
-                        uint32_t w[16];
-                        tmem_ld_32x16(acc_addr + out_bn + c, w);
-                        tc::tmem_ld_wait();
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(silu_mul(__uint_as_float(v[e]), __uint_as_float(w[e])));
-                    } else {
-                        tc::tmem_ld_wait();
-                    }
-                    if (mine)
-#pragma unroll
-                        for (int x = 0; x < 2; ++x)
-                            if (g.n0 + c + 8 * x < a.n_out) put_own8(g.n0 + c + 8 * x, reinterpret_cast<float(&)[8]>(v[8 * x]));
-                }
-                if (any_own) {
+                const int c_mid = (out_bn / 2 + 31) & ~31, c0 = part == 0 ? 0 : c_mid, n_cols = (part == 0 ? c_mid : out_bn) - c0;
+                if (any_own) {   // rows whose adapter has a B with an Inf or NaN get their delta here; 8 columns at a time
                     tc::OddRow odd;
                     if (own_pass) {
                         const int k = a.row_adapter[row];
@@ -672,23 +581,101 @@ gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                         odd.n = a.adapters[k * a.ad_stride];
                     }
 #pragma unroll 1
-                    for (int c8 = part == 0 ? 0 : c_mid; c8 < c_end && g.n0 + c8 < a.n_out; c8 += 8) {
+                    for (int c = 0; c < n_cols && g.n0 + c0 + c < a.n_out; c += 8) {
+                        const int col = g.n0 + c0 + c;
                         uint32_t v[8], w[8];
-                        tc::tmem_ld_32x8(acc_addr + c8, v);
-                        if (kMode == kDuoGlu) tc::tmem_ld_32x8(acc_addr + out_bn + c8, w);
+                        tc::tmem_ld_32x8(acc_addr + c0 + c, v);
+                        if (kMode == kDuoGlu) tc::tmem_ld_32x8(acc_addr + out_bn + c0 + c, w);
                         tc::tmem_ld_wait();
-                        if (!own_pass) continue;
-                        const int col = g.n0 + c8;
-                        odd.add8(reinterpret_cast<float(&)[8]>(v), col, kMode != kDuoQkv || col < a.Nq ? 0 : (col < a.Nq + a.Nkv ? 1 : 2));
+                        if (own_pass) {
+                            odd.add8(reinterpret_cast<float(&)[8]>(v), col, kMode != kDuoQkv || col < a.Nq ? 0 : (col < a.Nq + a.Nkv ? 1 : 2));
+                            if (kMode == kDuoGlu) odd.add8(reinterpret_cast<float(&)[8]>(w), a.N / 2 + col, 1);
+                        }
                         if (kMode == kDuoGlu) {
-                            odd.add8(reinterpret_cast<float(&)[8]>(w), a.N / 2 + col, 1);
 #pragma unroll
                             for (int e = 0; e < 8; ++e) v[e] = __float_as_uint(silu_mul(__uint_as_float(v[e]), __uint_as_float(w[e])));
                         }
-                        put_own8(col, reinterpret_cast<float(&)[8]>(v));
+                        if (row_ok) put_own8(col, reinterpret_cast<float(&)[8]>(v));
+                    }
+                    drained(h);
+                    continue;
+                }
+                // Chunks of 32 columns: in registers, packed, and only the last ones not yet packed when the half is given
+                // free for the next item; the rest runs underneath its MMAs.  (With the stores in between a half was taken
+                // up for 4 k cycles, with SwiGLU for 8 k, at 57 k for its MMAs.)
+                const bool res = kMode == kDuoLinear && a.residual != nullptr;
+                // this lane's row of the chunk at column `col`, rounded
+                auto pack32 = [&](int col, float (&f)[32], uint4 (&u)[4]) {
+                    const int cu = col + ql * 8;   // the columns of the quad's four rows that this lane reads
+                    if (res) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            u[j] = (row & ~3) + j < a.M && cu < a.n_out ? *reinterpret_cast<const uint4 *>(a.residual + (row4 + j) * a.ldo + cu) : make_uint4(0, 0, 0, 0);
+                        tc::quad_transpose(u, ql);
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) add_res8(reinterpret_cast<float(&)[8]>(f[8 * x]), u[x]);
+                    }
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) u[x] = pack8(reinterpret_cast<const float(&)[8]>(f[8 * x]));
+                };
+                auto put32 = [&](int k, uint4 (&u)[4]) {   // chunk k: 32 columns, 16, or none
+                    const int col = g.n0 + c0 + 32 * k, left = n_cols - 32 * k;
+                    if (left <= 0 || col >= a.n_out) return;
+                    if (left < 32) {
+                        if (row_ok)
+#pragma unroll
+                            for (int x = 0; x < 2; ++x)
+                                if (col + 8 * x < a.n_out) *reinterpret_cast<uint4 *>(a.out + (size_t)row * a.ldo + col + 8 * x) = u[x];
+                    } else if (kMode == kDuoQkv && a.kv_pool != nullptr && col >= a.Nq) {
+                        tc::quad_transpose(u, ql);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const long long at = __shfl_sync(0xffffffffu, kv_at, (lane & ~3) + j);   // (-1 for rows beyond the end)
+                            if (col + ql * 8 < a.n_out) kv_put(at, col + ql * 8, u[j]);
+                        }
+                    } else {
+                        // through shared memory and TMA, which cuts rows and columns off at the matrix's end
+                        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                        __syncwarp();
+                        const int b = n_out_bufs++ & 1;
+#pragma unroll
+                        for (int x = 0; x < 4; ++x)   // 64-byte swizzle
+                            *reinterpret_cast<uint4 *>(out_row + b * S::kOutBytes + ((x ^ ((lane >> 1) & 3)) << 4)) = u[x];
+                        tc::fence_proxy_async();
+                        __syncwarp();
+                        if (lane == 0) tma_store_2d(&tmO, out_buf + b * S::kOutBytes, col, row);
+                    }
+                };
+                constexpr int kFirst = kMode == kDuoGlu ? 1 : 2;   // chunks of a step: 64 columns of tensor memory
+                uint4 held[kFirst][4];
+#pragma unroll
+                for (int st = 0; st < 2; ++st) {
+                    uint32_t v[64];   // kDuoGlu: gate, up
+                    if (32 * kFirst * st < n_cols) {
+                        const uint32_t at = acc_addr + c0 + 32 * kFirst * st;
+                        tc::tmem_ld_32x32(at, reinterpret_cast<uint32_t(&)[32]>(v[0]));
+                        if (kMode == kDuoGlu) tc::tmem_ld_32x32(at + out_bn, reinterpret_cast<uint32_t(&)[32]>(v[32]));
+                        else if (32 * kFirst * st + 32 < n_cols) tc::tmem_ld_32x32(at + 32, reinterpret_cast<uint32_t(&)[32]>(v[32]));
+                        tc::tmem_ld_wait();
+                    }
+                    if (st == 1) {
+                        drained(h);
+                        if (!res)
+#pragma unroll
+                            for (int k = 0; k < kFirst; ++k) put32(k, held[k]);
+                    }
+                    if (kMode == kDuoGlu) {
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(silu_mul(__uint_as_float(v[e]), __uint_as_float(v[32 + e])));
+                    }
+#pragma unroll
+                    for (int k = 0; k < kFirst; ++k) {
+                        const int c = 32 * (kFirst * st + k);
+                        if (c >= n_cols) break;
+                        pack32(g.n0 + c0 + c, reinterpret_cast<float(&)[32]>(v[32 * k]), held[k]);
+                        if (st == 1 || res) put32(kFirst * st + k, held[k]);
                     }
                 }
-                drained(h);
             }
             if (ok && g.shrink && lane == 0) atomicAdd(a.t_ready + g.e0, 1);   // (behind each lane's fence and the warp's sync)
         }
