@@ -207,6 +207,8 @@ alora_status alora_create(const alora_config *cfg, alora_ctx **out) {
     ctx->max_quads = quad_bound(ctx, c.max_tokens, c.max_requests);
     if (c.dtype == ALORA_DTYPE_BF16) {
         ctx->t_slots = std::max(ctx->max_pairs, 3 * pair_bound(ctx, std::min(c.max_tokens, kSplitTTokens), c.max_requests));
+        // (per (quad, adapter) entry four row tiles, each summand)
+        ctx->t_slots = std::max(ctx->t_slots, 12 * quad_bound(ctx, std::min(c.max_tokens, kSplitTTokens), c.max_requests));
         if (c.max_tokens > kSplitTTokens) ctx->t_slots = std::max(ctx->t_slots, 4 * ctx->max_quads);
         alloc((void **)&ctx->d_quads, (size_t)ctx->max_quads * sizeof(TilePair));
         alloc((void **)&ctx->d_quad_off, (Tm / kQuadRows + 2) * 4);

@@ -199,7 +199,7 @@ struct alora_ctx {
     int32_t *d_group_done = nullptr;    // [max_split_rows / 16] finished key ranges per (stream, KV head), at its first partial row / 16
     int32_t max_split_items = 0, max_split_rows = 0, small_max_tokens = 0;
     void *d_t = nullptr;          // rank-r intermediate: fp32 [max_tokens][3][RP]; bf16 [pair][1 or 3 summands][128][3][RP], or
-                                  // [(quad, adapter) entry][512][3][RP]
+                                  // [(quad, adapter) entry][1 or 3 summands][512][3][RP]
     // few-row projection (batches of <= 128 rows): K-slice partial products and partial shrink results
     float *d_skinny_part = nullptr;   // [skinny_max_items][128][256] fp32
     float *d_skinny_t = nullptr;      // [slices of the q/k/v projection][128][skinny_p_cap][192] fp32

@@ -63,7 +63,7 @@ struct DuoArgs {
     const int32_t *any_odd;         // not 0: an adapter of the context may have b_odd set
     const __nv_bfloat16 *b_all;     // the launch's B rows of all adapters, [adapter][N][64] (read for rows of those)
     int32_t *t_ready;               // [entry] epilogue warps that have published their part of t
-    __nv_bfloat16 *t;               // [entry][512][t_cols]
+    __nv_bfloat16 *t;               // [entry][kParts][512][t_cols]
     // KV append fused into the epilogue (nullptr: off): the k and v columns then go to the page pool only
     __nv_bfloat16 *kv_pool;
     const int32_t *slot_map;
@@ -198,7 +198,7 @@ __device__ __forceinline__ bool touches(const DuoArgs &a, int n0, int blk) {
     return kMode != kDuoQkv || (n0 < blk_end(a, blk) && n0 + a.bn > blk_start(a, blk));
 }
 
-template <int kMode>
+template <int kMode, int kParts>   // kParts: bf16 summands of t
 __global__ void __launch_bounds__(kThreadsD, 1)
 gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                         const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmS,
@@ -345,8 +345,10 @@ gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                 if (!ok) break;
                 if (g.shrink) continue;
                 // expand: per adapter of the quad, one K block per adapted matrix that the column tile touches
+                int next_ad = g.e0 < g.e1 ? a.quads[g.e0].adapter : -1;
                 for (int e = g.e0; e < g.e1 && ok; ++e) {
-                    const int adapter = a.quads[e].adapter;
+                    const int adapter = next_ad;
+                    if (e + 1 < g.e1) next_ad = a.quads[e + 1].adapter;   // (in flight while this entry is waited for)
                     // t of this entry is written by shrink items (claimed by running clusters): wait until their sixteen
                     // epilogue warps have published, then order the TMA reads after it
                     const long long t0 = clock64();
@@ -357,9 +359,10 @@ gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                     asm volatile("fence.proxy.async.global;" ::: "memory");
                     for (int blk = 0; blk < kBlks; ++blk) {
                         if (!touches<kMode>(a, g.n0, blk)) continue;
+                        for (int p = 0; p < kParts; ++p) {   // (the summands of t meet the same B tile)
                         if (!begin_slot(all_bytes, sa, fb)) { ok = false; break; }
                         for (int h = 0; h < g.halves; ++h)
-                            tma2_load_2d(sa + h * kTileBytesD, &tmT, fb, blk * kTensorRP, (4 * e + 2 * h + (int)crank) * 128);
+                            tma2_load_2d(sa + h * kTileBytesD, &tmT, fb, blk * kTensorRP, (4 * (e * kParts + p) + 2 * h + (int)crank) * 128);
                         if (kMode == kDuoQkv)
                             tma2_load_3d(sa + 2 * kTileBytesD, blk == 0 ? &tmB0 : (blk == 1 ? &tmB1 : &tmB2), fb, 0,
                                          g.n0 + (int)crank * half_bn - blk_start(a, blk), adapter);
@@ -367,6 +370,8 @@ gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                             tma2_load_2d(sa + 2 * kTileBytesD, &tmB0, fb, 0, blk == (int)crank ? adapter * a.N + w_row : a.b_rows);
                         else
                             tma2_load_2d(sa + 2 * kTileBytesD, &tmB0, fb, 0, adapter * a.N + w_row);
+                        }
+                        if (!ok) break;
                     }
                 }
             }
@@ -448,8 +453,8 @@ gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                 for (int e = g.e0; e < g.e1 && ok; ++e) {
                     const int at = e - g.e0;
                     const int steps = at < 32 ? __shfl_sync(0xffffffffu, my_steps, at) : rank_steps(a, a.quads[e].adapter);
-                    for (int blk = 0; blk < kBlks; ++blk) {
-                        if (!touches<kMode>(a, g.n0, blk)) continue;
+                    for (int bp = 0; bp < kBlks * kParts; ++bp) {
+                        if (!touches<kMode>(a, g.n0, bp / kParts)) continue;
                         const int s = kc % S::kStages;
                         if (!wait_all(full_bar(s), (kc / S::kStages) & 1)) { ok = false; break; }
                         tc::tc_fence_after();
@@ -509,14 +514,14 @@ gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                     const bool use = row_ok && a.row_adapter[row] == g.adapter;
                     const float scale = __int_as_float(a.adapters[g.adapter * a.ad_stride + 1]);
                     const int rpad = a.adapters[g.adapter * a.ad_stride];
-                    __nv_bfloat16 *trow = a.t + ((size_t)(4 * g.e0 + 2 * (g.h0 + h) + (int)crank) * 128 + r) * a.t_cols;
+                    __nv_bfloat16 *trow = a.t + ((size_t)(4 * g.e0 * kParts + 2 * (g.h0 + h) + (int)crank) * 128 + r) * a.t_cols;
 #pragma unroll 1
                     for (int c = part * 32; c < a.t_cols; c += 64) {
                         if ((c & (kTensorRP - 1)) >= rpad) continue;   // (columns that no MMA step reads)
                         uint32_t v[32];
                         tc::tmem_ld_32x32(acc_addr + c, v);
                         tc::tmem_ld_wait();
-                        tc::store_t_warp(reinterpret_cast<float(&)[32]>(v), scale, use, trow + c, a.t_cols, 1, 0);
+                        tc::store_t_warp(reinterpret_cast<float(&)[32]>(v), scale, use, trow + c, a.t_cols, kParts, kQuadRows * a.t_cols);
                     }
                     // (published below: the rows are read by other blocks through TMA)
                     asm volatile("fence.proxy.async.global;" ::: "memory");
@@ -576,7 +581,8 @@ gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                         int e = g.e0;
                         while (e + 1 < g.e1 && a.quads[e].adapter != k) ++e;
                         ld_acquire_d(a.t_ready + e);   // (complete since the tile's K blocks were loaded; orders the reads)
-                        odd.t = a.t + ((size_t)(4 * e + 2 * (g.h0 + h) + (int)crank) * 128 + r) * a.t_cols;
+                        odd.t = a.t + ((size_t)(4 * e * kParts + 2 * (g.h0 + h) + (int)crank) * 128 + r) * a.t_cols;
+                        odd.parts = kParts; odd.part_stride = kQuadRows * a.t_cols;
                         odd.b = a.b_all + (size_t)k * a.N * kTensorRP;
                         odd.n = a.adapters[k * a.ad_stride];
                     }
@@ -710,13 +716,15 @@ static int duo_pick_bn(const alora_ctx *ctx, int T, int K, int n_cols, bool glu,
     for (int bn = kMaxBn; bn >= 128; bn -= 32) {   // (the instruction takes multiples of 32)
         const int out_bn = glu ? bn / 2 : bn, items = ((T + kQuadRows - 1) / kQuadRows) * ((n_cols + out_bn - 1) / out_bn) + entries;
         const long long kblock = std::max(4 * bn, (65536 + 192 * bn) / 128);
-        const long long c = (long long)((items + clusters - 1) / clusters) * ((K + kBKd - 1) / kBKd * kblock + 24 * bn);
+        const int rounds = (items + clusters - 1) / clusters;
+        // (shrink items of 512 rows end with the first round's column tiles, which then wait for their t)
+        const long long c = rounds * ((K + kBKd - 1) / kBKd * kblock + 24 * bn) + (items + entries > rounds * clusters ? 10000 : 0);
         if (best == 0 || c < *cycles) { best = bn; *cycles = c; }
     }
     return best;
 }
 
-template <int kMode>
+template <int kMode, int kParts>
 static int launch_duo(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap &tmW, const CUtensorMap &tmT, const CUtensorMap &tmS,
                       const CUtensorMap (&tmB)[3], const DuoArgs &g, int max_entries, cudaStream_t s) {
     // the output in boxes of 32 rows x 32 columns, 64-byte swizzle
@@ -733,7 +741,7 @@ static int launch_duo(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap 
     static bool attr_set[64] = {};   // one per instantiation
     const int dev = ctx->cfg.device;
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        if (cudaFuncSetAttribute(gemm_duo_tcgen05_kernel<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, DuoSmem::kTotal) != cudaSuccess) return -1;
+        if (cudaFuncSetAttribute(gemm_duo_tcgen05_kernel<kMode, kParts>, cudaFuncAttributeMaxDynamicSharedMemorySize, DuoSmem::kTotal) != cudaSuccess) return -1;
         attr_set[dev] = true;
     }
     const int out_bn = kMode == kDuoGlu ? g.bn / 2 : g.bn;
@@ -747,26 +755,35 @@ static int launch_duo(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap 
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, gemm_duo_tcgen05_kernel<kMode>, tmX, tmW, tmT, tmS, tmB[0], tmB[1], tmB[2], tmO, g) == cudaSuccess ? 1 : -1;
+    return cudaLaunchKernelEx(&cfg, gemm_duo_tcgen05_kernel<kMode, kParts>, tmX, tmW, tmT, tmS, tmB[0], tmB[1], tmB[2], tmO, g) == cudaSuccess ? 1 : -1;
 }
 
 bool shrink_apart(const alora_ctx *ctx, int T, int R, int items);   // gemm_tcgen05.cu
 
 // q/k/v projection of a batch.  Returns the kernels launched, 0 when the batch is better served by the 128-row kernel (nothing
-// launched) or -1 on error.  Only for batches of more than kSplitTTokens rows (one summand of t; the decision must not depend on
-// the mode, so that rows with a closed gate come out bit-identical to the base-only projection of the same batch).
+// launched) or -1 on error.  The decision must not depend on the mode, so that rows with a closed gate come out bit-identical to the
+// base-only projection of the same batch.
 int launch_project_duo_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int R, void *qkv, cudaStream_t s,
                           void *kv_pool, int num_pages) {
     const Dims &d = ctx->d;
-    if (T <= kSplitTTokens || ctx->sm_count < 2 || d.H % 8 != 0 || d.N % 8 != 0 || d.Nq % 32 != 0 || d.Nkv % 32 != 0) return 0;
-    const int G = ctx->sm_count;
+    if (T <= kQuadRows || ctx->sm_count < 2 || d.H % 8 != 0 || d.N % 8 != 0 || d.Nq % 32 != 0 || d.Nkv % 32 != 0) return 0;
+    const int G = ctx->sm_count, t_parts = T <= kSplitTTokens ? 3 : 1;
     // against the 128 x 256 tiles of gemm_tcgen05.cu, 790 cycles a K block
     const bool have_adapters = ctx->layer_has_adapter[layer] != 0;
     long long here = 0;
     const int bn = duo_pick_bn(ctx, T, d.H, d.N, false, have_adapters ? quad_bound(ctx, T, R) : 0, &here);
-    const int items128 = ((T + 127) / 128) * ((d.N + 255) / 256), shrink128 = have_adapters && !shrink_apart(ctx, T, R, items128) ? pair_bound(ctx, T, R) : 0;
+    const int items128 = ((T + 127) / 128) * ((d.N + 255) / 256);
+    const bool apart = have_adapters && shrink_apart(ctx, T, R, items128);
+    const int shrink128 = have_adapters && !apart ? pair_bound(ctx, T, R) : 0;
     const long long other = (long long)((items128 + shrink128 + G - 1) / G) * ((d.H + kBKd - 1) / kBKd) * 790;
-    if (here > other) return 0;
+    // With three summands of t (few rows) what follows the K loop counts: 15 k cycles for each adapter of a quad here, 8 k for each of
+    // a row tile there, 30 k for a shrink kernel of its own.  One layer call, us, there / here: 777 rows and one adapter 101 / 87,
+    // 1000 rows and two 80 / 66 (the projection alone), 753 rows of 48 requests and four 69 / 81.
+    const int n_m = (T + 127) / 128, n_q = (n_m + 3) / 4;
+    const bool few = have_adapters && t_parts == 3;
+    const long long late_here = few ? 15000ll * ((quad_bound(ctx, T, R) + n_q - 1) / n_q) : 0;
+    const long long late_other = few ? 8000ll * ((pair_bound(ctx, T, R) + n_m - 1) / n_m) + (apart ? 30000 : 0) : 0;
+    if (here + late_here > other + late_other) return 0;
     const void *W = ctx->layers[layer].wqkv;
     CUtensorMap tmX, tmW, tmT, tmS, tmB[3];
     if (!make_tensor_map_bf16(&tmX, hidden, T, d.H, d.H, 128)) return -1;
@@ -807,7 +824,9 @@ int launch_project_duo_tc(alora_ctx *ctx, int layer, const void *hidden, int T, 
         g.kv_page_size = d.page; g.kv_num_pages = num_pages;
     }
     g.status = ctx->d_status;
-    return launch_duo<kDuoQkv>(ctx, tmX, tmW, tmT, tmS, tmB, g, have_adapters ? 2 * quad_bound(ctx, T, R) : 0, s);
+    const int max_items = have_adapters ? 2 * quad_bound(ctx, T, R) : 0;
+    return t_parts == 3 ? launch_duo<kDuoQkv, 3>(ctx, tmX, tmW, tmT, tmS, tmB, g, max_items, s)
+                        : launch_duo<kDuoQkv, 1>(ctx, tmX, tmW, tmT, tmS, tmB, g, max_items, s);
 }
 
 // Plain dense projection y = x W^T (+ residual), or with `glu` y = silu(x Wg^T) * (x Wu^T) for W = [Wg; Wu]; optionally with a gated
@@ -848,8 +867,8 @@ int launch_linear_duo_tc(alora_ctx *ctx, const void *x, const void *W, int T, in
         g.row_adapter = delta->row_adapter; g.t_ready = ctx->d_quad_ready; g.t = (__nv_bfloat16 *)delta->t;
         g.any_odd = ctx->d_counts + kOddAdapters; g.b_all = (const __nv_bfloat16 *)delta->B;
     }
-    return glu ? launch_duo<kDuoGlu>(ctx, tmX, tmW, tmT, tmA, tmB, g, 2 * max_entries, s)
-               : launch_duo<kDuoLinear>(ctx, tmX, tmW, tmT, tmA, tmB, g, 2 * max_entries, s);
+    return glu ? launch_duo<kDuoGlu, 1>(ctx, tmX, tmW, tmT, tmA, tmB, g, 2 * max_entries, s)
+               : launch_duo<kDuoLinear, 1>(ctx, tmX, tmW, tmT, tmA, tmB, g, 2 * max_entries, s);
 }
 
 }  // namespace alora

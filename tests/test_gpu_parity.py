@@ -959,3 +959,40 @@ def test_projection_on_pairs_of_sms(oracle64, S):
     assert not np.isfinite(odd[own][:, [7, shape.Nq + 100]]).any()
     others = np.setdiff1d(np.arange(shape.N), [7, shape.Nq + 100])
     hp.assert_close(odd[own][:, others], finite[own][:, others], 2e-2, "the adapter's own rows")
+
+
+@pytest.mark.parametrize("n_req,each", [(1, 777), (8, 112), (5, 204)])
+def test_projection_of_600_to_1024_rows_on_pairs_of_sms_loses_nothing_of_t(n_req, each):
+    """The whole numbers of the test above at the 8B widths, where batches of these sizes with one or two adapters go to the
+    pairs of SMs: t takes up to 21 bits, three summands hold it, two would not."""
+    shape = wl.SHAPE_8B
+    rng = np.random.default_rng(111 + n_req)
+    whole = lambda n, *d: rng.integers(-n, n + 1, d).astype(np.float32)  # noqa: E731
+    w = whole(63, shape.N, shape.hidden)
+    starts = (0, shape.Nq, shape.Nq + shape.Nkv)
+    ads = []
+    for times in (1, 2)[:1 if n_req == 1 else 2]:
+        a = wl.make_adapter(shape, 32, rng)
+        for name, s in zip("qkv", starts):
+            b_m = np.zeros_like(getattr(a, "B" + name))
+            b_m[:32] = -times * np.eye(32, dtype=np.float32)
+            setattr(a, "B" + name, b_m)
+            setattr(a, "A" + name, w[s:s + 32].copy())
+        ads.append(a)
+    ids = [r % len(ads) if n_req == 1 else (r % 3) - 1 for r in range(n_req)]
+    b = wl.make_batch(shape, [40] * n_req, [each] * n_req, ids, rng)
+    b.hidden[:] = whole(255, b.T, shape.hidden)
+    y = b.hidden.astype(np.float64) @ w.astype(np.float64).T
+    assert 2 ** 18 < np.abs(y[:, :32]).max() and np.abs(y).max() * 4 < 2 ** 24
+    for s in starts:
+        y[:, s:s + 32] *= (1 - (np.repeat(np.array(ids), each) + 1))[:, None]
+    g = hp.GpuLayers(shape, [dict(wqkv=w)], [ads], b.T, b.R)
+    try:
+        d = hp.DevBatch(b, shape.dtype)
+        out = g.empty(b.T, shape.N)
+        ab.alora_project_qkv(g.ctx, 0, ab.MODE_ALORA, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, d.T, d.R, out)
+        assert g.status() == 0
+        got = hp.to_host(out)
+    finally:
+        g.close()
+    assert np.array_equal(got, wl.bf16_round(y.astype(np.float32)))
