@@ -6,7 +6,7 @@
 // as give every SM a block, stream their part of W and x through a TMA ring and accumulate in tensor memory
 // (tcgen05.mma 128 x tile x 16).  The partial products then go to each block's shared memory, and after a cluster barrier
 // every block adds up its share of the tile's columns over the cluster's shared memory, in slice order, and finishes them:
-// delta, residual, bf16, k / v columns to the cache slots.
+// delta, residual or SwiGLU, bf16, k / v columns to the cache slots.
 // Measured against the two kernels it replaces (the second one read the partials back from L2), hidden 4096: q/k/v of 128
 // rows with one adapter 38 -> 26 us, of 64 rows with four 34 -> 24; o_proj of 40 rows 13.7 -> 11.7, gate/up 46 -> 41 (35 us of
 // HBM time), down 27.7 -> 24 (18); against 48 tiles of 128 x 256 on the dense route, 194 rows: 52 -> 42 with the metadata.
@@ -46,6 +46,7 @@ struct FewArgs {
     const __nv_bfloat16 *residual;
     __nv_bfloat16 *out;
     int ldo;
+    int glu;                      // W = [gate; up]: a tile holds bn / 2 rows of each, out = silu(gate) * up
     __nv_bfloat16 *kv_pool;
     const int32_t *slot_map;
     int kv_hd_shift, kv_heads, kv_page_size, kv_num_pages;
@@ -124,19 +125,27 @@ gemm_few_cluster_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
     const int kb0 = sl * kb_base + min(sl, kb_rem), nkb = kb_base + (sl < kb_rem ? 1 : 0);
     tc::grid_dep_launch();
     const int w_ahead = min(nkb, n_stages);
+    auto load_w = [&](uint32_t dst, uint32_t bar, int k) {
+        if (!a.glu) {
+            tc::tma_load_2d(dst, &tmW, bar, k, tile * a.bn);
+        } else {
+            tc::tma_load_2d(dst, &tmW, bar, k, tile * (a.bn / 2));
+            tc::tma_load_2d(dst + w_bytes / 2, &tmW, bar, k, a.N / 2 + tile * (a.bn / 2));
+        }
+    };
     if (threadIdx.x == 0) {
         tc::tma_prefetch_desc(&tmW);
         for (int s = 0; s < w_ahead; ++s) {
             tc::mbar_expect_tx(full_bar(s), w_bytes);
-            tc::tma_load_2d(smem_base + s * a.stage_bytes + x_bytes, &tmW, full_bar(s), (kb0 + s) * kFcBK, tile * a.bn);
+            load_w(smem_base + s * a.stage_bytes + x_bytes, full_bar(s), (kb0 + s) * kFcBK);
         }
     }
     // x and the adapter facts are written by earlier kernels of the stream.  Where only the facts come from the kernel before,
     // W x does not wait for them, and the A rows take a second pass over x (from L2) once the facts are there.
     constexpr bool second_pass = kSecondPass;
     if (!kSecondPass && !a.x_early) tc::grid_dep_wait();
-    const int col0 = tile * a.bn;
-    const int v0 = sl * (a.bn / 8) / a.ksplit, v1 = (sl + 1) * (a.bn / 8) / a.ksplit;   // this block's share: 8-column vectors
+    const int out_bn = a.glu ? a.bn / 2 : a.bn, n_out = a.glu ? a.N / 2 : a.N, col0 = tile * out_bn;
+    const int v0 = sl * (out_bn / 8) / a.ksplit, v1 = (sl + 1) * (out_bn / 8) / a.ksplit;   // this block's share: 8-column vectors
     const int share = (v1 - v0) * 8;
     const int blk = col0 < a.Nq ? 0 : (col0 < a.Nq + a.Nkv ? 1 : 2);
     // over the ring, once the accumulators are complete, column-major with the rows contiguous:
@@ -168,7 +177,7 @@ gemm_few_cluster_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                     tc::mbar_arrive_expect_tx(full_bar(s), x_bytes + n_chunk * kFcChunkBytes);
                 } else {
                     tc::mbar_arrive_expect_tx(full_bar(s), x_bytes + w_bytes + n_chunk * kFcChunkBytes);
-                    tc::tma_load_2d(sw, &tmW, full_bar(s), k, col0);
+                    load_w(sw, full_bar(s), k);
                 }
                 tc::tma_load_2d(sx, &tmX, full_bar(s), k, row0);
                 a_rows(sw + w_bytes, s, k);
@@ -392,8 +401,9 @@ gemm_few_cluster_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
     __syncwarp();
     cluster_arrive();
     if (a.ksplit > 1)   // in place: only this block reads its own share of its own partials
-        add_slices(tc::smem_u32(part), v0 * 8 << rv_shift, v1 * 8 << rv_shift,
-                   [&](int i, const float4 &f) { *reinterpret_cast<float4 *>(part + 4 * i) = f; });
+        for (int c = 0; c < a.bn; c += out_bn)
+            add_slices(tc::smem_u32(part), c + v0 * 8 << rv_shift, c + v1 * 8 << rv_shift,
+                       [&](int i, const float4 &f) { *reinterpret_cast<float4 *>(part + 4 * i) = f; });
     cp_async_wait_all();
     __syncwarp();
     cluster_wait();     // t is complete
@@ -403,10 +413,14 @@ gemm_few_cluster_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
     //    by 16 x 8 x 16 matrix instructions, an adapter at a time, took as long for one adapter and twice as long for four.)
     for (int u = threadIdx.x; u < (v1 - v0) << a.rows_shift; u += kFcThreads) {
         const int row = u & (rs - 1), v = v0 + (u >> a.rows_shift), col = col0 + v * 8;
-        if (col >= a.N || row >= T) continue;
+        if (col >= n_out || row >= T) continue;
         float f[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) f[e] = part[((v * 8 + e) << a.rows_shift) + row];
+        if (a.glu) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) f[e] = __fdividef(f[e], 1.f + __expf(-f[e])) * part[((out_bn + v * 8 + e) << a.rows_shift) + row];
+        }
         const int slot = n_present > 0 ? slot_s[row] : -1;
         if (slot >= 0) {   // only rows with an applied adapter add anything (a gated-off row never sees "+ 0")
             const int vecs = rpad_s[slot] / 8;
@@ -566,17 +580,18 @@ bool few_cluster_route(const alora_ctx *ctx, int T, int R, int N, int K, bool lo
     return few_plan(ctx, T, R, N, K, lora, Nq, Nkv, false, a);
 }
 
-// Returns kernels launched, or -1.  `meta`: the batch's adapter facts of the layer (with the layer's A rows as tensor
+// Returns kernels launched, or -1.  `glu`: W holds gate and up rows, the output is silu(gate) * up (a kernel for that behind 40
+// rows x 28672: 4 us).  `meta`: the batch's adapter facts of the layer (with the layer's A rows as tensor
 // maps and its B slab), or nullptr for a plain dense projection.
 int launch_few_cluster(alora_ctx *ctx, const void *x, const void *W, const RankMaps *tmA, const FewRowMeta *meta,
                        const void *b_all, int T, int R, int K, int N, int Nq, int Nkv, void *out, const void *residual, void *kv_pool,
-                       int num_pages, bool x_early, cudaStream_t s) {
+                       int num_pages, bool x_early, cudaStream_t s, bool glu) {
     FewArgs a{};
     if (!few_plan(ctx, T, R, N, K, meta != nullptr, Nq, Nkv, x_early, a)) return -1;
     CUtensorMap tmX, tmW;
-    if (!make_tensor_map_bf16(&tmX, x, T, K, K, 1 << a.rows_shift) || !make_tensor_map_bf16(&tmW, W, N, K, K, a.bn)) return -1;
+    if (!make_tensor_map_bf16(&tmX, x, T, K, K, 1 << a.rows_shift) || !make_tensor_map_bf16(&tmW, W, N, K, K, glu ? a.bn / 2 : a.bn)) return -1;
     a.meta = meta; a.b_all = (const __nv_bfloat16 *)b_all; a.Nq = Nq; a.Nkv = Nkv;
-    a.residual = (const __nv_bfloat16 *)residual; a.out = (__nv_bfloat16 *)out; a.ldo = N; a.status = ctx->d_status;
+    a.residual = (const __nv_bfloat16 *)residual; a.out = (__nv_bfloat16 *)out; a.ldo = glu ? N / 2 : N; a.glu = glu ? 1 : 0; a.status = ctx->d_status;
     if (kv_pool != nullptr) {
         int shift = 0;
         while ((1 << shift) < ctx->d.hd) ++shift;

@@ -560,7 +560,7 @@ int launch_skinny_tc(alora_ctx *ctx, const void *x, const CUtensorMap &tmW, cons
 bool few_cluster_route(const alora_ctx *ctx, int T, int R, int N, int K, bool lora, int Nq, int Nkv);   // gemm_few_cluster.cu
 int launch_few_cluster(alora_ctx *ctx, const void *x, const void *W, const RankMaps *tmA, const FewRowMeta *meta,
                        const void *b_all, int T, int R, int K, int N, int Nq, int Nkv, void *out, const void *residual, void *kv_pool,
-                       int num_pages, bool x_early, cudaStream_t s);
+                       int num_pages, bool x_early, cudaStream_t s, bool glu = false);
 
 // More than 128 rows take the one-launch route only in a context without adapters on the MLP block: those need the (row tile,
 // adapter) pairs, which that route's metadata step does not build, and a call in which none of them applies has to take the
@@ -705,9 +705,16 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
     return ok ? 1 : -1;
 }
 
-// Gate and up projection with SwiGLU in the epilogue, for the batches that the pairs of SMs serve; 0: nothing launched.
+// Gate and up projection with SwiGLU in the epilogue, for the batches of the few-row kernel and of the pairs of SMs; 0: nothing
+// launched.  Not for few rows where the context has adapters on the MLP block: their expand step wants the rounded gate and up rows,
+// and a call in which none of them applies has to take the route of the others.
 int launch_glu_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y, cudaStream_t s, const LinearDelta *delta) {
-    if (T == 0 || (delta == nullptr && few_cluster_rows(ctx, T) && few_cluster_route(ctx, T, 0, N, K, false, N, 0))) return 0;
+    if (T == 0 || N % 16 != 0) return 0;
+    if (delta == nullptr && few_cluster_rows(ctx, T) && few_cluster_route(ctx, T, 0, N, K, false, N, 0)) {
+        for (int n : ctx->mlp_n_adapters) if (n > 0) return 0;
+        ProfScope prof(ctx, KK_LINEAR, s);
+        return launch_few_cluster(ctx, x, W, nullptr, nullptr, nullptr, T, 0, K, N, N, 0, y, nullptr, nullptr, 0, false, s, true);
+    }
     ProfScope prof(ctx, KK_LINEAR, s);
     return launch_linear_duo_tc(ctx, x, W, T, K, N, y, nullptr, delta, true, s);
 }

@@ -996,3 +996,26 @@ def test_projection_of_600_to_1024_rows_on_pairs_of_sms_loses_nothing_of_t(n_req
     finally:
         g.close()
     assert np.array_equal(got, wl.bf16_round(y.astype(np.float32)))
+
+
+@pytest.mark.parametrize("T,inter", [(1, 1096), (17, 2048), (40, 1096), (128, 4744), (200, 2048)])
+def test_few_rows_through_gate_and_up_with_swiglu_in_the_epilogue(oracle64, T, inter):
+    """One layer of a few rows: gate / up in one launch with SwiGLU, at the row boxes' edges, with a last column tile that is cut
+    off (1096, 4744: half tiles of 64 .. 128 columns) and over two row tiles."""
+    shape = wl.LayerShape(hidden=1024, n_q_heads=8, n_kv_heads=2, head_dim=128, page_size=16, dtype="bf16", intermediate=inter)
+    rng = np.random.default_rng(120 + T)
+    layers = [wl.make_stack_weights(shape, rng)]
+    b = wl.make_batch(shape, [0], [T], [-1], rng, shuffle_pages=True)
+    g = hp.GpuLayers(shape, layers, [[]], T, 1)
+    try:
+        d = hp.DevBatch(b, shape.dtype)
+        hout = g.empty(T, shape.hidden)
+        ab.alora_forward_stack(g.ctx, ab.MODE_BASE, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, [g.new_pool(b.num_pages)],
+                               d.bt, d.max_blocks, b.num_pages, d.T, d.R, hout)
+        assert g.status() == 0
+        x, _ = oracle64.decoder_layer(b.hidden.astype(np.float64), layers[0], shape.Nq, shape.Nkv, shape.n_q_heads, shape.n_kv_heads,
+                                      shape.head_dim, 1e-5, b.positions, b.query_start_loc, b.activation_offsets, b.adapter_ids, [],
+                                      [None], [None])
+        hp.assert_close(hp.to_host(hout), x, 2e-2, "a layer of few rows", block=shape.head_dim)
+    finally:
+        g.close()
