@@ -687,9 +687,15 @@ alora_status alora_forward_stack(alora_ctx *ctx, int mode, const void *d_hidden_
     // one token per request (the decode entry passes the context's own 0, 1, ..., R as query_start_loc): every request
     // is on the few-row attention list, the tensor-core attention kernel has nothing to do and is not launched
     b.all_small = (d_query_start_loc == ctx->d_iota && T == R) ? 1 : 0;
-    if (d_hidden_out != d_hidden_in && T > 0)
-        ALORA_CUDA(ctx, cudaMemcpyAsync(d_hidden_out, d_hidden_in, (size_t)T * d.H * ctx->esize, cudaMemcpyDeviceToDevice, s));
     char *h = (char *)d_hidden_out;  // residual stream, updated in place
+    // The first layer reads the caller's rows where they are (a copy of 2048 rows took 7 us, of 40 rows 3); buffers that overlap in
+    // part or are not aligned for the kernels' vectors are copied first.
+    const char *h_in = (const char *)d_hidden_in;
+    const size_t h_bytes = (size_t)T * d.H * ctx->esize;
+    if (h_in != h && T > 0 && (!aligned16(h_in) || (h_in < h + h_bytes && h < h_in + h_bytes))) {
+        ALORA_CUDA(ctx, cudaMemcpyAsync(h, h_in, h_bytes, cudaMemcpyDeviceToDevice, s));
+        h_in = h;
+    }
     int n = 0, k;
     // a launcher that returns < 0 has launched nothing (unsupported shape, failed tensor map or launch): the call
     // stops there with the residual stream as the completed steps left it
@@ -713,10 +719,11 @@ alora_status alora_forward_stack(alora_ctx *ctx, int mode, const void *d_hidden_
     for (int l = 0; l < ctx->cfg.n_layers; ++l) {
         const LayerWeights &lw = ctx->layers[l];
         if (l > 0) b.facts_ready = kMetaAttention | (one_route ? kMetaProjection : 0);
-        ALORA_STEP(launch_rmsnorm(ctx, h, lw.norm_attn, T, ctx->d_act[0], s));
+        const char *res = l == 0 ? h_in : h;
+        ALORA_STEP(launch_rmsnorm(ctx, res, lw.norm_attn, T, ctx->d_act[0], s));
         st = run_layer(ctx, l, ctx->d_act[0], b, h_paged_kv_layers[l], ctx->d_act[1], s);
         if (st != ALORA_OK) return st;
-        ALORA_STEP(launch_linear(ctx, ctx->d_act[1], lw.wo, T, d.Nq, d.H, h, h, s));           // h += o_proj(attn)
+        ALORA_STEP(launch_linear(ctx, ctx->d_act[1], lw.wo, T, d.Nq, d.H, h, res, s));           // h = res + o_proj(attn)
         ALORA_STEP(launch_rmsnorm(ctx, h, lw.norm_mlp, T, ctx->d_act[0], s));
         for (int t0 = 0; t0 < T; t0 += kMlpChunk) {                                        // MLP, token chunks
             const int tc = std::min(kMlpChunk, T - t0);

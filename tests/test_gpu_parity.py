@@ -1019,3 +1019,35 @@ def test_few_rows_through_gate_and_up_with_swiglu_in_the_epilogue(oracle64, T, i
         hp.assert_close(hp.to_host(hout), x, 2e-2, "a layer of few rows", block=shape.head_dim)
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+def test_stack_input_and_output_buffers(dtype):
+    """The stack call reads its input where it is: the same result in a buffer of its own, in place, and from rows that are not
+    16-byte aligned (copied first); the input stays as it was unless it is the output."""
+    import torch
+    shape = wl.LayerShape(hidden=256, n_q_heads=4, n_kv_heads=2, head_dim=64, page_size=16, dtype=dtype, intermediate=512)
+    rng = np.random.default_rng(131)
+    layers = [wl.make_stack_weights(shape, rng) for _ in range(2)]
+    b = wl.make_batch(shape, [0, 0], [30, 21], [-1, -1], rng)
+    g = hp.GpuLayers(shape, layers, [[], []], b.T, b.R)
+    try:
+        d = hp.DevBatch(b, dtype)
+        x, n = d.hidden.clone(), b.T * shape.hidden
+
+        def run(src, dst):
+            ab.alora_forward_stack(g.ctx, ab.MODE_BASE, src, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens,
+                                   [g.new_pool(b.num_pages) for _ in range(2)], d.bt, d.max_blocks, b.num_pages, d.T, d.R, dst)
+            assert g.status() == 0
+            return dst.clone()
+
+        want = run(x, g.empty(b.T, shape.hidden))
+        assert torch.equal(x, d.hidden) and not torch.equal(want, x)
+        y = x.clone()
+        assert torch.equal(run(y, y), want)
+        buf = torch.empty(n + 8192, dtype=x.dtype, device="cuda")
+        src, dst = buf[1:1 + n].view(b.T, -1), torch.empty_like(x)
+        src.copy_(x)
+        assert torch.equal(run(src, dst), want) and torch.equal(src, x)
+    finally:
+        g.close()
