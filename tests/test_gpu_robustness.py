@@ -117,3 +117,46 @@ def test_bounded_wait_gives_up_and_the_context_stays_usable(oracle64):
         hp.assert_close(hp.to_host(out), want["out"], 2e-2, "layer call after an expired wait", block=SHAPE.head_dim)
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("new", [7, 90])
+def test_a_captured_call_behind_a_copy_replays(dtype, new):
+    """The first launch of a call is a programmatic dependent one: in a captured graph it follows a copy (no kernel) and then
+    the last kernel of another call; replays on new input rows equal direct calls."""
+    import torch
+    shape = wl.LayerShape(hidden=256, n_q_heads=4, n_kv_heads=2, head_dim=64, page_size=16, dtype=dtype)
+    rng = np.random.default_rng(17)
+    w = wl.make_wqkv(shape, rng)
+    ads = [wl.make_adapter(shape, 8, rng)]
+    b = wl.make_batch(shape, [40, 9], [new, new], [0, -1], rng)
+    g = hp.GpuLayers(shape, [dict(wqkv=w)], [ads], b.T, b.R)
+    try:
+        d = hp.DevBatch(b, dtype)
+        fill = wl.random_kv_pool(shape, b.num_pages, rng)
+        pool, src, x, out = g.new_pool(b.num_pages, fill), d.hidden.clone(), d.hidden.clone(), [g.empty(b.T, shape.Nq) for _ in range(2)]
+
+        def call(dst):
+            ab.alora_prefill_layer(g.ctx, 0, x, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, pool, d.bt, d.max_blocks, b.num_pages,
+                                   d.T, d.R, dst)
+
+        call(out[0])
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            x.copy_(src)
+            call(out[0])
+            call(out[1])
+        for k in range(3):
+            src.copy_(d.hidden * (k + 1))
+            graph.replay()
+            torch.cuda.synchronize()
+            got = [o.clone() for o in out]
+            assert torch.equal(x, src)
+            call(out[0])
+            torch.cuda.synchronize()
+            assert g.status() == 0
+            assert torch.equal(got[0], out[0]) and torch.equal(got[1], out[0])
+        del graph
+    finally:
+        g.close()
