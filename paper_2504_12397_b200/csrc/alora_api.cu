@@ -106,7 +106,7 @@ static alora_status run_layer(alora_ctx *ctx, int layer, const void *hidden, con
     bool kv_appended = false;
     const bool rope = ctx->d_rope_inv_freq != nullptr;   // the rotation comes between projection and append
     ctx->pending_attn_meta = (b.facts_ready & kMetaAttention) || (ctx->d_attn_items == nullptr && ctx->d_split_items == nullptr) ? nullptr : &b;   // (no lists in fp32)
-    // (that launch is an ordinary one: it began when x was complete; in a stack call, whose facts of all layers take longer
+    // (that launch lets the next one start only when x is complete; in a stack call, whose facts of all layers take longer
     // but come once, the second pass over x that this brings does not pay)
     ctx->x_before_facts = b.n_layers == 1 && !(b.facts_ready & kMetaProjection);
     k = launch_project(ctx, layer, hidden, b.T, b.R, ctx->d_qkv, s, rope ? nullptr : pool, b.num_pages, &kv_appended);

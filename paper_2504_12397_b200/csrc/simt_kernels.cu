@@ -538,11 +538,11 @@ attn_simt_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ posi
     tc::grid_dep_launch();
     const int t = blockIdx.x, kvh = blockIdx.y, h0 = (int)blockIdx.z * HC, nh = min(HC, G - h0);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, stream = warp * 4 + (lane >> 3), d0 = (lane & 7) * 4;
-    // The caller's arrays and the cached keys of earlier calls were complete before the preceding kernel of the call let this one
-    // start: they are fetched beside it, the new rows after it.
+    // The caller's arrays were complete before the preceding kernel of the call let this one start: they are read beside it.  Rows of the
+    // page pool are read after it, those before this request's new tokens too: another request of the call may have appended them.
     const RowFacts f = row_facts(t, positions, nullptr, nullptr, qsl, seq_lens, block_tables, max_blocks, num_pages, page_size, 0, R,
                                  ALORA_MODE_BASE, status);
-    const int r = f.req, p = f.pos, first_new = p - (t - qsl[r]);
+    const int r = f.req, p = f.pos;
     float *orow = out + (size_t)t * Nq + (size_t)(kvh * G + h0) * HD;
     if (f.slot < 0) {  // a token that the metadata step rejects: defined output, no cache access
         tc::grid_dep_wait();
@@ -553,26 +553,21 @@ attn_simt_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ posi
     float m[HC], l[HC];
     const size_t plane = (size_t)Hkv * page_size * HD;
     const int32_t *table = block_tables + (size_t)r * max_blocks;
-    float4 kv[U][V], vv[U][V];
-    bool on[U];
-    // keys j0 + 32 u of a stream, either those in the cache before this call or the new ones
-    auto load = [&](int j0, bool cached) {
+    int page[U];   // of the stream's next keys
+    auto fetch_pages = [&](int j0) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int j = j0 + 32 * u;
-            if ((j < first_new) != cached) continue;
-            const int page = j <= p ? table[j / page_size] : -1;
-            on[u] = page >= 0 && page < num_pages;
-            if (j <= p && !on[u]) report(status, ALORA_ERR_PAGE_RANGE);
-            const float *kr = pool + ((size_t)(on[u] ? page : 0) * 2 * Hkv + kvh) * page_size * HD + (size_t)(j % page_size) * HD + d0;
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                kv[u][v] = on[u] ? *reinterpret_cast<const float4 *>(kr + 32 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
-                vv[u][v] = on[u] ? *reinterpret_cast<const float4 *>(kr + plane + 32 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
+            page[u] = j <= p ? table[j / page_size] : -1;
+            if (j <= p && (page[u] < 0 || page[u] >= num_pages)) report(status, ALORA_ERR_PAGE_RANGE);
         }
     };
-    load(stream, true);
+    auto key_row = [&](int u, int j) { return pool + ((size_t)page[u] * 2 * Hkv + kvh) * page_size * HD + (size_t)(j % page_size) * HD; };
+    fetch_pages(stream);
+#pragma unroll
+    for (int u = 0; u < U; ++u)   // the first keys and values on their way to L2 (a lane a line of 32 elements)
+        if (page[u] >= 0 && page[u] < num_pages && (lane & 7) < 2 * V)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(key_row(u, stream + 32 * u) + ((lane & 7) < V ? (lane & 7) * 32 : plane + ((lane & 7) - V) * 32)));
     tc::grid_dep_wait();
 #pragma unroll
     for (int c = 0; c < HC; ++c) {
@@ -585,8 +580,19 @@ attn_simt_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ posi
         }
     }
     for (int j0 = stream; j0 - stream <= p; j0 += 32 * U) {
-        if (j0 != stream) load(j0, true);
-        load(j0, false);
+        float4 kv[U][V], vv[U][V];
+        bool on[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            on[u] = page[u] >= 0 && page[u] < num_pages;
+            const float *kr = on[u] ? key_row(u, j0 + 32 * u) + d0 : pool;
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                kv[u][v] = on[u] ? *reinterpret_cast<const float4 *>(kr + 32 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
+                vv[u][v] = on[u] ? *reinterpret_cast<const float4 *>(kr + plane + 32 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+        fetch_pages(j0 + 32 * U);
 #pragma unroll
         for (int c = 0; c < HC; ++c) {
             float s[U], mx = m[c];

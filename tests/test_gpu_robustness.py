@@ -160,3 +160,28 @@ def test_a_captured_call_behind_a_copy_replays(dtype, new):
         del graph
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("first,second", [(48, 7), (16, 1), (320, 90)])
+def test_a_request_may_read_the_rows_that_another_one_of_its_call_appends(dtype, first, second):
+    """A base request and an adapter invocation on its pages in one call, on an empty pool: every row is in the cache before the
+    attention reads one, so that the same call again, on the pool that the first one filled, gives the same bits."""
+    import torch
+    shape = wl.LayerShape(hidden=256, n_q_heads=4, n_kv_heads=2, head_dim=64, page_size=16, dtype=dtype)
+    rng = np.random.default_rng(23)
+    b = wl.make_batch(shape, [0, first], [first, second], [-1, 0], rng)
+    b.block_tables[1, :first // 16] = b.block_tables[0, :first // 16]
+    g = hp.GpuLayers(shape, [dict(wqkv=wl.make_wqkv(shape, rng))], [[wl.make_adapter(shape, 8, rng)]], b.T, b.R)
+    try:
+        d = hp.DevBatch(b, dtype)
+        for _ in range(5):
+            pool, out = g.new_pool(b.num_pages), [g.empty(b.T, shape.Nq) for _ in range(2)]
+            for o in out:
+                ab.alora_prefill_layer(g.ctx, 0, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, pool, d.bt, d.max_blocks,
+                                       b.num_pages, d.T, d.R, o)
+            torch.cuda.synchronize()
+            assert g.status() == 0
+            assert torch.equal(out[0], out[1])
+    finally:
+        g.close()
