@@ -88,6 +88,7 @@ static alora_status run_layer(alora_ctx *ctx, int layer, const void *hidden, con
     int n = 0, k;
     if (simt_small_layer(ctx, b.T)) {   // few fp32 rows: facts, shrink, projection and append in one launch
         const bool rotate = ctx->d_rope_inv_freq != nullptr;
+        b.own_facts = true;
         if ((k = launch_project_small_simt(ctx, layer, hidden, b, ctx->d_qkv, rotate ? nullptr : pool, s)) < 0) return ALORA_ERR_UNSUPPORTED;
         n += k;
         if (rotate) {

@@ -277,6 +277,7 @@ struct BatchArgs {
     int few_row = 0; // the projection of this batch takes the few-row route: build FewRowMeta instead of row tiles
     int n_layers = 1; // layers from `layer` on that the projection's facts are built for (a stack call: all of them at once)
     int facts_ready = 0; // bits (kMetaProjection, kMetaAttention): built by an earlier layer of the same stack call
+    bool own_facts = false;    // no metadata step in front of the fp32 attention: it reads the caller's arrays itself
     bool lists_shared = false; // the attention lists built for this layer serve other layers of the call too
 };
 

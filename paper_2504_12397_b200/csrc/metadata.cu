@@ -25,7 +25,8 @@ __device__ __forceinline__ int find_request(const int32_t *qsl, int R, int t) {
 // offset; always open in full-LoRA mode, always closed in base mode), and the token slot
 // page * page_size + position % page_size.  Findings (inconsistent positions, page id out of
 // range, adapter id out of range) go to the status word; the row then gets adapter -1 / slot -1 so that later kernels
-// skip it.  (Whether the adapter is registered on a layer is not looked at here: one that is not has rank 0 there.)
+// skip it.  The small fp32 layers find the same facts in a kernel of theirs (row_facts() in simt_kernels.cu): a change
+// here is one there.  (Whether the adapter is registered on a layer is not looked at here: one that is not has rank 0 there.)
 template <typename Hook>
 __device__ __forceinline__ int metadata_token(int t, int p,
                                       const int32_t *__restrict__ a_req,

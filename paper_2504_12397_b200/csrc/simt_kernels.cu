@@ -187,8 +187,9 @@ linear_simt_kernel(const float *__restrict__ x, const float *__restrict__ W, int
 }
 
 // ---------------------------------------------------------------------------------------------
-// What a new token's row needs to know, from the caller's arrays (the same findings as the batch-metadata step): request, position,
-// applied adapter (the gate of Eq. 5; -1: none) and cache slot (-1: rejected).  Called by whole warps.
+// What a new token's row needs to know, from the caller's arrays (the same findings as the batch-metadata step; a change there or
+// here is one in both): request, position, applied adapter (the gate of Eq. 5; -1: none) and cache slot (-1: rejected).
+// Called by whole warps.
 // ---------------------------------------------------------------------------------------------
 struct RowFacts { int req, pos, adapter, slot; };
 __device__ __forceinline__ RowFacts row_facts(int t, const int32_t *__restrict__ positions, const int32_t *__restrict__ a_req,
@@ -198,8 +199,13 @@ __device__ __forceinline__ RowFacts row_facts(int t, const int32_t *__restrict__
     const int lane = threadIdx.x & 31;
     RowFacts f;
     f.pos = positions[t];
-    int r = 0;   // the last request that starts at or before t (empty requests start where their successor does)
-    for (int i = 1; i < R; i += 32) r += __popc(__ballot_sync(0xffffffffu, i + lane < R && qsl[i + lane] <= t));
+    int r = 0;   // the last request that starts at or before t (empty requests start where their successor does): 32 places a step
+    for (int n = R; n > 1;) {   // among requests r .. r + n - 1; r itself starts at or before t
+        const int step = (n + 31) >> 5, at = lane * step;
+        const int before = __popc(__ballot_sync(0xffffffffu, at < n && (lane == 0 || qsl[r + at] <= t))) - 1;
+        r += before * step;
+        n = min(step, n - before * step);
+    }
     f.req = r;
     const int len = seq_lens[r], next = qsl[r + 1], first_open = a_req != nullptr && mode == ALORA_MODE_ALORA ? a_req[r] : 0;
     int k = mode != ALORA_MODE_BASE && adapter_ids != nullptr ? adapter_ids[r] : -1;
@@ -527,9 +533,13 @@ int launch_rope(alora_ctx *ctx, void *qkv, const int32_t *positions, int T, void
 // head that scored a key per lane, element by element, and went over the values one key after the other took 24 us for 16
 // tokens on 64 cached ones, 27 with its launch: 4 us.)
 // ---------------------------------------------------------------------------------------------
-template <int HD, int HC>
+// kOwnFacts: the kernel finds its token's request and slot itself, beside the small layer's projection kernel in front of it; else they
+// come from the metadata step.  (Where every block of every fp32 call looked for its request, 4096 one-token requests of 4 heads
+// took 180 us instead of 90, 64 requests of 64 tokens 116 instead of 98.)
+template <int HD, int HC, bool kOwnFacts>
 __global__ void __launch_bounds__(256)
-attn_simt_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ positions, const int32_t *__restrict__ qsl,
+attn_simt_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ token_req, const int32_t *__restrict__ slot_map,
+                 const int32_t *__restrict__ positions, const int32_t *__restrict__ qsl,
                  const int32_t *__restrict__ seq_lens, const int32_t *__restrict__ block_tables, int max_blocks, int num_pages,
                  int page_size, int N, int Nq, int Hkv, int G, int R, float scale, const float *pool,
                  float *__restrict__ out, int32_t *status) {
@@ -538,14 +548,20 @@ attn_simt_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ posi
     tc::grid_dep_launch();
     const int t = blockIdx.x, kvh = blockIdx.y, h0 = (int)blockIdx.z * HC, nh = min(HC, G - h0);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, stream = warp * 4 + (lane >> 3), d0 = (lane & 7) * 4;
-    // The caller's arrays were complete before the preceding kernel of the call let this one start: they are read beside it.  Rows of the
-    // page pool are read after it, those before this request's new tokens too: another request of the call may have appended them.
-    const RowFacts f = row_facts(t, positions, nullptr, nullptr, qsl, seq_lens, block_tables, max_blocks, num_pages, page_size, 0, R,
-                                 ALORA_MODE_BASE, status);
+    // kOwnFacts: the caller's arrays were complete before the preceding kernel of the call let this one start: they are read beside it.  Rows
+    // of the page pool are read after it, those before this request's new tokens too: another request of the call may have appended them.
+    RowFacts f;
+    if constexpr (kOwnFacts) {
+        f = row_facts(t, positions, nullptr, nullptr, qsl, seq_lens, block_tables, max_blocks, num_pages, page_size, 0, R,
+                      ALORA_MODE_BASE, status);
+    } else {
+        tc::grid_dep_wait();
+        f.req = token_req[t]; f.pos = positions[t]; f.slot = slot_map[t];
+    }
     const int r = f.req, p = f.pos;
     float *orow = out + (size_t)t * Nq + (size_t)(kvh * G + h0) * HD;
     if (f.slot < 0) {  // a token that the metadata step rejects: defined output, no cache access
-        tc::grid_dep_wait();
+        if (kOwnFacts) tc::grid_dep_wait();
         for (int d = threadIdx.x; d < nh * HD; d += 256) orow[d] = 0.f;
         return;
     }
@@ -564,11 +580,13 @@ attn_simt_kernel(const float *__restrict__ qkv, const int32_t *__restrict__ posi
     };
     auto key_row = [&](int u, int j) { return pool + ((size_t)page[u] * 2 * Hkv + kvh) * page_size * HD + (size_t)(j % page_size) * HD; };
     fetch_pages(stream);
+    if (kOwnFacts) {
 #pragma unroll
-    for (int u = 0; u < U; ++u)   // the first keys and values on their way to L2 (a lane a line of 32 elements)
-        if (page[u] >= 0 && page[u] < num_pages && (lane & 7) < 2 * V)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(key_row(u, stream + 32 * u) + ((lane & 7) < V ? (lane & 7) * 32 : plane + ((lane & 7) - V) * 32)));
-    tc::grid_dep_wait();
+        for (int u = 0; u < U; ++u)   // the first keys and values on their way to L2 (a lane a line of 32 elements)
+            if (page[u] >= 0 && page[u] < num_pages && (lane & 7) < 2 * V)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(key_row(u, stream + 32 * u) + ((lane & 7) < V ? (lane & 7) * 32 : plane + ((lane & 7) - V) * 32)));
+        tc::grid_dep_wait();
+    }
 #pragma unroll
     for (int c = 0; c < HC; ++c) {
         m[c] = -INFINITY; l[c] = 0.f;
@@ -863,15 +881,18 @@ int launch_attend_simt(alora_ctx *ctx, const void *qkv, const BatchArgs &b, cons
     const Dims &d = ctx->d;
     ProfScope prof(ctx, KK_ATTENTION, s);
     auto go = [&](auto kernel, int hc) {
-        return launch_kernel(kernel, dim3(b.T, d.Hkv, (d.G + hc - 1) / hc), dim3(256), 0, s, true, (const float *)qkv, b.positions,
-                             b.query_start_loc, b.seq_lens, b.block_tables, b.max_blocks, b.num_pages,
+        return launch_kernel(kernel, dim3(b.T, d.Hkv, (d.G + hc - 1) / hc), dim3(256), 0, s, true, (const float *)qkv,
+                             (const int32_t *)ctx->d_token_req, (const int32_t *)ctx->d_slot, b.positions, b.query_start_loc, b.seq_lens, b.block_tables, b.max_blocks, b.num_pages,
                              d.page, d.N, d.Nq, d.Hkv, d.G, b.R, d.softmax_scale, (const float *)pool, (float *)out, ctx->d_status);
     };
-    const bool two = d.G > 1;
-    const cudaError_t e = d.hd == 32 ? (two ? go(attn_simt_kernel<32, 2>, 2) : go(attn_simt_kernel<32, 1>, 1))
-                          : d.hd == 64 ? (two ? go(attn_simt_kernel<64, 2>, 2) : go(attn_simt_kernel<64, 1>, 1))
-                                       : (two ? go(attn_simt_kernel<128, 2>, 2) : go(attn_simt_kernel<128, 1>, 1));
-    return e == cudaSuccess ? 1 : -1;
+    auto go_hd = [&](auto own) {
+        constexpr bool kOwn = decltype(own)::value;
+        const bool two = d.G > 1;
+        return d.hd == 32 ? (two ? go(attn_simt_kernel<32, 2, kOwn>, 2) : go(attn_simt_kernel<32, 1, kOwn>, 1))
+               : d.hd == 64 ? (two ? go(attn_simt_kernel<64, 2, kOwn>, 2) : go(attn_simt_kernel<64, 1, kOwn>, 1))
+                            : (two ? go(attn_simt_kernel<128, 2, kOwn>, 2) : go(attn_simt_kernel<128, 1, kOwn>, 1));
+    };
+    return (b.own_facts ? go_hd(std::true_type{}) : go_hd(std::false_type{})) == cudaSuccess ? 1 : -1;
 }
 
 }  // namespace alora

@@ -143,6 +143,69 @@ def test_fp32_layer_tile_and_head_edges(oracle64, hidden, heads, kv_heads, hd, n
         g.close()
 
 
+@pytest.mark.parametrize("hidden,n_req", [(64, 32), (64, 33), (64, 70), (64, 1030), (1028, 33), (1028, 70)])
+def test_fp32_layer_of_many_requests(oracle64, hidden, n_req):
+    """More requests than a warp has lanes, and than it has lanes squared, with empty ones in between and at the end: each token's
+    request is found by the small layer's own kernels (hidden 64) and by the metadata step (1028)."""
+    shape = wl.LayerShape(hidden=hidden, n_q_heads=2, n_kv_heads=1, head_dim=32, page_size=16, dtype="fp32")
+    rng = np.random.default_rng(n_req)
+    w = wl.make_wqkv(shape, rng)
+    ads = [wl.make_adapter(shape, 3, rng), wl.make_adapter(shape, 8, rng, scale=2.0)]
+    P = [(i * 7) % 40 for i in range(n_req)]
+    S = [(1, 0, 2, 1, 0)[i % 5] for i in range(n_req)]
+    S[0], S[-1] = 0, (0 if n_req % 2 else 1)
+    b = wl.make_batch(shape, P, S, [(i % 3) - 1 for i in range(n_req)], rng, activation_offsets=[p + (i % 4 == 1) for i, p in enumerate(P)],
+                      shuffle_pages=True)
+    fill = wl.random_kv_pool(shape, b.num_pages, rng)
+    g = hp.GpuLayers(shape, [dict(wqkv=w)], [ads], b.T, b.R)
+    try:
+        d = hp.DevBatch(b, shape.dtype)
+        pool, out = g.new_pool(b.num_pages, fill), g.empty(b.T, shape.Nq)
+        ab.alora_prefill_layer(g.ctx, 0, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, pool, d.bt, d.max_blocks,
+                               b.num_pages, d.T, d.R, out)
+        assert g.status() == 0
+        kv = [oracle64.paged_gather(fill, b.block_tables[r], P[r], shape.n_kv_heads, shape.page_size, shape.head_dim) if P[r] else (None, None)
+              for r in range(n_req)]
+        want = hp.oracle_block(oracle64, shape, w, ads, b, [k for k, _ in kv], [v for _, v in kv])
+        hp.assert_close(hp.to_host(out), want["out"], 1e-5, "")   # the bound of the other fp32 layer tests
+        slots = oracle64.slot_mapping(b.positions, b.query_start_loc, b.block_tables, shape.page_size)
+        got, old = hp.to_host(pool).swapaxes(1, 3).reshape(-1, shape.n_kv_heads, 2, shape.head_dim), fill.swapaxes(1, 3).reshape(-1, shape.n_kv_heads, 2, shape.head_dim)
+        hp.assert_close(got[slots][:, 0, 0], want["qkv"][:, shape.Nq:shape.Nq + shape.Nkv], 1e-5, "")
+        rest = np.setdiff1d(np.arange(len(got)), slots)
+        assert np.array_equal(got[rest], old[rest])
+    finally:
+        g.close()
+
+
+def test_fp32_attention_of_many_requests_costs_what_few_cost():
+    """4096 one-token requests against 512 of eight tokens, the same number of rows and fewer keys: the attention does not look for
+    its request among all of them in every block (1.6 times as long where it did, 1.0 now)."""
+    import torch
+    shape = wl.LayerShape(hidden=64, n_q_heads=4, n_kv_heads=2, head_dim=64, page_size=16, dtype="fp32")
+    rng = np.random.default_rng(3)
+    T, times = 4096, []
+    g = hp.GpuLayers(shape, [dict(wqkv=wl.make_wqkv(shape, rng))], [[]], T, T)
+    try:
+        for n_req in (512, 4096):
+            b = wl.make_batch(shape, [0] * n_req, [T // n_req] * n_req, [-1] * n_req, rng, with_hidden=False)
+            d = hp.DevBatch(b, shape.dtype)
+            pool, qkv, out = g.new_pool(b.num_pages), torch.randn(T, shape.N, device="cuda"), g.empty(T, shape.Nq)
+            best = float("inf")
+            for i in range(8):
+                ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+                ev[0].record()
+                for _ in range(20):
+                    ab.alora_attend(g.ctx, qkv, d.positions, d.qsl, d.seq_lens, pool, d.bt, d.max_blocks, b.num_pages, T, n_req, out)
+                ev[1].record()
+                torch.cuda.synchronize()
+                best = min(best, ev[0].elapsed_time(ev[1])) if i >= 2 else best
+            times.append(best)
+        assert g.status() == 0
+    finally:
+        g.close()
+    assert times[1] < 1.3 * times[0], times
+
+
 def test_ragged_multi_adapter_layer_bf16(oracle64):
     """Projection, append and attention on a ragged multi-adapter batch with mid-chunk activation."""
     w, ads, b = _mid_workload()
