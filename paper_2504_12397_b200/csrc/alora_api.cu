@@ -16,7 +16,7 @@ alora_status cuda_fail(alora_ctx *ctx, cudaError_t e, const char *what) {
 
 int launch_project_simt(alora_ctx *, int, const void *, int, void *, cudaStream_t, void *, int);
 int launch_linear_simt(alora_ctx *, const void *, const void *, int, int, int, void *, const void *, cudaStream_t);
-bool simt_small_layer(const alora_ctx *, int);
+bool simt_small_layer(const alora_ctx *, const BatchArgs &);
 int launch_project_small_simt(alora_ctx *, int, const void *, const BatchArgs &, void *, void *, cudaStream_t);
 int launch_attend_simt(alora_ctx *, const void *, const BatchArgs &, const void *, void *, cudaStream_t);
 
@@ -86,7 +86,7 @@ static alora_status run_layer(alora_ctx *ctx, int layer, const void *hidden, con
     b.layer = layer;
     b.few_row = project_is_few_row(ctx, layer, b.T, b.R) ? 1 : 0;   // (n_layers > 1 only where all of them take that route)
     int n = 0, k;
-    if (simt_small_layer(ctx, b.T)) {   // few fp32 rows: facts, shrink, projection and append in one launch
+    if (simt_small_layer(ctx, b)) {   // few fp32 rows: facts, shrink, projection and append in one launch
         const bool rotate = ctx->d_rope_inv_freq != nullptr;
         b.own_facts = true;
         if ((k = launch_project_small_simt(ctx, layer, hidden, b, ctx->d_qkv, rotate ? nullptr : pool, s)) < 0) return ALORA_ERR_UNSUPPORTED;
@@ -393,6 +393,8 @@ alora_status alora_register_adapter(alora_ctx *ctx, int adapter_id, int layer, i
     ctx->layer_has_adapter[layer] = 1;
     AdapterDev rec{A, B, rank, (rank + 15) / 16 * 16, scale, 0};
     ctx->h_adapters[idx] = rec;
+    ctx->largest_rank = 0;
+    for (const AdapterDev &a : ctx->h_adapters) ctx->largest_rank = std::max(ctx->largest_rank, a.rank);
     // the table entry is a kernel argument of later launches on this stream: order the update after
     // earlier work by copying on the same stream (source is context-owned host memory).
     ALORA_CUDA(ctx, cudaMemcpyAsync(ctx->d_adapters + idx, &ctx->h_adapters[idx], sizeof(AdapterDev),

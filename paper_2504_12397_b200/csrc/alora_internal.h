@@ -142,6 +142,7 @@ struct alora_ctx {
     size_t esize = 2;
     std::vector<alora::LayerWeights> layers;
     std::vector<alora::AdapterDev> h_adapters;  // [layer * max_adapters + id], mirrors d_adapters
+    int largest_rank = 0;                        // of all registered adapters, on any layer
     alora::AdapterDev *d_adapters = nullptr;
     std::vector<void *> adapter_storage;         // context-owned A/B buffers, same indexing, 2 per entry
 

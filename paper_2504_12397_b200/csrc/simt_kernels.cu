@@ -232,6 +232,7 @@ __device__ __forceinline__ RowFacts row_facts(int t, const int32_t *__restrict__
 // by every column tile, so this is for few rows and short rows of x (simt_small_layer()).
 // ---------------------------------------------------------------------------------------------
 constexpr int kSmallVecs = 8;   // 16-byte vectors of x a lane holds: hidden <= 1024
+constexpr long long kSmallRankHidden = 16384;
 __global__ void __launch_bounds__(768)
 project_small_simt_kernel(const float *__restrict__ x, const float *__restrict__ W, int Tn, int K, int N, int Nq, int Nkv, int RP,
                           const AdapterDev *__restrict__ adapters, const int32_t *__restrict__ positions,
@@ -847,13 +848,19 @@ int launch_project_simt(alora_ctx *ctx, int layer, const void *hidden, int T, vo
     return e == cudaSuccess ? 2 : -1;
 }
 
-// Whether a layer call takes project_small_simt_kernel: x rows that a warp holds in registers, and at most two blocks an SM (the t
-// that every column tile forms again costs as much as its base sums from rank 32 on).  A rule of sizes: all modes take the
-// same route.
-bool simt_small_layer(const alora_ctx *ctx, int T) {
+// Whether a layer call takes project_small_simt_kernel: x rows that a warp holds in registers, and few enough blocks (one is resident on
+// an SM, so up to two rounds).  Every column tile forms t of its rows again, one warp a row: where an adapter may apply, hidden x
+// rank is limited as well.  Calls against those with metadata, shrink and projection as launches of their own, us, 1 and 16
+// tokens on 64 cached ones, N 768: hidden 256, rank 8 12 and 13 / 16 and 21, rank 64 21 and 27 / 21 and 37; hidden 512, rank 32
+// 23 and 27 / 24 and 33, rank 64 34 and 41 / 25 and 41; hidden 1024, rank 16 28 and 32 / 33 and 36, rank 64 58 and 67 / 35 and 51.  Two
+// rounds: 192 tokens, hidden 1024, base model 59 / 62.  Both routes form the same base sums, so the rows without an adapter keep their
+// bits whichever one a mode takes.
+bool simt_small_layer(const alora_ctx *ctx, const BatchArgs &b) {
     const Dims &d = ctx->d;
-    return ctx->cfg.dtype == ALORA_DTYPE_FP32 && T > 0 && d.H % 4 == 0 && d.H <= 128 * kSmallVecs &&
-           (long long)((d.N + 31) / 32) * ((T + 15) / 16) <= 2ll * ctx->sm_count;
+    const bool may_adapt = b.mode != ALORA_MODE_BASE && b.adapter_ids != nullptr;
+    return ctx->cfg.dtype == ALORA_DTYPE_FP32 && b.T > 0 && d.H % 4 == 0 && d.H <= 128 * kSmallVecs &&
+           (!may_adapt || (long long)d.H * ctx->largest_rank <= kSmallRankHidden) &&
+           (long long)((d.N + 31) / 32) * ((b.T + 15) / 16) <= 2ll * ctx->sm_count;
 }
 int launch_project_small_simt(alora_ctx *ctx, int layer, const void *hidden, const BatchArgs &b, void *qkv, void *kv_pool, cudaStream_t s) {
     const Dims &d = ctx->d;

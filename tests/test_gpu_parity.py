@@ -206,6 +206,43 @@ def test_fp32_attention_of_many_requests_costs_what_few_cost():
     assert times[1] < 1.3 * times[0], times
 
 
+@pytest.mark.parametrize("hidden,rank,launches", [(256, 64, 2), (260, 64, 4), (1024, 16, 2), (1024, 17, 4)])
+def test_fp32_small_layer_at_its_rank_limit(oracle64, hidden, rank, launches):
+    """The one-launch projection of small fp32 layers is taken up to hidden x rank = 16384 of the largest registered adapter, metadata
+    and shrink as launches of their own beyond (from there on t formed by every column tile costs more).  Calls without adapters take
+    it anyway; rows whose gate is closed have the same bits on either route."""
+    shape = wl.LayerShape(hidden=hidden, n_q_heads=4, n_kv_heads=2, head_dim=64, page_size=16, dtype="fp32")
+    rng = np.random.default_rng(rank)
+    w = wl.make_wqkv(shape, rng)
+    ads = [wl.make_adapter(shape, 8, rng), wl.make_adapter(shape, rank, rng)]
+    b = wl.make_batch(shape, [5, 9], [20, 17], [0, 1], rng, activation_offsets=[5 + 11, 9 + 4], with_prefix_hidden=True)
+    g = hp.GpuLayers(shape, [dict(wqkv=w)], [ads], 64, 4)
+    try:
+        d = hp.DevBatch(b, shape.dtype)
+        pools = [g.new_pool(b.num_pages) for _ in range(2)]
+        for pool in pools:
+            _run_base_prefill(g, shape, b, pool)
+        outs = [g.empty(b.T, shape.Nq) for _ in range(2)]
+        n = [ab.alora_launch_count(g.ctx)]
+        for ids, pool, out in ((d.ids, pools[0], outs[0]), (None, pools[1], outs[1])):
+            ab.alora_prefill_layer(g.ctx, 0, d.hidden, d.positions, d.a_req, ids, d.qsl, d.seq_lens, pool, d.bt, d.max_blocks,
+                                   b.num_pages, d.T, d.R, out)
+            n.append(ab.alora_launch_count(g.ctx))
+        assert g.status() == 0
+        assert (n[1] - n[0], n[2] - n[1]) == (launches, 2)
+        Ks, Vs = hp.oracle_base_prefix(oracle64, shape, w, b)
+        want = hp.oracle_block(oracle64, shape, w, ads, b, Ks, Vs)
+        hp.assert_close(hp.to_host(outs[0]), want["out"], 1e-5, "")
+        off = want["gate"] == 0
+        assert 0 < off.sum() < b.T
+        assert np.array_equal(hp.to_host(outs[0])[off].view(np.uint32), hp.to_host(outs[1])[off].view(np.uint32))
+        slots = oracle64.slot_mapping(b.positions, b.query_start_loc, b.block_tables, shape.page_size)[off]
+        kept = [hp.to_host(p).swapaxes(1, 3).reshape(-1, 2 * shape.Nkv)[slots] for p in pools]
+        assert np.array_equal(kept[0].view(np.uint32), kept[1].view(np.uint32))
+    finally:
+        g.close()
+
+
 def test_ragged_multi_adapter_layer_bf16(oracle64):
     """Projection, append and attention on a ragged multi-adapter batch with mid-chunk activation."""
     w, ads, b = _mid_workload()
