@@ -232,7 +232,6 @@ __device__ __forceinline__ RowFacts row_facts(int t, const int32_t *__restrict__
 // by every column tile, so this is for few rows and short rows of x (simt_small_layer()).
 // ---------------------------------------------------------------------------------------------
 constexpr int kSmallVecs = 8;   // 16-byte vectors of x a lane holds: hidden <= 1024
-constexpr long long kSmallRankHidden = 16384;
 __global__ void __launch_bounds__(768)
 project_small_simt_kernel(const float *__restrict__ x, const float *__restrict__ W, int Tn, int K, int N, int Nq, int Nkv, int RP,
                           const AdapterDev *__restrict__ adapters, const int32_t *__restrict__ positions,
@@ -849,18 +848,22 @@ int launch_project_simt(alora_ctx *ctx, int layer, const void *hidden, int T, vo
 }
 
 // Whether a layer call takes project_small_simt_kernel: x rows that a warp holds in registers, and few enough blocks (one is resident on
-// an SM, so up to two rounds).  Every column tile forms t of its rows again, one warp a row: where an adapter may apply, hidden x
-// rank is limited as well.  Calls against those with metadata, shrink and projection as launches of their own, us, 1 and 16
-// tokens on 64 cached ones, N 768: hidden 256, rank 8 12 and 13 / 16 and 21, rank 64 21 and 27 / 21 and 37; hidden 512, rank 32
-// 23 and 27 / 24 and 33, rank 64 34 and 41 / 25 and 41; hidden 1024, rank 16 28 and 32 / 33 and 36, rank 64 58 and 67 / 35 and 51.  Two
-// rounds: 192 tokens, hidden 1024, base model 59 / 62.  Both routes form the same base sums, so the rows without an adapter keep their
-// bits whichever one a mode takes.
+// an SM, so up to two rounds).  Every column tile forms t of its rows again, one warp a row, which for few rows and a large
+// hidden x rank costs more than metadata, shrink and projection as launches of their own.  Those in turn take twice as long where the
+// shrink's blocks and the tiles, which start beside them, are more than there are SMs.  Calls on 64 cached tokens, N 768, here / there, us:
+//   hidden x rank      1 token   4          16         32         40
+//   512 x 32           23 / 25   23 / 25    28 / 33    28 / 33    29 / 66
+//   768 x 32           30 / 29   31 / 31    35 / 37    36 / 39    37 / 80
+//   512 x 64           34 / 25   34 / 28    41 / 41    42 / 43    42 / 86
+//   1024 x 64          58 / 35   59 / 37    67 / 51    68 / 53    69 / 115
+// Both routes form the same base sums, so the rows without an adapter keep their bits whichever one a mode takes.
 bool simt_small_layer(const alora_ctx *ctx, const BatchArgs &b) {
     const Dims &d = ctx->d;
+    if (ctx->cfg.dtype != ALORA_DTYPE_FP32 || b.T <= 0 || d.H % 4 != 0 || d.H > 128 * kSmallVecs) return false;
+    const long long tiles = (long long)((d.N + 31) / 32) * ((b.T + 15) / 16), work = (long long)d.H * ctx->largest_rank;
     const bool may_adapt = b.mode != ALORA_MODE_BASE && b.adapter_ids != nullptr;
-    return ctx->cfg.dtype == ALORA_DTYPE_FP32 && b.T > 0 && d.H % 4 == 0 && d.H <= 128 * kSmallVecs &&
-           (!may_adapt || (long long)d.H * ctx->largest_rank <= kSmallRankHidden) &&
-           (long long)((d.N + 31) / 32) * ((b.T + 15) / 16) <= 2ll * ctx->sm_count;
+    if (may_adapt && work > (b.T <= 4 ? 18432 : 30720) && 3 * b.T + tiles <= ctx->sm_count) return false;
+    return tiles <= 2ll * ctx->sm_count;
 }
 int launch_project_small_simt(alora_ctx *ctx, int layer, const void *hidden, const BatchArgs &b, void *qkv, void *kv_pool, cudaStream_t s) {
     const Dims &d = ctx->d;

@@ -206,16 +206,17 @@ def test_fp32_attention_of_many_requests_costs_what_few_cost():
     assert times[1] < 1.3 * times[0], times
 
 
-@pytest.mark.parametrize("hidden,rank,launches", [(256, 64, 2), (260, 64, 4), (1024, 16, 2), (1024, 17, 4)])
-def test_fp32_small_layer_at_its_rank_limit(oracle64, hidden, rank, launches):
-    """The one-launch projection of small fp32 layers is taken up to hidden x rank = 16384 of the largest registered adapter, metadata
-    and shrink as launches of their own beyond (from there on t formed by every column tile costs more).  Calls without adapters take
-    it anyway; rows whose gate is closed have the same bits on either route."""
+@pytest.mark.parametrize("hidden,rank,S,launches", [(512, 36, (2, 2), 2), (512, 37, (2, 2), 4), (512, 60, (3, 2), 2), (512, 61, (3, 2), 4),
+                                                    (1024, 64, (20, 13), 4), (1024, 64, (20, 14), 2)])
+def test_fp32_small_layer_at_its_limits(oracle64, hidden, rank, S, launches):
+    """Few rows and a large hidden x rank (of the largest registered adapter) take metadata, shrink and projection as launches of their
+    own, as long as their blocks fit on the SMs (148) side by side; else a small fp32 layer is two launches.  Calls without adapters take
+    those anyway; rows whose gate is closed have the same bits on either route."""
     shape = wl.LayerShape(hidden=hidden, n_q_heads=4, n_kv_heads=2, head_dim=64, page_size=16, dtype="fp32")
     rng = np.random.default_rng(rank)
     w = wl.make_wqkv(shape, rng)
     ads = [wl.make_adapter(shape, 8, rng), wl.make_adapter(shape, rank, rng)]
-    b = wl.make_batch(shape, [5, 9], [20, 17], [0, 1], rng, activation_offsets=[5 + 11, 9 + 4], with_prefix_hidden=True)
+    b = wl.make_batch(shape, [5, 9], list(S), [0, 1], rng, activation_offsets=[5 + S[0] // 2, 9 + 1], with_prefix_hidden=True)
     g = hp.GpuLayers(shape, [dict(wqkv=w)], [ads], 64, 4)
     try:
         d = hp.DevBatch(b, shape.dtype)
