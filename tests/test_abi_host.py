@@ -32,6 +32,13 @@ def test_every_declared_symbol_is_exported(lib):
         assert hasattr(raw, n), f"{n} declared in alora.h but not exported"
 
 
+def test_a_changed_header_makes_the_library_stale(lib, monkeypatch):
+    from paper_2504_12397_b200 import build
+    for changed, stale in ((".cuh", True), (".h", True), (".cu", True), (".py", False)):
+        monkeypatch.setattr(build.os.path, "getmtime", lambda p, c=changed: 2.0 if p.endswith(c) else 1.0)
+        assert build._stale() is stale, changed
+
+
 def test_status_strings(lib):
     seen = {ab.status_string(i) for i in range(10)}
     assert len(seen) == 10 and "ok" in seen
