@@ -145,7 +145,6 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, uint32_t sr
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];\n\tcp.async.bulk.commit_group;"
                  ::"l"((uint64_t)map), "r"(src), "r"(c0), "r"(c1) : "memory");
 }
-__device__ __forceinline__ float silu_mul(float g, float u) { return __fdividef(g, 1.f + __expf(-g)) * u; }
 
 // (none for a B with an Inf or NaN: see TilePair)
 __device__ __forceinline__ int rank_steps(const DuoArgs &a, int adapter) {
@@ -599,7 +598,7 @@ gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                         }
                         if (kMode == kDuoGlu) {
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) v[e] = __float_as_uint(silu_mul(__uint_as_float(v[e]), __uint_as_float(w[e])));
+                            for (int e = 0; e < 8; ++e) v[e] = __float_as_uint(tc::silu_mul(__uint_as_float(v[e]), __uint_as_float(w[e])));
                         }
                         if (row_ok) put_own8(col, reinterpret_cast<float(&)[8]>(v));
                     }
@@ -672,7 +671,7 @@ gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                     }
                     if (kMode == kDuoGlu) {
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(silu_mul(__uint_as_float(v[e]), __uint_as_float(v[32 + e])));
+                        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(tc::silu_mul(__uint_as_float(v[e]), __uint_as_float(v[32 + e])));
                     }
 #pragma unroll
                     for (int k = 0; k < kFirst; ++k) {

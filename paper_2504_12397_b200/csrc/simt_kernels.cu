@@ -712,7 +712,7 @@ __global__ void swiglu_kernel(const T *__restrict__ gate_up, int I, size_t total
          i += (size_t)gridDim.x * blockDim.x) {
         const size_t row = i / I, c = i % I;
         const float g = ldf(gate_up + row * 2 * I + c), u = ldf(gate_up + row * 2 * I + I + c);
-        stf(y + i, g / (1.f + __expf(-g)) * u);
+        stf(y + i, tc::silu_mul(g, u));
     }
 }
 
@@ -787,7 +787,7 @@ __global__ void __launch_bounds__(256) swiglu_bf16_kernel(const __nv_bfloat16 *_
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const float2 g = __bfloat1622float2(pg[e]), u = __bfloat1622float2(pu[e]);
-            po[e] = __floats2bfloat162_rn(g.x / (1.f + __expf(-g.x)) * u.x, g.y / (1.f + __expf(-g.y)) * u.y);
+            po[e] = __floats2bfloat162_rn(tc::silu_mul(g.x, u.x), tc::silu_mul(g.y, u.y));
         }
         *reinterpret_cast<uint4 *>(y + row * I + c) = o;
     }

@@ -1122,6 +1122,41 @@ def test_few_rows_through_gate_and_up_with_swiglu_in_the_epilogue(oracle64, T, i
         g.close()
 
 
+@pytest.mark.parametrize("dtype,T,inter", [("bf16", 8, 2048), ("bf16", 200, 2048), ("bf16", 300, 1024), ("bf16", 2048, 2048), ("fp32", 8, 64)])
+def test_swiglu_of_large_negative_gates(dtype, T, inter):
+    """A gate of -88 with an up value of 2^120: silu(-88) = -5.3e-37 is a normal number, the product -0.71.  On every route of the
+    gate / up projection (few rows, pairs of SMs, SwiGLU in a kernel of its own, fp32), with rows of ones that only column 0 of the
+    weights reads; the down projection hands every second column of the MLP on."""
+    import torch
+    H = 1024
+    shape = wl.LayerShape(hidden=H, n_q_heads=4, n_kv_heads=2, head_dim=64, page_size=16, dtype=dtype, intermediate=inter)
+    lw = dict(wqkv=np.zeros((shape.N, H), np.float32), wo=np.zeros((H, shape.Nq), np.float32), wgate_up=np.zeros((2 * inter, H), np.float32),
+              wdown=np.zeros((H, inter), np.float32), norm_attn=np.ones(H, np.float32), norm_mlp=np.ones(H, np.float32))
+    lw["wgate_up"][:inter, 0] = -88.0
+    lw["wgate_up"][inter:, 0] = 2.0 ** 120
+    n = min(H, inter) // 2
+    lw["wdown"][2 * np.arange(n), 2 * np.arange(n)] = 1.0
+    b = wl.make_batch(shape, [0], [T], [-1], np.random.default_rng(7))
+    b.hidden[:] = 1.0
+    g = hp.GpuLayers(shape, [lw], [[]], T, 1)
+    try:
+        d = hp.DevBatch(b, dtype)
+        hout = g.empty(T, H)
+        ab.alora_forward_stack(g.ctx, ab.MODE_BASE, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, [g.new_pool(b.num_pages)],
+                               d.bt, d.max_blocks, b.num_pages, T, 1, hout)
+        assert g.status() == 0
+        got = hp.to_host(hout)
+    finally:
+        g.close()
+    want = np.ones((T, H))
+    gate, up = -88.0 / np.sqrt(1 + 1e-5), 2.0 ** 120 / np.sqrt(1 + 1e-5)   # (of the norm; bf16 rows read 1)
+    if dtype == "bf16":
+        gate, up = -88.0, 2.0 ** 120
+    want[:, 2 * np.arange(n)] += gate / (1 + np.exp(-gate)) * up
+    # bf16: one rounding of the product (2^-9 x 0.71) and one of the sum; fp32: exp of an argument rounded to 2^-18
+    assert np.abs(got - want).max() < (4e-3 if dtype == "bf16" else 1e-4)
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 def test_stack_input_and_output_buffers(dtype):
     """The stack call reads its input where it is: the same result in a buffer of its own, in place, and from rows that are not
