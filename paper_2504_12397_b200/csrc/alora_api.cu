@@ -691,12 +691,15 @@ alora_status alora_forward_stack(alora_ctx *ctx, int mode, const void *d_hidden_
     // is on the few-row attention list, the tensor-core attention kernel has nothing to do and is not launched
     b.all_small = (d_query_start_loc == ctx->d_iota && T == R) ? 1 : 0;
     char *h = (char *)d_hidden_out;  // residual stream, updated in place
-    // The first layer reads the caller's rows where they are (a copy of 2048 rows took 7 us, of 40 rows 3); buffers that overlap in
-    // part or are not aligned for the kernels' vectors are copied first.
+    // The first layer reads the caller's rows where they are (a copy of 2048 rows took 7 us, of 40 rows 3).  Rows that are not aligned for
+    // the kernels' vectors are copied first, and rows that overlap the output in part through the workspace (a copy between ranges that
+    // overlap is not defined).
     const char *h_in = (const char *)d_hidden_in;
     const size_t h_bytes = (size_t)T * d.H * ctx->esize;
-    if (h_in != h && T > 0 && (!aligned16(h_in) || (h_in < h + h_bytes && h < h_in + h_bytes))) {
-        ALORA_CUDA(ctx, cudaMemcpyAsync(h, h_in, h_bytes, cudaMemcpyDeviceToDevice, s));
+    const bool overlap = h_in != h && h_in < h + h_bytes && h < h_in + h_bytes;
+    if (T > 0 && (overlap || (h_in != h && !aligned16(h_in)))) {
+        if (overlap) ALORA_CUDA(ctx, cudaMemcpyAsync(ctx->d_act[0], h_in, h_bytes, cudaMemcpyDeviceToDevice, s));
+        ALORA_CUDA(ctx, cudaMemcpyAsync(h, overlap ? ctx->d_act[0] : h_in, h_bytes, cudaMemcpyDeviceToDevice, s));
         h_in = h;
     }
     int n = 0, k;

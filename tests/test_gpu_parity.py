@@ -1159,8 +1159,9 @@ def test_swiglu_of_large_negative_gates(dtype, T, inter):
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 def test_stack_input_and_output_buffers(dtype):
-    """The stack call reads its input where it is: the same result in a buffer of its own, in place, and from rows that are not
-    16-byte aligned (copied first); the input stays as it was unless it is the output."""
+    """The stack call reads its input where it is: the same result in a buffer of its own, in place, from rows that are not 16-byte
+    aligned (copied first), and from rows that overlap the output in part, on either side (copied through the workspace); the
+    input stays as it was unless the output covers it."""
     import torch
     shape = wl.LayerShape(hidden=256, n_q_heads=4, n_kv_heads=2, head_dim=64, page_size=16, dtype=dtype, intermediate=512)
     rng = np.random.default_rng(131)
@@ -1185,5 +1186,9 @@ def test_stack_input_and_output_buffers(dtype):
         src, dst = buf[1:1 + n].view(b.T, -1), torch.empty_like(x)
         src.copy_(x)
         assert torch.equal(run(src, dst), want) and torch.equal(src, x)
+        for at_src, at_dst in ((0, 8), (8, 0), (1, 8), (9, 0), (0, 4096), (4096, 0)):   # elements into the buffer
+            src, dst = buf[at_src:at_src + n].view(b.T, -1), buf[at_dst:at_dst + n].view(b.T, -1)
+            src.copy_(x)
+            assert torch.equal(run(src, dst), want), (at_src, at_dst)
     finally:
         g.close()
