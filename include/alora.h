@@ -257,7 +257,8 @@ alora_status alora_full_lora_prefill_layer(alora_ctx *ctx, int layer, const void
  * All n_layers decoder layers (pre-norm residual: h += o_proj(attn(norm(h))); h += down(silu(gate)
  * * up) of norm(h)), adapters on q/k/v only, MLP and o_proj with base weights.  d_paged_kv_layers
  * is a HOST array of n_layers device pointers (one pool per layer, same block tables).
- * d_hidden_in[T][H] -> d_hidden_out[T][H] (may alias).  `mode` selects Eq. 5 / Eq. 4 / Eq. 2.
+ * d_hidden_in[T][H] -> d_hidden_out[T][H] (may alias or overlap; the output of bf16 layers has to be 16-byte aligned, else
+ * ALORA_ERR_INVALID_ARG).  `mode` selects Eq. 5 / Eq. 4 / Eq. 2.
  * A step whose shape the kernels do not serve (for the tensor-core path: hidden, Nq or intermediate not a
  * multiple of 8) or whose launch fails ends the call there with ALORA_ERR_UNSUPPORTED / ALORA_ERR_CUDA; the
  * steps before it have been enqueued and d_hidden_out then holds an unfinished residual stream.

@@ -677,6 +677,7 @@ alora_status alora_forward_stack(alora_ctx *ctx, int mode, const void *d_hidden_
         return ALORA_ERR_INVALID_ARG;
     if (mode < ALORA_MODE_ALORA || mode > ALORA_MODE_BASE) return ALORA_ERR_INVALID_ARG;
     if (mode == ALORA_MODE_ALORA && d_adapter_ids && !d_activation_offsets) return ALORA_ERR_INVALID_ARG;
+    if (ctx->cfg.dtype == ALORA_DTYPE_BF16 && !aligned16(d_hidden_out)) return ALORA_ERR_INVALID_ARG;   // (16-byte stores; fp32 has single ones)
     if (ctx->d.I <= 0) return ALORA_ERR_UNSUPPORTED;
     for (int l = 0; l < ctx->cfg.n_layers; ++l) {
         const LayerWeights &lw = ctx->layers[l];

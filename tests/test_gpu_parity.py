@@ -1190,5 +1190,14 @@ def test_stack_input_and_output_buffers(dtype):
             src, dst = buf[at_src:at_src + n].view(b.T, -1), buf[at_dst:at_dst + n].view(b.T, -1)
             src.copy_(x)
             assert torch.equal(run(src, dst), want), (at_src, at_dst)
+        # an output that is not aligned: fp32 rows are stored element by element, bf16 rows are refused before any launch
+        src, dst = x.clone(), buf[1:1 + n].view(b.T, -1)
+        if dtype == "fp32":
+            assert torch.equal(run(src, dst), want)
+        else:
+            launches = ab.alora_launch_count(g.ctx)
+            with pytest.raises(ab.AloraError) as e:
+                run(src, dst)
+            assert e.value.status == 1 and ab.alora_launch_count(g.ctx) == launches
     finally:
         g.close()
