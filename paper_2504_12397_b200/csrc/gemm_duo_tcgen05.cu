@@ -754,6 +754,7 @@ static int launch_duo(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap 
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
+    ProfScope prof(ctx, kMode == kDuoQkv ? KK_PROJECT : KK_LINEAR, s);
     return cudaLaunchKernelEx(&cfg, gemm_duo_tcgen05_kernel<kMode, kParts>, tmX, tmW, tmT, tmS, tmB[0], tmB[1], tmB[2], tmO, g) == cudaSuccess ? 1 : -1;
 }
 

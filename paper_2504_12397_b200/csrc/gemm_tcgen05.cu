@@ -603,8 +603,7 @@ int launch_project_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int 
                                 have_adapters ? ads : nullptr, ctx->tc_b_all[layer], T, d.H, d.N, d.Nq, d.Nkv, qkv,
                                 kv_pool, num_pages, layer, s);
     }
-    {   // many rows: pairs of SMs
-        ProfScope prof(ctx, KK_PROJECT, s);
+    {   // many rows: pairs of SMs (bracketed for the profile there, once the route is decided)
         const int r = launch_project_duo_tc(ctx, layer, hidden, T, R, qkv, s, kv_pool, num_pages);
         if (r != 0) return r;
     }
@@ -671,13 +670,15 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
     if (T == 0) return 0;
     if (K % 8 != 0 || N % 8 != 0) return -1;
     if (delta != nullptr && (T <= kFewRowMax || (N / delta->n_blk) % 256 != 0)) return -1;
-    ProfScope prof(ctx, KK_LINEAR, s);
-    if (delta == nullptr && few_cluster_rows(ctx, T) && few_cluster_route(ctx, T, 0, N, K, false, N, 0))
+    if (delta == nullptr && few_cluster_rows(ctx, T) && few_cluster_route(ctx, T, 0, N, K, false, N, 0)) {
+        ProfScope prof(ctx, KK_LINEAR, s);
         return launch_few_cluster(ctx, x, W, nullptr, nullptr, nullptr, T, 0, K, N, N, 0, y, residual, nullptr, 0, false, s);
+    }
     {
         const int r = launch_linear_duo_tc(ctx, x, W, T, K, N, y, residual, delta, false, s);   // many rows: pairs of SMs
         if (r != 0) return r;
     }
+    ProfScope prof(ctx, KK_LINEAR, s);
     const int BN = N % 256 == 0 || N > 1024 ? 256 : 128;
     CUtensorMap tmX, tmW;
     if (!make_tensor_map_bf16(&tmX, x, T, K, K, kBM)) return -1;
@@ -715,7 +716,6 @@ int launch_glu_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K, in
         ProfScope prof(ctx, KK_LINEAR, s);
         return launch_few_cluster(ctx, x, W, nullptr, nullptr, nullptr, T, 0, K, N, N, 0, y, nullptr, nullptr, 0, false, s, true);
     }
-    ProfScope prof(ctx, KK_LINEAR, s);
     return launch_linear_duo_tc(ctx, x, W, T, K, N, y, nullptr, delta, true, s);
 }
 

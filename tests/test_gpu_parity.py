@@ -758,6 +758,31 @@ def test_stack_layer_at_the_8b_shape_with_1024_rows(oracle64):
         g.close()
 
 
+@pytest.mark.parametrize("T", [200, 600, 2048])
+def test_profile_counts_only_groups_that_launched(T):
+    """One layer with adapters on the MLP block, whose rows take the row tiles or the pairs of SMs: a launcher that passes a batch on
+    to the next one leaves no empty group behind."""
+    shape = wl.LayerShape(hidden=1024, n_q_heads=8, n_kv_heads=2, head_dim=128, page_size=16, dtype="bf16", intermediate=2048)
+    rng = np.random.default_rng(3)
+    b = wl.make_batch(shape, [0, 0], [T - 70, 70], [0, -1], rng)
+    g = hp.GpuLayers(shape, [wl.make_stack_weights(shape, rng)], [[wl.make_adapter(shape, 8, rng)]], T, 2,
+                     mlp_adapters_per_layer=[[wl.make_mlp_adapter(shape, 8, rng)]])
+    try:
+        d = hp.DevBatch(b, shape.dtype)
+        pool, hout = g.new_pool(b.num_pages), g.empty(T, shape.hidden)
+        ab.alora_profile_enable(g.ctx, True)
+        n = ab.alora_launch_count(g.ctx)
+        ab.alora_forward_stack(g.ctx, ab.MODE_ALORA, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, [pool], d.bt, d.max_blocks,
+                               b.num_pages, T, 2, hout)
+        n = ab.alora_launch_count(g.ctx) - n
+        groups = {k: v[1] for k, v in ab.alora_profile_read(g.ctx).items()}
+        assert g.status() == 0
+    finally:
+        g.close()
+    assert groups["project_qkv"] == 1 and groups["linear"] == 3, groups   # o_proj, gate / up, down
+    assert sum(groups.values()) <= n, (groups, n)
+
+
 def test_empty_and_degenerate_batches():
     w, ads, b = _mid_workload()
     g = hp.GpuLayers(MID, [dict(wqkv=w)], [ads], 256, 8)
