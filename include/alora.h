@@ -388,6 +388,14 @@ alora_status alora_selftest_claim_order(int grid, int n_shrink, int n_row_tiles,
                                         int *completed);
 
 /*
+ * Which kernel serves one matrix of a layer for a batch of T tokens and R requests (host only, nothing is launched; the paper has no
+ * counterpart).  `matrix`: 0 q/k/v, 1 o_proj, 2 gate / up, 3 down (1 .. 3: at most 8192 of a stack call's tokens at a time);
+ * `adapted` != 0: the call applies adapters on the MLP block.  *tile = the column tile of the kernel that works on pairs of SMs, 0
+ * where another kernel is taken.
+ */
+alora_status alora_selftest_pair_tile(const alora_ctx *ctx, int layer, int matrix, int T, int R, int adapted, int *tile);
+
+/*
  * Optional per-kernel timing (a measurement aid; the paper has no counterpart).  While enabled,
  * every kernel family launched by this context is bracketed by CUDA events on the launching stream.
  * alora_profile_enable(ctx, 1) clears what was accumulated and starts, (ctx, 0) stops.

@@ -288,6 +288,16 @@ def alora_cow_tail_pages(ctx, query_start_loc, seq_lens, block_tables, max_block
                   _ptr(fresh_pages), _ptr(paged_kv), _stream(stream)), "alora_cow_tail_pages")
 
 
+def alora_selftest_pair_tile(ctx, layer: int, matrix: int, T: int, R: int, adapted: bool = False) -> int:
+    """Column tile of the kernel on pairs of SMs for one matrix of a layer (0 q/k/v, 1 o_proj, 2 gate / up, 3 down); 0: another kernel."""
+    f = load_library().alora_selftest_pair_tile
+    f.argtypes = [C.c_void_p] + [C.c_int] * 5 + [C.POINTER(C.c_int)]
+    f.restype = C.c_int
+    tile = C.c_int(-1)
+    _check(ctx, f(ctx, layer, matrix, T, R, int(bool(adapted)), C.byref(tile)), "alora_selftest_pair_tile")
+    return tile.value
+
+
 def alora_selftest_wait_timeout(ctx, limit_cycles: int, stream=None) -> None:
     f = load_library().alora_selftest_wait_timeout
     f.argtypes = [C.c_void_p, C.c_int64, _VP]

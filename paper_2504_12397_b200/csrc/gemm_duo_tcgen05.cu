@@ -760,14 +760,12 @@ static int launch_duo(alora_ctx *ctx, const CUtensorMap &tmX, const CUtensorMap 
 
 bool shrink_apart(const alora_ctx *ctx, int T, int R, int items);   // gemm_tcgen05.cu
 
-// q/k/v projection of a batch.  Returns the kernels launched, 0 when the batch is better served by the 128-row kernel (nothing
-// launched) or -1 on error.  The decision must not depend on the mode, so that rows with a closed gate come out bit-identical to the
-// base-only projection of the same batch.
-int launch_project_duo_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int R, void *qkv, cudaStream_t s,
-                          void *kv_pool, int num_pages) {
+// The column tile that the q/k/v projection of a batch takes here, 0: it is better served by the 128-row kernel.  The decision must not
+// depend on the mode, so that rows with a closed gate come out bit-identical to the base-only projection of the same batch.
+int duo_project_tile(const alora_ctx *ctx, int layer, int T, int R) {
     const Dims &d = ctx->d;
     if (T <= kQuadRows || ctx->sm_count < 2 || d.H % 8 != 0 || d.N % 8 != 0 || d.Nq % 32 != 0 || d.Nkv % 32 != 0) return 0;
-    const int G = ctx->sm_count, t_parts = T <= kSplitTTokens ? 3 : 1;
+    const int G = ctx->sm_count;
     // against the 128 x 256 tiles of gemm_tcgen05.cu, 790 cycles a K block
     const bool have_adapters = ctx->layer_has_adapter[layer] != 0;
     long long here = 0;
@@ -780,10 +778,19 @@ int launch_project_duo_tc(alora_ctx *ctx, int layer, const void *hidden, int T, 
     // a row tile there, 30 k for a shrink kernel of its own.  One layer call, us, there / here: 777 rows and one adapter 101 / 87,
     // 1000 rows and two 80 / 66 (the projection alone), 753 rows of 48 requests and four 69 / 81.
     const int n_m = (T + 127) / 128, n_q = (n_m + 3) / 4;
-    const bool few = have_adapters && t_parts == 3;
+    const bool few = have_adapters && T <= kSplitTTokens;
     const long long late_here = few ? 15000ll * ((quad_bound(ctx, T, R) + n_q - 1) / n_q) : 0;
     const long long late_other = few ? 8000ll * ((pair_bound(ctx, T, R) + n_m - 1) / n_m) + (apart ? 30000 : 0) : 0;
-    if (here + late_here > other + late_other) return 0;
+    return here + late_here > other + late_other ? 0 : bn;
+}
+
+// q/k/v projection of a batch.  Returns the kernels launched, 0 when the batch is not for this kernel (nothing launched) or -1 on error.
+int launch_project_duo_tc(alora_ctx *ctx, int layer, const void *hidden, int T, int R, void *qkv, cudaStream_t s,
+                          void *kv_pool, int num_pages) {
+    const Dims &d = ctx->d;
+    const int bn = duo_project_tile(ctx, layer, T, R), t_parts = T <= kSplitTTokens ? 3 : 1;
+    const bool have_adapters = ctx->layer_has_adapter[layer] != 0;
+    if (bn == 0) return 0;
     const void *W = ctx->layers[layer].wqkv;
     CUtensorMap tmX, tmW, tmT, tmS, tmB[3];
     if (!make_tensor_map_bf16(&tmX, hidden, T, d.H, d.H, 128)) return -1;
@@ -829,10 +836,12 @@ int launch_project_duo_tc(alora_ctx *ctx, int layer, const void *hidden, int T, 
                         : launch_duo<kDuoQkv, 1>(ctx, tmX, tmW, tmT, tmS, tmB, g, max_items, s);
 }
 
-// Plain dense projection y = x W^T (+ residual), or with `glu` y = silu(x Wg^T) * (x Wu^T) for W = [Wg; Wu]; optionally with a gated
-// low-rank delta.  Returns 1 (launched), 0 (shape better served by the 128-row kernel: not launched) or -1 (error).
-int launch_linear_duo_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
-                         const void *residual, const LinearDelta *delta, bool glu, cudaStream_t s) {
+static int duo_max_entries(const alora_ctx *ctx, int T) {
+    return std::min(ctx->max_quads, (T + kQuadRows - 1) / kQuadRows * std::max(1, ctx->cfg.max_adapters));
+}
+// The column tile that a dense projection of T rows takes here, 0: it is better served by the 128-row kernel.  (The choice of the
+// kernel must not depend on the mode; that of the tile may, a row's sums are the same in all of them.)
+int duo_linear_tile(const alora_ctx *ctx, int T, int K, int N, bool glu, bool adapted) {
     const int G = ctx->sm_count, n_out = glu ? N / 2 : N;
     // Against rounds over the blocks x 790 cycles of the 128 x 256 tile's K block.  That
     // kernel walks the column tiles of a row tile first, so a W that L2 does not hold is streamed from HBM (3400 bytes a cycle)
@@ -841,13 +850,22 @@ int launch_linear_duo_tc(alora_ctx *ctx, const void *x, const void *W, int T, in
     const long long rounds128 = (items128 + G - 1) / G;
     const long long w_cycles = (long long)N * K * 2 > (64ll << 20) ? (n_n >= G ? (T + 127) / 128 : rounds128) * N * (2 * kBKd) / 3400 : 0;
     const long long other = std::max(rounds128 * 790, w_cycles) * ((K + kBKd - 1) / kBKd);
-    if (delta != nullptr && (delta->n_blk != (glu ? 2 : 1) || delta->tile0 % 4 != 0)) return 0;
-    if (T <= 256 || G < 2 || K % 8 != 0 || N % 8 != 0 || (glu && (N % 16 != 0 || residual != nullptr))) return 0;
+    if (T <= 256 || G < 2 || K % 8 != 0 || N % 8 != 0 || (glu && N % 16 != 0)) return 0;
     long long here = 0;
-    int bn = duo_pick_bn(ctx, T, K, n_out, glu, 0, &here);   // (the choice of the kernel must not depend on the mode)
+    const int bn = duo_pick_bn(ctx, T, K, n_out, glu, 0, &here);
     if (here > other) return 0;
-    const int max_entries = delta == nullptr ? 0 : std::min(ctx->max_quads, (T + kQuadRows - 1) / kQuadRows * std::max(1, ctx->cfg.max_adapters));
-    if (max_entries > 0) bn = duo_pick_bn(ctx, T, K, n_out, glu, max_entries, &here);
+    return adapted ? duo_pick_bn(ctx, T, K, n_out, glu, duo_max_entries(ctx, T), &here) : bn;
+}
+
+// Plain dense projection y = x W^T (+ residual), or with `glu` y = silu(x Wg^T) * (x Wu^T) for W = [Wg; Wu]; optionally with a gated
+// low-rank delta.  Returns 1 (launched), 0 (not for this kernel: nothing launched) or -1 (error).
+int launch_linear_duo_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y,
+                         const void *residual, const LinearDelta *delta, bool glu, cudaStream_t s) {
+    const int n_out = glu ? N / 2 : N;
+    if (delta != nullptr && (delta->n_blk != (glu ? 2 : 1) || delta->tile0 % 4 != 0)) return 0;
+    if (glu && residual != nullptr) return 0;
+    const int bn = duo_linear_tile(ctx, T, K, N, glu, delta != nullptr), max_entries = delta == nullptr ? 0 : duo_max_entries(ctx, T);
+    if (bn == 0) return 0;
     CUtensorMap tmX, tmW, tmT, tmA, tmB[3];
     if (!make_tensor_map_bf16(&tmX, x, T, K, K, 128)) return -1;
     if (!make_tensor_map_bf16(&tmW, W, N, K, K, bn / 2)) return -1;

@@ -719,6 +719,23 @@ int launch_glu_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K, in
     return launch_linear_duo_tc(ctx, x, W, T, K, N, y, nullptr, delta, true, s);
 }
 
+int duo_project_tile(const alora_ctx *ctx, int layer, int T, int R);                       // gemm_duo_tcgen05.cu
+int duo_linear_tile(const alora_ctx *ctx, int T, int K, int N, bool glu, bool adapted);
+
+// The column tile of the kernel on pairs of SMs for one matrix of a layer (0 q/k/v, 1 o_proj, 2 gate / up with SwiGLU, 3 down), 0 where
+// another kernel serves it: the order of the launchers above.
+int pair_tile(const alora_ctx *ctx, int layer, int matrix, int T, int R, bool adapted) {
+    const Dims &d = ctx->d;
+    if (T == 0) return 0;
+    if (matrix == 0) {
+        if (project_few_cluster(ctx, layer, T, R) || skinny_route(ctx, T, d.N, d.H, ctx->layer_has_adapter[layer], d.Nq, d.Nkv)) return 0;
+        return duo_project_tile(ctx, layer, T, R);
+    }
+    const int K = matrix == 1 ? d.Nq : matrix == 2 ? d.H : d.I, N = matrix == 2 ? 2 * d.I : d.H;
+    if (!adapted && few_cluster_rows(ctx, T) && few_cluster_route(ctx, T, 0, N, K, false, N, 0)) return 0;
+    return duo_linear_tile(ctx, T, K, N, matrix == 2, adapted);
+}
+
 // Tensor maps that depend only on registered weights; (re)built when weights or adapters are set.
 bool build_layer_maps(alora_ctx *ctx, int layer) {
     const Dims &d = ctx->d;

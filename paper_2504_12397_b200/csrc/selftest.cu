@@ -23,7 +23,16 @@ __global__ void __launch_bounds__(32) wait_timeout_selftest_kernel(long long lim
     if (threadIdx.x == 0 && (!done || abort_flag)) report(status, ALORA_ERR_TIMEOUT);
 }
 
+int pair_tile(const alora_ctx *ctx, int layer, int matrix, int T, int R, bool adapted);   // gemm_tcgen05.cu
 }  // namespace alora
+
+extern "C" alora_status alora_selftest_pair_tile(const alora_ctx *ctx, int layer, int matrix, int T, int R, int adapted, int *tile) {
+    if (!ctx || !tile || layer < 0 || layer >= ctx->cfg.n_layers || matrix < 0 || matrix > 3 || T < 0 || R < 0) return ALORA_ERR_INVALID_ARG;
+    if (T > ctx->cfg.max_tokens || R > ctx->cfg.max_requests) return ALORA_ERR_CAPACITY;
+    if (matrix > 0 && ctx->d.I <= 0) return ALORA_ERR_UNSUPPORTED;
+    *tile = ctx->cfg.dtype == ALORA_DTYPE_BF16 ? alora::pair_tile(ctx, layer, matrix, T, R, adapted != 0 && matrix >= 2) : 0;
+    return ALORA_OK;
+}
 
 extern "C" alora_status alora_selftest_wait_timeout(alora_ctx *ctx, int64_t limit_cycles, void *stream) {
     if (!ctx) return ALORA_ERR_INVALID_ARG;

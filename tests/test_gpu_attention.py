@@ -204,8 +204,18 @@ def test_leading_keys_with_scores_of_minus_infinity(oracle64, S, dead):
 
 @pytest.mark.parametrize("S", [[33], [32, 64, 65, 31], [127, 128, 129], [33, 64] * 19, [40, 33] * 45])
 def test_blocks_of_half_size_and_claimed_items(oracle64, S):
-    """Few items: blocks of 32 tokens instead of 64, at the edges of both; 38 requests that fill the blocks exactly with
-    halves; 90 requests with more items than blocks, which the blocks claim."""
+    """Few items: blocks of 32 tokens instead of 64, at the edges of both; 38 requests in blocks of 64, nearly one a block; 90 requests
+    with more items than blocks, which the blocks claim."""
     P = [(i * 613) % 1500 for i in range(len(S))]
     err, _, _ = _attend_case(oracle64, SHAPE_G4, P, S, seed=700 + len(S))
+    assert err <= 2e-2
+
+
+@pytest.mark.parametrize("more", [0, 1])
+def test_blocks_of_half_size_up_to_one_an_sm(oracle64, more):
+    """The largest list of half-size blocks (two a request, two KV heads: one item an SM), and the first batch that keeps whole ones."""
+    import torch
+    n = torch.cuda.get_device_properties(0).multi_processor_count // 4 + more
+    P = [(i * 613) % 1500 for i in range(n)]
+    err, _, _ = _attend_case(oracle64, SHAPE_G4, P, [33 + (i * 7) % 32 for i in range(n)], seed=800 + more)
     assert err <= 2e-2

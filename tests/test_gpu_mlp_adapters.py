@@ -181,6 +181,44 @@ def test_mlp_adapters_across_token_chunks_of_the_mlp(oracle64):
         g.close()
 
 
+def test_mlp_adapters_across_token_chunks_on_pairs_of_sms(oracle64):
+    """A second MLP pass of 1048 rows whose gate / up and down are on pairs of SMs as well (entries of the batch's quads 16 .. 18, the last
+    one of 24 rows), gates open on both sides of row 8192; the same comparison, and closed rows keep the bits of the base mode."""
+    shape = wl.LayerShape(hidden=768, n_q_heads=4, n_kv_heads=2, head_dim=64, page_size=16, dtype="bf16", intermediate=2304)
+    rng = np.random.default_rng(46)
+    layers = [wl.make_stack_weights(shape, rng)]
+    ads = [[wl.make_adapter(shape, r, rng) for r in (16, 8)]]
+    mlps = [[wl.make_mlp_adapter(shape, r, rng, scale=s) for r, s in ((16, 1.0), (40, 0.5))]]
+    for m in mlps[0]:
+        for n in ("Bg", "Bu", "Bd"):
+            setattr(m, n, wl.bf16_round(getattr(m, n) * 8))
+    R, S = 22, 420
+    ids = [(r + 1) % 3 - 1 for r in range(R)]     # request 19 holds row 8192: adapter 1
+    a_req = [0 if r % 3 else 100 for r in range(R)]
+    b = wl.make_batch(shape, [0] * R, [S] * R, ids, rng, activation_offsets=a_req, shuffle_pages=True)
+    assert b.T == 9240 and ids[8192 // S] == 1
+    g = hp.GpuLayers(shape, layers, ads, b.T, R, mlp_adapters_per_layer=mlps)
+    try:
+        assert all(ab.alora_selftest_pair_tile(g.ctx, 0, m, rows, R, True) for m in (2, 3) for rows in (8192, b.T - 8192))
+        d = hp.DevBatch(b, shape.dtype)
+        outs = []
+        for mode in (ab.MODE_ALORA, ab.MODE_BASE):
+            pools, hout = [g.new_pool(b.num_pages)], g.empty(b.T, shape.hidden)
+            ab.alora_forward_stack(g.ctx, mode, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, pools, d.bt, d.max_blocks,
+                                   b.num_pages, d.T, d.R, hout)
+            outs.append(hp.to_host(hout))
+        assert g.status() == 0
+    finally:
+        g.close()
+    x, _ = oracle64.decoder_layer(b.hidden.astype(np.float64), layers[0], shape.Nq, shape.Nkv, shape.n_q_heads, shape.n_kv_heads,
+                                  shape.head_dim, 1e-5, b.positions, b.query_start_loc, b.activation_offsets, b.adapter_ids,
+                                  hp.oracle_adapters(ads[0]), [None] * R, [None] * R, mlp_adapters=hp.oracle_mlp_adapters(mlps[0]))
+    hp.assert_close(outs[0], x, 2e-2, "two MLP passes on pairs of SMs", block=shape.head_dim)
+    closed = (np.repeat(np.array(ids), S) < 0) | (b.positions < np.repeat(np.array(a_req), S))
+    assert np.array_equal(outs[0][closed].view(np.uint32), outs[1][closed].view(np.uint32))
+    assert hp.rel_err(outs[0][~closed], outs[1][~closed]) > 0.02
+
+
 def test_one_layer_at_the_8b_shape(oracle64):
     """One decoder layer at the 8B layer shape (hidden 4096, intermediate 14336: gate / up rows of 57 KB, a down
     projection with K = 14336) with adapters on q/k/v and on the MLP: three requests (rank 32 and rank 8 adapters and
@@ -304,11 +342,13 @@ def test_non_finite_mlp_adapter_values_stay_in_the_rows_that_use_them(each):
         assert not np.isfinite(odd[own]).all(), n
 
 
-def test_dense_matrices_on_pairs_of_sms(oracle64):
-    """One layer of 4900 rows (three row tiles in the last quad, the last one partial): o_proj, gate / up with SwiGLU in the
-    epilogue (column tiles of 96, the last one cut off) and down on pairs of SMs, with MLP adapters; closed rows keep the bits of
-    the base-mode call, and a non-finite B reaches only the rows that use it."""
-    shape = wl.LayerShape(hidden=1024, n_q_heads=8, n_kv_heads=2, head_dim=128, page_size=16, dtype="bf16", intermediate=1280)
+@pytest.mark.parametrize("inter,tiles", [(1280, (192, 256)), (768, (224, 160)), (1024, (160, 192))])
+def test_dense_matrices_on_pairs_of_sms(oracle64, inter, tiles):
+    """One layer of 4900 rows (three row tiles in the last quad, the last one partial): o_proj, gate / up with SwiGLU in the epilogue
+    and down on pairs of SMs, with MLP adapters.  The column tiles of gate / up are of 96, 112 and 80 columns in the base mode and
+    128, 80 and 96 with the adapters' items; the last one is cut off but for 128, and of 80 in the base mode.  Closed rows keep the
+    bits of the base-mode call, and a non-finite B reaches only the rows that use it."""
+    shape = wl.LayerShape(hidden=1024, n_q_heads=8, n_kv_heads=2, head_dim=128, page_size=16, dtype="bf16", intermediate=inter)
     rng = np.random.default_rng(52)
     layers = [wl.make_stack_weights(shape, rng)]
     ads = [[wl.make_adapter(shape, r, rng) for r in (32, 8)]]
@@ -323,6 +363,8 @@ def test_dense_matrices_on_pairs_of_sms(oracle64):
     def run(mode=ab.MODE_ALORA):
         g = hp.GpuLayers(shape, layers, ads, b.T, b.R, mlp_adapters_per_layer=mlps)
         try:
+            assert tuple(ab.alora_selftest_pair_tile(g.ctx, 0, 2, b.T, b.R, adapted) for adapted in (False, True)) == tiles
+            assert ab.alora_selftest_pair_tile(g.ctx, 0, 1, b.T, b.R) and ab.alora_selftest_pair_tile(g.ctx, 0, 3, b.T, b.R, True)
             d = hp.DevBatch(b, shape.dtype)
             pools, hout = [g.new_pool(b.num_pages)], g.empty(b.T, shape.hidden)
             ab.alora_forward_stack(g.ctx, mode, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, pools, d.bt,

@@ -330,9 +330,12 @@ def _boosted_adapters(shape, rng, spec):
     return ads
 
 
-def _check_projection(oracle64, shape, w, ads, b, n_off_expected=None):
+def _check_projection(oracle64, shape, w, ads, b, n_off_expected=None, on_pairs=None):
+    """on_pairs: whether the kernel on pairs of SMs has to serve the batch (None: not looked at)."""
     g = hp.GpuLayers(shape, [dict(wqkv=w)], [ads], b.T, b.R)
     try:
+        if on_pairs is not None:
+            assert (ab.alora_selftest_pair_tile(g.ctx, 0, 0, b.T, b.R) > 0) == on_pairs
         d = hp.DevBatch(b, shape.dtype)
         qkv, base, again = g.empty(b.T, shape.N), g.empty(b.T, shape.N), g.empty(b.T, shape.N)
         for mode, dst in ((ab.MODE_ALORA, qkv), (ab.MODE_BASE, base), (ab.MODE_ALORA, again)):
@@ -366,17 +369,15 @@ def test_projection_row_tile_route_with_fused_shrink(oracle64):
     _check_projection(oracle64, MID, w, ads, b, n_off_expected=130 + 130 + 195)
 
 
-def test_projection_of_many_rows_two_row_tiles_per_block(oracle64):
-    """Many rows (and enough tiles to fill the blocks): the projection takes 256 x 192 tiles (two row tiles per block).  With this shape's
-    blocks of 1024 / 256 / 256 columns the 192-wide column tiles straddle the q | k and k | v boundaries, some
-    row tiles are partial, one request runs on the base model and gates open in the middle of requests."""
+def test_projection_of_many_rows_on_single_sms(oracle64):
+    """Many rows on tiles of 128 x 256, one a block, where those take fewer rounds than the tiles of pairs of SMs, with the shrink as leading
+    work items: 36 row tiles in two rounds, one request on the base model, gates that open in the middle of requests."""
     rng = np.random.default_rng(45)
     w = wl.make_wqkv(MID, rng)
     ads = _boosted_adapters(MID, rng, ((8, 1.0), (64, 0.5), (32, 2.0)))
     b = wl.make_batch(MID, [0, 300, 20, 5, 0], [1500, 1390, 530, 760, 428], [1, 0, -1, 2, 0], rng,
                       activation_offsets=[130, 300, 0, 200, 77])
-    assert b.T == 4608   # 18 row pairs x 8 column tiles = 144 items for 148 blocks: the launcher prefers this tile shape
-    _check_projection(oracle64, MID, w, ads, b, n_off_expected=130 + 530 + 195 + 77)
+    _check_projection(oracle64, MID, w, ads, b, n_off_expected=130 + 530 + 195 + 77, on_pairs=False)
 
 
 def test_projection_row_wise_route_many_short_requests(oracle64):
@@ -703,9 +704,9 @@ def test_two_layer_stack(oracle64):
         g.close()
 
 
-def test_stack_layer_with_many_rows_takes_the_256_row_gemm(oracle64):
-    """One decoder layer on 2048 tokens with a wide MLP: gate/up (2048 x 9472 outputs = 296 tiles of 256 x 256) runs
-    on the 256-row GEMM kernel, o_proj and down (one column tile) on the 128-row kernel."""
+def test_stack_layer_with_many_rows_and_a_short_k(oracle64):
+    """One decoder layer on 2048 tokens with a wide MLP and a hidden size of 256: gate / up (2048 x 9472 outputs = 592 tiles of 128 x 256) on
+    the 128-row kernel with SwiGLU in a kernel of its own, as are o_proj and q/k/v; down (K 4736, two column tiles) on pairs of SMs."""
     shape = wl.LayerShape(hidden=256, n_q_heads=4, n_kv_heads=2, head_dim=64, page_size=16, dtype="bf16",
                           intermediate=4736)
     rng = np.random.default_rng(41)
@@ -714,6 +715,7 @@ def test_stack_layer_with_many_rows_takes_the_256_row_gemm(oracle64):
     b = wl.make_batch(shape, [0] * 8, [256] * 8, [0, -1] * 4, rng, activation_offsets=[100] * 8, shuffle_pages=True)
     g = hp.GpuLayers(shape, layers, ads, 2048, 8)
     try:
+        assert [ab.alora_selftest_pair_tile(g.ctx, 0, m, b.T, b.R) > 0 for m in range(4)] == [False, False, False, True]
         d = hp.DevBatch(b, shape.dtype)
         pools = [g.new_pool(b.num_pages)]
         hout = g.empty(b.T, shape.hidden)
@@ -730,9 +732,9 @@ def test_stack_layer_with_many_rows_takes_the_256_row_gemm(oracle64):
 
 
 def test_stack_layer_at_the_8b_shape_with_1024_rows(oracle64):
-    """One decoder layer at the 8B layer shape on 4 x 256 new tokens: q/k/v on the 128-row tile route with the fused
-    shrink, o_proj, gate / up (28672 columns) and down (K = 14336) on the 256 x 256 dense kernel, the 16-byte norm and
-    SwiGLU kernels at their real row lengths.  Every row against the oracle (about 0.23 TFLOP of oracle work)."""
+    """One decoder layer at the 8B layer shape on 4 x 256 new tokens: q/k/v with its adapter, o_proj, gate / up (28672 columns, SwiGLU in
+    the epilogue) and down (K = 14336) on pairs of SMs, the 16-byte norm kernel at its real row length.  Every row against the
+    oracle (about 0.23 TFLOP of oracle work)."""
     shape = wl.SHAPE_8B
     rng = np.random.default_rng(48)
     layers = [wl.make_stack_weights(shape, rng)]
@@ -743,6 +745,7 @@ def test_stack_layer_at_the_8b_shape_with_1024_rows(oracle64):
                       shuffle_pages=True)
     g = hp.GpuLayers(shape, layers, ads, 1024, 4)
     try:
+        assert all(ab.alora_selftest_pair_tile(g.ctx, 0, m, b.T, b.R) for m in range(4))
         d = hp.DevBatch(b, shape.dtype)
         pools = [g.new_pool(b.num_pages)]
         hout = g.empty(b.T, shape.hidden)
@@ -939,6 +942,39 @@ def test_stack_layers_on_different_projection_routes_share_the_attention_list(or
         g.close()
 
 
+def test_stack_layers_hand_the_claim_counter_of_the_attention_on(oracle64):
+    """Four layers on a batch with more attention items (180) than blocks, which the blocks claim from a counter: layers 0 and 2 use one
+    counter, 1 and 3 the other, each cleared by the layer in between.  A second call begins with what the first one left."""
+    shape = wl.LayerShape(hidden=256, n_q_heads=4, n_kv_heads=2, head_dim=64, page_size=16, dtype="bf16", intermediate=256)
+    rng = np.random.default_rng(67)
+    n, R = 4, 90
+    layers = [wl.make_stack_weights(shape, rng) for _ in range(n)]
+    P = [int(p) for p in rng.integers(0, 400, R)]
+    b = wl.make_batch(shape, P, [int(s) for s in rng.integers(33, 65, R)], [-1] * R, rng, shuffle_pages=True)
+    pools_np = [wl.random_kv_pool(shape, b.num_pages, rng) for _ in range(n)]
+    g = hp.GpuLayers(shape, layers, [[]] * n, b.T, R)
+    try:
+        d = hp.DevBatch(b, shape.dtype)
+        outs = []
+        for _ in range(2):
+            pools, hout = [g.new_pool(b.num_pages, fill=p) for p in pools_np], g.empty(b.T, shape.hidden)
+            ab.alora_forward_stack(g.ctx, ab.MODE_BASE, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, pools, d.bt, d.max_blocks,
+                                   b.num_pages, d.T, d.R, hout)
+            assert g.status() == 0
+            outs.append(hp.to_host(hout))
+        assert np.array_equal(outs[0].view(np.uint32), outs[1].view(np.uint32))
+        x = b.hidden.astype(np.float64)
+        for l in range(n):
+            kv = [oracle64.paged_gather(pools_np[l], b.block_tables[r], P[r], shape.n_kv_heads, shape.page_size, shape.head_dim) if P[r]
+                  else (None, None) for r in range(R)]
+            x, _ = oracle64.decoder_layer(x, layers[l], shape.Nq, shape.Nkv, shape.n_q_heads, shape.n_kv_heads, shape.head_dim, 1e-5,
+                                          b.positions, b.query_start_loc, b.activation_offsets, b.adapter_ids, [],
+                                          [k for k, _ in kv], [v for _, v in kv])
+        hp.assert_close(outs[0], x, 2e-2, "four layers, items claimed", block=shape.head_dim)
+    finally:
+        g.close()
+
+
 @pytest.mark.parametrize("n_req,each,kv_heads,slots", [(9, 12, 2, 3), (9, 12, 2, 5), (20, 30, 2, 3), (20, 30, 2, 5), (47, 17, 2, 5),
                                                        (30, 45, 2, 3), (11, 50, 1, 5)])
 def test_non_finite_adapter_values_stay_in_the_rows_that_use_them(oracle64, n_req, each, kv_heads, slots):
@@ -1057,7 +1093,7 @@ def test_projection_on_pairs_of_sms(oracle64, S):
     ids = ([1, 0, -1, 2, 1])[:R]
     b = wl.make_batch(shape, [20] * R, S, ids, rng, activation_offsets=[150, 20, 20, 220, 20][:R])
     assert (b.T + 127) // 128 in (26, 27, 29)
-    _check_projection(oracle64, shape, w, ads, b)
+    _check_projection(oracle64, shape, w, ads, b, on_pairs=True)
 
     def run():
         g = hp.GpuLayers(shape, [dict(wqkv=w)], [ads], b.T, b.R)
@@ -1114,6 +1150,7 @@ def test_projection_of_600_to_1024_rows_on_pairs_of_sms_loses_nothing_of_t(n_req
         y[:, s:s + 32] *= (1 - (np.repeat(np.array(ids), each) + 1))[:, None]
     g = hp.GpuLayers(shape, [dict(wqkv=w)], [ads], b.T, b.R)
     try:
+        assert ab.alora_selftest_pair_tile(g.ctx, 0, 0, b.T, b.R) > 0
         d = hp.DevBatch(b, shape.dtype)
         out = g.empty(b.T, shape.N)
         ab.alora_project_qkv(g.ctx, 0, ab.MODE_ALORA, d.hidden, d.positions, d.a_req, d.ids, d.qsl, d.seq_lens, d.T, d.R, out)
