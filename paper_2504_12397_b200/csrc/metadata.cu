@@ -817,13 +817,11 @@ int launch_metadata(alora_ctx *ctx, const BatchArgs &b, cudaStream_t s, int phas
             b.num_pages, ctx->d.page, ctx->cfg.max_adapters, b.T, b.R, b.mode, ctx->d_token_req, ctx->d_row_adapter,
             ctx->d_slot, ads, few, ctx->few_tiles, ctx->d_status) == cudaSuccess ? 1 : -1;
     }
-    // (one token a request: launch_attend_tc does not launch the kernel that reads this list)
-    AttnWork *const attn_items = b.all_small && ctx->max_split_items > 0 ? nullptr : ctx->d_attn_items;
     const cudaError_t e = launch_kernel(metadata_kernel, dim3(grid), dim3(threads), 0, s, true,
         b.positions, b.activation_offsets, b.adapter_ids, b.query_start_loc, b.seq_lens, b.block_tables,
         b.max_blocks, b.num_pages, ctx->d.page, ctx->cfg.max_adapters, b.T, b.R, b.mode, ctx->d_token_req,
         ctx->d_row_adapter, ctx->d_slot, ctx->max_pairs, ctx->d_pairs, ctx->d_pair_off, ctx->max_quads, ctx->d_quads, ctx->d_quad_off, ctx->d_counts, ctx->d_seg_scratch,
-        ctx->d.Hkv, ctx->attn_q_block, ctx->max_attn_items, attn_items, ctx->d_attn_off, ctx->d.G,
+        ctx->d.Hkv, ctx->attn_q_block, ctx->max_attn_items, ctx->d_attn_items, ctx->d_attn_off, ctx->d.G,
         ctx->sm_count, ctx->small_max_tokens, ctx->max_split_items, ctx->max_split_rows, ctx->d_split_items,
         ctx->d_req_scratch, ctx->d_group_done,
         ctx->d_attn_cta_start, ads, b.n_layers, phases, ctx->d_prefix_groups, ctx->d_status);
