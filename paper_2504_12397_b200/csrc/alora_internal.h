@@ -178,7 +178,7 @@ struct alora_ctx {
                                   // [8] attention items taken whole (the first ones), [9] key tiles of those,
                                   // [10], [11] next unclaimed projection item and blocks done, [12] few-row attention blocks done,
                                   // [13] an adapter with a non-finite B has been registered (kOddAdapters),
-                                  // [14] (quad, adapter) entries, [15], [16] tensor-core attention items claimed (even, odd layers)
+                                  // [15], [16] tensor-core attention items claimed (even, odd layers)
     int32_t *d_seg_scratch = nullptr;  // [14*max_requests+5] per-request values and merged row runs of the current batch
     int32_t *d_t_ready = nullptr;      // [max_pairs] per pair: epilogue warps that have published t (zero between launches)
     int32_t *d_iota = nullptr;         // 0..max_requests: query_start_loc of a decode batch

@@ -898,7 +898,6 @@ int launch_attend_tc(alora_ctx *ctx, const void *qkv, const BatchArgs &b, const 
 
 static int launch_attend_long(alora_ctx *ctx, const void *qkv, const BatchArgs &b, const void *pool, void *out,
                               cudaStream_t s) {
-    const int n_small = 0;
     const Dims &d = ctx->d;
     const bool page_ok = d.page >= 8 && d.page <= 128 && (d.page & (d.page - 1)) == 0;
     if ((d.hd != 64 && d.hd != 128) || 128 % d.G != 0 || !page_ok) return -1;
@@ -970,11 +969,11 @@ static int launch_attend_long(alora_ctx *ctx, const void *qkv, const BatchArgs &
     else le = hi ? launch_kernel(attn_tcgen05_kernel<128, false>, g3, b3, AttnSmem<128>::kTotal, s, true, tmQ, tmKV, a)
                  : launch_kernel(attn_tcgen05_kernel<64, false>, g3, b3, AttnSmem<64>::kTotal, s, true, tmQ, tmKV, a);
     if (le != cudaSuccess) return -1;
-    if (!runs) return 1 + n_small;
+    if (!runs) return 1;
     const cudaError_t me = hi ? launch_kernel(attn_merge_kernel<128>, dim3(2 * (grid - 1), 4), dim3(512), 0, s, true, a)
                               : launch_kernel(attn_merge_kernel<64>, dim3(2 * (grid - 1), 4), dim3(512), 0, s, true, a);
     if (me != cudaSuccess) return -1;
-    return 2 + n_small;
+    return 2;
 }
 
 }  // namespace alora

@@ -104,7 +104,7 @@ __device__ __forceinline__ void metadata_pairs(const int32_t *__restrict__ a_req
     const int n_tiles = (T + tile_rows - 1) / tile_rows;
     if (!any) {   // base model only
         for (int i = threadIdx.x; i <= n_tiles; i += blockDim.x) pair_off[i] = 0;
-        if (threadIdx.x == 0) *n_pairs = 0;
+        if (threadIdx.x == 0 && n_pairs != nullptr) *n_pairs = 0;
         return;
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = (int)blockDim.x >> 5;
@@ -163,7 +163,7 @@ __device__ __forceinline__ void metadata_pairs(const int32_t *__restrict__ a_req
     if (threadIdx.x == 0) {
         if (carry > max_pairs) report(status, ALORA_ERR_CAPACITY);
         pair_off[n_tiles] = min(carry, max_pairs);
-        *n_pairs = min(carry, max_pairs);
+        if (n_pairs != nullptr) *n_pairs = min(carry, max_pairs);
     }
 }
 
@@ -736,7 +736,7 @@ metadata_kernel(const int32_t *__restrict__ positions, const int32_t *a_req, con
                        seg_scratch, adapters, n_layers, status);
         __syncthreads();  // a builder that follows in this block reuses the scratch
     } else if ((int)blockIdx.x == b_quads) {
-        metadata_pairs(a_req, adapter_ids, qsl, seq_lens, R, mode, max_adapters, T, kQuadRows, max_quads, quads, quad_off, counts + 14,
+        metadata_pairs(a_req, adapter_ids, qsl, seq_lens, R, mode, max_adapters, T, kQuadRows, max_quads, quads, quad_off, nullptr,
                        seg_scratch == smem_scratch ? smem_scratch : seg_scratch + 3 * R, nullptr, 0, status);
     }
     if ((int)blockIdx.x == b_attn && items != nullptr && block_tables != nullptr) {
