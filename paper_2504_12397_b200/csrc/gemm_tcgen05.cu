@@ -709,6 +709,7 @@ int launch_linear_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K,
 // Gate and up projection with SwiGLU in the epilogue, for the batches of the few-row kernel and of the pairs of SMs; 0: nothing
 // launched.  Not for few rows where the context has adapters on the MLP block: their expand step wants the rounded gate and up rows,
 // and a call in which none of them applies has to take the route of the others.
+// (So a stack call of few rows rounds gate and up before SwiGLU in such a context, and does not in one without these adapters.)
 int launch_glu_tc(alora_ctx *ctx, const void *x, const void *W, int T, int K, int N, void *y, cudaStream_t s, const LinearDelta *delta) {
     if (T == 0 || N % 16 != 0) return 0;
     if (delta == nullptr && few_cluster_rows(ctx, T) && few_cluster_route(ctx, T, 0, N, K, false, N, 0)) {

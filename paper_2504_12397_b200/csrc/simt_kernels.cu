@@ -229,7 +229,8 @@ __device__ __forceinline__ RowFacts row_facts(int t, const int32_t *__restrict__
 // for the tile's 32 columns, which lie in one of the q / k / v blocks (a column a lane).  Batch metadata, shrink and projection
 // as launches of their own are chains of two to four fetches each, one after the other: 16 tokens at hidden 256 took 17 us
 // until the projection was done, of 22 for the call; here the chains run side by side (call: 13 us).  t is formed again
-// by every column tile, so this is for few rows and short rows of x (simt_small_layer()).
+// by every column tile, so this is for few rows and short rows of x (simt_small_layer()).  80 registers at 768 threads, one block an
+// SM; 80 bytes are spilled around the batch facts.
 // ---------------------------------------------------------------------------------------------
 constexpr int kSmallVecs = 8;   // 16-byte vectors of x a lane holds: hidden <= 1024
 __global__ void __launch_bounds__(768)
