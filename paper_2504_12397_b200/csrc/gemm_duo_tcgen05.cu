@@ -598,7 +598,8 @@ gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                         }
                         if (kMode == kDuoGlu) {
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) v[e] = __float_as_uint(tc::silu_mul(__uint_as_float(v[e]), __uint_as_float(w[e])));
+                            for (int e = 0; e < 8; e += 2)
+                                tc::silu_mul2(reinterpret_cast<float &>(v[e]), reinterpret_cast<float &>(v[e + 1]), __uint_as_float(w[e]), __uint_as_float(w[e + 1]));
                         }
                         if (row_ok) put_own8(col, reinterpret_cast<float(&)[8]>(v));
                     }
@@ -671,7 +672,8 @@ gemm_duo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                     }
                     if (kMode == kDuoGlu) {
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(tc::silu_mul(__uint_as_float(v[e]), __uint_as_float(v[32 + e])));
+                        for (int e = 0; e < 32; e += 2)
+                            tc::silu_mul2(reinterpret_cast<float &>(v[e]), reinterpret_cast<float &>(v[e + 1]), __uint_as_float(v[32 + e]), __uint_as_float(v[33 + e]));
                     }
 #pragma unroll
                     for (int k = 0; k < kFirst; ++k) {

@@ -419,7 +419,8 @@ gemm_few_cluster_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
         for (int e = 0; e < 8; ++e) f[e] = part[((v * 8 + e) << a.rows_shift) + row];
         if (a.glu) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) f[e] = tc::silu_mul(f[e], part[((out_bn + v * 8 + e) << a.rows_shift) + row]);
+            for (int e = 0; e < 8; e += 2)
+                tc::silu_mul2(f[e], f[e + 1], part[((out_bn + v * 8 + e) << a.rows_shift) + row], part[((out_bn + v * 8 + e + 1) << a.rows_shift) + row]);
         }
         const int slot = n_present > 0 ? slot_s[row] : -1;
         if (slot >= 0) {   // only rows with an applied adapter add anything (a gated-off row never sees "+ 0")

@@ -308,6 +308,26 @@ __device__ __forceinline__ float silu_mul(float g, float u) {
     return g * q * u;
 }
 
+// The same of two gates and ups at once, in place of the gates, bit for bit: two values an instruction except for the exponential, the
+// reciprocal and the choice of m (signs so that none has to be turned: -m, -(1 + p) and its reciprocal).  A decode step of 40 requests
+// through four layers 676 us one by one, 674 in pairs.
+__device__ __forceinline__ void silu_mul2(float &g0, float &g1, float u0, float u1) {
+    auto both = [](float a, float b) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; };
+    auto mul = [](uint64_t a, uint64_t b) { uint64_t r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; };
+    auto add = [](uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; };
+    auto fma = [](uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; };
+    const float p0 = __expf(-fabsf(g0)), p1 = __expf(-fabsf(g1));
+    const uint64_t p = both(p0, p1), neg1 = both(-1.f, -1.f), nm = both(g0 < 0.f ? -p0 : -1.f, g1 < 0.f ? -p1 : -1.f);
+    float d0, d1;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(fma(p, neg1, neg1)));
+    asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(d0));
+    asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(d1));
+    const uint64_t nr = both(d0, d1);
+    uint64_t q = mul(nm, nr);
+    q = fma(fma(p, q, add(nm, q)), nr, q);
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(g0), "=f"(g1) : "l"(mul(mul(both(g0, g1), q), both(u0, u1))));
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t *>(&v);
